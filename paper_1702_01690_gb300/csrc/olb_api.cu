@@ -44,7 +44,7 @@ bool olb::tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int
 {
     static_assert(sizeof(TmaMap) == sizeof(CUtensorMap), "TmaMap must hold a CUtensorMap");
     const size_t elt = fp64 ? 8 : 4;
-    const unsigned hx = (unsigned)tx + 8, hy = (unsigned)ty + 6;
+    const unsigned hx = (unsigned)region_pitch(tx, fp64), hy = (unsigned)ty + 6;
     // the box's rows must be whole 16-byte units, and its x start x0 - 4
     // (x0 a multiple of tx) must sit on a 16-byte boundary for every tile
     if ((hx * elt) % 16 != 0 || ((size_t)tx * elt) % 16 != 0 || (4 * elt) % 16 != 0) return false;
@@ -364,15 +364,13 @@ static cudaError_t prepare_tile(olb_ctx *c)
     return cudaSuccess;
 }
 
-// Default shape, the fastest measured on a GB300 for each precision.  FP64:
-// 8 x 8 nodes with 4 velocity lanes (its faces of all 25 velocities fit in
-// shared memory, so a stage has one face pass and one barrier), except that
-// small grids take 7 x 8 tiles with 8 lanes when that lowers the most nodes
-// any SM has to advance (1024 x 8: 147 tiles of 56 nodes rather than 128 of
-// 64 on 152 SMs).  FP32 (compensated pairs, twice the staged bytes of plain
-// FP32): 8 x 8 nodes with 8 lanes on every grid (4096^2: 10.2 ms per stage
-// against 11.0 for 8 x 8 x 4, 14.0 for 16 x 8 x 2 and 14.2 for 32 x 16 x 1),
-// 4 lanes with learned weights.  olb_set_tile overrides.
+// Default shape, the fastest measured on a GB300 for each precision: 8 x 8
+// nodes with 5 velocity lanes (the faces of all 25 velocities fit in shared
+// memory, so a stage has one face pass and one barrier; FP64: the 320 strips of
+// the face pass are one per thread), except that small FP64 grids take 7 x 8
+// tiles with 8 lanes when that lowers the most nodes any SM has to advance
+// (1024 x 8: 147 tiles of 56 nodes rather than 128 of 64 on 152 SMs).  Learned
+// weights: 4 lanes.  olb_set_tile overrides.
 static void default_tile(olb_ctx *c)
 {
     int dev = 0, sms = 0;
@@ -385,8 +383,8 @@ static void default_tile(olb_ctx *c)
         return (long long)((c->geo.nx + TILE_X[k] - 1) / TILE_X[k]) * ((c->geo.ny + TILE_Y[k] - 1) / TILE_Y[k]);
     };
     auto most_nodes = [&](int k) { return (tiles(k) + sms - 1) / sms * TILE_X[k] * TILE_Y[k]; };
-    int k = fp64 || learned ? 0 : 7;
-    if (fp64 && !learned && most_nodes(narrow) < most_nodes(0)) k = narrow;
+    int k = learned ? 0 : 7;
+    if (fp64 && !learned && most_nodes(narrow) < most_nodes(k)) k = narrow;
     c->tx = TILE_X[k];
     c->ty = TILE_Y[k];
     c->kp = TILE_K[k];

@@ -74,10 +74,12 @@ template <typename real, int TX, int TY, int KP>
 struct FusedSmem {
     // LS: threads per velocity lane, the tile's nodes rounded up to whole
     // warps (so that every lane starts on a warp); NT threads in all
+    // HP: pitch of a staged row of populations (region_pitch)
     static constexpr int HX = TX + 8, HY = TY + 6, NN = TX * TY, LS = (NN + 31) / 32 * 32, NT = LS * KP;
+    static constexpr int HP = region_pitch(TX, sizeof(real) == 8);
     using fld = typename FieldT<real>::type;
-    real pop[NK][HY][HX];
-    PopLo<real, HY, HX> pl;
+    real pop[NK][HY][HP];
+    PopLo<real, HY, HP> pl;
     fld n[HY][HX];
     fld dp[HY][HX];
     real ux[TY][TX];
@@ -124,15 +126,15 @@ __device__ __forceinline__ real sel5(const real v[NQ], int k)
     return r;
 }
 
-// Face value of one upwind-ordered stencil: Jiang-Shu weights, or the
+// Face value of one upwind-ordered FP64 stencil: Jiang-Shu weights, or the
 // learned network's (parameters in shared memory) when LEARNED.
-template <typename real, bool LEARNED>
-__device__ __forceinline__ real face_value(const float *mlp, real v0, real v1, real v2, real v3, real v4)
+template <bool LEARNED>
+__device__ __forceinline__ double face_value(const float *mlp, double v0, double v1, double v2, double v3, double v4)
 {
     if constexpr (LEARNED)
-        return weno5_learned<real>(mlp, v0, v1, v2, v3, v4);
+        return weno5_learned(mlp, v0, v1, v2, v3, v4);
     else
-        return weno5(v0, v1, v2, v3, v4);
+        return weno5_face(v2, v1 - v0, v2 - v1, v3 - v2, v4 - v3);
 }
 
 // FP32 pairs: the correction c (face value minus the upwind node v2) of the
@@ -419,7 +421,7 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
                                            const StageFields<real> *fields = nullptr)
 {
     using S = FusedSmem<real, TX, TY, KP>;
-    constexpr int NT = S::NT, NN = S::NN, HX = S::HX, HY = S::HY;
+    constexpr int NT = S::NT, NN = S::NN, HX = S::HX, HY = S::HY, HP = S::HP;
 
     // thread = (tile node, velocity lane): KP velocities are advanced at once
     const int tid = threadIdx.x;
@@ -623,7 +625,7 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
             const real g1 = fma(real(6), a0, fma(real(-8), a1, real(3) * a2));
             if (c0 - dc >= 0 && c0 - dc < HX) sm.pop[k][tr + 3][c0 - dc] = g0;
             if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) sm.pop[k][tr + 3][c0 - 2 * dc] = g1;
-            wf = t.R[k1] * face_value<real, LEARNED>(mlp, a2, a1, a0, g0, g1);
+            wf = t.R[k1] * face_value<LEARNED>(mlp, a2, a1, a0, g0, g1);
         } else {
             // pairs: the ghosts 3a0 - 3a1 + a2 and 6a0 - 8a1 + 3a2 as a0 plus
             // combinations of the differences D1 = a0 - a1, D2 = a1 - a2, and
@@ -900,23 +902,23 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
                                  : face_corr<LEARNED>(mlp, pd(c + 5, c + 6), pd(c + 4, c + 5), pd(c + 3, c + 4), pd(c + 2, c + 3));
                 } else {
                     sm.fx[slot][r][c] =
-                        (k1 > 2) ? face_value<real, LEARNED>(mlp, row[c + 1], row[c + 2], row[c + 3], row[c + 4], row[c + 5])
-                                 : face_value<real, LEARNED>(mlp, row[c + 6], row[c + 5], row[c + 4], row[c + 3], row[c + 2]);
+                        (k1 > 2) ? face_value<LEARNED>(mlp, row[c + 1], row[c + 2], row[c + 3], row[c + 4], row[c + 5])
+                                 : face_value<LEARNED>(mlp, row[c + 6], row[c + 5], row[c + 4], row[c + 3], row[c + 2]);
                 }
             }
         } else if (x0 + c < g.nx && y0 + r <= g.ny) {
             // face at y = y0 + r: rows y0+r-3 .. y0+r+2 are rows r .. r+5
             const int cc4 = 4 + c;
-            const real(*P)[HX] = sm.pop[k];
+            const real(*P)[HP] = sm.pop[k];
             if constexpr (F32) {
-                const float(*Lo)[HX] = sm.pl.lo[k];
+                const float(*Lo)[HP] = sm.pl.lo[k];
                 auto pd = [&](int a_, int b_) { return pdiff(P[a_][cc4], Lo[a_][cc4], P[b_][cc4], Lo[b_][cc4]); };
                 sm.fy[slot][r][c] = (k2 > 2) ? face_corr<LEARNED>(mlp, pd(r + 1, r), pd(r + 2, r + 1), pd(r + 3, r + 2), pd(r + 4, r + 3))
                                              : face_corr<LEARNED>(mlp, pd(r + 4, r + 5), pd(r + 3, r + 4), pd(r + 2, r + 3), pd(r + 1, r + 2));
             } else {
-                sm.fy[slot][r][c] = (k2 > 2) ? face_value<real, LEARNED>(mlp, P[r][cc4], P[r + 1][cc4], P[r + 2][cc4],
+                sm.fy[slot][r][c] = (k2 > 2) ? face_value<LEARNED>(mlp, P[r][cc4], P[r + 1][cc4], P[r + 2][cc4],
                                                                         P[r + 3][cc4], P[r + 4][cc4])
-                                            : face_value<real, LEARNED>(mlp, P[r + 5][cc4], P[r + 4][cc4], P[r + 3][cc4],
+                                            : face_value<LEARNED>(mlp, P[r + 5][cc4], P[r + 4][cc4], P[r + 3][cc4],
                                                                         P[r + 2][cc4], P[r + 1][cc4]);
             }
         }
@@ -939,22 +941,16 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
             p0 = (k2 > 2) ? r : r + 5;
             step = (k2 > 2) ? 1 : -1;
         }
-        real d[4] = {0, 0, 0, 0}, v2 = 0;
+        real d[4] = {0, 0, 0, 0};
         if (valid) {
             const real *P = &sm.pop[k][0][0];
-            auto at = [&](int m) { return along_x ? (3 + r) * HX + p0 + m * step : (p0 + m * step) * HX + 4 + c; };
+            auto at = [&](int m) { return along_x ? (3 + r) * HP + p0 + m * step : (p0 + m * step) * HP + 4 + c; };
             if constexpr (F32) {
                 const float *Lo = &sm.pl.lo[k][0][0];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) d[m] = pdiff(P[at(m + 1)], Lo[at(m + 1)], P[at(m)], Lo[at(m)]);
-            } else {
-#pragma unroll
-                for (int m = 0; m < 4; ++m) d[m] = P[at(m + 1)] - P[at(m)];
-                v2 = P[at(2)];
             }
         }
-        // the guard in the population precision, the network's input and
-        // correction in FP32 from the rounded differences
         const bool acts = learned_guard<real>(d[0], d[1], d[2], d[3]);
         const float e[4] = {(float)d[0], (float)d[1], (float)d[2], (float)d[3]};
         float x[MLP_IN], w[MLP_OUT] = {0.0f, 0.0f, 0.0f};
@@ -962,13 +958,7 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
         // the whole warp skips the network when none of its stencils needs it
         if (__any_sync(0xffffffffu, acts)) mlp_weights_warp(mlp, x, w, mlp_sc);
         if (valid) {
-            real res;
-            if (acts) {
-                res = v2 + (real)learned_corr_from(w, e);
-            } else {
-                const real q12 = d[1] * d[1], q23 = d[2] * d[2];
-                res = weno5_core(d[0], d[1], d[2], d[3], q23, real(2.5) * q12, real(2.5) * q23, v2);
-            }
+            const real res = acts ? learned_corr_from(w, e) : weno5_corr(e[0], e[1], e[2], e[3]);
             if (along_x) sm.fx[slot][r][c] = res;
             else sm.fy[slot][r][c] = res;
         }
@@ -991,8 +981,8 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
         if constexpr (F32) {
             // flux difference = difference of the upwind nodes of the two
             // faces (a first difference of pairs) + difference of corrections
-            const float(*P)[HX] = sm.pop[k];
-            const float(*Lo)[HX] = sm.pl.lo[k];
+            const float(*P)[HP] = sm.pop[k];
+            const float(*Lo)[HP] = sm.pl.lo[k];
             float adv = 0.0f;
             if (k1 != 2) {
                 const int cu = k1 > 2 ? c : c + 1;
@@ -1128,17 +1118,41 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
                     const int rs = (f / TX) * SY, c = f - (f / TX) * TX;
                     // face at y = y0 + r reads rows r .. r+4 (xi_y > 0) or r+5 .. r+1
                     if (k % NQ > 2)
-                        weno5_strip_c<SY>(&sm.pop[k][rs][4 + c], &sm.pl.lo[k][rs][4 + c], HX, &sm.fy[k][rs][c], TX);
+                        weno5_strip_c<SY>(&sm.pop[k][rs][4 + c], &sm.pl.lo[k][rs][4 + c], HP, &sm.fy[k][rs][c], TX);
                     else
-                        weno5_strip_c<SY>(&sm.pop[k][rs + SY + 4][4 + c], &sm.pl.lo[k][rs + SY + 4][4 + c], -HX,
+                        weno5_strip_c<SY>(&sm.pop[k][rs + SY + 4][4 + c], &sm.pl.lo[k][rs + SY + 4][4 + c], -HP,
                                           &sm.fy[k][rs + SY - 1][c], -TX);
                 }
             }
             // (faces outside the grid are computed from staged values and never read)
+        } else if constexpr (Sf::ALL_FACES && !LEARNED) {
+            // FP64: a strip is a whole tile row (x faces of the 20 velocities
+            // with xi_x != 0) or column (y faces of the 20 with xi_y != 0), in
+            // the upwind direction: 1.5 first differences per node and axis, the
+            // only FP64 operations of a face besides the sum with its upwind
+            // node.  An 8 x 8 tile has 320 strips, one for each thread of the
+            // shape with five lanes.
+            for (int e = tid; e < 20 * (TY + TX); e += NT) {
+                if (e < 20 * TY) {
+                    const int kx = e / TY, r = e - kx * TY;
+                    const int k = kx < 2 * NQ ? kx : kx + NQ;
+                    const real *row = &sm.pop[k][3 + r][0];
+                    // one call for both directions: the code of a strip is long
+                    const bool up = k / NQ > 2;
+                    weno5_strip_ff<TX + 1>(row + (up ? 1 : TX + 6), up ? 1 : -1, &sm.fx[k][r][up ? 0 : TX], up ? 1 : -1);
+                } else {
+                    const int e2 = e - 20 * TY, ky = e2 / TX, c = e2 - ky * TX, q = ky & 3;
+                    const int k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
+                    const bool up = k % NQ > 2;
+                    weno5_strip_ff<TY + 1>(&sm.pop[k][up ? 0 : TY + 5][4 + c], up ? HP : -HP, &sm.fy[k][up ? 0 : TY][c],
+                                           up ? TX : -TX);
+                }
+            }
+            // (faces outside the grid are computed from staged values and never read)
         } else if constexpr (Sf::ALL_FACES) {
-            // every face of every velocity once, enumerated densely: the x faces
-            // of the 20 velocities with xi_x != 0 (k1 != 2), then the y faces of
-            // the 20 with xi_y != 0 (k2 != 2)
+            // learned weights: every face of every velocity once, enumerated
+            // densely: the x faces of the 20 velocities with xi_x != 0, then the
+            // y faces of the 20 with xi_y != 0
             for (int e = tid; e < 20 * (nfx + nfy); e += NT) {
                 if (e < 20 * nfx) {
                     const int kx = e / nfx, f = e - kx * nfx;

@@ -87,6 +87,11 @@ struct alignas(64) TmaArg {
     TmaMap map;
     int on;
 };
+// Pitch (elements) of a staged row of a tile's region, TX + 8 nodes wide: FP64
+// rows of even tiles get two more, so that the strips of the eight rows of a
+// tile start 4 banks apart (rows of TX + 8 doubles are whole multiples of the 32
+// banks or halves of it, and the strips of a warp would queue for two banks).
+__host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 8 + (fp64 && tx % 2 == 0 ? 2 : 0); }
 // Encode the map of buffer `base` for tile shape tx x ty (olb_api.cu); false
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);

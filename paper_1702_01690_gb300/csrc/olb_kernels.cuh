@@ -5,6 +5,7 @@
 // (double, or float stored as hi + lo pairs).
 #pragma once
 
+#include "olb_ff.cuh"
 #include "olb_internal.cuh"
 
 namespace olb {
@@ -67,20 +68,11 @@ __device__ __forceinline__ double recip_nr1(double d)
     return fma(r, fma(-d, r, 1.0), r);
 }
 
-// v0..v4 = f_{i-2} .. f_{i+2} in the upwind orientation; returns the WENO-5
-// interface value sum_q wbar_q Fhat^q (without p/m).
-//
-// In terms of the first differences d01 = v1 - v0, ..., d34 = v4 - v3, the
-// indicators of Eq. weno5_sigma (13/12 a_q^2 + 1/4 b_q^2, a_q and b_q linear
-// in two neighbouring differences) are positive-definite quadratic forms:
-//   12 sigma_1 / 16 = d01^2 - 11/4 d01 d12 + 5/2 d12^2
-//   12 sigma_2 / 16 = d12^2 + d23^2 - 5/4 d12 d23 = d12 (d12 - 5/4 d23) + d23^2
-//   12 sigma_3 / 16 = d34^2 - 11/4 d23 d34 + 5/2 d23^2
-// (the weights only depend on ratios of the sigma_q, so the common factor
-// 12/16 is dropped), and 6 (Fhat^q - v2) of Eq. weno5_flux are
-//   6 G_1 = 5 d12 - 2 d01,  6 G_2 = d12 + 2 d23,  6 G_3 = 4 d23 - d34.
-// A form vanishes exactly when both of its differences do (the case of
-// Table tab:weno).
+// Jiang-Shu value of an interface in FP64, for the stencils that the learned
+// weights leave to Jiang-Shu in FP64 contexts: a warp takes this beside the
+// network, which fills the FP32 pipe, so it stays on the FP64 pipe (as weno5_ff
+// it measured 50.6 ms against 43.8 ms for two steps of 1024^2).  Same forms as
+// weno5_ff (olb_ff.cuh).
 //
 // Weights: wbar_q is proportional to delta_q / sigma_q^2.  Multiplying every
 // term by 10 (sigma_1 sigma_2 sigma_3)^2 gives weights proportional to
@@ -90,11 +82,6 @@ __device__ __forceinline__ double recip_nr1(double d)
 // two or three vanish; those cases take Table tab:weno (the ideal weights of
 // the vanishing set).  If the products underflow without an exact zero the
 // min-scaled form delta_q (s/sigma_q)^2 is used instead.
-//
-// weno5_core takes the first differences, q23 = d23^2 and h12 = 2.5 d12^2,
-// h23 = 2.5 d23^2; weno5 (one face) and weno5_strip
-// (consecutive faces, carrying those values from face to face) both end in
-// it, with the same operations on the same operands, so they agree bit for bit.
 __device__ __forceinline__ double weno5_core(double d01, double d12, double d23, double d34, double q23, double h12,
                                              double h23, double v2)
 {
@@ -128,19 +115,26 @@ __device__ __forceinline__ double weno5_core(double d01, double d12, double d23,
     }
     return fma(fma(A1, G1, fma(A2, G2, A3 * G3)), recip_nr1(6.0 * den), v2);
 }
-__device__ __forceinline__ double weno5(double v0, double v1, double v2, double v3, double v4)
-{
-    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3;
-    const double q12 = d12 * d12, q23 = d23 * d23;
-    return weno5_core(d01, d12, d23, d34, q23, 2.5 * q12, 2.5 * q23, v2);
-}
-
-// FP32 form (same forms and candidates): the products of four squared
-// indicators underflow in single precision, so the weights are always the
-// min-scaled 10 delta_q (s/sigma_q)^2 (same normalised weights), with Table
-// tab:weno when an indicator vanishes.
-__device__ __forceinline__ float weno5_core(float d01, float d12, float d23, float d34, float q23, float h12, float h23,
-                                            float v2)
+// FP32 populations: the correction c of an interface value (the value minus
+// its upwind node v2, sum_q wbar_q (Fhat^q - v2)) from the first differences
+// d01 = v1 - v0, ..., d34 = v4 - v3 of the stencil v0..v4 = f_{i-2} .. f_{i+2} in
+// the upwind orientation.  (FP64 populations: weno5_ff in olb_ff.cuh.)
+//
+// The indicators of Eq. weno5_sigma (13/12 a_q^2 + 1/4 b_q^2, a_q and b_q linear
+// in two neighbouring differences) are positive-definite quadratic forms:
+//   12 sigma_1 / 16 = d01^2 - 11/4 d01 d12 + 5/2 d12^2
+//   12 sigma_2 / 16 = d12^2 + d23^2 - 5/4 d12 d23 = d12 (d12 - 5/4 d23) + d23^2
+//   12 sigma_3 / 16 = d34^2 - 11/4 d23 d34 + 5/2 d23^2
+// (the weights only depend on ratios of the sigma_q, so the common factor
+// 12/16 is dropped), and 6 (Fhat^q - v2) of Eq. weno5_flux are
+//   6 G_1 = 5 d12 - 2 d01,  6 G_2 = d12 + 2 d23,  6 G_3 = 4 d23 - d34.
+// A form vanishes exactly when both of its differences do (the case of
+// Table tab:weno).  The products of four squared indicators underflow in
+// single precision, so the weights are the min-scaled 10 delta_q (s/sigma_q)^2,
+// with Table tab:weno (the ideal weights of the vanishing set) when an
+// indicator vanishes.  q23 = d23^2, h12 = 2.5 d12^2, h23 = 2.5 d23^2: strips of
+// consecutive faces carry those values from face to face.
+__device__ __forceinline__ float weno5_core(float d01, float d12, float d23, float d34, float q23, float h12, float h23)
 {
     const float s1 = fmaf(d01, fmaf(-2.75f, d12, d01), h12);
     const float s2 = fmaf(d12, fmaf(-1.25f, d23, d12), q23);
@@ -160,42 +154,8 @@ __device__ __forceinline__ float weno5_core(float d01, float d12, float d23, flo
         w2 = (s2 == 0.0f) ? 6.0f : 0.0f;
         w3 = (s3 == 0.0f) ? 3.0f : 0.0f;
     }
-    return fmaf(fmaf(w1, G1, fmaf(w2, G2, w3 * G3)), __fdividef(1.0f, 6.0f * (w1 + w2 + w3)), v2);
+    return fmaf(fmaf(w1, G1, fmaf(w2, G2, w3 * G3)), __fdividef(1.0f, 6.0f * (w1 + w2 + w3)), 0.0f);
 }
-__device__ __forceinline__ float weno5(float v0, float v1, float v2, float v3, float v4)
-{
-    const float d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3;
-    const float q12 = d12 * d12, q23 = d23 * d23;
-    return weno5_core(d01, d12, d23, d34, q23, 2.5f * q12, 2.5f * q23, v2);
-}
-
-// S consecutive faces along a row or column, in the upwind direction: the
-// stencil v_0 .. v_4 of face j is p[(j + m) step], m = 0..4, and its value
-// goes to out[j ostep].  Neighbouring faces share three first differences
-// and one scaled square, which are carried instead of recomputed (4 fewer
-// operations per face after the first).
-template <int S, typename real>
-__device__ __forceinline__ void weno5_strip(const real *p, int step, real *out, int ostep)
-{
-    real v2 = p[2 * step], v3 = p[3 * step];
-    const real v1 = p[step];
-    real d01 = v1 - p[0], d12 = v2 - v1, d23 = v3 - v2;
-    real h12 = real(2.5) * (d12 * d12);
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-        const real v4 = p[(j + 4) * step];
-        const real d34 = v4 - v3;
-        const real q23 = d23 * d23, h23 = real(2.5) * q23;
-        out[j * ostep] = weno5_core(d01, d12, d23, d34, q23, h12, h23, v2);
-        d01 = d12;
-        d12 = d23;
-        d23 = d34;
-        h12 = h23;
-        v2 = v3;
-        v3 = v4;
-    }
-}
-
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ int wrap(int i, int n)
 {
@@ -350,12 +310,13 @@ __device__ __forceinline__ f2 pair_sum5(const float h[NQ], const float l[NQ])
 __device__ __forceinline__ float weno5_corr(float d01, float d12, float d23, float d34)
 {
     const float q12 = d12 * d12, q23 = d23 * d23;
-    return weno5_core(d01, d12, d23, d34, q23, 2.5f * q12, 2.5f * q23, 0.0f);
+    return weno5_core(d01, d12, d23, d34, q23, 2.5f * q12, 2.5f * q23);
 }
 
-// weno5_strip for pairs: the stencil of face j is (ph, pl)[(j + m) step],
-// m = 0..4, the corrections go to out[j ostep]; the first differences of the
-// pairs are carried from face to face.
+// S consecutive faces along a row or column, in the upwind direction: the
+// stencil of face j is (ph, pl)[(j + m) step], m = 0..4, the corrections go to
+// out[j ostep].  Neighbouring faces share three first differences of the pairs
+// and one scaled square, which are carried instead of recomputed.
 template <int S>
 __device__ __forceinline__ void weno5_strip_c(const float *ph, const float *pl, int step, float *out, int ostep)
 {
@@ -367,7 +328,7 @@ __device__ __forceinline__ void weno5_strip_c(const float *ph, const float *pl, 
     for (int j = 0; j < S; ++j) {
         const float d34 = pdiff(ph[(j + 4) * step], pl[(j + 4) * step], ph[(j + 3) * step], pl[(j + 3) * step]);
         const float q23 = d23 * d23, h23 = 2.5f * q23;
-        out[j * ostep] = weno5_core(d01, d12, d23, d34, q23, h12, h23, 0.0f);
+        out[j * ostep] = weno5_core(d01, d12, d23, d34, q23, h12, h23);
         d01 = d12;
         d12 = d23;
         d23 = d34;

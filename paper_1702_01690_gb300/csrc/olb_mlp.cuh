@@ -171,22 +171,21 @@ __device__ __forceinline__ float learned_corr_net(const float *__restrict__ th, 
 // where any smoothness indicator vanishes the Jiang-Shu weights with Table
 // tab:weno apply (constant ghost layers keep their exact flux), and so do
 // they where the stencil is smooth (min sigma_q >= MLP_GUARD max sigma_q);
-// otherwise v2 + sum_q w_q G_q with the network's weights.  The guard is
-// taken in the population precision; the network and the correction
+// otherwise v2 + sum_q w_q G_q with the network's weights.  FP64 populations: the guard is
+// taken in FP64; the network and the correction
 // sum_q w_q G_q run in FP32 (the weights carry FP32 error anyway), and the
-// correction is added to v2 in the population precision.
-template <typename real>
-__device__ __forceinline__ real weno5_learned(const float *__restrict__ th, real v0, real v1, real v2, real v3,
-                                              real v4)
+// correction is added to v2 in FP64.
+__device__ __forceinline__ double weno5_learned(const float *__restrict__ th, double v0, double v1, double v2, double v3,
+                                                double v4)
 {
-    const real d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3;
-    if (!learned_guard<real>(d01, d12, d23, d34)) {
-        // Jiang-Shu on the same differences (the operations of weno5)
-        const real q12 = d12 * d12, q23 = d23 * d23;
-        return weno5_core(d01, d12, d23, d34, q23, real(2.5) * q12, real(2.5) * q23, v2);
+    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3;
+    if (!learned_guard<double>(d01, d12, d23, d34)) {
+        // Jiang-Shu on the same differences
+        const double q12 = d12 * d12, q23 = d23 * d23;
+        return weno5_core(d01, d12, d23, d34, q23, 2.5 * q12, 2.5 * q23, v2);
     }
     const float e[4] = {(float)d01, (float)d12, (float)d23, (float)d34};
-    return v2 + (real)learned_corr_net(th, e);
+    return v2 + (double)learned_corr_net(th, e);
 }
 
 // The same for the compensated FP32 storage: the correction sum_q w_q G_q (the
