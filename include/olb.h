@@ -220,7 +220,8 @@ int olb_profile(olb_ctx *ctx, int nsteps, double *ms, int *launches);
  * (32,16,1), (8,8,8), (7,8,8), (8,8,5); olb_create picks one from the
  * grid size ((8,8,5), FP64: or (7,8,8) when that lowers the most nodes one SM
  * advances; (8,8,4) with learned weights).  With
- * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  olb_set_tile returns
+ * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  FP64 tiles of more than
+ * 64 nodes are advanced as 8 x 8 tiles by CTAs of their own.  olb_set_tile returns
  * OLB_ERR_ARG for any other shape; results do not depend on the shape.
  * Not part of the paper (a tuning knob). */
 int olb_set_tile(olb_ctx *ctx, int tx, int ty, int kp);

@@ -119,6 +119,25 @@ double host_g(const HostTables &t, int k, double u, double T)
     return s;
 }
 
+ff ff_of(double v)
+{
+    const float h = (float)v;
+    return {h, (float)(v - (double)h)};
+}
+
+StageK stage_constants(const Geo &g, StageCoef c)
+{
+    HostTables h;
+    host_tables(&h);
+    StageK k{};
+    k.cit = ff_of(c.cc * g.inv_tau);
+    k.ca = ff_of(c.ca);
+    k.kp = ff_of(c.cc * g.inv_ds / 5040.0);
+    k.kn = ff_of(c.cc * g.sigma * g.inv_ds3 / 2160.0);
+    for (int m = 0; m < 3; ++m) k.adv[m] = ff_of(c.cc * g.inv_ds * h.R[2 + m] / 6.0);
+    return k;
+}
+
 template <typename real>
 void fill_tab(Tab<real> *tab, const HostTables &h, const double Tw[2], const double uw[2])
 {
@@ -131,6 +150,15 @@ void fill_tab(Tab<real> *tab, const HostTables &h, const double Tw[2], const dou
             tab->wHe[k][q] = (real)h.wHe[k][q];
         }
     }
+    if constexpr (sizeof(real) == 8)
+        for (int m = 0; m < 3; ++m) {
+            const double *D = h.D[2 + m];
+            for (int q = 1; q < 3; ++q) {
+                tab->ff.E[m][q - 1] = ff_of(0.5 * (D[2 + q] - D[2 - q]));
+                if (m > 0) tab->ff.O[m - 1][q] = ff_of(0.5 * (D[2 + q] + D[2 - q]));
+            }
+            if (m > 0) tab->ff.O[m - 1][0] = ff_of(D[2]);
+        }
     for (int s = 0; s < 2; ++s) {
         double den = 0.0;
         for (int k1 = 0; k1 < NQ; ++k1)
@@ -358,9 +386,10 @@ static cudaError_t prepare_tile(olb_ctx *c)
     // TMA maps of the three buffers for this shape (tiles whose region lies
     // inside the grid then load it with one copy); without them every tile
     // takes the per-element loads
+    const Shape s = stage_shape(is_fp64(c), learned, c->tx, c->ty, c->kp);
     c->tma_ok = true;
     for (int k = 0; k < 3 && c->tma_ok; ++k)
-        c->tma_ok = tma_encode(&c->tma[k], c->f[k], is_fp64(c), c->geo, c->tx, c->ty);
+        c->tma_ok = tma_encode(&c->tma[k], c->f[k], is_fp64(c), c->geo, s.tx, s.ty);
     return cudaSuccess;
 }
 

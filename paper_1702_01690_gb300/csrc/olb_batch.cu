@@ -88,10 +88,11 @@ static cudaError_t batch_upload(olb_batch *b)
     const size_t rb = b_fp64(b) ? batch_run_bytes((double *)nullptr) : batch_run_bytes((float *)nullptr);
     std::vector<char> host(rb * b->count);
     std::vector<int> start(b->count + 1);
+    const Shape sh = stage_shape(b_fp64(b), false, b->tx, b->ty, b->kp);
     int acc = 0;
     for (int r = 0; r < b->count; ++r) {
         const Geo &g = b->geo[r];
-        const int ntx = (g.nx + b->tx - 1) / b->tx, nty = (g.ny + b->ty - 1) / b->ty;
+        const int ntx = (g.nx + sh.tx - 1) / sh.tx, nty = (g.ny + sh.ty - 1) / sh.ty;
         start[r] = acc;
         acc += ntx * nty;
         if (b_fp64(b))
@@ -108,7 +109,7 @@ static cudaError_t batch_upload(olb_batch *b)
     for (int k = 0; k < 3 && b->tma_ok; ++k)
         for (int r = 0; r < b->count && b->tma_ok; ++r)
             b->tma_ok = tma_encode(&maps[(size_t)k * b->count + r], (const char *)b->f[k] + b->off[r] * b->elt,
-                                   b_fp64(b), b->geo[r], b->tx, b->ty);
+                                   b_fp64(b), b->geo[r], sh.tx, sh.ty);
     cudaError_t e = cudaMemcpyAsync(b->runs, host.data(), host.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->tile_start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream);
@@ -140,7 +141,7 @@ static cudaError_t batch_stage(olb_batch *b, int st, cudaStream_t s)
     // src[st] is buffer st: its maps are row st of tmaps
     const TmaMap *maps = b->tma_ok ? b->tmaps + (size_t)st * b->count : nullptr;
     return launch_fused_batch(src[st], f0, dst[st], b->status, b->runs, b->tile_start, b->count, b->total_tiles,
-                              batch_tab(b, (real *)nullptr), coef[st], b->tx, b->ty, b->kp, b->fields, b->node_start,
+                              batch_tab(b, (real *)nullptr), coef[st], st, b->tx, b->ty, b->kp, b->fields, b->node_start,
                               b->total_nodes, maps, s);
 }
 
@@ -252,7 +253,7 @@ extern "C" int olb_batch_create(const olb_params *runs, int count, void *stream,
         b->max_nodes = std::max(b->max_nodes, (long long)g.nx * g.ny);
     }
     b->total_elems = acc;
-    // default shape: as for a single grid of the batch's total size
+    // default shape
     const bool fp64 = b_fp64(b);
     b->tx = 16;
     b->ty = 8;
@@ -514,6 +515,8 @@ extern "C" int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, in
             b->tx = TILE_X[q];
             b->ty = TILE_Y[q];
             b->kp = TILE_K[q];
+            const Shape sh = stage_shape(b_fp64(b), false, b->tx, b->ty, b->kp);
+            if (sh.tx != b->tx || sh.ty != b->ty) continue;  // advanced as another shape of the list
             if (batch_prepare(b) != cudaSuccess) {
                 cudaGetLastError();
                 continue;  // shape does not fit this precision

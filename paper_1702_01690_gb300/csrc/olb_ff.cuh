@@ -15,16 +15,15 @@
 // 2^-41 to 2^-42.6), so faces are more accurate than they were.
 //
 // Measured on a 4096^2 grid (one step, three stages): 236.1 ms with 30 FP64
-// operations a face, 106.6 ms with 1.3 differences and 3 more a face.
+// operations a face, 106.6 ms with 1.3 differences and 3 more a face (the force
+// and the node updates still in FP64; see olb_stage64.cuh for those).
 #pragma once
 
-#include <cuda_runtime.h>
+#include <type_traits>
+
+#include "olb_internal.cuh"
 
 namespace olb {
-
-struct ff {
-    float h, l;
-};
 
 // FP64 <-> bit patterns and the FP32 seed of a reciprocal.  (Host versions
 // exist so that the arithmetic can be checked on a CPU.)
@@ -91,45 +90,59 @@ __host__ __device__ __forceinline__ float rcp_seed(float v)
 }
 
 // ---------------------------------------------------------------- FP64 to float-float and back
-// The differences of one strip of faces are scaled by a common power of two,
-// which puts the largest at FF_EXP: squares and weights then stay in FP32's
-// range whatever the populations' units.  FfScale holds the scale of a strip
-// as the high words of FP64 numbers: emax the exponent field of its largest
-// difference, thr the smallest high word that is kept (a difference below
-// 2^-132 of the largest, or subnormal, counts as zero).
-constexpr int FF_EXP = 157;  // FP32 exponent field of the largest difference
+// Values are scaled by a power of two that puts the largest density of a tile
+// at 2^45: a tile's differences, from 2^-66 of it (an ulp of a population 2^-13
+// of it) to 2^18 times it, then have squares and weights inside FP32's range
+// whatever the populations' units.
+constexpr int FF_EXP = 127 + 45;  // FP32 exponent field of the largest density
 struct FfScale {
-    int emax, thr;
+    int off;     // added to an FP64 high word: exponent field e - emax + FF_EXP
+    int lo, hi;  // high words of the smallest value that is kept (2^-60 scaled: smaller ones
+                 // and zero become it, far below every rounding) and of the first beyond FP32
 };
-// top: the largest high word (sign cleared) of the strip's differences.
+// top: high word (sign cleared) of the largest density.
 __host__ __device__ __forceinline__ FfScale ff_scale(int top)
 {
-    const int emax = top & 0x7ff00000, thr = emax - (132 << 20);
-    return {emax, thr > 0x00100000 ? thr : 0x00100000};
+    const int off = (FF_EXP << 20) - (top & 0x7ff00000);
+    return {off, max((67 << 20) - off, 1 << 20), (255 << 20) - off};
 }
-// d scaled: h its leading 24 bits, l the next 23 (both truncated, so of one sign).
+// An int as a float (rounded).
+__host__ __device__ __forceinline__ float f32_of(int v)
+{
+#ifdef __CUDA_ARCH__
+    return __int2float_rn(v);
+#else
+    return (float)v;
+#endif
+}
+// d scaled: h is d rounded to 24 bits, l the rest (29 bits and a sign) rounded
+// to 24; not finite for infinities, NaN and what FP32 cannot hold.
+// (Zero becomes 2^-60: sigma_q then never vanishes, and nothing divides by
+// zero.  Where all differences of a sub-stencil vanish its weight takes over as
+// in Table tab:weno, and which of several vanishing ones does is no matter,
+// since their candidates agree.)
 __host__ __device__ __forceinline__ ff ff_split(double d, FfScale s)
 {
     const int hw = f64_hi(d);
-    const unsigned lw = (unsigned)f64_lo(d);
-    const bool keep = (hw & 0x7fffffff) >= s.thr;
-    // exponent field e - emax + FF_EXP, formed in the high word and moved to
-    // FP32's place by the shift (its upper bits and the sign fall off)
-    const unsigned e = (unsigned)(hw - s.emax + (FF_EXP << 20));
-    const unsigned b = ((e << 3) | (lw >> 29));
-    const unsigned h = (b & 0x7fffffffu) | ((unsigned)hw & 0x80000000u);
-    const unsigned base = (h & 0xff800000u) - (23u << 23);
-    const float l = f32_make(base | ((lw >> 6) & 0x007fffffu)) - f32_make(base);
-    return {keep ? f32_make(h) : 0.0f, keep ? l : 0.0f};
+    const unsigned lw = (unsigned)f64_lo(d), sign = (unsigned)hw & 0x80000000u;
+    const int a = min(max(hw & 0x7fffffff, s.lo), s.hi);
+    // half an ulp of h added to the magnitude
+    const unsigned lr = lw + 0x10000000u, e = (unsigned)(a + s.off) + (lr < lw ? 1u : 0u);
+    const unsigned h = ((e << 3) | (lr >> 29)) | sign;
+    // the last 29 bits, less 2^29 where h was rounded up; 8 of their units are 2^-49 of d's leading bit
+    const unsigned unit = ((unsigned)(a + s.off - (55 << 20)) << 3) & 0x7f800000u;
+    return {f32_make(h), f32_of((int)(lw << 3)) * f32_make(unit | sign)};
 }
-// The scaled float v as FP64, scale undone (zero below FP64's normal range).
-__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s)
+// A scaled float as FP64, scale undone (FP64's smallest normal number where it
+// would be less); l: a low part, whose high part carries an infinity or NaN.
+__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s, bool l)
 {
-    const unsigned b = f32_bits(v), a = b & 0x7fffffffu;
-    const int hw = (int)(a >> 3) + (s.emax - (FF_EXP << 20));
-    const bool zero = a < 0x00800000u || hw < 0x00100000;
-    return f64_make(zero ? 0 : (int)((unsigned)hw | (b & 0x80000000u)), zero ? 0 : (int)(b << 29));
+    const unsigned b = f32_bits(v);
+    const int a = (int)(b & 0x7fffffffu), least = (max(s.off, 0) + (1 << 20)) << 3;
+    const int m = max(a, least), hw = (m >> 3) - s.off;
+    return f64_make(!l && a >= 0x7f800000 ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
 }
+__host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s) { return ff_widen(v.h, s, false) + ff_widen(v.l, s, true); }
 
 // ---------------------------------------------------------------- float-float arithmetic
 // (error-free transformations of Dekker and Knuth; -fmad=false keeps every
@@ -203,13 +216,12 @@ __host__ __device__ __forceinline__ ff ff_inv2(ff s, float m)
 }
 
 // ---------------------------------------------------------------- WENO-5
-// 6 c of one face, c its correction (face value minus the upwind node v2),
-// from the first differences d0 .. d3 (v1 - v0, ..., v4 - v3): the candidates
-// of Eq. weno5_flux are 6 G_1 = 5 d1 - 2 d0, 6 G_2 = d1 + 2 d2,
-// 6 G_3 = 4 d2 - d3, so with the third differences t0 = d0 - 2 d1 + d2 and
-// t1 = d1 - 2 d2 + d3
-//   6 (G_1 - G_2) = -2 t0,  6 (G_3 - G_2) = -t1,
-//   6 c = d1 + 2 d2 - (2 W_1 t0 + W_3 t1) / (W_1 + W_2 + W_3),
+// The part of one face's value that is not linear, from the first differences
+// d0 .. d3 (v1 - v0, ..., v4 - v3) of its stencil.  The candidates of Eq.
+// weno5_flux are 6 (G_1 - v2) = 5 d1 - 2 d0, 6 (G_2 - v2) = d1 + 2 d2,
+// 6 (G_3 - v2) = 4 d2 - d3, so with the third differences t0 = d0 - 2 d1 + d2 and
+// t1 = d1 - 2 d2 + d3 the face value F has
+//   6 (F - v2) = d1 + 2 d2 - z,  z = (2 W_1 t0 + W_3 t1) / (W_1 + W_2 + W_3),
 // W_q = delta_q / sigma_q^2 (up to a factor) with the indicators of
 // Eq. weno5_sigma as the quadratic forms
 //   sigma_1 = d0^2 - 11/4 d0 d1 + 5/2 d1^2,  sigma_2 = d1^2 - 5/4 d1 d2 + d2^2,
@@ -218,25 +230,14 @@ __host__ __device__ __forceinline__ ff ff_inv2(ff s, float m)
 // x_j = d_j d_{j+1} are shared by the faces of a strip.  Weights are scaled by
 // the power of two m below the smallest indicator.  Where an indicator
 // vanishes (both its differences are zero) the weights are those of Table
-// tab:weno: the ideal weights of the vanishing set.
-__host__ __device__ __forceinline__ ff weno5_ff(ff d1, ff d2, ff q0, ff q1, ff q2, ff q3, ff x0, ff x1, ff x2, ff t0,
-                                                ff t1)
+// tab:weno (see ff_split).  Returns z.
+__host__ __device__ __forceinline__ ff weno5_ff(ff q0, ff q1, ff q2, ff q3, ff x0, ff x1, ff x2, ff t0, ff t1)
 {
     const ff s1 = ff_form(q0, 2.5f, q1, 2.75f, x0);
     const ff s2 = ff_form(q1, 1.0f, q2, 1.25f, x1);
     const ff s3 = ff_form(q3, 2.5f, q2, 2.75f, x2);
-    const float lo = fminf(s1.h, fminf(s2.h, s3.h));
-    ff w1, w2, w3;  // (m / sigma_q)^2
-    if (lo > 0.0f) {
-        const float m = f32_make(f32_bits(lo) & 0x7f800000u);
-        w1 = ff_inv2(s1, m);
-        w2 = ff_inv2(s2, m);
-        w3 = ff_inv2(s3, m);
-    } else {
-        w1 = {s1.h == 0.0f ? 1.0f : 0.0f, 0.0f};
-        w2 = {s2.h == 0.0f ? 1.0f : 0.0f, 0.0f};
-        w3 = {s3.h == 0.0f ? 1.0f : 0.0f, 0.0f};
-    }
+    const float m = f32_make(f32_bits(fminf(s1.h, fminf(s2.h, s3.h))) & 0x7f800000u);
+    const ff w1 = ff_inv2(s1, m), w2 = ff_inv2(s2, m), w3 = ff_inv2(s3, m);  // (m / sigma_q)^2
     // weights 1 : 6 : 3 times w (delta_q times 10)
     ff den = {w1.h, fmaf(3.0f, w3.l, fmaf(6.0f, w2.l, w1.l))};
     ff_acck(den, 6.0f, w2.h);
@@ -247,70 +248,86 @@ __host__ __device__ __forceinline__ ff weno5_ff(ff d1, ff d2, ff q0, ff q1, ff q
     ff_acc(num, b3);
     // num / den: quotient of the leading parts and its remainder
     const float r = rcp_seed(den.h), z = num.h * r;
-    const float zl = fmaf(-z, den.l, fmaf(-z, den.h, num.h) + num.l) * r;
-    ff c = {d1.h, fmaf(2.0f, d2.l, d1.l) - zl};
-    ff_acck(c, 2.0f, d2.h);
-    ff_acc(c, -z);
-    return ff_norm(c);
+    return {z, (fmaf(-z, den.l, fmaf(-z, den.h, num.h)) + num.l) * r};
 }
 
-// The face value v2 + c from a scaled 6 c.
-__host__ __device__ __forceinline__ double weno5_value(double v2, ff c6, FfScale s)
+// The flux difference across a node, in the upwind direction and times 6: the
+// value of the face ahead minus that of the face behind, whose non-linear parts
+// are z1 and z0.  With v the node, db = v - (node behind), d = the difference
+// before db's and da = (node ahead) - v, the linear parts add up to
+// 2 da + 5 db - dbb.
+__host__ __device__ __forceinline__ ff weno5_flux6(ff dbb, ff db, ff da, ff z0, ff z1)
 {
-    return fma(1.0 / 6.0, ff_widen(c6.h, s) + ff_widen(c6.l, s), v2);
+    const float b5 = 5.0f * db.h;
+    ff s = {2.0f * da.h, fmaf(2.0f, da.l, fmaf(5.0f, db.l, fmaf(5.0f, db.h, -b5))) - dbb.l + (z0.l - z1.l)};
+    ff_acc(s, b5);
+    ff_acc(s, -dbb.h);
+    ff_acc(s, z0.h);
+    ff_acc(s, -z1.h);
+    return ff_norm(s);
 }
 
-// The value of one face from its upwind node and first differences.
-__host__ __device__ __forceinline__ double weno5_face(double v2, double d0, double d1, double d2, double d3)
+// The value of one face from its upwind node and first differences, in FP64.
+__host__ __device__ __forceinline__ double weno5_face(double v2, double d0, double d1, double d2, double d3, FfScale s)
 {
-    const int a0 = f64_hi(d0) & 0x7fffffff, a1 = f64_hi(d1) & 0x7fffffff, a2 = f64_hi(d2) & 0x7fffffff,
-              a3 = f64_hi(d3) & 0x7fffffff;
-    const int top = max(max(a0, a1), max(a2, a3));
-    if (top >= 0x7ff00000) return f64_make(0x7ff80000, 0);  // an infinity or NaN among the differences
-    const FfScale s = ff_scale(top);
     const ff f0 = ff_split(d0, s), f1 = ff_split(d1, s), f2 = ff_split(d2, s), f3 = ff_split(d3, s);
-    const ff c = weno5_ff(f1, f2, ff_sqr(f0), ff_sqr(f1), ff_sqr(f2), ff_sqr(f3), ff_mul(f0, f1), ff_mul(f1, f2),
+    const ff z = weno5_ff(ff_sqr(f0), ff_sqr(f1), ff_sqr(f2), ff_sqr(f3), ff_mul(f0, f1), ff_mul(f1, f2),
                           ff_mul(f2, f3), ff_diff2(f0, f1, f2), ff_diff2(f1, f2, f3));
-    return weno5_value(v2, c, s);
+    ff c = {f1.h, fmaf(2.0f, f2.l, f1.l) - z.l};
+    ff_acc(c, 2.0f * f2.h);
+    ff_acc(c, -z.h);
+    return fma(1.0 / 6.0, ff_widen(c, s), v2);
 }
 
-// S consecutive faces along a row or column, in the upwind direction: the
-// stencil v_0 .. v_4 of face j is p[(j + m) step], m = 0..4, and its value goes
-// to out[j ostep].  Differences, their squares and products and the third
-// differences are formed once per strip; every face has the operations of
-// weno5_face on the same operands (up to the common power of two), so that
-// strips of any length agree bit for bit.
-template <int S>
-__device__ __forceinline__ void weno5_strip_ff(const double *p, int step, double *out, int ostep)
+// A row or column of N nodes in the upwind direction: node i is p[(i + 3) step]
+// (three nodes behind the row and two ahead of it are read), and the flux
+// difference across it (weno5_flux6) goes to out[i ostep].  Differences, their
+// squares and products and the third differences are formed once for the row.
+// Z: gives the non-linear part of face j instead of the Jiang-Shu weights.
+// The loop over the faces is unrolled by three: unrolled whole, a row is some
+// 2000 instructions and the warps waited for the instruction cache.
+struct NoFaces {};
+template <int N, typename Z = NoFaces>
+__device__ __forceinline__ void weno5_row(const double *p, int step, ff *out, int ostep, FfScale s, Z given = {})
 {
-    double v[S + 4], d[S + 3];
-    int top = 0;
-    v[0] = p[0];
-#pragma unroll
-    for (int j = 0; j < S + 3; ++j) {
-        v[j + 1] = p[(j + 1) * step];
-        d[j] = v[j + 1] - v[j];
-        top = max(top, f64_hi(d[j]) & 0x7fffffff);
+    constexpr bool JS = std::is_same<Z, NoFaces>::value;
+    double v = p[0];
+    auto next = [&] {
+        p += step;
+        const double b = *p;
+        const ff d = ff_split(b - v, s);
+        v = b;
+        return d;
+    };
+    ff f0 = next(), f1 = next(), f2 = next();
+    ff q0, q1, q2, x0, x1, t0, z0 = {0.0f, 0.0f};
+    if constexpr (JS) {
+        q0 = ff_sqr(f0);
+        q1 = ff_sqr(f1);
+        q2 = ff_sqr(f2);
+        x0 = ff_mul(f0, f1);
+        x1 = ff_mul(f1, f2);
+        t0 = ff_diff2(f0, f1, f2);
     }
-    if (top >= 0x7ff00000) {  // an infinity or NaN among the differences
-#pragma unroll
-        for (int j = 0; j < S; ++j) out[j * ostep] = weno5_face(v[j + 2], d[j], d[j + 1], d[j + 2], d[j + 3]);
-        return;
-    }
-    const FfScale s = ff_scale(top);
-    ff f0 = ff_split(d[0], s), f1 = ff_split(d[1], s), f2 = ff_split(d[2], s);
-    ff q0 = ff_sqr(f0), q1 = ff_sqr(f1), q2 = ff_sqr(f2);
-    ff x0 = ff_mul(f0, f1), x1 = ff_mul(f1, f2), t0 = ff_diff2(f0, f1, f2);
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-        const ff f3 = ff_split(d[j + 3], s);
-        const ff q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);
-        const ff c = weno5_ff(f1, f2, q0, q1, q2, q3, x0, x1, x2, t0, t1);
-        out[j * ostep] = weno5_value(v[j + 2], c, s);
+#pragma unroll 3
+    for (int j = 0; j <= N; ++j) {
+        const ff f3 = next();
+        ff z1;
+        if constexpr (JS) {
+            const ff q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);
+            z1 = weno5_ff(q0, q1, q2, q3, x0, x1, x2, t0, t1);
+            q0 = q1; q1 = q2; q2 = q3;
+            x0 = x1; x1 = x2;
+            t0 = t1;
+        } else {
+            z1 = given(j);
+        }
+        if (j > 0) {
+            *out = weno5_flux6(f0, f1, f2, z0, z1);
+            out += ostep;
+        }
+        z0 = z1;
         f0 = f1; f1 = f2; f2 = f3;
-        q0 = q1; q1 = q2; q2 = q3;
-        x0 = x1; x1 = x2;
-        t0 = t1;
     }
 }
 

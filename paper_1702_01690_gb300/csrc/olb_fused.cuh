@@ -33,6 +33,7 @@
 #pragma once
 
 #include "olb_mlp.cuh"
+#include "olb_stage64.cuh"
 
 namespace olb {
 
@@ -61,58 +62,60 @@ __device__ __forceinline__ float field_diff(float2 a, float2 b) { return (a.x - 
 __device__ __forceinline__ double field_val(double a) { return a; }
 __device__ __forceinline__ float field_val(float2 a) { return a.x + a.y; }
 
-// lo parts of the staged populations (FP32 only; FP64 has none)
-template <typename real, int HY, int HX>
-struct PopLo {
-    real lo[NK][HY][HX];
-};
-template <int HY, int HX>
-struct PopLo<double, HY, HX> {
-};
-
-template <typename real, int TX, int TY, int KP>
-struct FusedSmem {
+// Shared memory of an FP32 tile (FP64: Smem64 in olb_stage64.cuh).
+template <int TX, int TY, int KP>
+struct Smem32 {
     // LS: threads per velocity lane, the tile's nodes rounded up to whole
-    // warps (so that every lane starts on a warp); NT threads in all
+    // warps (so that every lane starts on a warp); NT threads in all;
     // HP: pitch of a staged row of populations (region_pitch)
     static constexpr int HX = TX + 8, HY = TY + 6, NN = TX * TY, LS = (NN + 31) / 32 * 32, NT = LS * KP;
-    static constexpr int HP = region_pitch(TX, sizeof(real) == 8);
-    using fld = typename FieldT<real>::type;
-    real pop[NK][HY][HP];
-    PopLo<real, HY, HP> pl;
+    static constexpr int HP = region_pitch(TX, false);
+    using fld = FieldT<float>::type;
+    float pop[NK][HY][HP];
+    struct {
+        float lo[NK][HY][HP];  // lo parts of the staged populations
+    } pl;
     fld n[HY][HX];
     fld dp[HY][HX];
-    real ux[TY][TX];
-    real uy[TY][TX];
-    fld T[TY][TX];  // FP32: hi + lo pair
-    // FP32: e = sum |p|^2 f at the tile nodes as a double-float pair (the
-    // target energy of the equilibrium's correction); unused in FP64
-    fld eng[sizeof(real) == 4 ? TY : 1][sizeof(real) == 4 ? TX : 1];
+    float ux[TY][TX];
+    float uy[TY][TX];
+    fld T[TY][TX];    // hi + lo pair
+    // e = sum |p|^2 f at the tile nodes as a double-float pair (the target
+    // energy of the equilibrium's correction)
+    fld eng[TY][TX];
     // per tile node, shared by the KP velocity lanes (with one lane they stay
     // in registers): the stencil sums of grad(Delta p) and grad(Laplacian n),
-    // inv_ds / n, E_q = (c/tau) n g_q(u_x, T) and g_q(u_y, T) (FP32: the
-    // even and odd parts n ge_q(u_x, T), n go_q(u_x, T), ge_q(u_y, T),
-    // go_q(u_y, T) instead), and, on tiles that keep every face, G_x = c F_x
-    // and G_y in L_G, L_G + 1
-    static constexpr int NEQ = sizeof(real) == 8 ? 2 : 4;  // equilibrium factor sets
+    // inv_ds / n, the even and odd equilibrium parts n ge_q(u_x, T),
+    // n go_q(u_x, T), ge_q(u_y, T), go_q(u_y, T), and, on tiles that keep
+    // every face, G_x = c F_x and G_y in L_G, L_G + 1, then the correction
+    static constexpr int NEQ = 4;  // equilibrium factor sets
     static constexpr int L_DDX = 0, L_DDY = 1, L_LDX = 2, L_LDY = 3, L_DN = 4, L_E = 5, L_GY = 5 + NQ,
                          L_OX = 5 + 2 * NQ, L_OY = 5 + 3 * NQ, L_G = 5 + NEQ * NQ,
-                         L_CA = 7 + NEQ * NQ, L_CB = 8 + NEQ * NQ, L_CC = 9 + NEQ * NQ;  // FP32: the correction
-    real loc[KP > 1 ? 7 + NEQ * NQ + (sizeof(real) == 4 ? 3 : 0) : 1][KP > 1 ? NN : 1];
+                         L_CA = 7 + NEQ * NQ, L_CB = 8 + NEQ * NQ, L_CC = 9 + NEQ * NQ;
+    float loc[KP > 1 ? 10 + NEQ * NQ : 1][KP > 1 ? NN : 1];
     // WENO-5 face values.  Small tiles (at most 64 nodes) hold the faces of
     // all 25 velocities, so one pass computes them all and the node updates
     // follow without further barriers; larger tiles hold KP velocities'.
     static constexpr bool ALL_FACES = TX * TY <= 64;
     static constexpr int KF = ALL_FACES ? NK : KP;
     union {
-        real fx[KF][TY][TX + 1];
+        float fx[KF][TY][TX + 1];
         // wall density n_w of each tile row at the left and right diffuse wall
         // (Eq. nw): written and read between the moments and the force,
         // before any face value is stored
-        real wnw[2][TY];
+        float wnw[2][TY];
     };
-    real fy[KF][TY + 1][TX];
+    float fy[KF][TY + 1][TX];
     unsigned long long mbar;  // completion barrier of the TMA copy of phase 1
+};
+
+template <typename real, int TX, int TY, int KP, bool LEARNED>
+struct StageSmem {
+    using type = Smem32<TX, TY, KP>;
+};
+template <int TX, int TY, int KP, bool LEARNED>
+struct StageSmem<double, TX, TY, KP, LEARNED> {
+    using type = Smem64<TX, TY, KP, LEARNED>;
 };
 
 template <typename real>
@@ -132,9 +135,13 @@ template <bool LEARNED>
 __device__ __forceinline__ double face_value(const float *mlp, double v0, double v1, double v2, double v3, double v4)
 {
     if constexpr (LEARNED)
-        return weno5_learned(mlp, v0, v1, v2, v3, v4);
+        return v2 + weno5_learned_corr64(mlp, v1 - v0, v2 - v1, v3 - v2, v4 - v3);
     else
-        return weno5_face(v2, v1 - v0, v2 - v1, v3 - v2, v4 - v3);
+    {
+        auto high = [](double v) { return __double2hiint(v) & 0x7fffffff; };
+        const FfScale s = ff_scale(max(max(max(high(v0), high(v1)), max(high(v3), high(v4))), high(v2)));
+        return weno5_face(v2, v1 - v0, v2 - v1, v3 - v2, v4 - v3, s);
+    }
 }
 
 // FP32 pairs: the correction c (face value minus the upwind node v2) of the
@@ -357,7 +364,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
 
 // Phase 1 for a tile whose staged region lies inside the grid: one TMA copy
 // of the box (HX, HY, planes) at (gx0, gy0, 0) of the tensor map into the
-// staging arrays (pop, then the lo planes in FP32, contiguous in FusedSmem in
+// staging arrays (pop, then the lo planes in FP32, contiguous in the tile's shared memory in
 // the box's order), completion tracked by an mbarrier.  tma_issue starts the
 // copy (all threads call it; it synchronises); tma_finish waits for it with
 // the bounded wait.  If the wait runs out, bit 1 of the status word is set,
@@ -365,10 +372,10 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
 // caller leaves the tile untouched and the CTA stops.  After a completed copy
 // the barrier is invalidated, so that a CTA that stages several tiles
 // initialises it afresh for each.
-template <typename real, int TX, int TY, int KP>
-__device__ __forceinline__ void tma_issue(FusedSmem<real, TX, TY, KP> &sm, const TmaMap *tmap, int gx0, int gy0)
+template <typename Smem>
+__device__ __forceinline__ void tma_issue(Smem &sm, const TmaMap *tmap, int gx0, int gy0)
 {
-    constexpr unsigned bytes = sizeof(sm.pop) + (sizeof(real) == 4 ? sizeof(sm.pop) : 0);
+    constexpr unsigned bytes = sizeof(sm.pop) * (sizeof(sm.pop[0][0][0]) == 4 ? 2 : 1);  // FP32: the lo planes too
     const unsigned mbar = (unsigned)__cvta_generic_to_shared(&sm.mbar);
     const unsigned dst = (unsigned)__cvta_generic_to_shared(&sm.pop[0][0][0]);
     if (threadIdx.x == 0) {
@@ -384,8 +391,8 @@ __device__ __forceinline__ void tma_issue(FusedSmem<real, TX, TY, KP> &sm, const
     }
     __syncthreads();  // the barrier is initialised before anyone waits on it
 }
-template <typename real, int TX, int TY, int KP>
-__device__ __forceinline__ bool tma_finish(FusedSmem<real, TX, TY, KP> &sm, int *status)
+template <typename Smem>
+__device__ __forceinline__ bool tma_finish(Smem &sm, int *status)
 {
     const unsigned mbar = (unsigned)__cvta_generic_to_shared(&sm.mbar);
     const bool ok = mbar_wait(mbar, 0);
@@ -396,6 +403,468 @@ __device__ __forceinline__ bool tma_finish(FusedSmem<real, TX, TY, KP> &sm, int 
     }
     // every thread has passed its wait (the barrier above)
     if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(mbar) : "memory");
+    return true;
+}
+
+// ---------------------------------------------------------------- force and update of an FP32 tile
+// Phases 4 and 5 for FP32 populations (FP64: advance64 in olb_stage64.cuh), same
+// contract.
+template <int TX, int TY, int KP, bool LEARNED, typename Wait>
+__device__ __forceinline__ bool advance32(Smem32<TX, TY, KP> &sm, const float *fn, float *out, const Geo &g,
+                                          const Tab<float> &t, int x0, int y0, float ca, float cb, float cc, float ca_lo,
+                                          float cb_lo, const float *mlp, Wait wait)
+{
+    using real = float;
+    using S = Smem32<TX, TY, KP>;
+    constexpr int NT = S::NT, NN = S::NN, HP = S::HP;
+    const int tid = threadIdx.x;
+    const int node = tid % S::LS, lane_k = tid / S::LS;
+    const int tx = node % TX, ty = node / TX;
+    const bool active = (node < NN) && (x0 + tx < g.nx) && (y0 + ty < g.ny);
+
+    // ---- 4. force and equilibrium factors at the tile nodes.  The four
+    // stencil sums and the two factor sets are split over the velocity lanes
+    // (KP = 4: ddx | ddy | ldx, g(u_x) | ldy, g(u_y); KP = 2: x | y parts).
+    constexpr int cy = 3, cx = 4;
+    auto grad_sum = [&](bool along_x) {
+        real acc = 0;
+#pragma unroll
+        for (int l = 1; l <= 3; ++l)
+#pragma unroll
+            for (int m = -3; m <= 3; ++m) {
+                const int am = m < 0 ? -m : m;
+                if (grad_w(l, am) != 0.0) {
+                    const real w = real(l * grad_w(l, am));
+                    acc = along_x ? fma(w, field_diff(sm.dp[ty + cy + m][tx + cx + l], sm.dp[ty + cy + m][tx + cx - l]), acc)
+                                  : fma(w, field_diff(sm.dp[ty + cy + l][tx + cx + m], sm.dp[ty + cy - l][tx + cx + m]), acc);
+                }
+            }
+        return acc;
+    };
+    auto glap_sum = [&](bool along_x) {
+        real acc = 0;
+        {
+            // the stencil cancels its O(ds) terms down to O(ds^3) (a
+            // factor ~1/(ds k)^2 on fine grids), so the weighted differences
+            // are summed in double-float arithmetic with double-float weights
+            // (exact products of the hi parts, TwoSum accumulation): the sum
+            // keeps FP32 accuracy of itself, not of its terms
+            f2 sum{0.0f, 0.0f};
+#pragma unroll
+            for (int l = 1; l <= 3; ++l)
+#pragma unroll
+                for (int m = -3; m <= 3; ++m) {
+                    const int am = m < 0 ? -m : m;
+                    if (glap_c(am, l) != 0.0) {
+                        const float wh = (float)glap_c(am, l);
+                        const float wl = (float)(glap_c(am, l) - (double)(float)glap_c(am, l));
+                        const float2 a = along_x ? sm.n[ty + cy + m][tx + cx + l] : sm.n[ty + cy + l][tx + cx + m];
+                        const float2 b = along_x ? sm.n[ty + cy + m][tx + cx - l] : sm.n[ty + cy - l][tx + cx + m];
+                        const f2 dh = two_sum(a.x, -b.x);
+                        const float dl = dh.lo + (a.y - b.y);
+                        const float p = wh * dh.hi;
+                        const float e = fmaf(wh, dh.hi, -p);
+                        const float tl = fmaf(wh, dl, fmaf(wl, dh.hi, e));
+                        const f2 t2 = two_sum(sum.hi, p);
+                        sum = f2{t2.hi, t2.lo + (sum.lo + tl)};
+                    }
+                }
+            acc = sum.hi + sum.lo;
+        }
+        return acc;
+    };
+    // With c the stage's coefficient of dt L (Eq. rk3), the node update below
+    // needs per node G = c F and n ge_q(u_x, T), n go_q(u_x, T), ge_q(u_y, T),
+    // go_q(u_y, T), the even and odd parts of the factors, in E, Ox, gy, Oy.
+    const real sg3 = real(g.sigma) * real(g.inv_ds3);
+    const real cit = cc * real(g.inv_tau);
+    real Gx = 0, Gy = 0, E[NQ], gy[NQ], Ox[NQ], Oy[NQ];
+    real qa = 0, qb = 0, qc = 0;  // alpha, beta, gamma of the equilibrium's correction (eq_correction)
+    // equilibrium factor sets of the node at (tx_, ty_): x (scaled by n) into
+    // ex, ox and y into ey, oy
+    auto eq_sets = [&](bool x_set, real *a, real *b) {
+        if (x_set) {
+            eq_factors_split(t, sm.ux[ty][tx], sm.T[ty][tx], a, b);
+            const real nn = sm.n[ty + 3][tx + 4].x;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                a[q] = nn * a[q];
+                b[q] = nn * b[q];
+            }
+        } else {
+            eq_factors_split(t, sm.uy[ty][tx], sm.T[ty][tx], a, b);
+        }
+    };
+    if constexpr (KP == 1) {
+        if (active) {
+            const real ddx = grad_sum(true), ddy = grad_sum(false);
+            const real ldx = glap_sum(true), ldy = glap_sum(false);
+            const real nn = field_val(sm.n[ty + cy][tx + cx]);
+            const real dn = real(g.inv_ds) / nn;
+            Gx = cc * fma(ddx, dn, sg3 * ldx);
+            Gy = cc * fma(ddy, dn, sg3 * ldy);
+            eq_sets(true, E, Ox);
+            eq_sets(false, gy, Oy);
+            eq_correction(t, E, gy, sm.n[ty + 3][tx + 4], sm.eng[ty][tx], sm.ux[ty][tx], sm.uy[ty][tx], qa, qb, qc);
+        }
+    } else {
+        static_assert(KP == 2 || KP == 4 || KP == 5 || KP == 8, "velocity lanes: 1, 2, 4, 5 or 8");
+        using Sm = Smem32<TX, TY, KP>;
+        if (active) {
+            // KP = 8: lanes 0..5 take ddx, ddy, ldx, ldy, E, g(u_y);
+            // KP = 5: lanes 0..3 ddx, ddy, ldx, ldy, lane 4 E and g(u_y);
+            // KP = 4: lane 0 ddx, lane 1 ddy, lane 2 ldx + E, lane 3 ldy + g(u_y);
+            // KP = 2: lane 0 the x parts, lane 1 the y parts
+            const bool lane_ldx = KP == 2 ? lane_k == 0 : lane_k == 2;
+            const bool lane_ldy = KP == 2 ? lane_k == 1 : lane_k == 3;
+            const bool lane_gx = KP == 2 ? lane_k == 0 : (KP == 4 ? lane_k == 2 : lane_k == 4);
+            const bool lane_gy = KP == 2 ? lane_k == 1 : (KP == 4 ? lane_k == 3 : (KP == 5 ? lane_k == 4 : lane_k == 5));
+            if (lane_k == 0) {
+                sm.loc[Sm::L_DDX][node] = grad_sum(true);
+                sm.loc[Sm::L_DN][node] = real(g.inv_ds) / field_val(sm.n[ty + cy][tx + cx]);
+            }
+            if (lane_k == 1) sm.loc[Sm::L_DDY][node] = grad_sum(false);
+            if (lane_ldx) sm.loc[Sm::L_LDX][node] = glap_sum(true);
+            if (lane_ldy) sm.loc[Sm::L_LDY][node] = glap_sum(false);
+            if (lane_gx) {
+                eq_sets(true, E, Ox);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    sm.loc[Sm::L_E + q][node] = E[q];
+                    sm.loc[Sm::L_OX + q][node] = Ox[q];
+                }
+            }
+            if (lane_gy) {
+                eq_sets(false, gy, Oy);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    sm.loc[Sm::L_GY + q][node] = gy[q];
+                    sm.loc[Sm::L_OY + q][node] = Oy[q];
+                }
+            }
+            {
+                // the equilibrium's mass and energy correction, on a lane with
+                // little else to do (KP = 8: lane 6; KP = 5, 4, 2: lane 1), from
+                // the same factors the other lanes store (same operations)
+                if (lane_k == (KP == 8 ? 6 : 1)) {
+                    real ex[NQ], ox[NQ], ey[NQ], oy[NQ];
+                    eq_sets(true, ex, ox);
+                    eq_sets(false, ey, oy);
+                    eq_correction(t, ex, ey, sm.n[ty + 3][tx + 4], sm.eng[ty][tx], sm.ux[ty][tx], sm.uy[ty][tx], qa,
+                                  qb, qc);
+                    sm.loc[Sm::L_CA][node] = qa;
+                    sm.loc[Sm::L_CB][node] = qb;
+                    sm.loc[Sm::L_CC][node] = qc;
+                }
+            }
+        }
+        __syncthreads();
+        // G = c F at the node: in registers of each lane, or, on tiles that
+        // keep every face, once per node in shared memory (read after the
+        // barrier that ends the face pass)
+        if (active && (!Sm::ALL_FACES || lane_k == 0)) {
+            const real dn = sm.loc[Sm::L_DN][node];
+            Gx = cc * fma(sm.loc[Sm::L_DDX][node], dn, sg3 * sm.loc[Sm::L_LDX][node]);
+            Gy = cc * fma(sm.loc[Sm::L_DDY][node], dn, sg3 * sm.loc[Sm::L_LDY][node]);
+            if constexpr (Sm::ALL_FACES) {
+                sm.loc[Sm::L_G][node] = Gx;
+                sm.loc[Sm::L_G + 1][node] = Gy;
+            }
+        }
+    }
+
+    // ---- 5. advection, collision and RK combination, KP velocities at a time
+    const int nfx = (TX + 1) * TY, nfy = TX * (TY + 1);
+    const real cadv = cc * real(g.inv_ds);
+    using Sf = Smem32<TX, TY, KP>;
+    constexpr int KF = Sf::KF;
+    // one face value: x face (r, c) or y face (r, c) of velocity k, stored in
+    // slot (FP32: its WENO correction, from first differences of the pairs)
+    auto face = [&](int k, int slot, bool along_x, int r, int c) {
+        const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
+        if (along_x) {
+            if (y0 + r < g.ny && x0 + c <= g.nx) {
+                // face at x = x0 + c: nodes x0+c-3 .. x0+c+2 are columns c+1 .. c+6
+                const real *row = &sm.pop[k][3 + r][0];
+                const float *lo = &sm.pl.lo[k][3 + r][0];
+                auto pd = [&](int a_, int b_) { return pdiff(row[a_], lo[a_], row[b_], lo[b_]); };
+                sm.fx[slot][r][c] =
+                    (k1 > 2) ? face_corr<LEARNED>(mlp, pd(c + 2, c + 1), pd(c + 3, c + 2), pd(c + 4, c + 3), pd(c + 5, c + 4))
+                             : face_corr<LEARNED>(mlp, pd(c + 5, c + 6), pd(c + 4, c + 5), pd(c + 3, c + 4), pd(c + 2, c + 3));
+            }
+        } else if (x0 + c < g.nx && y0 + r <= g.ny) {
+            // face at y = y0 + r: rows y0+r-3 .. y0+r+2 are rows r .. r+5
+            const int cc4 = 4 + c;
+            const real(*P)[HP] = sm.pop[k];
+            const float(*Lo)[HP] = sm.pl.lo[k];
+            auto pd = [&](int a_, int b_) { return pdiff(P[a_][cc4], Lo[a_][cc4], P[b_][cc4], Lo[b_][cc4]); };
+            sm.fy[slot][r][c] = (k2 > 2) ? face_corr<LEARNED>(mlp, pd(r + 1, r), pd(r + 2, r + 1), pd(r + 3, r + 2), pd(r + 4, r + 3))
+                                         : face_corr<LEARNED>(mlp, pd(r + 4, r + 5), pd(r + 3, r + 4), pd(r + 2, r + 3), pd(r + 1, r + 2));
+        }
+    };
+    // learned weights: the face of item (k, slot, along_x,
+    // r, c), or none (valid false); every lane of the warp calls it together,
+    // from a single call site, since the warp evaluates the network of its 32
+    // stencils on the tensor pipe
+    float *const mlp_sc = LEARNED ? const_cast<float *>(mlp) + MLP_SCRATCH_OFF + (tid >> 5) * MLP_WARP_SCRATCH : nullptr;
+    auto learned_face = [&](int k, int slot, bool along_x, int r, int c, bool valid) {
+        const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
+        valid = valid && (along_x ? (y0 + r < g.ny && x0 + c <= g.nx) : (x0 + c < g.nx && y0 + r <= g.ny));
+        // the stencil v0 .. v4 in the upwind orientation, as positions of the
+        // staged region: x faces along row 3 + r, y faces along column 4 + c
+        int p0 = 0, step = 1;
+        if (along_x) {
+            p0 = (k1 > 2) ? c + 1 : c + 6;
+            step = (k1 > 2) ? 1 : -1;
+        } else {
+            p0 = (k2 > 2) ? r : r + 5;
+            step = (k2 > 2) ? 1 : -1;
+        }
+        real d[4] = {0, 0, 0, 0};
+        if (valid) {
+            const real *P = &sm.pop[k][0][0];
+            auto at = [&](int m) { return along_x ? (3 + r) * HP + p0 + m * step : (p0 + m * step) * HP + 4 + c; };
+            const float *Lo = &sm.pl.lo[k][0][0];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) d[m] = pdiff(P[at(m + 1)], Lo[at(m + 1)], P[at(m)], Lo[at(m)]);
+        }
+        const bool acts = learned_guard(d[0], d[1], d[2], d[3]);
+        float x[MLP_IN], w[MLP_OUT] = {0.0f, 0.0f, 0.0f};
+        learned_input_x(d, acts, x);
+        // the whole warp skips the network when none of its stencils needs it
+        if (__any_sync(0xffffffffu, acts)) mlp_weights_warp(mlp, x, w, mlp_sc);
+        if (valid) {
+            const real res = acts ? learned_corr_from(w, d) : weno5_corr(d[0], d[1], d[2], d[3]);
+            if (along_x) sm.fx[slot][r][c] = res;
+            else sm.fy[slot][r][c] = res;
+        }
+    };
+    // node update of velocity k (faces in slot) at tile node (tx_, ty_) with
+    // Ek = n ge(k1), oxk = n go(k1), gyk = ge(k2), oyk = go(k2)
+    auto update = [&](int k1, int k2, int slot, int tx_, int ty_, real Gx_, real Gy_, real Ek, real gyk, real oxk,
+                      real oyk, real qa_, real qb_, real qc_) {
+        const int k = NQ * k1 + k2;
+        const int r = ty_ + 3, c = tx_ + 4;
+        real dx = 0, dy = 0;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            dx = fma(t.D[k1][q], sm.pop[NQ * q + k2][r][c], dx);
+            dy = fma(t.D[k2][q], sm.pop[NQ * k1 + q][r][c], dy);
+        }
+        const real f = sm.pop[k][r][c];
+        const long long o = (long long)(y0 + ty_) * g.pitch + (x0 + tx_);
+        // flux difference = difference of the upwind nodes of the two
+        // faces (a first difference of pairs) + difference of corrections
+        const float(*P)[HP] = sm.pop[k];
+        const float(*Lo)[HP] = sm.pl.lo[k];
+        float adv = 0.0f;
+        if (k1 != 2) {
+            const int cu = k1 > 2 ? c : c + 1;
+            adv = t.R[k1] * (pdiff(P[r][cu], Lo[r][cu], P[r][cu - 1], Lo[r][cu - 1]) +
+                             (sm.fx[slot][ty_][tx_ + 1] - sm.fx[slot][ty_][tx_]));
+        }
+        if (k2 != 2) {
+            const int ru = k2 > 2 ? r : r + 1;
+            adv = fmaf(t.R[k2], pdiff(P[ru][c], Lo[ru][c], P[ru - 1][c], Lo[ru - 1][c]) +
+                                    (sm.fy[slot][ty_ + 1][tx_] - sm.fy[slot][ty_][tx_]), adv);
+        }
+        // f - f^eq with f^eq = n (ge ge + ge go + go (ge + go)) - c: the
+        // exactly symmetric part first, then the parts odd in p_y and in
+        // p_x (each exactly odd after rounding), so that FP32 rounding of
+        // the equilibrium carries no momentum; c (eq_correction) restores
+        // its mass and energy
+        const float fl = Lo[r][c];
+        const float corr =
+            (t.wHe[k1][0] * t.wHe[k2][0]) * fmaf(qc_, t.R2[k1] - t.R2[k2], fmaf(qb_, t.R2[k1] + t.R2[k2], qa_));
+        const float neq = ((((f - Ek * gyk) + fl) - Ek * oyk) - oxk * (gyk + oyk)) + corr;
+        // c L = -c xi.grad f - c F.grad_p f - (c/tau)(f - f^eq), then
+        // out = ca f_n + cb f_s + c L (Eq. rk3) in double-float arithmetic
+        const float inc = -fmaf(cit, neq, fmaf(Gx_, dx, fmaf(Gy_, dy, cadv * adv)));
+        f2 acc = f2_cmul(f2{cb, cb_lo}, f, fl);
+        if (ca != 0.0f) {
+            const f2 an = f2_cmul(f2{ca, ca_lo}, fn[k * g.plane + o], fn[(NK + k) * g.plane + o]);
+            const f2 sh = two_sum(acc.hi, an.hi);
+            acc = f2{sh.hi, sh.lo + (acc.lo + an.lo)};
+        }
+        const f2 si = two_sum(acc.hi, inc);
+        const f2 v = fast_two_sum(si.hi, si.lo + acc.lo);
+        out[k * g.plane + o] = v.hi;
+        out[(NK + k) * g.plane + o] = v.lo;
+    };
+    if (!wait()) return false;  // the populations of phase 1
+    for (int kb = 0; kb < NK; kb += KF) {
+        __syncthreads();  // loc ready / the previous velocities' faces are consumed
+        if constexpr (LEARNED) {
+            // learned weights: the network on the tensor pipe, one warp per 32
+            // stencils (FP64 evaluates it per thread).  The faces of this pass (all 25 velocities' on small tiles, else
+            // those of velocities kb .. kb+KP-1), enumerated as below, on
+            // whole warps: items past the end take part in the network only.
+            // Small tiles: the x faces of the 20 velocities with xi_x != 0,
+            // then the y faces of the 20 with xi_y != 0, located by division
+            // (as in the dense pass below); otherwise the KP velocities'
+            // faces, located in their prefix table
+            int end[KF], total = 0;
+            if constexpr (Sf::ALL_FACES) {
+                total = 20 * (nfx + nfy);
+            } else {
+#pragma unroll
+                for (int sub = 0; sub < KF; ++sub) {
+                    const int k = kb + sub;
+                    if (k < NK) total += (k / NQ != 2 ? nfx : 0) + (k % NQ != 2 ? nfy : 0);
+                    end[sub] = total;
+                }
+            }
+            const int padded = (total + 31) & ~31;
+            for (int e = tid; e < padded; e += NT) {
+                int k, sub, f;
+                bool valid = e < total;
+                if constexpr (Sf::ALL_FACES) {
+                    const int ee = valid ? e : 0;
+                    if (ee < 20 * nfx) {
+                        const int kx = ee / nfx;
+                        k = kx < 2 * NQ ? kx : kx + NQ;
+                        f = ee - kx * nfx;
+                    } else {
+                        const int e2 = ee - 20 * nfx, ky = e2 / nfy, q = ky & 3;
+                        k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
+                        f = nfx + e2 - ky * nfy;
+                    }
+                    sub = k;
+                } else {
+                    int start = 0;
+                    sub = 0;
+#pragma unroll
+                    for (int q = 0; q + 1 < KF; ++q)
+                        if (e >= end[q]) {
+                            sub = q + 1;
+                            start = end[q];
+                        }
+                    k = kb + sub;
+                    f = e - start;
+                    if (k / NQ == 2) f += nfx;
+                    valid = valid && k < NK;
+                }
+                const bool along_x = f < nfx;
+                const int r = along_x ? f / (TX + 1) : (f - nfx) / TX;
+                const int c = along_x ? f - r * (TX + 1) : f - nfx - r * TX;
+                // one call site: the warp's network must run as one instruction
+                // stream (mma.sync needs every lane at the same instruction)
+                learned_face(k, sub, along_x, valid ? r : 0, valid ? c : 0, valid);
+            }
+        } else if constexpr (Sf::ALL_FACES) {
+            // (issue-bound) every face of every velocity once, in strips
+            // of SX (SY) consecutive faces along a tile row (column), each
+            // strip in the upwind direction of its velocity: the x strips of
+            // the 20 velocities with xi_x != 0 (k1 != 2), then the y strips of
+            // the 20 with xi_y != 0 (k2 != 2).
+            constexpr int SX = (TX + 1) % 4 == 0 ? 4 : ((TX + 1) % 3 == 0 ? 3 : 1);
+            constexpr int SY = (TY + 1) % 4 == 0 ? 4 : ((TY + 1) % 3 == 0 ? 3 : 1);
+            constexpr int NSX = (TX + 1) / SX, NSY = (TY + 1) / SY;    // strips per row, per column
+            constexpr int nsx = NSX * TY, nsy = NSY * TX;              // strips per velocity
+            for (int e = tid; e < 20 * (nsx + nsy); e += NT) {
+                if (e < 20 * nsx) {
+                    const int kx = e / nsx, f = e - kx * nsx;
+                    const int k = kx < 2 * NQ ? kx : kx + NQ;
+                    const int r = f / NSX, cs = (f - r * NSX) * SX;
+                    // face at x = x0 + c reads columns c+1 .. c+5 (xi_x > 0) or c+6 .. c+2
+                    const real *row = &sm.pop[k][3 + r][0];
+                    const real *rlo = &sm.pl.lo[k][3 + r][0];
+                    if (k / NQ > 2) weno5_strip_c<SX>(row + cs + 1, rlo + cs + 1, 1, &sm.fx[k][r][cs], 1);
+                    else weno5_strip_c<SX>(row + cs + SX + 5, rlo + cs + SX + 5, -1, &sm.fx[k][r][cs + SX - 1], -1);
+                } else {
+                    const int e2 = e - 20 * nsx, ky = e2 / nsy, f = e2 - ky * nsy, q = ky & 3;
+                    const int k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
+                    const int rs = (f / TX) * SY, c = f - (f / TX) * TX;
+                    // face at y = y0 + r reads rows r .. r+4 (xi_y > 0) or r+5 .. r+1
+                    if (k % NQ > 2)
+                        weno5_strip_c<SY>(&sm.pop[k][rs][4 + c], &sm.pl.lo[k][rs][4 + c], HP, &sm.fy[k][rs][c], TX);
+                    else
+                        weno5_strip_c<SY>(&sm.pop[k][rs + SY + 4][4 + c], &sm.pl.lo[k][rs + SY + 4][4 + c], -HP,
+                                          &sm.fy[k][rs + SY - 1][c], -TX);
+                }
+            }
+            // (faces outside the grid are computed from staged values and never read)
+        } else {
+            // faces of the KP velocities kb .. kb+KP-1, each computed once and
+            // enumerated densely: x faces of the tile rows unless xi_x = 0
+            // (k1 = 2), then y faces of the tile columns unless xi_y = 0 (k2 = 2)
+            int end[KP], total = 0;
+#pragma unroll
+            for (int sub = 0; sub < KP; ++sub) {
+                const int k = kb + sub;
+                if (k < NK) total += (k / NQ != 2 ? nfx : 0) + (k % NQ != 2 ? nfy : 0);
+                end[sub] = total;
+            }
+            for (int e = tid; e < total; e += NT) {
+                int sub = 0, start = 0;
+#pragma unroll
+                for (int q = 0; q + 1 < KP; ++q)
+                    if (e >= end[q]) {
+                        sub = q + 1;
+                        start = end[q];
+                    }
+                const int k = kb + sub;
+                int f = e - start;
+                if (k / NQ == 2) f += nfx;
+                if (f < nfx) {
+                    const int r = f / (TX + 1);
+                    face(k, sub, true, r, f - r * (TX + 1));
+                } else {
+                    const int r = (f - nfx) / TX;
+                    face(k, sub, false, r, f - nfx - r * TX);
+                }
+            }
+        }
+        __syncthreads();
+        if constexpr (Sf::ALL_FACES && KP == NQ) {
+            // (issue-bound) node updates with five lanes: thread (node,
+            // lane k2) advances the five velocities 5 k1 + k2, k1 unrolled,
+            // so that the k1 tables are immediate operands and the node's
+            // factors are read once
+            if (active) {
+                const int k2 = lane_k;
+                const real Gx_ = sm.loc[Sf::L_G][node], Gy_ = sm.loc[Sf::L_G + 1][node];
+                const real qa_ = sm.loc[Sf::L_CA][node], qb_ = sm.loc[Sf::L_CB][node], qc_ = sm.loc[Sf::L_CC][node];
+                const real gyk = sm.loc[Sf::L_GY + k2][node], oyk = sm.loc[Sf::L_OY + k2][node];
+#pragma unroll
+                for (int k1 = 0; k1 < NQ; ++k1)
+                    update(k1, k2, NQ * k1 + k2, tx, ty, Gx_, Gy_, sm.loc[Sf::L_E + k1][node], gyk,
+                           sm.loc[Sf::L_OX + k1][node], oyk, qa_, qb_, qc_);
+            }
+        } else if constexpr (Sf::ALL_FACES) {
+            // node updates, enumerated densely over (velocity, tile node)
+            for (int e = tid; e < NK * NN; e += NT) {
+                const int k = e / NN, nd = e - k * NN;
+                const int tx_ = nd % TX, ty_ = nd / TX;
+                if (x0 + tx_ >= g.nx || y0 + ty_ >= g.ny) continue;
+                const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
+                update(k1, k2, k, tx_, ty_, sm.loc[Sf::L_G][nd], sm.loc[Sf::L_G + 1][nd], sm.loc[Sf::L_E + k1][nd],
+                       sm.loc[Sf::L_GY + k2][nd], sm.loc[Sf::L_OX + k1][nd], sm.loc[Sf::L_OY + k2][nd],
+                       sm.loc[Sf::L_CA][nd], sm.loc[Sf::L_CB][nd], sm.loc[Sf::L_CC][nd]);
+            }
+        } else {
+            const int k = kb + lane_k;
+            if (active && k < NK) {
+                const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
+                real Ek, gyk, oxk = 0, oyk = 0, qa_ = qa, qb_ = qb, qc_ = qc;
+                if constexpr (KP > 1) {
+                    Ek = sm.loc[Sf::L_E + k1][node];
+                    gyk = sm.loc[Sf::L_GY + k2][node];
+                    oxk = sm.loc[Sf::L_OX + k1][node];
+                    oyk = sm.loc[Sf::L_OY + k2][node];
+                    qa_ = sm.loc[Sf::L_CA][node];
+                    qb_ = sm.loc[Sf::L_CB][node];
+                    qc_ = sm.loc[Sf::L_CC][node];
+                } else {
+                    Ek = sel5(E, k1);
+                    gyk = sel5(gy, k2);
+                    oxk = sel5(Ox, k1);
+                    oyk = sel5(Oy, k2);
+                }
+                update(k1, k2, lane_k, tx, ty, Gx, Gy, Ek, gyk, oxk, oyk, qa_, qb_, qc_);
+            }
+        }
+    }
     return true;
 }
 
@@ -412,23 +881,18 @@ __device__ __forceinline__ bool tma_finish(FusedSmem<real, TX, TY, KP> &sm, int 
 // or nullptr; fields: the moments of fs from k_fields, or nullptr to compute
 // them here.  Returns false when the TMA copy timed out (the CTA must stop).
 template <typename real, int TX, int TY, int KP, bool LEARNED = false>
-__device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, const real *__restrict__ fs,
+__device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, LEARNED>::type &sm, const real *__restrict__ fs,
                                            const real *fn, real *out, int *__restrict__ status, const Geo &g,
                                            const Tab<real> &t, const Tab<real> &tw, const int x0, const int y0,
                                            const real ca,
                                            const real cb, const real cc, const real ca_lo, const real cb_lo,
-                                           const float *mlp = nullptr, const TmaMap *tmap = nullptr,
+                                           const StageK &sk, const float *mlp = nullptr, const TmaMap *tmap = nullptr,
                                            const StageFields<real> *fields = nullptr)
 {
-    using S = FusedSmem<real, TX, TY, KP>;
-    constexpr int NT = S::NT, NN = S::NN, HX = S::HX, HY = S::HY, HP = S::HP;
+    using S = typename StageSmem<real, TX, TY, KP, LEARNED>::type;
+    constexpr int NT = S::NT, HX = S::HX, HY = S::HY;
 
-    // thread = (tile node, velocity lane): KP velocities are advanced at once
     const int tid = threadIdx.x;
-    const int node = tid % S::LS, lane_k = tid / S::LS;
-    const int tx = node % TX, ty = node / TX;
-    const int i = x0 + tx, j = y0 + ty;
-    const bool active = (node < NN) && (i < g.nx) && (j < g.ny);
 
     // ---- 1. populations of the region (c <-> x = x0 - 4 + c, r <-> y = y0 - 3 + r)
     //    A region inside the grid comes in one TMA copy.  Otherwise:
@@ -440,7 +904,10 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
     // the pre-pass fields of this thread's first moment position (phase 2's
     // item e = tid) are fetched into registers now, so that their latency
     // overlaps the staging of the populations
-    using fld = typename S::fld;
+    using fld = typename FieldT<real>::type;
+    if constexpr (sizeof(real) == 8) {
+        if (tid == 0) sm.top = 0;  // ordered before phase 2 by phase 1's barrier
+    }
     fld pf_n{}, pf_dp{}, pf_T{}, pf_E{};
     real pf_ux = 0, pf_uy = 0;
     bool pf_ok = false, pf_node = false;
@@ -542,11 +1009,20 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
     // wall-flux items start on the first warp after the moment positions
     constexpr int e_flux = (HY * (HX - 2) + 31) / 32 * 32;
     const int nflux = ((int)left_wall + (int)right_wall) * TY * 16;
+    // FP64: high word of this thread's largest finite n (the tile's scale)
+    int top = 0;
+    auto note_n = [&](fld n) {
+        if constexpr (sizeof(real) == 8) {
+            const int a = __double2hiint(n) & 0x7fffffff;
+            top = max(top, a < 0x7ff00000 ? a : 0);
+        }
+    };
     if (fields != nullptr) {
         // moments from the per-node pre-pass (k_fields): n and Delta p on the
         // region, u, T (FP32: and e) at the tile nodes; item tid was fetched
         // before phase 1
         if (pf_ok) {
+            note_n(pf_n);
             sm.n[pf_r][pf_c] = pf_n;
             sm.dp[pf_r][pf_c] = pf_dp;
             if (pf_node) {
@@ -562,7 +1038,9 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
             if (g.walls && (gx < 0 || gx >= g.nx)) continue;
             if (g.spec_y && (gyr < 0 || gyr >= g.ny)) continue;
             const long long o = (long long)wrap(gyr, g.ny) * g.pitch + wrap(gx, g.nx);
-            sm.n[r][c] = fields->n[o];
+            const fld n = fields->n[o];
+            note_n(n);
+            sm.n[r][c] = n;
             sm.dp[r][c] = fields->dp[o];
             const int tr = r - 3, tc = c - 4;
             if (tr >= 0 && tr < TY && tc >= 0 && tc < TX) {
@@ -587,6 +1065,7 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
             else
                 m = node_moments<real>([&](int k) { return make_float2(sm.pop[k][r][c], sm.pl.lo[k][r][c]); }, g,
                                        t);
+            note_n(m.n);
             sm.n[r][c] = m.n;
             sm.dp[r][c] = m.dp;
             if (tile_node) {
@@ -597,6 +1076,10 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
                 if (own && !m.ok) atomicOr(status, 1);
             }
         }
+    }
+    if constexpr (sizeof(real) == 8) {
+        top = __reduce_max_sync(0xffffffffu, top);
+        if ((tid & 31) == 0) atomicMax(&sm.top, top);
     }
     // wall flux item f runs on thread (e_flux + f) mod NT: on the warps after
     // those with moment positions.  Each tile row of a wall takes a
@@ -703,562 +1186,12 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
     }
     __syncthreads();
 
-    // ---- 4. force and equilibrium factors at the tile nodes.  The four
-    // stencil sums and the two factor sets are split over the velocity lanes
-    // (KP = 4: ddx | ddy | ldx, g(u_x) | ldy, g(u_y); KP = 2: x | y parts).
-    constexpr int cy = 3, cx = 4;
-    auto grad_sum = [&](bool along_x) {
-        real acc = 0;
-#pragma unroll
-        for (int l = 1; l <= 3; ++l)
-#pragma unroll
-            for (int m = -3; m <= 3; ++m) {
-                const int am = m < 0 ? -m : m;
-                if (grad_w(l, am) != 0.0) {
-                    const real w = real(l * grad_w(l, am));
-                    acc = along_x ? fma(w, field_diff(sm.dp[ty + cy + m][tx + cx + l], sm.dp[ty + cy + m][tx + cx - l]), acc)
-                                  : fma(w, field_diff(sm.dp[ty + cy + l][tx + cx + m], sm.dp[ty + cy - l][tx + cx + m]), acc);
-                }
-            }
-        return acc;
-    };
-    auto glap_sum = [&](bool along_x) {
-        real acc = 0;
-        if constexpr (sizeof(real) == 4) {
-            // FP32: the stencil cancels its O(ds) terms down to O(ds^3) (a
-            // factor ~1/(ds k)^2 on fine grids), so the weighted differences
-            // are summed in double-float arithmetic with double-float weights
-            // (exact products of the hi parts, TwoSum accumulation): the sum
-            // keeps FP32 accuracy of itself, not of its terms
-            f2 sum{0.0f, 0.0f};
-#pragma unroll
-            for (int l = 1; l <= 3; ++l)
-#pragma unroll
-                for (int m = -3; m <= 3; ++m) {
-                    const int am = m < 0 ? -m : m;
-                    if (glap_c(am, l) != 0.0) {
-                        const float wh = (float)glap_c(am, l);
-                        const float wl = (float)(glap_c(am, l) - (double)(float)glap_c(am, l));
-                        const float2 a = along_x ? sm.n[ty + cy + m][tx + cx + l] : sm.n[ty + cy + l][tx + cx + m];
-                        const float2 b = along_x ? sm.n[ty + cy + m][tx + cx - l] : sm.n[ty + cy - l][tx + cx + m];
-                        const f2 dh = two_sum(a.x, -b.x);
-                        const float dl = dh.lo + (a.y - b.y);
-                        const float p = wh * dh.hi;
-                        const float e = fmaf(wh, dh.hi, -p);
-                        const float tl = fmaf(wh, dl, fmaf(wl, dh.hi, e));
-                        const f2 t2 = two_sum(sum.hi, p);
-                        sum = f2{t2.hi, t2.lo + (sum.lo + tl)};
-                    }
-                }
-            acc = sum.hi + sum.lo;
-        } else {
-#pragma unroll
-            for (int l = 1; l <= 3; ++l)
-#pragma unroll
-                for (int m = -3; m <= 3; ++m) {
-                    const int am = m < 0 ? -m : m;
-                    if (glap_c(am, l) != 0.0) {
-                        const real w = real(glap_c(am, l));
-                        acc = along_x ? fma(w, field_diff(sm.n[ty + cy + m][tx + cx + l], sm.n[ty + cy + m][tx + cx - l]), acc)
-                                      : fma(w, field_diff(sm.n[ty + cy + l][tx + cx + m], sm.n[ty + cy - l][tx + cx + m]), acc);
-                    }
-                }
-        }
-        return acc;
-    };
-    // With c the stage's coefficient of dt L (Eq. rk3), the node update below
-    // needs per node G = c F, E_q = (c/tau) n g_q(u_x, T) and g_q(u_y, T)
-    // (FP32: n ge_q(u_x, T), n go_q(u_x, T), ge_q(u_y, T), go_q(u_y, T), the
-    // even and odd parts of the factors, in E, Ox, gy, Oy).
-    const real sg3 = real(g.sigma) * real(g.inv_ds3);
-    const real cit = cc * real(g.inv_tau);
-    constexpr bool F32 = sizeof(real) == 4;
-    real Gx = 0, Gy = 0, E[NQ], gy[NQ], Ox[NQ], Oy[NQ];
-    real qa = 0, qb = 0, qc = 0;  // FP32: alpha, beta, gamma of the equilibrium's correction (eq_correction)
-    // equilibrium factor sets of the node at (tx_, ty_): x (scaled by n, and
-    // for FP64 by c/tau) into ex, ox and y into ey, oy
-    auto eq_sets = [&](bool x_set, real *a, real *b) {
-        if constexpr (F32) {
-            if (x_set) {
-                eq_factors_split(t, sm.ux[ty][tx], sm.T[ty][tx], a, b);
-                const real nn = sm.n[ty + 3][tx + 4].x;
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    a[q] = nn * a[q];
-                    b[q] = nn * b[q];
-                }
-            } else {
-                eq_factors_split(t, sm.uy[ty][tx], sm.T[ty][tx], a, b);
-            }
-        } else {
-            if (x_set) {
-                eq_factors<real>(t, sm.ux[ty][tx], sm.T[ty][tx], a);
-                const real cn = cit * field_val(sm.n[ty + 3][tx + 4]);
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) a[q] = cn * a[q];
-            } else {
-                eq_factors<real>(t, sm.uy[ty][tx], sm.T[ty][tx], a);
-            }
-        }
-    };
-    if constexpr (KP == 1) {
-        if (active) {
-            const real ddx = grad_sum(true), ddy = grad_sum(false);
-            const real ldx = glap_sum(true), ldy = glap_sum(false);
-            const real nn = field_val(sm.n[ty + cy][tx + cx]);
-            const real dn = real(g.inv_ds) / nn;
-            Gx = cc * fma(ddx, dn, sg3 * ldx);
-            Gy = cc * fma(ddy, dn, sg3 * ldy);
-            eq_sets(true, E, Ox);
-            eq_sets(false, gy, Oy);
-            if constexpr (F32)
-                eq_correction(t, E, gy, sm.n[ty + 3][tx + 4], sm.eng[ty][tx], sm.ux[ty][tx], sm.uy[ty][tx], qa, qb, qc);
-        }
-    } else {
-        static_assert(KP == 2 || KP == 4 || KP == 5 || KP == 8, "velocity lanes: 1, 2, 4, 5 or 8");
-        using Sm = FusedSmem<real, TX, TY, KP>;
-        if (active) {
-            // KP = 8: lanes 0..5 take ddx, ddy, ldx, ldy, E, g(u_y);
-            // KP = 5: lanes 0..3 ddx, ddy, ldx, ldy, lane 4 E and g(u_y);
-            // KP = 4: lane 0 ddx, lane 1 ddy, lane 2 ldx + E, lane 3 ldy + g(u_y);
-            // KP = 2: lane 0 the x parts, lane 1 the y parts
-            const bool lane_ldx = KP == 2 ? lane_k == 0 : lane_k == 2;
-            const bool lane_ldy = KP == 2 ? lane_k == 1 : lane_k == 3;
-            const bool lane_gx = KP == 2 ? lane_k == 0 : (KP == 4 ? lane_k == 2 : lane_k == 4);
-            const bool lane_gy = KP == 2 ? lane_k == 1 : (KP == 4 ? lane_k == 3 : (KP == 5 ? lane_k == 4 : lane_k == 5));
-            if (lane_k == 0) {
-                sm.loc[Sm::L_DDX][node] = grad_sum(true);
-                sm.loc[Sm::L_DN][node] = real(g.inv_ds) / field_val(sm.n[ty + cy][tx + cx]);
-            }
-            if (lane_k == 1) sm.loc[Sm::L_DDY][node] = grad_sum(false);
-            if (lane_ldx) sm.loc[Sm::L_LDX][node] = glap_sum(true);
-            if (lane_ldy) sm.loc[Sm::L_LDY][node] = glap_sum(false);
-            if (lane_gx) {
-                eq_sets(true, E, Ox);
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    sm.loc[Sm::L_E + q][node] = E[q];
-                    if constexpr (F32) sm.loc[Sm::L_OX + q][node] = Ox[q];
-                }
-            }
-            if (lane_gy) {
-                eq_sets(false, gy, Oy);
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    sm.loc[Sm::L_GY + q][node] = gy[q];
-                    if constexpr (F32) sm.loc[Sm::L_OY + q][node] = Oy[q];
-                }
-            }
-            if constexpr (F32) {
-                // the equilibrium's mass and energy correction, on a lane with
-                // little else to do (KP = 8: lane 6; KP = 5, 4, 2: lane 1), from
-                // the same factors the other lanes store (same operations)
-                if (lane_k == (KP == 8 ? 6 : 1)) {
-                    real ex[NQ], ox[NQ], ey[NQ], oy[NQ];
-                    eq_sets(true, ex, ox);
-                    eq_sets(false, ey, oy);
-                    eq_correction(t, ex, ey, sm.n[ty + 3][tx + 4], sm.eng[ty][tx], sm.ux[ty][tx], sm.uy[ty][tx], qa,
-                                  qb, qc);
-                    sm.loc[Sm::L_CA][node] = qa;
-                    sm.loc[Sm::L_CB][node] = qb;
-                    sm.loc[Sm::L_CC][node] = qc;
-                }
-            }
-        }
-        __syncthreads();
-        // G = c F at the node: in registers of each lane, or, on tiles that
-        // keep every face, once per node in shared memory (read after the
-        // barrier that ends the face pass)
-        if (active && (!Sm::ALL_FACES || lane_k == 0)) {
-            const real dn = sm.loc[Sm::L_DN][node];
-            Gx = cc * fma(sm.loc[Sm::L_DDX][node], dn, sg3 * sm.loc[Sm::L_LDX][node]);
-            Gy = cc * fma(sm.loc[Sm::L_DDY][node], dn, sg3 * sm.loc[Sm::L_LDY][node]);
-            if constexpr (Sm::ALL_FACES) {
-                sm.loc[Sm::L_G][node] = Gx;
-                sm.loc[Sm::L_G + 1][node] = Gy;
-            }
-        }
-    }
-
-    // ---- 5. advection, collision and RK combination, KP velocities at a time
-    const int nfx = (TX + 1) * TY, nfy = TX * (TY + 1);
-    const real cf = cb - cit;
-    const real cadv = cc * real(g.inv_ds);
-    using Sf = FusedSmem<real, TX, TY, KP>;
-    constexpr int KF = Sf::KF;
-    // one face value: x face (r, c) or y face (r, c) of velocity k, stored in
-    // slot (FP32: its WENO correction, from first differences of the pairs)
-    auto face = [&](int k, int slot, bool along_x, int r, int c) {
-        const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
-        if (along_x) {
-            if (y0 + r < g.ny && x0 + c <= g.nx) {
-                // face at x = x0 + c: nodes x0+c-3 .. x0+c+2 are columns c+1 .. c+6
-                const real *row = &sm.pop[k][3 + r][0];
-                if constexpr (F32) {
-                    const float *lo = &sm.pl.lo[k][3 + r][0];
-                    auto pd = [&](int a_, int b_) { return pdiff(row[a_], lo[a_], row[b_], lo[b_]); };
-                    sm.fx[slot][r][c] =
-                        (k1 > 2) ? face_corr<LEARNED>(mlp, pd(c + 2, c + 1), pd(c + 3, c + 2), pd(c + 4, c + 3), pd(c + 5, c + 4))
-                                 : face_corr<LEARNED>(mlp, pd(c + 5, c + 6), pd(c + 4, c + 5), pd(c + 3, c + 4), pd(c + 2, c + 3));
-                } else {
-                    sm.fx[slot][r][c] =
-                        (k1 > 2) ? face_value<LEARNED>(mlp, row[c + 1], row[c + 2], row[c + 3], row[c + 4], row[c + 5])
-                                 : face_value<LEARNED>(mlp, row[c + 6], row[c + 5], row[c + 4], row[c + 3], row[c + 2]);
-                }
-            }
-        } else if (x0 + c < g.nx && y0 + r <= g.ny) {
-            // face at y = y0 + r: rows y0+r-3 .. y0+r+2 are rows r .. r+5
-            const int cc4 = 4 + c;
-            const real(*P)[HP] = sm.pop[k];
-            if constexpr (F32) {
-                const float(*Lo)[HP] = sm.pl.lo[k];
-                auto pd = [&](int a_, int b_) { return pdiff(P[a_][cc4], Lo[a_][cc4], P[b_][cc4], Lo[b_][cc4]); };
-                sm.fy[slot][r][c] = (k2 > 2) ? face_corr<LEARNED>(mlp, pd(r + 1, r), pd(r + 2, r + 1), pd(r + 3, r + 2), pd(r + 4, r + 3))
-                                             : face_corr<LEARNED>(mlp, pd(r + 4, r + 5), pd(r + 3, r + 4), pd(r + 2, r + 3), pd(r + 1, r + 2));
-            } else {
-                sm.fy[slot][r][c] = (k2 > 2) ? face_value<LEARNED>(mlp, P[r][cc4], P[r + 1][cc4], P[r + 2][cc4],
-                                                                        P[r + 3][cc4], P[r + 4][cc4])
-                                            : face_value<LEARNED>(mlp, P[r + 5][cc4], P[r + 4][cc4], P[r + 3][cc4],
-                                                                        P[r + 2][cc4], P[r + 1][cc4]);
-            }
-        }
-    };
-    // learned weights (FP32 instances): the face of item (k, slot, along_x,
-    // r, c), or none (valid false); every lane of the warp calls it together,
-    // from a single call site, since the warp evaluates the network of its 32
-    // stencils on the tensor pipe
-    float *const mlp_sc = (LEARNED && F32) ? const_cast<float *>(mlp) + MLP_SCRATCH_OFF + (tid >> 5) * MLP_WARP_SCRATCH : nullptr;
-    auto learned_face = [&](int k, int slot, bool along_x, int r, int c, bool valid) {
-        const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
-        valid = valid && (along_x ? (y0 + r < g.ny && x0 + c <= g.nx) : (x0 + c < g.nx && y0 + r <= g.ny));
-        // the stencil v0 .. v4 in the upwind orientation, as positions of the
-        // staged region: x faces along row 3 + r, y faces along column 4 + c
-        int p0 = 0, step = 1;
-        if (along_x) {
-            p0 = (k1 > 2) ? c + 1 : c + 6;
-            step = (k1 > 2) ? 1 : -1;
-        } else {
-            p0 = (k2 > 2) ? r : r + 5;
-            step = (k2 > 2) ? 1 : -1;
-        }
-        real d[4] = {0, 0, 0, 0};
-        if (valid) {
-            const real *P = &sm.pop[k][0][0];
-            auto at = [&](int m) { return along_x ? (3 + r) * HP + p0 + m * step : (p0 + m * step) * HP + 4 + c; };
-            if constexpr (F32) {
-                const float *Lo = &sm.pl.lo[k][0][0];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) d[m] = pdiff(P[at(m + 1)], Lo[at(m + 1)], P[at(m)], Lo[at(m)]);
-            }
-        }
-        const bool acts = learned_guard<real>(d[0], d[1], d[2], d[3]);
-        const float e[4] = {(float)d[0], (float)d[1], (float)d[2], (float)d[3]};
-        float x[MLP_IN], w[MLP_OUT] = {0.0f, 0.0f, 0.0f};
-        learned_input_x(e, acts, x);
-        // the whole warp skips the network when none of its stencils needs it
-        if (__any_sync(0xffffffffu, acts)) mlp_weights_warp(mlp, x, w, mlp_sc);
-        if (valid) {
-            const real res = acts ? learned_corr_from(w, e) : weno5_corr(e[0], e[1], e[2], e[3]);
-            if (along_x) sm.fx[slot][r][c] = res;
-            else sm.fy[slot][r][c] = res;
-        }
-    };
-    // node update of velocity k (faces in slot) at tile node (tx_, ty_):
-    // FP64 with Ek = E_q(k1), gyk = g_q(k2); FP32 with Ek = n ge(k1),
-    // oxk = n go(k1), gyk = ge(k2), oyk = go(k2)
-    auto update = [&](int k1, int k2, int slot, int tx_, int ty_, real Gx_, real Gy_, real Ek, real gyk, real oxk,
-                      real oyk, real qa_, real qb_, real qc_) {
-        const int k = NQ * k1 + k2;
-        const int r = ty_ + 3, c = tx_ + 4;
-        real dx = 0, dy = 0;
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            dx = fma(t.D[k1][q], sm.pop[NQ * q + k2][r][c], dx);
-            dy = fma(t.D[k2][q], sm.pop[NQ * k1 + q][r][c], dy);
-        }
-        const real f = sm.pop[k][r][c];
-        const long long o = (long long)(y0 + ty_) * g.pitch + (x0 + tx_);
-        if constexpr (F32) {
-            // flux difference = difference of the upwind nodes of the two
-            // faces (a first difference of pairs) + difference of corrections
-            const float(*P)[HP] = sm.pop[k];
-            const float(*Lo)[HP] = sm.pl.lo[k];
-            float adv = 0.0f;
-            if (k1 != 2) {
-                const int cu = k1 > 2 ? c : c + 1;
-                adv = t.R[k1] * (pdiff(P[r][cu], Lo[r][cu], P[r][cu - 1], Lo[r][cu - 1]) +
-                                 (sm.fx[slot][ty_][tx_ + 1] - sm.fx[slot][ty_][tx_]));
-            }
-            if (k2 != 2) {
-                const int ru = k2 > 2 ? r : r + 1;
-                adv = fmaf(t.R[k2], pdiff(P[ru][c], Lo[ru][c], P[ru - 1][c], Lo[ru - 1][c]) +
-                                        (sm.fy[slot][ty_ + 1][tx_] - sm.fy[slot][ty_][tx_]), adv);
-            }
-            // f - f^eq with f^eq = n (ge ge + ge go + go (ge + go)) - c: the
-            // exactly symmetric part first, then the parts odd in p_y and in
-            // p_x (each exactly odd after rounding), so that FP32 rounding of
-            // the equilibrium carries no momentum; c (eq_correction) restores
-            // its mass and energy
-            const float fl = Lo[r][c];
-            const float corr =
-                (t.wHe[k1][0] * t.wHe[k2][0]) * fmaf(qc_, t.R2[k1] - t.R2[k2], fmaf(qb_, t.R2[k1] + t.R2[k2], qa_));
-            const float neq = ((((f - Ek * gyk) + fl) - Ek * oyk) - oxk * (gyk + oyk)) + corr;
-            // c L = -c xi.grad f - c F.grad_p f - (c/tau)(f - f^eq), then
-            // out = ca f_n + cb f_s + c L (Eq. rk3) in double-float arithmetic
-            const float inc = -fmaf(cit, neq, fmaf(Gx_, dx, fmaf(Gy_, dy, cadv * adv)));
-            f2 acc = f2_cmul(f2{cb, cb_lo}, f, fl);
-            if (ca != 0.0f) {
-                const f2 an = f2_cmul(f2{ca, ca_lo}, fn[k * g.plane + o], fn[(NK + k) * g.plane + o]);
-                const f2 sh = two_sum(acc.hi, an.hi);
-                acc = f2{sh.hi, sh.lo + (acc.lo + an.lo)};
-            }
-            const f2 si = two_sum(acc.hi, inc);
-            const f2 v = fast_two_sum(si.hi, si.lo + acc.lo);
-            out[k * g.plane + o] = v.hi;
-            out[(NK + k) * g.plane + o] = v.lo;
-        } else {
-            real adv = 0;
-            if (k1 != 2) adv = t.R[k1] * (sm.fx[slot][ty_][tx_ + 1] - sm.fx[slot][ty_][tx_]);
-            if (k2 != 2) adv = fma(t.R[k2], sm.fy[slot][ty_ + 1][tx_] - sm.fy[slot][ty_][tx_], adv);
-            // c L = -c xi.grad f - c F.grad_p f - (c/tau)(f - f^eq) with f^eq = n g g
-            // (Eqs. feq, g_alpha), combined with b f (and a f_n) as in Eq. rk3
-            real v = fma(cf, f, fma(Ek, gyk, -fma(Gx_, dx, fma(Gy_, dy, cadv * adv))));
-            if (ca != real(0)) v = fma(ca, fn[k * g.plane + o], v);
-            out[k * g.plane + o] = v;
-        }
-    };
-    if (defer && !tma_finish(sm, status)) return false;  // the populations of phase 1
-    for (int kb = 0; kb < NK; kb += KF) {
-        __syncthreads();  // loc ready / the previous velocities' faces are consumed
-        if constexpr (LEARNED && sizeof(real) == 4) {
-            // FP32 with learned weights: the network on the tensor pipe, one
-            // warp per 32 stencils (FP64 instances, bound by the FP64 pipe,
-            // evaluate it per thread in the loop further down: the warp
-            // network measured no faster there, and its scratch does not fit
-            // the largest FP64 tile).  The faces of this pass (all 25 velocities' on small tiles, else
-            // those of velocities kb .. kb+KP-1), enumerated as below, on
-            // whole warps: items past the end take part in the network only.
-            // Small tiles: the x faces of the 20 velocities with xi_x != 0,
-            // then the y faces of the 20 with xi_y != 0, located by division
-            // (as in the dense pass below); otherwise the KP velocities'
-            // faces, located in their prefix table
-            int end[KF], total = 0;
-            if constexpr (Sf::ALL_FACES) {
-                total = 20 * (nfx + nfy);
-            } else {
-#pragma unroll
-                for (int sub = 0; sub < KF; ++sub) {
-                    const int k = kb + sub;
-                    if (k < NK) total += (k / NQ != 2 ? nfx : 0) + (k % NQ != 2 ? nfy : 0);
-                    end[sub] = total;
-                }
-            }
-            const int padded = (total + 31) & ~31;
-            for (int e = tid; e < padded; e += NT) {
-                int k, sub, f;
-                bool valid = e < total;
-                if constexpr (Sf::ALL_FACES) {
-                    const int ee = valid ? e : 0;
-                    if (ee < 20 * nfx) {
-                        const int kx = ee / nfx;
-                        k = kx < 2 * NQ ? kx : kx + NQ;
-                        f = ee - kx * nfx;
-                    } else {
-                        const int e2 = ee - 20 * nfx, ky = e2 / nfy, q = ky & 3;
-                        k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
-                        f = nfx + e2 - ky * nfy;
-                    }
-                    sub = k;
-                } else {
-                    int start = 0;
-                    sub = 0;
-#pragma unroll
-                    for (int q = 0; q + 1 < KF; ++q)
-                        if (e >= end[q]) {
-                            sub = q + 1;
-                            start = end[q];
-                        }
-                    k = kb + sub;
-                    f = e - start;
-                    if (k / NQ == 2) f += nfx;
-                    valid = valid && k < NK;
-                }
-                const bool along_x = f < nfx;
-                const int r = along_x ? f / (TX + 1) : (f - nfx) / TX;
-                const int c = along_x ? f - r * (TX + 1) : f - nfx - r * TX;
-                // one call site: the warp's network must run as one instruction
-                // stream (mma.sync needs every lane at the same instruction)
-                learned_face(k, sub, along_x, valid ? r : 0, valid ? c : 0, valid);
-            }
-        } else if constexpr (Sf::ALL_FACES && sizeof(real) == 4) {
-            // FP32 (issue-bound): every face of every velocity once, in strips
-            // of SX (SY) consecutive faces along a tile row (column), each
-            // strip in the upwind direction of its velocity: the x strips of
-            // the 20 velocities with xi_x != 0 (k1 != 2), then the y strips of
-            // the 20 with xi_y != 0 (k2 != 2).  (In FP64 the FP64 unit paces
-            // each warp, and the fewer, longer strip items leave too few warps
-            // per sub-partition at the end of the pass: single faces are faster.)
-            constexpr int SX = (TX + 1) % 4 == 0 ? 4 : ((TX + 1) % 3 == 0 ? 3 : 1);
-            constexpr int SY = (TY + 1) % 4 == 0 ? 4 : ((TY + 1) % 3 == 0 ? 3 : 1);
-            constexpr int NSX = (TX + 1) / SX, NSY = (TY + 1) / SY;    // strips per row, per column
-            constexpr int nsx = NSX * TY, nsy = NSY * TX;              // strips per velocity
-            for (int e = tid; e < 20 * (nsx + nsy); e += NT) {
-                if (e < 20 * nsx) {
-                    const int kx = e / nsx, f = e - kx * nsx;
-                    const int k = kx < 2 * NQ ? kx : kx + NQ;
-                    const int r = f / NSX, cs = (f - r * NSX) * SX;
-                    // face at x = x0 + c reads columns c+1 .. c+5 (xi_x > 0) or c+6 .. c+2
-                    const real *row = &sm.pop[k][3 + r][0];
-                    const real *rlo = &sm.pl.lo[k][3 + r][0];
-                    if (k / NQ > 2) weno5_strip_c<SX>(row + cs + 1, rlo + cs + 1, 1, &sm.fx[k][r][cs], 1);
-                    else weno5_strip_c<SX>(row + cs + SX + 5, rlo + cs + SX + 5, -1, &sm.fx[k][r][cs + SX - 1], -1);
-                } else {
-                    const int e2 = e - 20 * nsx, ky = e2 / nsy, f = e2 - ky * nsy, q = ky & 3;
-                    const int k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
-                    const int rs = (f / TX) * SY, c = f - (f / TX) * TX;
-                    // face at y = y0 + r reads rows r .. r+4 (xi_y > 0) or r+5 .. r+1
-                    if (k % NQ > 2)
-                        weno5_strip_c<SY>(&sm.pop[k][rs][4 + c], &sm.pl.lo[k][rs][4 + c], HP, &sm.fy[k][rs][c], TX);
-                    else
-                        weno5_strip_c<SY>(&sm.pop[k][rs + SY + 4][4 + c], &sm.pl.lo[k][rs + SY + 4][4 + c], -HP,
-                                          &sm.fy[k][rs + SY - 1][c], -TX);
-                }
-            }
-            // (faces outside the grid are computed from staged values and never read)
-        } else if constexpr (Sf::ALL_FACES && !LEARNED) {
-            // FP64: a strip is a whole tile row (x faces of the 20 velocities
-            // with xi_x != 0) or column (y faces of the 20 with xi_y != 0), in
-            // the upwind direction: 1.5 first differences per node and axis, the
-            // only FP64 operations of a face besides the sum with its upwind
-            // node.  An 8 x 8 tile has 320 strips, one for each thread of the
-            // shape with five lanes.
-            for (int e = tid; e < 20 * (TY + TX); e += NT) {
-                if (e < 20 * TY) {
-                    const int kx = e / TY, r = e - kx * TY;
-                    const int k = kx < 2 * NQ ? kx : kx + NQ;
-                    const real *row = &sm.pop[k][3 + r][0];
-                    // one call for both directions: the code of a strip is long
-                    const bool up = k / NQ > 2;
-                    weno5_strip_ff<TX + 1>(row + (up ? 1 : TX + 6), up ? 1 : -1, &sm.fx[k][r][up ? 0 : TX], up ? 1 : -1);
-                } else {
-                    const int e2 = e - 20 * TY, ky = e2 / TX, c = e2 - ky * TX, q = ky & 3;
-                    const int k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
-                    const bool up = k % NQ > 2;
-                    weno5_strip_ff<TY + 1>(&sm.pop[k][up ? 0 : TY + 5][4 + c], up ? HP : -HP, &sm.fy[k][up ? 0 : TY][c],
-                                           up ? TX : -TX);
-                }
-            }
-            // (faces outside the grid are computed from staged values and never read)
-        } else if constexpr (Sf::ALL_FACES) {
-            // learned weights: every face of every velocity once, enumerated
-            // densely: the x faces of the 20 velocities with xi_x != 0, then the
-            // y faces of the 20 with xi_y != 0
-            for (int e = tid; e < 20 * (nfx + nfy); e += NT) {
-                if (e < 20 * nfx) {
-                    const int kx = e / nfx, f = e - kx * nfx;
-                    const int k = kx < 2 * NQ ? kx : kx + NQ;
-                    const int r = f / (TX + 1);
-                    face(k, k, true, r, f - r * (TX + 1));
-                } else {
-                    const int e2 = e - 20 * nfx, ky = e2 / nfy, f = e2 - ky * nfy, q = ky & 3;
-                    const int k = (ky >> 2) * NQ + (q < 2 ? q : q + 1);
-                    const int r = f / TX;
-                    face(k, k, false, r, f - r * TX);
-                }
-            }
-        } else {
-            // faces of the KP velocities kb .. kb+KP-1, each computed once and
-            // enumerated densely: x faces of the tile rows unless xi_x = 0
-            // (k1 = 2), then y faces of the tile columns unless xi_y = 0 (k2 = 2)
-            int end[KP], total = 0;
-#pragma unroll
-            for (int sub = 0; sub < KP; ++sub) {
-                const int k = kb + sub;
-                if (k < NK) total += (k / NQ != 2 ? nfx : 0) + (k % NQ != 2 ? nfy : 0);
-                end[sub] = total;
-            }
-            for (int e = tid; e < total; e += NT) {
-                int sub = 0, start = 0;
-#pragma unroll
-                for (int q = 0; q + 1 < KP; ++q)
-                    if (e >= end[q]) {
-                        sub = q + 1;
-                        start = end[q];
-                    }
-                const int k = kb + sub;
-                int f = e - start;
-                if (k / NQ == 2) f += nfx;
-                if (f < nfx) {
-                    const int r = f / (TX + 1);
-                    face(k, sub, true, r, f - r * (TX + 1));
-                } else {
-                    const int r = (f - nfx) / TX;
-                    face(k, sub, false, r, f - nfx - r * TX);
-                }
-            }
-        }
-        __syncthreads();
-        if constexpr (Sf::ALL_FACES && F32 && KP == NQ) {
-            // FP32 (issue-bound) node updates with five lanes: thread (node,
-            // lane k2) advances the five velocities 5 k1 + k2, k1 unrolled,
-            // so that the k1 tables are immediate operands and the node's
-            // factors are read once
-            if (active) {
-                const int k2 = lane_k;
-                const real Gx_ = sm.loc[Sf::L_G][node], Gy_ = sm.loc[Sf::L_G + 1][node];
-                const real qa_ = sm.loc[Sf::L_CA][node], qb_ = sm.loc[Sf::L_CB][node], qc_ = sm.loc[Sf::L_CC][node];
-                const real gyk = sm.loc[Sf::L_GY + k2][node], oyk = sm.loc[Sf::L_OY + k2][node];
-#pragma unroll
-                for (int k1 = 0; k1 < NQ; ++k1)
-                    update(k1, k2, NQ * k1 + k2, tx, ty, Gx_, Gy_, sm.loc[Sf::L_E + k1][node], gyk,
-                           sm.loc[Sf::L_OX + k1][node], oyk, qa_, qb_, qc_);
-            }
-        } else if constexpr (Sf::ALL_FACES) {
-            // node updates, enumerated densely over (velocity, tile node)
-            for (int e = tid; e < NK * NN; e += NT) {
-                const int k = e / NN, nd = e - k * NN;
-                const int tx_ = nd % TX, ty_ = nd / TX;
-                if (x0 + tx_ >= g.nx || y0 + ty_ >= g.ny) continue;
-                const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
-                real oxk = 0, oyk = 0, qa_ = 0, qb_ = 0, qc_ = 0;
-                if constexpr (F32) {
-                    oxk = sm.loc[Sf::L_OX + k1][nd];
-                    oyk = sm.loc[Sf::L_OY + k2][nd];
-                    qa_ = sm.loc[Sf::L_CA][nd];
-                    qb_ = sm.loc[Sf::L_CB][nd];
-                    qc_ = sm.loc[Sf::L_CC][nd];
-                }
-                update(k1, k2, k, tx_, ty_, sm.loc[Sf::L_G][nd], sm.loc[Sf::L_G + 1][nd], sm.loc[Sf::L_E + k1][nd],
-                       sm.loc[Sf::L_GY + k2][nd], oxk, oyk, qa_, qb_, qc_);
-            }
-        } else {
-            const int k = kb + lane_k;
-            if (active && k < NK) {
-                const int k1 = k / NQ, k2 = k - NQ * (k / NQ);
-                real Ek, gyk, oxk = 0, oyk = 0, qa_ = qa, qb_ = qb, qc_ = qc;
-                if constexpr (KP > 1) {
-                    Ek = sm.loc[Sf::L_E + k1][node];
-                    gyk = sm.loc[Sf::L_GY + k2][node];
-                    if constexpr (F32) {
-                        oxk = sm.loc[Sf::L_OX + k1][node];
-                        oyk = sm.loc[Sf::L_OY + k2][node];
-                        qa_ = sm.loc[Sf::L_CA][node];
-                        qb_ = sm.loc[Sf::L_CB][node];
-                        qc_ = sm.loc[Sf::L_CC][node];
-                    }
-                } else {
-                    Ek = sel5(E, k1);
-                    gyk = sel5(gy, k2);
-                    if constexpr (F32) {
-                        oxk = sel5(Ox, k1);
-                        oyk = sel5(Oy, k2);
-                    }
-                }
-                update(k1, k2, lane_k, tx, ty, Gx, Gy, Ek, gyk, oxk, oyk, qa_, qb_, qc_);
-            }
-        }
-    }
-    return true;
+    // ---- 4, 5. force, fluxes, collision and RK-3 combination
+    auto wait = [&] { return !defer || tma_finish(sm, status); };
+    if constexpr (sizeof(real) == 8)
+        return advance64<TX, TY, KP, LEARNED>(sm, fn, out, g, t, t.ff, sk, x0, y0, mlp, wait);
+    else
+        return advance32<TX, TY, KP, LEARNED>(sm, fn, out, g, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, mlp, wait);
 }
 
 // Shared memory of the single-grid kernel: the tile staging, then (learned
@@ -1267,17 +1200,22 @@ __device__ __forceinline__ bool stage_tile(FusedSmem<real, TX, TY, KP> &sm, cons
 template <typename real, int TX, int TY, int KP>
 constexpr size_t mlp_offset()
 {
-    return (sizeof(FusedSmem<real, TX, TY, KP>) + 15) / 16 * 16;
+    return (sizeof(typename StageSmem<real, TX, TY, KP, true>::type) + 15) / 16 * 16;
 }
 template <typename real, int TX, int TY, int KP, bool LEARNED>
 constexpr size_t fused_smem_bytes()
 {
     // learned: the parameters; FP32 also the split W2 and MLP_WARP_SCRATCH
     // floats per warp
-    constexpr size_t mlp_floats = sizeof(real) == 4
-                                      ? MLP_SCRATCH_OFF + FusedSmem<real, TX, TY, KP>::NT / 32 * MLP_WARP_SCRATCH
-                                      : MLP_P + 1;
-    return LEARNED ? mlp_offset<real, TX, TY, KP>() + mlp_floats * sizeof(float) : sizeof(FusedSmem<real, TX, TY, KP>);
+    using S = typename StageSmem<real, TX, TY, KP, LEARNED>::type;
+    constexpr size_t mlp_floats = sizeof(real) == 4 ? MLP_SCRATCH_OFF + S::NT / 32 * MLP_WARP_SCRATCH : MLP_P + 1;
+    return LEARNED ? mlp_offset<real, TX, TY, KP>() + mlp_floats * sizeof(float) : sizeof(S);
+}
+// Threads of a shape's CTA: KP lanes of the tile's nodes, rounded up to warps.
+template <int TX, int TY, int KP>
+constexpr int stage_threads()
+{
+    return (TX * TY + 31) / 32 * 32 * KP;
 }
 
 // CTAs per SM that the register allocation must leave room for: as many as
@@ -1292,22 +1230,23 @@ constexpr int fused_min_ctas(size_t smem_bytes, int threads, int cap = 0)
     return n < 1 ? 1 : (cap > 0 && n > cap ? cap : n);
 }
 
-// Single grid: one CTA per tile.  Learned-weight instances leave their
-// network the registers it needs: FP32 (tensor-pipe network) at most two CTAs
-// per SM, FP64 (per-thread network) one.
+// Single grid: one CTA per tile.  FP64 takes two CTAs per SM (its strips need
+// the registers).  Learned-weight instances leave their network the registers
+// it needs: FP32 (tensor-pipe network) at most two CTAs per SM, FP64 (per-thread
+// network) one.
 template <typename real, int TX, int TY, int KP, bool LEARNED>
-__global__ void __launch_bounds__(FusedSmem<real, TX, TY, KP>::NT,
+__global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
                                   fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, LEARNED>(),
-                                                 FusedSmem<real, TX, TY, KP>::NT,
-                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : 0))
+                                                 stage_threads<TX, TY, KP>(),
+                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : (sizeof(real) == 4 ? 0 : 2)))
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
-        real cb_lo, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
+        real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
         const __grid_constant__ StageFields<real> fields)
 {
     // 128-byte aligned: the TMA copy of phase 1 lands at offset 0
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    auto &sm = *reinterpret_cast<FusedSmem<real, TX, TY, KP> *>(smem_raw);
+    auto &sm = *reinterpret_cast<typename StageSmem<real, TX, TY, KP, LEARNED>::type *>(smem_raw);
     float *mlp_sm = nullptr;
     if constexpr (LEARNED) {
         mlp_sm = reinterpret_cast<float *>(smem_raw + mlp_offset<real, TX, TY, KP>());
@@ -1319,7 +1258,7 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
         // made visible by the first barrier inside stage_tile
     }
     stage_tile<real, TX, TY, KP, LEARNED>(sm, fs, fn, out, status, g, t, t, blockIdx.x * TX, blockIdx.y * TY, ca, cb,
-                                          cc, ca_lo, cb_lo, mlp_sm, tma.on ? &tma.map : nullptr,
+                                          cc, ca_lo, cb_lo, sk, mlp_sm, tma.on ? &tma.map : nullptr,
                                           fields.n ? &fields : nullptr);
 }
 
@@ -1340,26 +1279,23 @@ struct __align__(16) BatchRun {
     long long off;   // populations: element offset in the three buffers
     long long foff;  // stage fields: byte offset in the fields buffer
     int ntx, pad;
+    StageK k[3];  // constants of the three RK-3 stages (FP64)
+    long long pad2;
 };
 static_assert(sizeof(BatchRun<double>) % 16 == 0, "BatchRun<double> must be a whole number of int4 words");
 static_assert(sizeof(BatchRun<float>) % 16 == 0, "BatchRun<float> must be a whole number of int4 words");
 
 template <typename real, int TX, int TY, int KP>
-__global__ void __launch_bounds__(FusedSmem<real, TX, TY, KP>::NT,
-                                  // FP64: at most two (more would spill the per-item
-                                  // state); FP32: as many as fit, like the single grid
-                                  sizeof(real) == 4
-                                      ? fused_min_ctas(sizeof(FusedSmem<real, TX, TY, KP>) + sizeof(BatchRun<real>),
-                                                       FusedSmem<real, TX, TY, KP>::NT)
-                                      : (fused_min_ctas(sizeof(FusedSmem<real, TX, TY, KP>) + sizeof(BatchRun<real>),
-                                                        FusedSmem<real, TX, TY, KP>::NT) > 1 ? 2 : 1))
+__global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
+                                  fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, false>() + sizeof(BatchRun<real>),
+                                                 stage_threads<TX, TY, KP>(), sizeof(real) == 4 ? 0 : 2))
 k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
               const BatchRun<real> *__restrict__ runs, const int *__restrict__ tile_start, int nruns,
-              const __grid_constant__ Tab<real> tv, real ca, real cb, real ccoef, real ca_lo, real cb_lo,
+              const __grid_constant__ Tab<real> tv, real ca, real cb, real ccoef, real ca_lo, real cb_lo, int st,
               char *fields, const TmaMap *__restrict__ tmaps)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    auto &sm = *reinterpret_cast<FusedSmem<real, TX, TY, KP> *>(smem_raw);
+    auto &sm = *reinterpret_cast<typename StageSmem<real, TX, TY, KP, false>::type *>(smem_raw);
     __shared__ __align__(16) BatchRun<real> run;
     const int item = blockIdx.x;
     int lo = 0, hi = nruns - 1;
@@ -1385,7 +1321,7 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
     if (tm && threadIdx.x == 0)
         asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm) : "memory");
     stage_tile<real, TX, TY, KP>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
-                                 ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, nullptr, tm, fields ? &fl : nullptr);
+                                 ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, run.k[st], nullptr, tm, fields ? &fl : nullptr);
 }
 
 // The moments pre-pass for a batch: one thread per node of every run (a
@@ -1437,7 +1373,7 @@ cudaError_t fused_prepare_one()
                                          (int)fused_smem_bytes<real, TX, TY, KP, LEARNED>());
     if (e != cudaSuccess || LEARNED) return e;
     return cudaFuncSetAttribute(k_fused_batch<real, TX, TY, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sizeof(FusedSmem<real, TX, TY, KP>));
+                                (int)fused_smem_bytes<real, TX, TY, KP, false>());
 }
 
 template <typename real, int TX, int TY, int KP, bool LEARNED = false>
@@ -1458,16 +1394,16 @@ cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *sta
         const long long N = (long long)g.nx * g.ny;
         k_fields<real><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
     }
-    k_fused<real, TX, TY, KP, LEARNED><<<grid, FusedSmem<real, TX, TY, KP>::NT, fused_smem_bytes<real, TX, TY, KP, LEARNED>(), s>>>(
+    k_fused<real, TX, TY, KP, LEARNED><<<grid, stage_threads<TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, LEARNED>(), s>>>(
         fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
-        (real)(c.cb - (double)(real)c.cb), mlp, tma, fl);
+        (real)(c.cb - (double)(real)c.cb), sizeof(real) == 8 ? stage_constants(g, c) : StageK{}, mlp, tma, fl);
     return cudaGetLastError();
 }
 
 template <typename real, int TX, int TY, int KP>
 cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, int *status, const void *runs,
                                    const int *tile_start, int nruns, int total, const Tab<real> &t, StageCoef c,
-                                   void *fields, const long long *node_start, long long total_nodes,
+                                   int st, void *fields, const long long *node_start, long long total_nodes,
                                    const TmaMap *tmaps, cudaStream_t s)
 {
     if (total < 1) return cudaSuccess;
@@ -1480,57 +1416,62 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
             fs, static_cast<char *>(fields), static_cast<const BatchRun<real> *>(runs), node_start, nruns, total_nodes,
             status);
     }
-    k_fused_batch<real, TX, TY, KP><<<total, FusedSmem<real, TX, TY, KP>::NT, sizeof(FusedSmem<real, TX, TY, KP>), s>>>(
+    k_fused_batch<real, TX, TY, KP><<<total, stage_threads<TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, false>(), s>>>(
         fs, fn, out, status, static_cast<const BatchRun<real> *>(runs), tile_start, nruns, t, (real)c.ca, (real)c.cb,
-        (real)c.cc, (real)(c.ca - (double)(real)c.ca), (real)(c.cb - (double)(real)c.cb), static_cast<char *>(fields),
+        (real)c.cc, (real)(c.ca - (double)(real)c.ca), (real)(c.cb - (double)(real)c.cb), st, static_cast<char *>(fields),
         tmaps);
     return cudaGetLastError();
 }
 
 // Shapes compiled for each precision: TX x TY nodes per CTA, KP velocities
-// advanced at once (KP lanes of TX*TY threads rounded up to whole warps).  Must match TILE_X/TILE_Y/TILE_K in
-// olb_internal.cuh.
-#define OLB_FUSED_SHAPE_CASES(real, DO) \
-    DO(real, 8, 8, 4) DO(real, 16, 8, 2) DO(real, 16, 8, 1) DO(real, 32, 8, 1) DO(real, 32, 16, 1) DO(real, 8, 8, 8) \
-    DO(real, 7, 8, 8) DO(real, 8, 8, 5)
-// Shapes with a learned-weights instance (the default shapes of both precisions).
-#define OLB_FUSED_LEARNED_CASES(real, DO) DO(real, 8, 8, 4) DO(real, 16, 8, 2) DO(real, 32, 16, 1)
+// advanced at once (KP lanes of TX*TY threads rounded up to whole warps).  FP32:
+// those of TILE_X/TILE_Y/TILE_K in olb_internal.cuh; FP64: those that
+// stage_shape maps them to.  OLB_FUSED_LEARNED_*: with learned weights.
+#define OLB_FUSED_SHAPES_float(DO) \
+    DO(float, 8, 8, 4) DO(float, 16, 8, 2) DO(float, 16, 8, 1) DO(float, 32, 8, 1) DO(float, 32, 16, 1) \
+    DO(float, 8, 8, 8) DO(float, 7, 8, 8) DO(float, 8, 8, 5)
+#define OLB_FUSED_SHAPES_double(DO) DO(double, 8, 8, 4) DO(double, 8, 8, 8) DO(double, 7, 8, 8) DO(double, 8, 8, 5)
+#define OLB_FUSED_LEARNED_float(DO) DO(float, 8, 8, 4) DO(float, 16, 8, 2) DO(float, 32, 16, 1)
+#define OLB_FUSED_LEARNED_double(DO) DO(double, 8, 8, 4)
 #define OLB_FUSED_PREP_CASE(real, A, B, C) \
-    if (!learned && tx == A && ty == B && kp == C) return fused_prepare_one<real, A, B, C>();
+    if (!learned && sh.tx == A && sh.ty == B && sh.kp == C) return fused_prepare_one<real, A, B, C>();
 #define OLB_FUSED_PREP_LEARNED(real, A, B, C) \
-    if (learned && tx == A && ty == B && kp == C) return fused_prepare_one<real, A, B, C, true>();
-#define OLB_FUSED_LAUNCH_CASE(real, A, B, C)           \
-    if (!mlp && tx == A && ty == B && kp == C)          \
+    if (learned && sh.tx == A && sh.ty == B && sh.kp == C) return fused_prepare_one<real, A, B, C, true>();
+#define OLB_FUSED_LAUNCH_CASE(real, A, B, C)                  \
+    if (!mlp && sh.tx == A && sh.ty == B && sh.kp == C)        \
         return fused_launch_one<real, A, B, C>(fs, fn, out, status, g, t, c, mlp, tma, fields, s);
-#define OLB_FUSED_LAUNCH_LEARNED(real, A, B, C)                 \
-    if (mlp && tx == A && ty == B && kp == C)                   \
+#define OLB_FUSED_LAUNCH_LEARNED(real, A, B, C)               \
+    if (mlp && sh.tx == A && sh.ty == B && sh.kp == C)         \
         return fused_launch_one<real, A, B, C, true>(fs, fn, out, status, g, t, c, mlp, tma, fields, s);
 #define OLB_FUSED_BATCH_CASE(real, A, B, C)                                                                  \
-    if (tx == A && ty == B && kp == C)                                                                       \
+    if (sh.tx == A && sh.ty == B && sh.kp == C)                                                              \
         return fused_batch_launch_one<real, A, B, C>(fs, fn, out, status, runs, tile_start, nruns, total, t,     \
-                                                     c, fields, node_start, total_nodes, tmaps, s);
+                                                     c, st, fields, node_start, total_nodes, tmaps, s);
 #define OLB_DEFINE_FUSED(real)                                                                                \
     cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned)                                   \
     {                                                                                                         \
-        OLB_FUSED_SHAPE_CASES(real, OLB_FUSED_PREP_CASE)                                                      \
-        OLB_FUSED_LEARNED_CASES(real, OLB_FUSED_PREP_LEARNED)                                                 \
+        const Shape sh = stage_shape(sizeof(real) == 8, learned, tx, ty, kp);                                 \
+        OLB_FUSED_SHAPES_##real(OLB_FUSED_PREP_CASE)                                                          \
+        OLB_FUSED_LEARNED_##real(OLB_FUSED_PREP_LEARNED)                                                      \
         return cudaErrorInvalidValue;                                                                         \
     }                                                                                                         \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,            \
                              const Tab<real> &t, StageCoef c, int tx, int ty, int kp, const float *mlp,       \
                              const TmaMap *tma, void *fields, cudaStream_t s)                                 \
     {                                                                                                         \
-        OLB_FUSED_SHAPE_CASES(real, OLB_FUSED_LAUNCH_CASE)                                                    \
-        OLB_FUSED_LEARNED_CASES(real, OLB_FUSED_LAUNCH_LEARNED)                                               \
+        const Shape sh = stage_shape(sizeof(real) == 8, mlp != nullptr, tx, ty, kp);                          \
+        OLB_FUSED_SHAPES_##real(OLB_FUSED_LAUNCH_CASE)                                                        \
+        OLB_FUSED_LEARNED_##real(OLB_FUSED_LAUNCH_LEARNED)                                                    \
         return cudaErrorInvalidValue;                                                                         \
     }                                                                                                         \
     cudaError_t launch_fused_batch(const real *fs, const real *fn, real *out, int *status, const void *runs,  \
                                    const int *tile_start, int nruns, int total, const Tab<real> &t,         \
-                                   StageCoef c, int tx, int ty, int kp, void *fields,                         \
+                                   StageCoef c, int st, int tx, int ty, int kp, void *fields,                 \
                                    const long long *node_start, long long total_nodes, const TmaMap *tmaps,   \
                                    cudaStream_t s)                                                            \
     {                                                                                                         \
-        OLB_FUSED_SHAPE_CASES(real, OLB_FUSED_BATCH_CASE)                                                     \
+        const Shape sh = stage_shape(sizeof(real) == 8, false, tx, ty, kp);                                   \
+        OLB_FUSED_SHAPES_##real(OLB_FUSED_BATCH_CASE)                                                         \
         return cudaErrorInvalidValue;                                                                         \
     }                                                                                                         \
     size_t batch_run_bytes(real *) { return sizeof(BatchRun<real>); }                                         \
@@ -1543,6 +1484,9 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
         r.off = off;                                                                                          \
         r.foff = foff;                                                                                        \
         r.ntx = ntx;                                                                                          \
+        const StageCoef c[3] = {{0.0, 1.0, g.dt}, {0.75, 0.25, 0.25 * g.dt}, {1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0 * g.dt}}; \
+        if (sizeof(real) == 8)                                                                                \
+            for (int st = 0; st < 3; ++st) r.k[st] = stage_constants(g, c[st]);                               \
         *static_cast<BatchRun<real> *>(dst) = r;                                                              \
     }
 

@@ -44,9 +44,34 @@ struct Geo {
     double ds, inv_ds, inv_ds3, dt, inv_tau, sigma, a, b;
 };
 
+// An unevaluated sum h + l of two floats (olb_ff.cuh).
+struct ff {
+    float h, l;
+};
+
+// The matrix D of the momentum derivative by parity, for FP64's stage kernel
+// (dp_line in olb_stage64.cuh), and the constants of one of its RK-3 stages, as
+// float-floats.
+struct FfTab {
+    ff E[3][2], O[2][3];
+};
+struct StageK {
+    ff cit;     // c / tau, c the coefficient of dt L
+    ff ca;      // the coefficient of f^n (cb = 1 - ca)
+    ff kp, kn;  // c / (5040 ds), c sigma / (2160 ds^3)
+    ff adv[3];  // c |xi| / (6 ds), |xi| the roots 2, 3, 4
+};
+template <typename real>
+struct TabFf {
+};
+template <>
+struct TabFf<double> {
+    FfTab ff;
+};
+
 // Velocity-space tables (Sec. 2.2, 2.3), in the population precision.
 template <typename real>
-struct Tab {
+struct Tab : TabFf<real> {
     real R[NQ];          // roots of He_5, ascending
     real R2[NQ];         // R^2
     real R2lo[NQ];       // R^2 - R2 (the remainder of R^2 in this precision; 0 in FP64)
@@ -65,6 +90,7 @@ double host_g(const HostTables &t, int k, double u, double T);
 
 template <typename real>
 void fill_tab(Tab<real> *tab, const HostTables &h, const double Tw[2], const double uw[2]);
+ff ff_of(double v);
 
 // Parameter validation of olb_create (OLB_OK / OLB_ERR_ARG / OLB_ERR_CFL)
 // and the mapping of CUDA errors to status codes (olb_api.cu).
@@ -96,10 +122,24 @@ __host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);
 
+// The compiled shape that advances tiles of a shape: FP64 tiles of more than 64
+// nodes are advanced as 8 x 8 tiles (their faces, factors and differences fit in
+// shared memory beside the populations; the larger shapes kept one velocity's
+// faces at a time and recomputed per-node terms 25 times).
+struct Shape {
+    int tx, ty, kp;
+};
+inline Shape stage_shape(bool fp64, bool learned, int tx, int ty, int kp)
+{
+    if (fp64 && tx * ty > 64) return {8, 8, learned ? 4 : 5};
+    return {tx, ty, kp};
+}
+
 // RK-3 stage coefficients: out = ca f^n + cb f_s + cc L[f_s] (Eq. rk3).
 struct StageCoef {
     double ca, cb, cc;
 };
+StageK stage_constants(const Geo &g, StageCoef c);
 
 // Launchers, one set per precision (olb_fp64.cu, olb_fp32.cu).  Output
 // pointers of launch_moments_out may be NULL to skip a field.  launch_fused
@@ -112,7 +152,7 @@ struct StageCoef {
                              const float *mlp, const TmaMap *tma, void *fields, cudaStream_t s);       \
     cudaError_t launch_fused_batch(const real *fs, const real *fn, real *out, int *status,             \
                                    const void *runs, const int *tile_start, int nruns, int total,      \
-                                   const Tab<real> &t, StageCoef c, int tx, int ty, int kp,            \
+                                   const Tab<real> &t, StageCoef c, int st, int tx, int ty, int kp,    \
                                    void *fields,                                                       \
                                    const long long *node_start, long long total_nodes,                 \
                                    const TmaMap *tmaps, cudaStream_t s);                               \

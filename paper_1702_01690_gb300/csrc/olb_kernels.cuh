@@ -68,10 +68,11 @@ __device__ __forceinline__ double recip_nr1(double d)
     return fma(r, fma(-d, r, 1.0), r);
 }
 
-// Jiang-Shu value of an interface in FP64, for the stencils that the learned
+// Jiang-Shu correction of an interface in FP64, for the stencils that the learned
 // weights leave to Jiang-Shu in FP64 contexts: a warp takes this beside the
 // network, which fills the FP32 pipe, so it stays on the FP64 pipe (as weno5_ff
-// it measured 50.6 ms against 43.8 ms for two steps of 1024^2).  Same forms as
+// it measured 50.6 ms against 43.8 ms for two steps of 1024^2, when the node
+// updates were in FP64).  Same forms as
 // weno5_ff (olb_ff.cuh).
 //
 // Weights: wbar_q is proportional to delta_q / sigma_q^2.  Multiplying every
@@ -83,7 +84,7 @@ __device__ __forceinline__ double recip_nr1(double d)
 // the vanishing set).  If the products underflow without an exact zero the
 // min-scaled form delta_q (s/sigma_q)^2 is used instead.
 __device__ __forceinline__ double weno5_core(double d01, double d12, double d23, double d34, double q23, double h12,
-                                             double h23, double v2)
+                                             double h23)
 {
     const double s1 = fma(d01, fma(-2.75, d12, d01), h12);
     const double s2 = fma(d12, fma(-1.25, d23, d12), q23);
@@ -113,7 +114,7 @@ __device__ __forceinline__ double weno5_core(double d01, double d12, double d23,
         }
         den = A1 + A2 + A3;
     }
-    return fma(fma(A1, G1, fma(A2, G2, A3 * G3)), recip_nr1(6.0 * den), v2);
+    return fma(A1, G1, fma(A2, G2, A3 * G3)) * recip_nr1(6.0 * den);
 }
 // FP32 populations: the correction c of an interface value (the value minus
 // its upwind node v2, sum_q wbar_q (Fhat^q - v2)) from the first differences

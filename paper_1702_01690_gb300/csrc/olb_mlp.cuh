@@ -167,25 +167,24 @@ __device__ __forceinline__ float learned_corr_net(const float *__restrict__ th, 
     return learned_corr_from(w, e);
 }
 
-// Learned WENO-5 interface value (without p/m) of the upwind-ordered stencil:
-// where any smoothness indicator vanishes the Jiang-Shu weights with Table
-// tab:weno apply (constant ghost layers keep their exact flux), and so do
-// they where the stencil is smooth (min sigma_q >= MLP_GUARD max sigma_q);
-// otherwise v2 + sum_q w_q G_q with the network's weights.  FP64 populations: the guard is
-// taken in FP64; the network and the correction
-// sum_q w_q G_q run in FP32 (the weights carry FP32 error anyway), and the
-// correction is added to v2 in FP64.
-__device__ __forceinline__ double weno5_learned(const float *__restrict__ th, double v0, double v1, double v2, double v3,
-                                                double v4)
+// Learned WENO-5 correction (interface value minus its upwind node, without p/m)
+// from the first differences of the upwind-ordered stencil: where any
+// smoothness indicator vanishes the Jiang-Shu weights with Table tab:weno apply
+// (constant ghost layers keep their exact flux), and so do they where the
+// stencil is smooth (min sigma_q >= MLP_GUARD max sigma_q); otherwise
+// sum_q w_q G_q with the network's weights.  FP64 populations: the guard is
+// taken in FP64; the network and sum_q w_q G_q run in FP32 (the weights carry
+// FP32 error anyway).
+__device__ __forceinline__ double weno5_learned_corr64(const float *__restrict__ th, double d01, double d12, double d23,
+                                                       double d34)
 {
-    const double d01 = v1 - v0, d12 = v2 - v1, d23 = v3 - v2, d34 = v4 - v3;
     if (!learned_guard<double>(d01, d12, d23, d34)) {
         // Jiang-Shu on the same differences
         const double q12 = d12 * d12, q23 = d23 * d23;
-        return weno5_core(d01, d12, d23, d34, q23, 2.5 * q12, 2.5 * q23, v2);
+        return weno5_core(d01, d12, d23, d34, q23, 2.5 * q12, 2.5 * q23);
     }
     const float e[4] = {(float)d01, (float)d12, (float)d23, (float)d34};
-    return v2 + (double)learned_corr_net(th, e);
+    return (double)learned_corr_net(th, e);
 }
 
 // The same for the compensated FP32 storage: the correction sum_q w_q G_q (the
