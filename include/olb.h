@@ -331,8 +331,8 @@ int olb_set_weno_mlp(olb_ctx *ctx, const float *theta);
  * cudaStream_t or NULL) and the call returns after it has completed, with
  * OLB_ERR_DIVERGED if an invalid moment was met, else OLB_OK.
  *
- * The two intermediate RK-3 buffers and the status word live in one
- * file-scope device array of 2 * 25 * OLB_STATIC_MAX_NODES doubles (6.6 MB)
+ * The two intermediate RK-3 buffers, the stage fields and the status word live in
+ * one file-scope device array of 55 * OLB_STATIC_MAX_NODES doubles (7.2 MB)
  * that every GPU which loads the library keeps until the process exits.  The
  * first call on a device looks up that array's device address (with the
  * device current).  All calls share the array and it keeps the last call's contents (the status

@@ -279,27 +279,29 @@ __host__ __device__ __forceinline__ double weno5_face(double v2, double d0, doub
     return fma(1.0 / 6.0, ff_widen(c, s), v2);
 }
 
-// A row or column of N nodes in the upwind direction: node i is p[(i + 3) step]
-// (three nodes behind the row and two ahead of it are read), and the flux
-// difference across it (weno5_flux6) goes to out[i ostep].  Differences, their
-// squares and products and the third differences are formed once for the row.
-// Z: gives the non-linear part of face j instead of the Jiang-Shu weights.
-// The loop over the faces is unrolled by three: unrolled whole, a row is some
-// 2000 instructions and the warps waited for the instruction cache.
+// A row or column of N nodes in the upwind direction: p0[0], p0[halo], p0[2 halo]
+// are the three nodes behind it, p1[i step] its nodes, p2[0] and p2[halo] the two
+// ahead.  The flux difference across node i (weno5_flux6) goes to out[i ostep].
+// Differences, their squares and products and the third differences are formed
+// once for the row.  Z: gives the non-linear part of face j instead of the
+// Jiang-Shu weights.  The loop over the faces is unrolled by three: unrolled
+// whole, a row is some 2000 instructions and the warps waited for the
+// instruction cache.
 struct NoFaces {};
 template <int N, typename Z = NoFaces>
-__device__ __forceinline__ void weno5_row(const double *p, int step, ff *out, int ostep, FfScale s, Z given = {})
+__device__ __forceinline__ void weno5_row(const double *p0, const double *p1, const double *p2, int halo, int step,
+                                          ff *out, int ostep, FfScale s, Z given = {})
 {
     constexpr bool JS = std::is_same<Z, NoFaces>::value;
-    double v = p[0];
-    auto next = [&] {
-        p += step;
+    double v = p0[0];
+    auto next = [&](const double *p) {
         const double b = *p;
         const ff d = ff_split(b - v, s);
         v = b;
         return d;
     };
-    ff f0 = next(), f1 = next(), f2 = next();
+    ff f0 = next(p0 + halo), f1 = next(p0 + 2 * halo), f2 = next(p1);
+    const double *p = p1 + step;
     ff q0, q1, q2, x0, x1, t0, z0 = {0.0f, 0.0f};
     if constexpr (JS) {
         q0 = ff_sqr(f0);
@@ -311,7 +313,12 @@ __device__ __forceinline__ void weno5_row(const double *p, int step, ff *out, in
     }
 #pragma unroll 3
     for (int j = 0; j <= N; ++j) {
-        const ff f3 = next();
+        if (j == N - 1) {
+            p = p2;
+            step = halo;
+        }
+        const ff f3 = next(p);
+        p += step;
         ff z1;
         if constexpr (JS) {
             const ff q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);

@@ -107,6 +107,12 @@ struct Smem32 {
     };
     float fy[KF][TY + 1][TX];
     unsigned long long mbar;  // completion barrier of the TMA copy of phase 1
+
+    // the staged population k at row r and column c of the region; planes lie
+    // plane(r) apart
+    __device__ __forceinline__ float *at(int k, int r, int c) { return &pop[k][r][c]; }
+    __device__ __forceinline__ static constexpr bool staged(int, int) { return true; }
+    __device__ __forceinline__ static constexpr int plane(int) { return HY * HP; }
 };
 
 template <typename real, int TX, int TY, int KP, bool LEARNED>
@@ -362,32 +368,54 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
     return false;
 }
 
-// Phase 1 for a tile whose staged region lies inside the grid: one TMA copy
-// of the box (HX, HY, planes) at (gx0, gy0, 0) of the tensor map into the
-// staging arrays (pop, then the lo planes in FP32, contiguous in the tile's shared memory in
-// the box's order), completion tracked by an mbarrier.  tma_issue starts the
-// copy (all threads call it; it synchronises); tma_finish waits for it with
-// the bounded wait.  If the wait runs out, bit 1 of the status word is set,
-// the copy is waited for once more (bounded) and false is returned: the
-// caller leaves the tile untouched and the CTA stops.  After a completed copy
-// the barrier is invalidated, so that a CTA that stages several tiles
-// initialises it afresh for each.
-template <typename Smem>
-__device__ __forceinline__ void tma_issue(Smem &sm, const TmaMap *tmap, int gx0, int gy0)
+// Phase 1 for a tile whose staged region lies inside the grid: TMA copies of the
+// boxes at (x0, y0) of the tensor maps (TmaMap) into the staging arrays (FP32:
+// pop, then the lo planes, contiguous in the box's order), completion tracked by
+// an mbarrier.  tma_issue starts the copies (all threads call it; it
+// synchronises); tma_finish waits for them with the bounded wait.  If the wait
+// runs out, bit 1 of the status word is set, the copies are waited for once more
+// (bounded) and false is returned: the caller leaves the tile untouched and the
+// CTA stops.  After completed copies the barrier is invalidated.
+__device__ __forceinline__ void tma_load(unsigned dst, const unsigned char *map, int x, int y, unsigned mbar)
 {
-    constexpr unsigned bytes = sizeof(sm.pop) * (sizeof(sm.pop[0][0][0]) == 4 ? 2 : 1);  // FP32: the lo planes too
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(0), "r"(mbar)
+        : "memory");
+}
+template <int TX, int TY, int KP>
+__device__ __forceinline__ unsigned tma_bytes(const Smem32<TX, TY, KP> &sm)
+{
+    return sizeof(sm.pop) + sizeof(sm.pl);
+}
+template <int TX, int TY, int KP>
+__device__ __forceinline__ void tma_copies(Smem32<TX, TY, KP> &sm, const TmaMap *m, int x0, int y0, unsigned mbar)
+{
+    tma_load((unsigned)__cvta_generic_to_shared(&sm.pop[0][0][0]), m->bytes[0], x0 - 4, y0 - 3, mbar);
+}
+template <int TX, int TY, int KP, bool LEARNED>
+__device__ __forceinline__ unsigned tma_bytes(const Smem64<TX, TY, KP, LEARNED> &sm)
+{
+    return sizeof(sm.mid) + sizeof(sm.below) + sizeof(sm.above);
+}
+template <int TX, int TY, int KP, bool LEARNED>
+__device__ __forceinline__ void tma_copies(Smem64<TX, TY, KP, LEARNED> &sm, const TmaMap *m, int x0, int y0, unsigned mbar)
+{
+    tma_load((unsigned)__cvta_generic_to_shared(&sm.mid[0][0][0]), m->bytes[0], x0 - 4, y0, mbar);
+    tma_load((unsigned)__cvta_generic_to_shared(&sm.below[0][0][0]), m->bytes[1], x0, y0 - 3, mbar);
+    tma_load((unsigned)__cvta_generic_to_shared(&sm.above[0][0][0]), m->bytes[1], x0, y0 + TY, mbar);
+}
+template <typename Smem>
+__device__ __forceinline__ void tma_issue(Smem &sm, const TmaMap *tmap, int x0, int y0)
+{
     const unsigned mbar = (unsigned)__cvta_generic_to_shared(&sm.mbar);
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(&sm.pop[0][0][0]);
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-            "[%5];" ::"r"(dst),
-            "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(gx0), "r"(gy0), "r"(0), "r"(mbar)
-            : "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(tma_bytes(sm)) : "memory");
+        tma_copies(sm, tmap, x0, y0, mbar);
     }
     __syncthreads();  // the barrier is initialised before anyone waits on it
 }
@@ -878,16 +906,15 @@ __device__ __forceinline__ bool advance32(Smem32<TX, TY, KP> &sm, const float *f
 // to all runs and passed as a kernel parameter; mlp: the learned network's
 // parameters in shared memory (LEARNED
 // only); tmap: TMA map of fs (of this run, in a batch) for this tile shape,
-// or nullptr; fields: the moments of fs from k_fields, or nullptr to compute
-// them here.  Returns false when the TMA copy timed out (the CTA must stop).
+// or nullptr; fields: the moments of fs from k_fields.  Returns false when the TMA copy timed out (the CTA must stop).
 template <typename real, int TX, int TY, int KP, bool LEARNED = false>
 __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, LEARNED>::type &sm, const real *__restrict__ fs,
                                            const real *fn, real *out, int *__restrict__ status, const Geo &g,
                                            const Tab<real> &t, const Tab<real> &tw, const int x0, const int y0,
                                            const real ca,
                                            const real cb, const real cc, const real ca_lo, const real cb_lo,
-                                           const StageK &sk, const float *mlp = nullptr, const TmaMap *tmap = nullptr,
-                                           const StageFields<real> *fields = nullptr)
+                                           const StageK &sk, const float *mlp, const TmaMap *tmap,
+                                           const StageFields<real> &fields)
 {
     using S = typename StageSmem<real, TX, TY, KP, LEARNED>::type;
     constexpr int NT = S::NT, HX = S::HX, HY = S::HY;
@@ -912,35 +939,35 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
     real pf_ux = 0, pf_uy = 0;
     bool pf_ok = false, pf_node = false;
     int pf_r = 0, pf_c = 0;
-    if (fields != nullptr && tid < HY * (HX - 2)) {
+    if (tid < HY * (HX - 2)) {
         pf_r = tid / (HX - 2);
         pf_c = tid - pf_r * (HX - 2) + 1;
         const int gx = x0 - 4 + pf_c, gyr = y0 - 3 + pf_r;
         pf_ok = !(g.walls && (gx < 0 || gx >= g.nx)) && !(g.spec_y && (gyr < 0 || gyr >= g.ny));
         if (pf_ok) {
             const long long o = (long long)wrap(gyr, g.ny) * g.pitch + wrap(gx, g.nx);
-            pf_n = fields->n[o];
-            pf_dp = fields->dp[o];
+            pf_n = fields.n[o];
+            pf_dp = fields.dp[o];
             const int tr = pf_r - 3, tc = pf_c - 4;
             pf_node = tr >= 0 && tr < TY && tc >= 0 && tc < TX;
             if (pf_node) {
-                pf_ux = fields->ux[o];
-                pf_uy = fields->uy[o];
-                pf_T = fields->T[o];
-                if constexpr (sizeof(real) == 4) pf_E = fields->E[o];
+                pf_ux = fields.ux[o];
+                pf_uy = fields.uy[o];
+                pf_T = fields.T[o];
+                if constexpr (sizeof(real) == 4) pf_E = fields.E[o];
             }
         }
     }
-    // With the moments from the pre-pass, a tile inside the grid touches its
-    // staged populations first in the face pass (no walls, no sides, no
-    // moments to compute), so phases 2-4 run while the copy is in flight
-    const bool defer = inside && fields != nullptr;
+    // A tile inside the grid touches its staged populations first in the face
+    // pass (no walls, no sides), so phases 2-4 run while the copy is in flight
     if (inside) {
-        tma_issue(sm, tmap, x0 - 4, y0 - 3);
-        if (!defer && !tma_finish(sm, status)) return false;
+        tma_issue(sm, tmap, x0, y0);
     } else {
         for (int e = tid; e < HY * HX; e += NT) {
             const int r = e / HX, c = e - r * HX;
+            if (!S::staged(r, c)) continue;
+            real *dst = sm.at(0, r, c);
+            const int dp = S::plane(r);
             int gy = y0 - 3 + r, gx = x0 - 4 + c;
             bool flip_x = false, flip_y = false, zero = false;
             if (gy < 0 || gy >= g.ny) {
@@ -967,7 +994,7 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
             if (zero) {
 #pragma unroll 5
                 for (int k = 0; k < NK; ++k) {
-                    sm.pop[k][r][c] = real(0);
+                    dst[k * dp] = real(0);
                     if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = 0.0f;
                 }
                 continue;
@@ -976,7 +1003,7 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
             if (!flip_x && !flip_y) {
 #pragma unroll 5
                 for (int k = 0; k < NK; ++k) {
-                    sm.pop[k][r][c] = __ldg(src + k * g.plane);
+                    dst[k * dp] = __ldg(src + k * g.plane);
                     if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = __ldg(src + (NK + k) * g.plane);
                 }
             } else {
@@ -985,7 +1012,7 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
 #pragma unroll
                     for (int k2 = 0; k2 < NQ; ++k2) {
                         const int kk = NQ * (flip_x ? NQ - 1 - k1 : k1) + (flip_y ? NQ - 1 - k2 : k2);
-                        sm.pop[NQ * k1 + k2][r][c] = __ldg(src + kk * g.plane);
+                        dst[(NQ * k1 + k2) * dp] = __ldg(src + kk * g.plane);
                         if constexpr (sizeof(real) == 4) sm.pl.lo[NQ * k1 + k2][r][c] = __ldg(src + (NK + kk) * g.plane);
                     }
             }
@@ -993,15 +1020,13 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
     }
     __syncthreads();
 
-    // ---- 2. moments at every fluid position of the region that the 7 x 7
+    // ---- 2. fields at every fluid position of the region that the 7 x 7
     // force stencils reach (columns 1 .. HX-2; ghost positions of walls and
     // specular sides take the reflected fields in phase 3).  A tile at a
     // diffuse wall also computes here, on warps of their own, the wall-face
     // flux of every outgoing velocity in every tile row (Sec. 3.4.2: the
     // WENO-5 face value at the wall from the three nearest fluid nodes and the
-    // two ghosts extrapolated from them) and stores those two ghosts; both
-    // need the phase-1 populations only, and the FP64 units of the
-    // sub-partitions with fewer moment warps have room.
+    // two ghosts extrapolated from them) and stores those two ghosts.
     const bool x_lo = g.walls && x0 == 0;                // ghost columns at x = 0
     const bool x_hi = g.walls && (x0 + TX + 3 >= g.nx);  // ghost columns at x = nx ds
     const bool left_wall = x_lo && g.wall_lo;
@@ -1017,64 +1042,36 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
             top = max(top, a < 0x7ff00000 ? a : 0);
         }
     };
-    if (fields != nullptr) {
-        // moments from the per-node pre-pass (k_fields): n and Delta p on the
-        // region, u, T (FP32: and e) at the tile nodes; item tid was fetched
-        // before phase 1
-        if (pf_ok) {
-            note_n(pf_n);
-            sm.n[pf_r][pf_c] = pf_n;
-            sm.dp[pf_r][pf_c] = pf_dp;
-            if (pf_node) {
-                sm.ux[pf_r - 3][pf_c - 4] = pf_ux;
-                sm.uy[pf_r - 3][pf_c - 4] = pf_uy;
-                sm.T[pf_r - 3][pf_c - 4] = pf_T;
-                if constexpr (sizeof(real) == 4) sm.eng[pf_r - 3][pf_c - 4] = pf_E;
-            }
+    // moments from the per-node pre-pass (k_fields): n and Delta p on the
+    // region, u, T (FP32: and e) at the tile nodes; item tid was fetched
+    // before phase 1
+    if (pf_ok) {
+        note_n(pf_n);
+        sm.n[pf_r][pf_c] = pf_n;
+        sm.dp[pf_r][pf_c] = pf_dp;
+        if (pf_node) {
+            sm.ux[pf_r - 3][pf_c - 4] = pf_ux;
+            sm.uy[pf_r - 3][pf_c - 4] = pf_uy;
+            sm.T[pf_r - 3][pf_c - 4] = pf_T;
+            if constexpr (sizeof(real) == 4) sm.eng[pf_r - 3][pf_c - 4] = pf_E;
         }
-        for (int e = tid + NT; e < HY * (HX - 2); e += NT) {
-            const int r = e / (HX - 2), c = e - r * (HX - 2) + 1;
-            const int gx = x0 - 4 + c, gyr = y0 - 3 + r;
-            if (g.walls && (gx < 0 || gx >= g.nx)) continue;
-            if (g.spec_y && (gyr < 0 || gyr >= g.ny)) continue;
-            const long long o = (long long)wrap(gyr, g.ny) * g.pitch + wrap(gx, g.nx);
-            const fld n = fields->n[o];
-            note_n(n);
-            sm.n[r][c] = n;
-            sm.dp[r][c] = fields->dp[o];
-            const int tr = r - 3, tc = c - 4;
-            if (tr >= 0 && tr < TY && tc >= 0 && tc < TX) {
-                sm.ux[tr][tc] = fields->ux[o];
-                sm.uy[tr][tc] = fields->uy[o];
-                sm.T[tr][tc] = fields->T[o];
-                if constexpr (sizeof(real) == 4) sm.eng[tr][tc] = fields->E[o];
-            }
-        }
-    } else {
-        for (int e = tid; e < HY * (HX - 2); e += NT) {
-            const int r = e / (HX - 2), c = e - r * (HX - 2) + 1;
-            const int gx = x0 - 4 + c, gyr = y0 - 3 + r;
-            if (g.walls && (gx < 0 || gx >= g.nx)) continue;
-            if (g.spec_y && (gyr < 0 || gyr >= g.ny)) continue;
-            const int tr = r - 3, tc = c - 4;
-            const bool tile_node = tr >= 0 && tr < TY && tc >= 0 && tc < TX;
-            const bool own = tile_node && x0 + tc < g.nx && y0 + tr < g.ny;
-            NodeMoments<real> m;
-            if constexpr (sizeof(real) == 8)
-                m = node_moments<real>([&](int k) { return sm.pop[k][r][c]; }, g, t);
-            else
-                m = node_moments<real>([&](int k) { return make_float2(sm.pop[k][r][c], sm.pl.lo[k][r][c]); }, g,
-                                       t);
-            note_n(m.n);
-            sm.n[r][c] = m.n;
-            sm.dp[r][c] = m.dp;
-            if (tile_node) {
-                sm.ux[tr][tc] = m.ux;
-                sm.uy[tr][tc] = m.uy;
-                sm.T[tr][tc] = m.T;
-                if constexpr (sizeof(real) == 4) sm.eng[tr][tc] = m.E;
-                if (own && !m.ok) atomicOr(status, 1);
-            }
+    }
+    for (int e = tid + NT; e < HY * (HX - 2); e += NT) {
+        const int r = e / (HX - 2), c = e - r * (HX - 2) + 1;
+        const int gx = x0 - 4 + c, gyr = y0 - 3 + r;
+        if (g.walls && (gx < 0 || gx >= g.nx)) continue;
+        if (g.spec_y && (gyr < 0 || gyr >= g.ny)) continue;
+        const long long o = (long long)wrap(gyr, g.ny) * g.pitch + wrap(gx, g.nx);
+        const fld n = fields.n[o];
+        note_n(n);
+        sm.n[r][c] = n;
+        sm.dp[r][c] = fields.dp[o];
+        const int tr = r - 3, tc = c - 4;
+        if (tr >= 0 && tr < TY && tc >= 0 && tc < TX) {
+            sm.ux[tr][tc] = fields.ux[o];
+            sm.uy[tr][tc] = fields.uy[o];
+            sm.T[tr][tc] = fields.T[o];
+            if constexpr (sizeof(real) == 4) sm.eng[tr][tc] = fields.E[o];
         }
     }
     if constexpr (sizeof(real) == 8) {
@@ -1102,12 +1099,12 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
         if (v >= 10) {
             // idle lane of the row's half-warp
         } else if constexpr (sizeof(real) == 8) {
-            const real a0 = sm.pop[k][tr + 3][c0], a1 = sm.pop[k][tr + 3][c0 + dc];
-            const real a2 = sm.pop[k][tr + 3][c0 + 2 * dc];
+            const real a0 = *sm.at(k, tr + 3, c0), a1 = *sm.at(k, tr + 3, c0 + dc);
+            const real a2 = *sm.at(k, tr + 3, c0 + 2 * dc);
             const real g0 = fma(real(3), a0 - a1, a2);
             const real g1 = fma(real(6), a0, fma(real(-8), a1, real(3) * a2));
-            if (c0 - dc >= 0 && c0 - dc < HX) sm.pop[k][tr + 3][c0 - dc] = g0;
-            if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) sm.pop[k][tr + 3][c0 - 2 * dc] = g1;
+            if (c0 - dc >= 0 && c0 - dc < HX) *sm.at(k, tr + 3, c0 - dc) = g0;
+            if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) *sm.at(k, tr + 3, c0 - 2 * dc) = g1;
             wf = t.R[k1] * face_value<LEARNED>(mlp, a2, a1, a0, g0, g1);
         } else {
             // pairs: the ghosts 3a0 - 3a1 + a2 and 6a0 - 8a1 + 3a2 as a0 plus
@@ -1179,7 +1176,7 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
                 const int c = side ? g.nx + m - (x0 - 4) : -1 - m - (x0 - 4);
                 if (c < 0 || c >= HX) continue;
                 const int k = NQ * (side ? v / 5 : 3 + v / 5) + v % 5;
-                sm.pop[k][tr + 3][c] = sm.wnw[side][tr] * tw.geqw[side][k];
+                *sm.at(k, tr + 3, c) = sm.wnw[side][tr] * tw.geqw[side][k];
                 if constexpr (sizeof(real) == 4) sm.pl.lo[k][tr + 3][c] = 0.0f;
             }
         }
@@ -1187,7 +1184,7 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
     __syncthreads();
 
     // ---- 4, 5. force, fluxes, collision and RK-3 combination
-    auto wait = [&] { return !defer || tma_finish(sm, status); };
+    auto wait = [&] { return !inside || tma_finish(sm, status); };
     if constexpr (sizeof(real) == 8)
         return advance64<TX, TY, KP, LEARNED>(sm, fn, out, g, t, t.ff, sk, x0, y0, mlp, wait);
     else
@@ -1230,15 +1227,18 @@ constexpr int fused_min_ctas(size_t smem_bytes, int threads, int cap = 0)
     return n < 1 ? 1 : (cap > 0 && n > cap ? cap : n);
 }
 
-// Single grid: one CTA per tile.  FP64 takes two CTAs per SM (its strips need
-// the registers).  Learned-weight instances leave their network the registers
+// FP64's lines of faces need more than the 40 registers that three CTAs of eight
+// lanes leave.
+constexpr int stage_cta_cap(bool fp64, int kp) { return fp64 && kp > 5 ? 2 : 0; }
+
+// Single grid: one CTA per tile.  Learned-weight instances leave their network the registers
 // it needs: FP32 (tensor-pipe network) at most two CTAs per SM, FP64 (per-thread
 // network) one.
 template <typename real, int TX, int TY, int KP, bool LEARNED>
 __global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
                                   fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, LEARNED>(),
                                                  stage_threads<TX, TY, KP>(),
-                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : (sizeof(real) == 4 ? 0 : 2)))
+                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : stage_cta_cap(sizeof(real) == 8, KP)))
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
         real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
@@ -1259,7 +1259,7 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
     }
     stage_tile<real, TX, TY, KP, LEARNED>(sm, fs, fn, out, status, g, t, t, blockIdx.x * TX, blockIdx.y * TY, ca, cb,
                                           cc, ca_lo, cb_lo, sk, mlp_sm, tma.on ? &tma.map : nullptr,
-                                          fields.n ? &fields : nullptr);
+                                          fields);
 }
 
 // Batch of independent runs (uneven grid sizes, own parameters): one CTA per
@@ -1288,7 +1288,7 @@ static_assert(sizeof(BatchRun<float>) % 16 == 0, "BatchRun<float> must be a whol
 template <typename real, int TX, int TY, int KP>
 __global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
                                   fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, false>() + sizeof(BatchRun<real>),
-                                                 stage_threads<TX, TY, KP>(), sizeof(real) == 4 ? 0 : 2))
+                                                 stage_threads<TX, TY, KP>(), stage_cta_cap(sizeof(real) == 8, KP)))
 k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
               const BatchRun<real> *__restrict__ runs, const int *__restrict__ tile_start, int nruns,
               const __grid_constant__ Tab<real> tv, real ca, real cb, real ccoef, real ca_lo, real cb_lo, int st,
@@ -1313,15 +1313,16 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
     __syncthreads();
     const int lt = item - __ldg(tile_start + lo);
     const int x0 = (lt % run.ntx) * TX, y0 = (lt / run.ntx) * TY;
-    const StageFields<real> fl = fields ? fields_of<real>(fields + run.foff, run.g) : StageFields<real>{};
+    const StageFields<real> fl = fields_of<real>(fields + run.foff, run.g);
     // the run's tensor map of fs lives in global memory, written by the host
     // before the launch: acquire it for the tensormap proxy before the thread
     // that issues the copy uses it
     const TmaMap *tm = tmaps ? tmaps + lo : nullptr;
     if (tm && threadIdx.x == 0)
-        asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm) : "memory");
+        for (int k = 0; k < 2; ++k)
+            asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm->bytes[k]) : "memory");
     stage_tile<real, TX, TY, KP>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
-                                 ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, run.k[st], nullptr, tm, fields ? &fl : nullptr);
+                                 ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, run.k[st], nullptr, tm, fl);
 }
 
 // The moments pre-pass for a batch: one thread per node of every run (a
@@ -1387,13 +1388,10 @@ cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *sta
         tma.map = *tmap;
         tma.on = 1;
     }
-    StageFields<real> fl{};
-    if (fields) {
-        // the moments of fs first (one thread per node), then the stage
-        fl = fields_of<real>(fields, g);
-        const long long N = (long long)g.nx * g.ny;
-        k_fields<real><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
-    }
+    // the moments of fs first (one thread per node), then the stage
+    const StageFields<real> fl = fields_of<real>(fields, g);
+    const long long N = (long long)g.nx * g.ny;
+    k_fields<real><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
     k_fused<real, TX, TY, KP, LEARNED><<<grid, stage_threads<TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, LEARNED>(), s>>>(
         fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
         (real)(c.cb - (double)(real)c.cb), sizeof(real) == 8 ? stage_constants(g, c) : StageK{}, mlp, tma, fl);
@@ -1407,7 +1405,7 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
                                    const TmaMap *tmaps, cudaStream_t s)
 {
     if (total < 1) return cudaSuccess;
-    if (fields && total_nodes > 0) {
+    if (total_nodes > 0) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -101,14 +101,18 @@ bool fields_admissible(const double *n, const double *ux, const double *uy, cons
 void set_sides(Geo *g, const ::olb_params *p);
 int cuda_status(cudaError_t e);
 
-// A TMA tensor map (CUtensorMap, 128 bytes, 64-byte aligned) over one
-// population buffer as a 3-D tensor [planes][ny][nx] with row stride pitch,
-// box (TX + 8) x (TY + 6) x planes: the staged region of a tile in one copy.
+// TMA tensor maps (CUtensorMap, 128 bytes, 64-byte aligned) over one population
+// buffer as a 3-D tensor [planes][ny][nx] with row stride pitch.  FP32: one box
+// (pitch of a staged row) x (TY + 6) x planes, the staged region of a tile.
+// FP64: the rows of the tile, (pitch of a staged row) x TY x planes, and the
+// three rows above or below its nodes, TX x 3 x planes: the corners of the
+// region, which no face reads, are left out (39 KB instead of 51 KB for an
+// 8 x 8 tile, and three CTAs on an SM instead of two).
 struct alignas(64) TmaMap {
-    unsigned char bytes[128];
+    unsigned char bytes[2][128];
 };
-// Kernel argument: the map and whether to use it (tiles whose staged region
-// lies inside the grid are loaded with one TMA copy when on != 0).
+// Kernel argument: the maps and whether to use them (tiles whose staged region
+// lies inside the grid are loaded by TMA when on != 0).
 struct alignas(64) TmaArg {
     TmaMap map;
     int on;
@@ -118,7 +122,7 @@ struct alignas(64) TmaArg {
 // tile start 4 banks apart (rows of TX + 8 doubles are whole multiples of the 32
 // banks or halves of it, and the strips of a warp would queue for two banks).
 __host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 8 + (fp64 && tx % 2 == 0 ? 2 : 0); }
-// Encode the map of buffer `base` for tile shape tx x ty (olb_api.cu); false
+// Encode the maps of buffer `base` for tile shape tx x ty (olb_api.cu); false
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);
 
@@ -143,8 +147,8 @@ StageK stage_constants(const Geo &g, StageCoef c);
 
 // Launchers, one set per precision (olb_fp64.cu, olb_fp32.cu).  Output
 // pointers of launch_moments_out may be NULL to skip a field.  launch_fused
-// with fields != NULL (a buffer of fields_bytes(g)) runs the per-node
-// moments pre-pass first and lets the stage kernel read its results.
+// runs the per-node moments pre-pass into fields (a buffer of fields_bytes(g)),
+// then the stage kernel, which reads them.
 #define OLB_DECLARE_LAUNCHERS(real)                                                                    \
     cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned);                           \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,     \

@@ -35,43 +35,63 @@ struct Smem64 {
     static constexpr int HX = TX + 8, HY = TY + 6, NN = TX * TY, LS = (NN + 31) / 32 * 32, NT = LS * KP;
     static constexpr int HP = region_pitch(TX, true);
     static_assert(NN <= 64, "FP64 tiles hold at most 64 nodes");
-    double pop[NK][HY][HP];
-    double n[HY][HX];
-    double dp[HY][HX];
-    double ux[TY][TX];
-    double uy[TY][TX];
-    double T[TY][TX];
+    // populations of the tile's rows (columns x0 - 4 ...) and of the three rows
+    // below and above its nodes
+    alignas(128) double mid[NK][TY][HP];
+    alignas(128) double below[NK][3][TX];
+    alignas(128) double above[NK][3][TX];
     double ex[NQ][NN];  // n g_q(u_x, T) and g_q(u_y, T) of the tile nodes
     double ey[NQ][NN];
-    ff sum[4][NN];      // stencil sums: Delta p along x, y, then n along x, y
     ff G[2][NN];        // c F
     union {
-        // differences v(+l) - v(-l), l = 1..3, of Delta p and n, along x for
-        // every row of the region and along y for every column that a stencil
-        // of the tile reaches: a value serves the seven nodes of a stencil row
+        // phases 2 to 4: fields of the region, and differences v(+l) - v(-l),
+        // l = 1..3, of Delta p and n, along x for every row of the region and
+        // along y for every column that a stencil of the tile reaches: a value
+        // serves the seven nodes of a stencil row
         struct {
+            double n[HY][HX];
+            double dp[HY][HX];
+            double ux[TY][TX];
+            double uy[TY][TX];
+            double T[TY][TX];
             ff dx[2][3][HY][TX];
             ff dy[2][3][TY][TX + 6];
         };
-        // flux differences times 6 (weno5_flux6) across the nodes of each row
-        // along x and column along y, of the 20 velocities that move along the
-        // axis (slot_x, slot_y; learned weights: first the faces' non-linear
-        // parts, one more than nodes, which the flux differences then replace);
-        // ax then holds the sum of a velocity's advection and y force terms
+        // phase 5: flux differences times 6 (weno5_flux6) across the nodes of
+        // each row along x and column along y, of the 20 velocities that move
+        // along the axis (slot_x, slot_y; learned weights: first the faces'
+        // non-linear parts, one more than nodes, which the flux differences then
+        // replace); then, in place of one of a velocity's flux differences (inc),
+        // the sum of its advection and y force terms
         struct {
-            ff ax[NK][TY][TX + 1];
+            ff ax[20][TY][TX + 1];
             ff ay[20][TX][TY + 1];
+            ff rest[NN];
         };
-        double wnw[2][TY];  // wall density of each tile row (Eq. nw), before the force
     };
-    ff f[NK][NN];       // populations of the tile nodes, scaled
+    double wnw[2][TY];        // wall density of each tile row (Eq. nw)
     int top;                  // high word of the largest n of the region (the tile's scale)
-    unsigned long long mbar;  // completion barrier of the TMA copy
+    unsigned long long mbar;  // completion barrier of the TMA copies
+
+    // the staged population k at row r and column c of the region; planes lie
+    // plane(r) apart; the corners of the region are not staged
+    __device__ __forceinline__ double *at(int k, int r, int c)
+    {
+        return r < 3 ? &below[k][r][c - 4] : r < TY + 3 ? &mid[k][r - 3][c] : &above[k][r - TY - 3][c - 4];
+    }
+    __device__ __forceinline__ static constexpr bool staged(int r, int c)
+    {
+        return (r >= 3 && r < TY + 3) || (c >= 4 && c < TX + 4);
+    }
+    __device__ __forceinline__ static constexpr int plane(int r) { return r >= 3 && r < TY + 3 ? TY * HP : 3 * TX; }
+    __device__ __forceinline__ ff &inc(int k1, int k2, int x, int y)
+    {
+        return k1 != 2 ? ax[NQ * (k1 < 2 ? k1 : k1 - 1) + k2][y][x] : k2 != 2 ? ay[8 + (k2 < 2 ? k2 : k2 - 1)][x][y] : rest[y * TX + x];
+    }
 };
 
-// Slots of ax for the velocities with xi_x != 0 (k1 != 2; the five others follow
-// them) and of ay for those with xi_y != 0.
-__device__ __forceinline__ int slot_x(int k1, int k2) { return NQ * (k1 < 2 ? k1 : k1 > 2 ? k1 - 1 : 4) + k2; }
+// Slots of ax for the velocities with xi_x != 0 and of ay for those with xi_y != 0.
+__device__ __forceinline__ int slot_x(int k1, int k2) { return NQ * (k1 < 2 ? k1 : k1 - 1) + k2; }
 __device__ __forceinline__ int slot_y(int k1, int k2) { return 4 * k1 + (k2 < 2 ? k2 : k2 - 1); }
 
 // ---------------------------------------------------------------- stencils
@@ -167,7 +187,7 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
     const int tid = threadIdx.x;
     const FfScale sc = ff_scale(sm.top);
 
-    // ---- 4a. differences of the fields; equilibrium factors on the last threads
+    // ---- 4a. differences of the fields
     constexpr int NX = 3 * HY * TX, NY = 3 * TY * (TX + 6);
     for (int e = tid; e < 2 * (NX + NY); e += NT) {
         const int field = e >= NX + NY;
@@ -182,47 +202,45 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
             (&sm.dy[field][0][0][0])[q] = ff_split(v[y + 3 + l][x + 1] - v[y + 3 - l][x + 1], sc);
         }
     }
-    for (int e = tid - (NT - 128); e < 2 * NN; e += NT) {
-        if (e < 0) continue;
-        const int node = e < NN ? e : e - NN, x = node % TX, y = node / TX;
-        double w[NQ];
-        eq_factors64(t, e < NN ? sm.ux[y][x] : sm.uy[y][x], sm.T[y][x], w);
-        const double n = e < NN ? sm.n[y + 3][x + 4] : 1.0;
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) (e < NN ? sm.ex : sm.ey)[q][node] = e < NN ? n * w[q] : w[q];
-    }
     __syncthreads();
 
-    // ---- 4b. stencil sums of grad(Delta p) and grad(Laplacian n)
-    for (int e = tid; e < 4 * NN; e += NT) {
-        const int which = e / NN, node = e - which * NN, x = node % TX, y = node / TX;
-        ff s;
-        if (which == 0) s = stencil_sum<false>([&](int l, int m) { return sm.dx[0][l - 1][y + 3 + m][x]; });
-        else if (which == 1) s = stencil_sum<false>([&](int l, int m) { return sm.dy[0][l - 1][y][x + 3 + m]; });
-        else if (which == 2) s = stencil_sum<true>([&](int l, int m) { return sm.dx[1][l - 1][y + 3 + m][x]; });
-        else s = stencil_sum<true>([&](int l, int m) { return sm.dy[1][l - 1][y][x + 3 + m]; });
-        sm.sum[which][node] = s;
-    }
-    if (!wait()) return false;
-    __syncthreads();
-
-    // ---- 4c. G = c F = (c/ds) sum_dp / n + (c sigma/ds^3) sum_n, with the
-    // scale that the fields' differences still carry taken out of 1/n and sum_n
-    for (int e = tid; e < 2 * NN; e += NT) {
-        const int a = e / NN, node = e - a * NN;
-        const ff n = ff_split(sm.n[node / TX + 3][node % TX + 4], sc);
+    // ---- 4b. on the first 128 threads G = c F = (c/ds) sum_dp / n + (c sigma/ds^3)
+    // sum_n from the stencil sums of grad(Delta p) and grad(Laplacian n), a node
+    // and axis a thread (the scale that the differences carry is taken out of
+    // 1/n and sum_n); on the next 128, meanwhile, the equilibrium factors (FP64)
+    static_assert(NT >= 256, "phase 4b takes 256 threads");
+    if (tid < 2 * NN) {
+        const int a = tid / NN, node = tid - a * NN, x = node % TX, y = node / TX;
+        ff sp, sn;
+        if (a == 0) {
+            sp = stencil_sum<false>([&](int l, int m) { return sm.dx[0][l - 1][y + 3 + m][x]; });
+            sn = stencil_sum<true>([&](int l, int m) { return sm.dx[1][l - 1][y + 3 + m][x]; });
+        } else {
+            sp = stencil_sum<false>([&](int l, int m) { return sm.dy[0][l - 1][y][x + 3 + m]; });
+            sn = stencil_sum<true>([&](int l, int m) { return sm.dy[1][l - 1][y][x + 3 + m]; });
+        }
+        const ff n = ff_split(sm.n[y + 3][x + 4], sc);
         const float r = rcp_seed(n.h);
         const ff inv = {r, r * fmaf(-r, n.l, fmaf(-r, n.h, 1.0f))};
-        ff v = ff_mul(ff_mul(sm.sum[a][node], inv), c.kp);
-        const ff w = ff_mul(sm.sum[2 + a][node], c.kn);
-        // sum_n in the populations' units is 2^-k of the scaled one
+        ff v = ff_mul(ff_mul(sp, inv), c.kp);
+        const ff w = ff_mul(sn, c.kn);
+        // sum_n in the populations' units is 2^k of the scaled one
         const int k = 127 - 1023 - (sc.off >> 20);
         const int k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
         const float u1 = f32_make((unsigned)(k1 + 127) << 23), u2 = f32_make((unsigned)(k2 + 127) << 23);
         v.l += w.l * u1 * u2;
         ff_acc(v, w.h * u1 * u2);
         sm.G[a][node] = ff_norm(v);
+    } else if (tid >= 128 && tid < 128 + 2 * NN) {
+        const int a = (tid - 128) / NN, node = tid - 128 - a * NN, x = node % TX, y = node / TX;
+        double w[NQ];
+        eq_factors64(t, a == 0 ? sm.ux[y][x] : sm.uy[y][x], sm.T[y][x], w);
+        const double n = sm.n[y + 3][x + 4];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) (a == 0 ? sm.ex : sm.ey)[q][node] = a == 0 ? n * w[q] : w[q];
     }
+    if (!wait()) return false;
+    __syncthreads();
 
     // ---- 5a. flux differences, a tile row or column a thread
     if constexpr (LEARNED) {
@@ -235,11 +253,10 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
             const int r = along_x ? f / (TX + 1) : f / TX, cc = along_x ? f - r * (TX + 1) : f - r * TX;
             if (along_x ? (y0 + r >= g.ny || x0 + cc > g.nx) : (x0 + cc >= g.nx || y0 + r > g.ny)) continue;
             const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-            const double *p = along_x ? &sm.pop[k][3 + r][up ? cc + 1 : cc + 6] : &sm.pop[k][up ? r : r + 5][4 + cc];
-            const int step = (along_x ? 1 : HP) * (up ? 1 : -1);
             double v[5];
 #pragma unroll
-            for (int m = 0; m < 5; ++m) v[m] = p[m * step];
+            for (int m = 0; m < 5; ++m)
+                v[m] = along_x ? sm.mid[k][r][up ? cc + 1 + m : cc + 6 - m] : *sm.at(k, up ? r + m : r + 5 - m, 4 + cc);
             const double d1 = v[2] - v[1], d2 = v[3] - v[2];
             const ff corr = ff_split(weno5_learned_corr64(mlp, v[1] - v[0], d1, d2, v[4] - v[3]), sc);
             // z = d1 + 2 d2 - 6 (F - v2)
@@ -258,15 +275,29 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
     auto line = [&](auto n, bool along_x, int q, int i) {
         const int k = along_x ? (q < 2 * NQ ? q : q + NQ) : (q >> 2) * NQ + ((q & 3) < 2 ? (q & 3) : (q & 3) + 1);
         const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-        const int step = along_x ? 1 : HP;
-        const double *p = &sm.pop[k][along_x ? 3 + i : 0][along_x ? 1 : 4 + i] + (up ? 0 : (decltype(n)::value + 5) * step);
+        constexpr int N = decltype(n)::value;
+        // the three nodes behind the line, its nodes, and the two ahead
+        const double *p0, *p1, *p2;
+        int step = up ? 1 : -1, halo = step;
+        if (along_x) {
+            const double *row = &sm.mid[k][i][0];
+            p0 = row + (up ? 1 : TX + 6);
+            p1 = row + (up ? 4 : TX + 3);
+            p2 = row + (up ? TX + 4 : 3);
+        } else {
+            halo = step * TX;
+            step *= HP;
+            p0 = up ? &sm.below[k][0][i] : &sm.above[k][2][i];
+            p1 = &sm.mid[k][up ? 0 : TY - 1][4 + i];
+            p2 = up ? &sm.above[k][0][i] : &sm.below[k][2][i];
+        }
         ff *o = along_x ? &sm.ax[q][i][0] : &sm.ay[q][i][0];
         // (the flux difference across a node takes the place of a face that it has used)
         if constexpr (LEARNED)
-            weno5_row<decltype(n)::value>(p, up ? step : -step, o + (up ? 0 : decltype(n)::value - 1), up ? 1 : -1, sc,
-                                          [&](int j) { return o[up ? j : decltype(n)::value - j]; });
+            weno5_row<N>(p0, p1, p2, halo, step, o + (up ? 0 : N - 1), up ? 1 : -1, sc,
+                         [&](int j) { return o[up ? j : N - j]; });
         else
-            weno5_row<decltype(n)::value>(p, up ? step : -step, o + (up ? 0 : decltype(n)::value - 1), up ? 1 : -1, sc);
+            weno5_row<N>(p0, p1, p2, halo, step, o + (up ? 0 : N - 1), up ? 1 : -1, sc);
     };
     for (int e = tid; e < 20 * (TY + TX); e += NT) {
         const bool along_x = e < 20 * TY;
@@ -295,12 +326,12 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
         }
 
     // ---- 5b. a row of velocities (k1; k2 = 0..4) of a node a thread: the y force
-    // term and both advection terms of its velocities, added up in ax
+    // term and both advection terms of its velocities
     for (int e = tid; e < NQ * NN; e += NT) {
         const int k1 = e / NN, node = e - k1 * NN, x = node % TX, y = node / TX;
         ff f[NQ], d[NQ];
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) sm.f[NQ * k1 + q][node] = f[q] = ff_split(sm.pop[NQ * k1 + q][y + 3][x + 4], sc);
+        for (int q = 0; q < NQ; ++q) f[q] = ff_split(sm.mid[NQ * k1 + q][y][x + 4], sc);
         dp_line(ft, f, d);
         const ff Gy = sm.G[1][node];
         const ff K1 = c.adv[k1 < 2 ? 2 - k1 : k1 - 2];
@@ -317,7 +348,7 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
                 s.l += v.l;
                 ff_acc(s, v.h);
             }
-            sm.ax[slot_x(k1, k2)][y][x] = s;
+            sm.inc(k1, k2, x, y) = s;
         }
     }
     __syncthreads();
@@ -332,8 +363,8 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
         ff f[NQ], d[NQ];
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            fv[q] = sm.pop[NQ * q + k2][y + 3][x + 4];
-            f[q] = sm.f[NQ * q + k2][node];
+            fv[q] = sm.mid[NQ * q + k2][y][x + 4];
+            f[q] = ff_split(fv[q], sc);
         }
         dp_line(ft, f, d);
         const ff Gx = sm.G[0][node];
@@ -350,7 +381,7 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
                 s.l += v.l;
                 ff_acc(s, v.h);
             }
-            const ff a = sm.ax[slot_x(k1, k2)][y][x], b = ff_mul(Gx, d[k1]);
+            const ff a = sm.inc(k1, k2, x, y), b = ff_mul(Gx, d[k1]);
             s.l -= a.l + b.l;
             ff_acc(s, -a.h);
             ff_acc(s, -b.h);

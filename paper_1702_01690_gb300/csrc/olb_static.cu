@@ -7,8 +7,8 @@
 // other work), and some host applications hand all device memory to their
 // own pool up front or run the library as a plug-in that may not touch the
 // allocator at all.  Such a caller owns the populations; the two
-// intermediate RK-3 buffers and the status word live in one file-scope
-// device array instead, sized for grids of at most OLB_STATIC_MAX_NODES
+// intermediate RK-3 buffers, the stage fields and the status word live in one
+// file-scope device array instead, sized for grids of at most OLB_STATIC_MAX_NODES
 // nodes, which every GPU that loads the library holds until the process ends.
 //
 // The array's name is only a host-side stand-in in host code; its device
@@ -25,8 +25,9 @@ using namespace olb;
 namespace {
 
 constexpr long long kMaxNodes = OLB_STATIC_MAX_NODES;
-// f^(1), f^(2) as [25][ny][nx] each, then 256 bytes for the status word.
-constexpr long long kScratchDoubles = 2LL * NK * kMaxNodes + 32;
+// f^(1), f^(2) as [25][ny][nx] each, then the stage fields (fields_bytes: five
+// values a node) and 256 bytes for the status word.
+constexpr long long kScratchDoubles = (2LL * NK + 5) * kMaxNodes + 32;
 
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
@@ -110,10 +111,11 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
 
     double *f1 = scratch;
     double *f2 = scratch + (long long)NK * g.plane;
-    int *status = reinterpret_cast<int *>(scratch + 2LL * NK * kMaxNodes);
+    double *fields = scratch + 2LL * NK * kMaxNodes;
+    int *status = reinterpret_cast<int *>(fields + 5 * kMaxNodes);
     cudaStream_t s = (cudaStream_t)stream;
 
-    // shape, as olb_create picks it for FP64: 8 x 8 nodes with 4 velocity
+    // shape, as olb_create picks it for FP64: 8 x 8 nodes with 5 velocity
     // lanes, or 7 x 8 nodes with 8 lanes when that lowers the most nodes one
     // SM advances (grids here have at most 256 tiles, a wave or two)
     int sms = 0;
@@ -126,7 +128,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
         return (tiles + sms - 1) / sms * tx_ * ty_;
     };
     const bool narrow = most_nodes(7, 8) < most_nodes(8, 8);
-    const int tx = narrow ? 7 : 8, ty = 8, kp = narrow ? 8 : 4;
+    const int tx = narrow ? 7 : 8, ty = 8, kp = narrow ? 8 : 5;
     cudaError_t e = prepare_fused((double *)nullptr, tx, ty, kp, false);
     // the scratch keeps the previous call's contents: the status word must start at zero
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
@@ -136,7 +138,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
     double *dst[3] = {f1, f2, f};
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k)
         for (int st = 0; st < 3 && e == cudaSuccess; ++st)
-            e = launch_fused(src[st], f, dst[st], status, g, tab, coef[st], tx, ty, kp, nullptr, nullptr, nullptr, s);
+            e = launch_fused(src[st], f, dst[st], status, g, tab, coef[st], tx, ty, kp, nullptr, nullptr, fields, s);
     int hstatus = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, status, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
