@@ -218,10 +218,11 @@ int olb_profile(olb_ctx *ctx, int nsteps, double *ms, int *launches);
  * at once (kp lanes of tx*ty threads, each rounded up to whole warps).
  * Compiled shapes (tx, ty, kp): (8,8,4), (16,8,2), (16,8,1), (32,8,1),
  * (32,16,1), (8,8,8), (7,8,8), (8,8,5); olb_create picks one from the
- * grid size ((8,8,5), FP64: or (7,8,8) when that lowers the most nodes one SM
- * advances; (8,8,4) with learned weights).  With
- * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  FP64 tiles of more than
- * 64 nodes are advanced as 8 x 8 tiles by CTAs of their own.  olb_set_tile returns
+ * grid size ((8,8,5), FP64: or (8,8,8) on grids of at most one tile an SM;
+ * (8,8,4) with learned weights).  With
+ * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  FP64 tiles are
+ * advanced as 8 x 8 tiles whatever the shape, by 320 threads each with kp = 8
+ * and by 160 otherwise (learned weights: 256).  olb_set_tile returns
  * OLB_ERR_ARG for any other shape; results do not depend on the shape.
  * Not part of the paper (a tuning knob). */
 int olb_set_tile(olb_ctx *ctx, int tx, int ty, int kp);
@@ -332,7 +333,7 @@ int olb_set_weno_mlp(olb_ctx *ctx, const float *theta);
  * OLB_ERR_DIVERGED if an invalid moment was met, else OLB_OK.
  *
  * The two intermediate RK-3 buffers, the stage fields and the status word live in
- * one file-scope device array of 55 * OLB_STATIC_MAX_NODES doubles (7.2 MB)
+ * one file-scope device array of 57 * OLB_STATIC_MAX_NODES doubles (7.5 MB)
  * that every GPU which loads the library keeps until the process exits.  The
  * first call on a device looks up that array's device address (with the
  * device current).  All calls share the array and it keeps the last call's contents (the status

@@ -396,12 +396,10 @@ static cudaError_t prepare_tile(olb_ctx *c)
 }
 
 // Default shape, the fastest measured on a GB300 for each precision: 8 x 8
-// nodes with 5 velocity lanes (the faces of all 25 velocities fit in shared
-// memory, so a stage has one face pass and one barrier; FP64: the 320 strips of
-// the face pass are one per thread), except that small FP64 grids take 7 x 8
-// tiles with 8 lanes when that lowers the most nodes any SM has to advance
-// (1024 x 8: 147 tiles of 56 nodes rather than 128 of 64 on 152 SMs).  Learned
-// weights: 4 lanes.  olb_set_tile overrides.
+// nodes with 5 velocity lanes (FP32: the faces of all 25 velocities fit in shared
+// memory, so a stage has one face pass and one barrier; FP64: 160 threads, two
+// nodes each), FP64 grids of at most one tile an SM 8 lanes (320 threads, Plan64
+// in olb_stage64.cuh).  Learned weights: 4 lanes.  olb_set_tile overrides.
 static void default_tile(olb_ctx *c)
 {
     int dev = 0, sms = 0;
@@ -409,13 +407,9 @@ static void default_tile(olb_ctx *c)
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
     const bool learned = c->p.weno_mode == OLB_WENO_LEARNED;
     const bool fp64 = is_fp64(c);
-    const int narrow = 6;
-    auto tiles = [&](int k) {
-        return (long long)((c->geo.nx + TILE_X[k] - 1) / TILE_X[k]) * ((c->geo.ny + TILE_Y[k] - 1) / TILE_Y[k]);
-    };
-    auto most_nodes = [&](int k) { return (tiles(k) + sms - 1) / sms * TILE_X[k] * TILE_Y[k]; };
+    const long long tiles = (long long)((c->geo.nx + 7) / 8) * ((c->geo.ny + 7) / 8);
     int k = learned ? 0 : 7;
-    if (fp64 && !learned && most_nodes(narrow) < most_nodes(k)) k = narrow;
+    if (fp64 && !learned && tiles <= sms) k = 5;
     c->tx = TILE_X[k];
     c->ty = TILE_Y[k];
     c->kp = TILE_K[k];
@@ -466,7 +460,7 @@ extern "C" int olb_create(const olb_params *p, void *stream, olb_ctx **out)
     c->mlp = p->weno_mode == OLB_WENO_LEARNED ? (float *)ctx_alloc(c, 1348 * sizeof(float)) : nullptr;
     // olb_totals: TOTALS_BLOCKS x 4 partial sums, then the 4 sums
     c->totals = (double *)ctx_alloc(c, (size_t)(4 * TOTALS_BLOCKS + 4) * sizeof(double));
-    c->fields = ctx_alloc(c, fields_bytes(g));
+    c->fields = ctx_alloc(c, fields_bytes(g, is_fp64(c)));
     default_tile(c);
     bool ok = c->f[0] && c->f[1] && c->f[2] && c->status && c->stage4 && c->totals && c->fields &&
               (p->weno_mode != OLB_WENO_LEARNED || c->mlp);

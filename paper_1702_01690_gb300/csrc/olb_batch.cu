@@ -51,6 +51,8 @@ struct olb_batch {
     void *fields = nullptr;              // stage fields of every run (moments pre-pass)
     std::vector<long long> foff;         // byte offset of each run's fields
     long long *node_start = nullptr;     // [count + 1] prefix sum of the runs' node counts
+    int *force_start = nullptr;          // [count + 1] prefix sum of the runs' force blocks (FP64)
+    int total_force = 0;
     long long total_nodes = 0;
     long long max_nodes = 0;
     TmaMap *tmaps = nullptr;             // [3][count] tensor maps (runs x buffers) for the current shape
@@ -142,7 +144,7 @@ static cudaError_t batch_stage(olb_batch *b, int st, cudaStream_t s)
     const TmaMap *maps = b->tma_ok ? b->tmaps + (size_t)st * b->count : nullptr;
     return launch_fused_batch(src[st], f0, dst[st], b->status, b->runs, b->tile_start, b->count, b->total_tiles,
                               batch_tab(b, (real *)nullptr), coef[st], st, b->tx, b->ty, b->kp, b->fields, b->node_start,
-                              b->total_nodes, maps, s);
+                              b->total_nodes, b->force_start, b->total_force, maps, s);
 }
 
 static cudaError_t batch_enqueue_steps(olb_batch *b, int n, cudaStream_t s)
@@ -181,6 +183,7 @@ static void batch_free(olb_batch *b)
     cudaFree(b->stage4);
     cudaFree(b->fields);
     cudaFree(b->node_start);
+    cudaFree(b->force_start);
     cudaFree(b->tmaps);
 }
 
@@ -227,6 +230,7 @@ extern "C" int olb_batch_create(const olb_params *runs, int count, void *stream,
     b->foff.resize(count);
     long long acc = 0, facc = 0;
     std::vector<long long> nstart(count + 1, 0);
+    std::vector<int> fstart(count + 1, 0);
     for (int r = 0; r < count; ++r) {
         const olb_params *p = &runs[r];
         Geo &g = b->geo[r];
@@ -248,8 +252,9 @@ extern "C" int olb_batch_create(const olb_params *runs, int count, void *stream,
         b->off[r] = acc;
         acc += ((long long)(b_fp64(b) ? pop_planes<double>() : pop_planes<float>()) * g.plane + 63) / 64 * 64;
         b->foff[r] = facc;
-        facc += ((long long)fields_bytes(g) + 255) / 256 * 256;
+        facc += ((long long)fields_bytes(g, b_fp64(b)) + 255) / 256 * 256;
         nstart[r + 1] = nstart[r] + (long long)g.nx * g.ny;
+        fstart[r + 1] = fstart[r] + force_blocks(g);
         b->max_nodes = std::max(b->max_nodes, (long long)g.nx * g.ny);
     }
     b->total_elems = acc;
@@ -275,7 +280,12 @@ extern "C" int olb_batch_create(const olb_params *runs, int count, void *stream,
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->node_start, nstart.data(), (size_t)(count + 1) * sizeof(long long),
                             cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&b->force_start, (size_t)(count + 1) * sizeof(int));
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->force_start, fstart.data(), (size_t)(count + 1) * sizeof(int), cudaMemcpyHostToDevice,
+                            b->stream);
     b->total_nodes = nstart[count];
+    b->total_force = fstart[count];
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMemsetAsync(b->f[k], 0, (size_t)acc * b->elt, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status, 0, (size_t)count * sizeof(int), b->stream);
     if (e == cudaSuccess) e = batch_prepare(b);
@@ -516,7 +526,7 @@ extern "C" int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, in
             b->ty = TILE_Y[q];
             b->kp = TILE_K[q];
             const Shape sh = stage_shape(b_fp64(b), false, b->tx, b->ty, b->kp);
-            if (sh.tx != b->tx || sh.ty != b->ty) continue;  // advanced as another shape of the list
+            if (sh.tx != b->tx || sh.ty != b->ty || sh.kp != b->kp) continue;  // advanced as another shape of the list
             if (batch_prepare(b) != cudaSuccess) {
                 cudaGetLastError();
                 continue;  // shape does not fit this precision

@@ -144,75 +144,202 @@ __host__ __device__ __forceinline__ double ff_widen(float v, FfScale s, bool l)
 }
 __host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s) { return ff_widen(v.h, s, false) + ff_widen(v.l, s, true); }
 
+// ---------------------------------------------------------------- one or two floats
+// The arithmetic below is written for a vector V of one float or of two (the
+// packed instructions fma.rn.f32x2 and so on of sm_100 and later: the same
+// operations as two scalar ones in one issue slot; measured on a GB300, FFMA
+// starts 114 lanes per clock and SM, FFMA2 63, and a negated operand is free in
+// both).  Results do not depend on V.
+struct vf1 {
+    static constexpr int W = 1;
+    float v;
+    __host__ __device__ __forceinline__ static vf1 all(float a) { return {a}; }
+    __host__ __device__ __forceinline__ static vf1 of(const float *a) { return {a[0]}; }
+    __host__ __device__ __forceinline__ float operator[](int) const { return v; }
+};
+__host__ __device__ __forceinline__ vf1 operator+(vf1 a, vf1 b) { return {a.v + b.v}; }
+__host__ __device__ __forceinline__ vf1 operator-(vf1 a, vf1 b) { return {a.v - b.v}; }
+__host__ __device__ __forceinline__ vf1 operator*(vf1 a, vf1 b) { return {a.v * b.v}; }
+__host__ __device__ __forceinline__ vf1 operator-(vf1 a) { return {-a.v}; }
+__host__ __device__ __forceinline__ vf1 vfma(vf1 a, vf1 b, vf1 c) { return {fmaf(a.v, b.v, c.v)}; }
+
+struct vf2 {
+    static constexpr int W = 2;
+    unsigned long long v;
+    __device__ __forceinline__ static vf2 pair(float a, float b)
+    {
+        vf2 r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+        return r;
+    }
+    __device__ __forceinline__ static vf2 all(float a) { return pair(a, a); }
+    __device__ __forceinline__ static vf2 of(const float *a) { return pair(a[0], a[1]); }
+    __device__ __forceinline__ float operator[](int i) const
+    {
+        float a, b;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+        return i ? b : a;
+    }
+};
+__device__ __forceinline__ vf2 operator+(vf2 a, vf2 b)
+{
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a.v) : "l"(b.v));
+    return a;
+}
+__device__ __forceinline__ vf2 operator-(vf2 a, vf2 b)
+{
+    asm("sub.rn.f32x2 %0, %0, %1;" : "+l"(a.v) : "l"(b.v));
+    return a;
+}
+__device__ __forceinline__ vf2 operator*(vf2 a, vf2 b)
+{
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(a.v) : "l"(b.v));
+    return a;
+}
+__device__ __forceinline__ vf2 operator-(vf2 a) { return vf2::pair(-a[0], -a[1]); }
+__device__ __forceinline__ vf2 vfma(vf2 a, vf2 b, vf2 c)
+{
+    vf2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+template <typename V, int = V::W>
+__host__ __device__ __forceinline__ V operator*(float a, V b)
+{
+    return V::all(a) * b;
+}
+template <typename V, int = V::W>
+__host__ __device__ __forceinline__ V vfma(float a, V b, V c)
+{
+    return vfma(V::all(a), b, c);
+}
+
+// W float-floats.
+template <typename V>
+struct ffv {
+    V h, l;
+};
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_all(ff a)
+{
+    return {V::all(a.h), V::all(a.l)};
+}
+template <typename V>
+__host__ __device__ __forceinline__ ff ff_lane(ffv<V> a, int i)
+{
+    return {a.h[i], a.l[i]};
+}
+// ff_split of W values
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_split(const double (&d)[V::W], FfScale s)
+{
+    float h[V::W], l[V::W];
+#pragma unroll
+    for (int i = 0; i < V::W; ++i) {
+        const ff f = ff_split(d[i], s);
+        h[i] = f.h;
+        l[i] = f.l;
+    }
+    return {V::of(h), V::of(l)};
+}
+
 // ---------------------------------------------------------------- float-float arithmetic
 // (error-free transformations of Dekker and Knuth; -fmad=false keeps every
 // product and sum as written)
 
 // (h, l) += b, with the rounding error of the sum kept in l (TwoSum).
-__host__ __device__ __forceinline__ void ff_acc(ff &s, float b)
+template <typename V>
+__host__ __device__ __forceinline__ void ff_acc(ffv<V> &s, V b)
 {
-    const float r = s.h + b, t = r - s.h;
-    s.l += (s.h - (r - t)) + (b - t);
+    const V r = s.h + b, t = r - s.h;
+    s.l = s.l + ((s.h - (r - t)) + (b - t));
     s.h = r;
+}
+template <typename V>
+__host__ __device__ __forceinline__ void ff_acc(ffv<V> &s, ffv<V> b)
+{
+    s.l = s.l + b.l;
+    ff_acc(s, b.h);
 }
 // (h, l) += k b for a short constant k: the sum's error as in TwoSum, with
 // the remainder of the unrounded product k b from an FMA.  Exact up to 2^-47 of
 // the larger term where h and k b have one sign, or k is a power of two.
-__host__ __device__ __forceinline__ void ff_acck(ff &s, float k, float b)
+template <typename V>
+__host__ __device__ __forceinline__ void ff_acck(ffv<V> &s, float k, V b)
 {
-    const float r = fmaf(k, b, s.h), t = r - s.h;
-    s.l += (s.h - (r - t)) + fmaf(k, b, -t);
+    const V r = vfma(k, b, s.h), t = r - s.h;
+    s.l = s.l + ((s.h - (r - t)) + vfma(k, b, -t));
     s.h = r;
 }
 // (h, l) -= k b where |h| >= |k b| is known (the product split exactly, then
 // Fast2Sum: with cancellation k b has to be a float for its sum to be exact).
-__host__ __device__ __forceinline__ void ff_subk_small(ff &s, float k, float b)
+template <typename V>
+__host__ __device__ __forceinline__ void ff_subk_small(ffv<V> &s, float k, V b)
 {
-    const float z = k * b, r = s.h - z, t = r - s.h;
-    s.l = (s.l - fmaf(k, b, -z)) - (z + t);
+    const V z = k * b, r = s.h - z, t = r - s.h;
+    s.l = (s.l - vfma(k, b, -z)) - (z + t);
     s.h = r;
 }
-__host__ __device__ __forceinline__ ff ff_norm(ff a)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_norm(ffv<V> a)
 {
-    const float s = a.h + a.l;
+    const V s = a.h + a.l;
     return {s, a.l - (s - a.h)};
 }
 // a b without the product of the low parts (below 2^-46 of a b)
-__host__ __device__ __forceinline__ ff ff_mul(ff a, ff b)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_mul(ffv<V> a, ffv<V> b)
 {
-    const float p = a.h * b.h;
-    return {p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
+    const V p = a.h * b.h;
+    return {p, vfma(a.l, b.h, vfma(a.h, b.l, vfma(a.h, b.h, -p)))};
 }
-__host__ __device__ __forceinline__ ff ff_sqr(ff a)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_mul(ff a, ffv<V> b)
 {
-    const float p = a.h * a.h;
-    return {p, fmaf(a.h + a.h, a.l, fmaf(a.h, a.h, -p))};
+    return ff_mul(ff_all<V>(a), b);
+}
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_sqr(ffv<V> a)
+{
+    const V p = a.h * a.h;
+    return {p, vfma(a.h + a.h, a.l, vfma(a.h, a.h, -p))};
 }
 // d0 - 2 d1 + d2
-__host__ __device__ __forceinline__ ff ff_diff2(ff d0, ff d1, ff d2)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_diff2(ffv<V> d0, ffv<V> d1, ffv<V> d2)
 {
-    ff s = {d0.h, fmaf(-2.0f, d1.l, d0.l + d2.l)};
+    ffv<V> s = {d0.h, vfma(-2.0f, d1.l, d0.l + d2.l)};
     ff_acc(s, d2.h);
     ff_acck(s, -2.0f, d1.h);
-    return ff_norm(s);
+    return s;  // (a sum that cancels leaves l as large as h: both only go into products)
 }
-// a p + b q - c x for the indicators (a, b >= 0, p, q squares, x the product of
-// their roots with |c x| <= a p + b q)
-__host__ __device__ __forceinline__ ff ff_form(ff p, float b, ff q, float c, ff x)
+// p + b q - c x for the indicators (p, q squares, x the product of their roots
+// with |c x| <= p + b q)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_form(ffv<V> p, float b, ffv<V> q, float c, ffv<V> x)
 {
-    ff s = {p.h, fmaf(-c, x.l, fmaf(b, q.l, p.l))};
+    ffv<V> s = {p.h, vfma(-c, x.l, vfma(b, q.l, p.l))};
     ff_acck(s, b, q.h);
     ff_subk_small(s, c, x.h);
     return s;
 }
+template <typename V, int = V::W>
+__host__ __device__ __forceinline__ V rcp_seed(V a)
+{
+    float r[V::W];
+#pragma unroll
+    for (int i = 0; i < V::W; ++i) r[i] = rcp_seed(a[i]);
+    return V::of(r);
+}
 // u with u u = (m / s)^2 up to 2^-44, as a float-float square: the seed
 // r ~ 1/s leaves e = 1 - r s, and (m r)^2 (1 + 2 e) is (m / s)^2 to O(e^2).
-__host__ __device__ __forceinline__ ff ff_inv2(ff s, float m)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> ff_inv2(ffv<V> s, V m)
 {
-    const float r = rcp_seed(s.h);
-    const float e = fmaf(-r, s.l, fmaf(-r, s.h, 1.0f));
-    const float a = m * r, p = a * a;
-    return {p, fmaf(p, e + e, fmaf(a, a, -p))};
+    const V r = rcp_seed(s.h);
+    const V e = vfma(-r, s.l, vfma(-r, s.h, V::all(1.0f)));
+    const V a = m * r, p = a * a;
+    return {p, vfma(p, e + e, vfma(a, a, -p))};
 }
 
 // ---------------------------------------------------------------- WENO-5
@@ -227,28 +354,33 @@ __host__ __device__ __forceinline__ ff ff_inv2(ff s, float m)
 //   sigma_1 = d0^2 - 11/4 d0 d1 + 5/2 d1^2,  sigma_2 = d1^2 - 5/4 d1 d2 + d2^2,
 //   sigma_3 = d3^2 - 11/4 d2 d3 + 5/2 d2^2,
 // each positive definite with condition number below 19.  q_j = d_j^2 and
-// x_j = d_j d_{j+1} are shared by the faces of a strip.  Weights are scaled by
+// x_j = d_j d_{j+1} are shared by the faces of a line.  Weights are scaled by
 // the power of two m below the smallest indicator.  Where an indicator
 // vanishes (both its differences are zero) the weights are those of Table
 // tab:weno (see ff_split).  Returns z.
-__host__ __device__ __forceinline__ ff weno5_ff(ff q0, ff q1, ff q2, ff q3, ff x0, ff x1, ff x2, ff t0, ff t1)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> weno5_ff(ffv<V> q0, ffv<V> q1, ffv<V> q2, ffv<V> q3, ffv<V> x0, ffv<V> x1,
+                                                    ffv<V> x2, ffv<V> t0, ffv<V> t1)
 {
-    const ff s1 = ff_form(q0, 2.5f, q1, 2.75f, x0);
-    const ff s2 = ff_form(q1, 1.0f, q2, 1.25f, x1);
-    const ff s3 = ff_form(q3, 2.5f, q2, 2.75f, x2);
-    const float m = f32_make(f32_bits(fminf(s1.h, fminf(s2.h, s3.h))) & 0x7f800000u);
-    const ff w1 = ff_inv2(s1, m), w2 = ff_inv2(s2, m), w3 = ff_inv2(s3, m);  // (m / sigma_q)^2
+    const ffv<V> s1 = ff_form(q0, 2.5f, q1, 2.75f, x0);
+    const ffv<V> s2 = ff_form(q1, 1.0f, q2, 1.25f, x1);
+    const ffv<V> s3 = ff_form(q3, 2.5f, q2, 2.75f, x2);
+    float mi[V::W];
+#pragma unroll
+    for (int i = 0; i < V::W; ++i) mi[i] = f32_make(f32_bits(fminf(s1.h[i], fminf(s2.h[i], s3.h[i]))) & 0x7f800000u);
+    const V m = V::of(mi);
+    const ffv<V> w1 = ff_inv2(s1, m), w2 = ff_inv2(s2, m), w3 = ff_inv2(s3, m);  // (m / sigma_q)^2
     // weights 1 : 6 : 3 times w (delta_q times 10)
-    ff den = {w1.h, fmaf(3.0f, w3.l, fmaf(6.0f, w2.l, w1.l))};
+    ffv<V> den = {w1.h, vfma(3.0f, w3.l, vfma(6.0f, w2.l, w1.l))};
     ff_acck(den, 6.0f, w2.h);
     ff_acck(den, 3.0f, w3.h);
-    const ff a = ff_mul(w1, t0), b = ff_mul(w3, t1);
-    const float b3 = 3.0f * b.h;
-    ff num = {a.h + a.h, fmaf(2.0f, a.l, fmaf(3.0f, b.l, fmaf(3.0f, b.h, -b3)))};
+    const ffv<V> a = ff_mul(w1, t0), b = ff_mul(w3, t1);
+    const V b3 = 3.0f * b.h;
+    ffv<V> num = {a.h + a.h, vfma(2.0f, a.l, vfma(3.0f, b.l, vfma(3.0f, b.h, -b3)))};
     ff_acc(num, b3);
     // num / den: quotient of the leading parts and its remainder
-    const float r = rcp_seed(den.h), z = num.h * r;
-    return {z, (fmaf(-z, den.l, fmaf(-z, den.h, num.h)) + num.l) * r};
+    const V r = rcp_seed(den.h), z = num.h * r;
+    return {z, (vfma(-z, den.l, vfma(-z, den.h, num.h)) + num.l) * r};
 }
 
 // The flux difference across a node, in the upwind direction and times 6: the
@@ -256,53 +388,65 @@ __host__ __device__ __forceinline__ ff weno5_ff(ff q0, ff q1, ff q2, ff q3, ff x
 // are z1 and z0.  With v the node, db = v - (node behind), d = the difference
 // before db's and da = (node ahead) - v, the linear parts add up to
 // 2 da + 5 db - dbb.
-__host__ __device__ __forceinline__ ff weno5_flux6(ff dbb, ff db, ff da, ff z0, ff z1)
+template <typename V>
+__host__ __device__ __forceinline__ ffv<V> weno5_flux6(ffv<V> dbb, ffv<V> db, ffv<V> da, ffv<V> z0, ffv<V> z1)
 {
-    const float b5 = 5.0f * db.h;
-    ff s = {2.0f * da.h, fmaf(2.0f, da.l, fmaf(5.0f, db.l, fmaf(5.0f, db.h, -b5))) - dbb.l + (z0.l - z1.l)};
+    const V b5 = 5.0f * db.h;
+    ffv<V> s = {2.0f * da.h, vfma(2.0f, da.l, vfma(5.0f, db.l, vfma(5.0f, db.h, -b5))) - dbb.l + (z0.l - z1.l)};
     ff_acc(s, b5);
     ff_acc(s, -dbb.h);
     ff_acc(s, z0.h);
     ff_acc(s, -z1.h);
-    return ff_norm(s);
+    return s;
 }
 
 // The value of one face from its upwind node and first differences, in FP64.
 __host__ __device__ __forceinline__ double weno5_face(double v2, double d0, double d1, double d2, double d3, FfScale s)
 {
-    const ff f0 = ff_split(d0, s), f1 = ff_split(d1, s), f2 = ff_split(d2, s), f3 = ff_split(d3, s);
-    const ff z = weno5_ff(ff_sqr(f0), ff_sqr(f1), ff_sqr(f2), ff_sqr(f3), ff_mul(f0, f1), ff_mul(f1, f2),
-                          ff_mul(f2, f3), ff_diff2(f0, f1, f2), ff_diff2(f1, f2, f3));
-    ff c = {f1.h, fmaf(2.0f, f2.l, f1.l) - z.l};
+    using F = ffv<vf1>;
+    const double d[4][1] = {{d0}, {d1}, {d2}, {d3}};
+    const F f0 = ff_split<vf1>(d[0], s), f1 = ff_split<vf1>(d[1], s), f2 = ff_split<vf1>(d[2], s),
+            f3 = ff_split<vf1>(d[3], s);
+    const F z = weno5_ff(ff_sqr(f0), ff_sqr(f1), ff_sqr(f2), ff_sqr(f3), ff_mul(f0, f1), ff_mul(f1, f2), ff_mul(f2, f3),
+                         ff_diff2(f0, f1, f2), ff_diff2(f1, f2, f3));
+    F c = {f1.h, vfma(2.0f, f2.l, f1.l) - z.l};
     ff_acc(c, 2.0f * f2.h);
     ff_acc(c, -z.h);
-    return fma(1.0 / 6.0, ff_widen(c, s), v2);
+    return fma(1.0 / 6.0, ff_widen(ff_lane(c, 0), s), v2);
 }
 
-// A row or column of N nodes in the upwind direction: p0[0], p0[halo], p0[2 halo]
-// are the three nodes behind it, p1[i step] its nodes, p2[0] and p2[halo] the two
-// ahead.  The flux difference across node i (weno5_flux6) goes to out[i ostep].
+// W rows or columns of N nodes (W the floats of V) in the upwind direction, each
+// `lane` elements after the one before: p0[0], p0[halo], p0[2 halo] are the three
+// nodes behind a line, p1[i step] its nodes, p2[0] and p2[halo] the two ahead.
+// store(i, v) takes the flux difference across node i (weno5_flux6).
 // Differences, their squares and products and the third differences are formed
-// once for the row.  Z: gives the non-linear part of face j instead of the
+// once for the line.  Z: gives the non-linear part of face j instead of the
 // Jiang-Shu weights.  The loop over the faces is unrolled by three: unrolled
-// whole, a row is some 2000 instructions and the warps waited for the
+// whole, a line is some 2000 instructions and the warps waited for the
 // instruction cache.
 struct NoFaces {};
-template <int N, typename Z = NoFaces>
-__device__ __forceinline__ void weno5_row(const double *p0, const double *p1, const double *p2, int halo, int step,
-                                          ff *out, int ostep, FfScale s, Z given = {})
+template <int N, typename V, typename Store, typename Z = NoFaces>
+__device__ __forceinline__ void weno5_line(const double *p0, const double *p1, const double *p2, int lane, int halo,
+                                           int step, FfScale s, Store store, Z given = {})
 {
     constexpr bool JS = std::is_same<Z, NoFaces>::value;
-    double v = p0[0];
+    double v[V::W];
+#pragma unroll
+    for (int i = 0; i < V::W; ++i) v[i] = p0[i * lane];
     auto next = [&](const double *p) {
-        const double b = *p;
-        const ff d = ff_split(b - v, s);
-        v = b;
-        return d;
+        double d[V::W];
+#pragma unroll
+        for (int i = 0; i < V::W; ++i) {
+            const double b = p[i * lane];
+            d[i] = b - v[i];
+            v[i] = b;
+        }
+        return ff_split<V>(d, s);
     };
-    ff f0 = next(p0 + halo), f1 = next(p0 + 2 * halo), f2 = next(p1);
+    ffv<V> f0 = next(p0 + halo), f1 = next(p0 + 2 * halo), f2 = next(p1);
     const double *p = p1 + step;
-    ff q0, q1, q2, x0, x1, t0, z0 = {0.0f, 0.0f};
+    const V zero = V::all(0.0f);
+    ffv<V> q0, q1, q2, x0, x1, t0, z0 = {zero, zero};
     if constexpr (JS) {
         q0 = ff_sqr(f0);
         q1 = ff_sqr(f1);
@@ -317,11 +461,11 @@ __device__ __forceinline__ void weno5_row(const double *p0, const double *p1, co
             p = p2;
             step = halo;
         }
-        const ff f3 = next(p);
+        const ffv<V> f3 = next(p);
         p += step;
-        ff z1;
+        ffv<V> z1;
         if constexpr (JS) {
-            const ff q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);
+            const ffv<V> q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);
             z1 = weno5_ff(q0, q1, q2, q3, x0, x1, x2, t0, t1);
             q0 = q1; q1 = q2; q2 = q3;
             x0 = x1; x1 = x2;
@@ -329,10 +473,7 @@ __device__ __forceinline__ void weno5_row(const double *p0, const double *p1, co
         } else {
             z1 = given(j);
         }
-        if (j > 0) {
-            *out = weno5_flux6(f0, f1, f2, z0, z1);
-            out += ostep;
-        }
+        if (j > 0) store(j - 1, weno5_flux6(f0, f1, f2, z0, z1));
         z0 = z1;
         f0 = f1; f1 = f2; f2 = f3;
     }

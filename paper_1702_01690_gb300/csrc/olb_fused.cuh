@@ -32,42 +32,19 @@
 // momentum), and the RK-3 combination is done in double-float arithmetic.
 #pragma once
 
-#include "olb_mlp.cuh"
+#include "olb_fields.cuh"
 #include "olb_stage64.cuh"
+#include "olb_tile.cuh"
 
 namespace olb {
 
-// n and Delta p of the region, kept for the 49-point stencils.  The stencils
-// cancel to O(ds^k) of their terms on fine grids, so the FP32 kernel keeps
-// each value as an unevaluated sum hi + lo of two floats (hi = the value
-// rounded to FP32, lo = the FP64 remainder rounded to FP32): differences of
-// neighbouring values then keep ~FP64 accuracy at FP32 cost.
-template <typename real>
-struct FieldT {
-    using type = double;
-};
-template <>
-struct FieldT<float> {
-    using type = float2;
-};
-
-__device__ __forceinline__ double make_field(double v, double) { return v; }
-__device__ __forceinline__ float2 make_field(double v, float)
-{
-    const float hi = __double2float_rn(v);
-    return make_float2(hi, __double2float_rn(v - (double)hi));
-}
-__device__ __forceinline__ double field_diff(double a, double b) { return a - b; }
-__device__ __forceinline__ float field_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
-__device__ __forceinline__ double field_val(double a) { return a; }
-__device__ __forceinline__ float field_val(float2 a) { return a.x + a.y; }
-
 // Shared memory of an FP32 tile (FP64: Smem64 in olb_stage64.cuh).
-template <int TX, int TY, int KP>
+template <int TX_, int TY_, int KP>
 struct Smem32 {
     // LS: threads per velocity lane, the tile's nodes rounded up to whole
     // warps (so that every lane starts on a warp); NT threads in all;
     // HP: pitch of a staged row of populations (region_pitch)
+    static constexpr int TX = TX_, TY = TY_;
     static constexpr int HX = TX + 8, HY = TY + 6, NN = TX * TY, LS = (NN + 31) / 32 * 32, NT = LS * KP;
     static constexpr int HP = region_pitch(TX, false);
     using fld = FieldT<float>::type;
@@ -113,6 +90,11 @@ struct Smem32 {
     __device__ __forceinline__ float *at(int k, int r, int c) { return &pop[k][r][c]; }
     __device__ __forceinline__ static constexpr bool staged(int, int) { return true; }
     __device__ __forceinline__ static constexpr int plane(int) { return HY * HP; }
+    static constexpr int TMA_BYTES = 2 * NK * HY * HP * 4;
+    __device__ __forceinline__ void tma(const TmaMap *m, int x0, int y0, unsigned mbar)
+    {
+        tma_load((unsigned)__cvta_generic_to_shared(&pop[0][0][0]), m->bytes[0], x0 - 4, y0 - 3, mbar);
+    }
 };
 
 template <typename real, int TX, int TY, int KP, bool LEARNED>
@@ -121,7 +103,8 @@ struct StageSmem {
 };
 template <int TX, int TY, int KP, bool LEARNED>
 struct StageSmem<double, TX, TY, KP, LEARNED> {
-    using type = Smem64<TX, TY, KP, LEARNED>;
+    static_assert(TX == 8 && TY == 8, "FP64 tiles are 8 x 8 (stage_shape)");
+    using type = Smem64<KP, LEARNED>;
 };
 
 template <typename real>
@@ -133,305 +116,6 @@ __device__ __forceinline__ real sel5(const real v[NQ], int k)
     r = (k == 3) ? v[3] : r;
     r = (k == 4) ? v[4] : r;
     return r;
-}
-
-// Face value of one upwind-ordered FP64 stencil: Jiang-Shu weights, or the
-// learned network's (parameters in shared memory) when LEARNED.
-template <bool LEARNED>
-__device__ __forceinline__ double face_value(const float *mlp, double v0, double v1, double v2, double v3, double v4)
-{
-    if constexpr (LEARNED)
-        return v2 + weno5_learned_corr64(mlp, v1 - v0, v2 - v1, v3 - v2, v4 - v3);
-    else
-    {
-        auto high = [](double v) { return __double2hiint(v) & 0x7fffffff; };
-        const FfScale s = ff_scale(max(max(max(high(v0), high(v1)), max(high(v3), high(v4))), high(v2)));
-        return weno5_face(v2, v1 - v0, v2 - v1, v3 - v2, v4 - v3, s);
-    }
-}
-
-// FP32 pairs: the correction c (face value minus the upwind node v2) of the
-// stencil with first differences d01 .. d34.
-template <bool LEARNED>
-__device__ __forceinline__ float face_corr(const float *mlp, float d01, float d12, float d23, float d34)
-{
-    if constexpr (LEARNED)
-        return weno5_learned_corr(mlp, d01, d12, d23, d34);
-    else
-        return weno5_corr(d01, d12, d23, d34);
-}
-
-// ---------------------------------------------------------------- moments of a node
-// n, u, T and Delta p of one node from its 25 populations (Sec. 2.2; T from
-// the trace of Eq. sigmaq_def; Delta p = n T - p^w, Eq. vdw), and whether they
-// are admissible (finite, n > 0, T > 0, b n < 1).  get(k) returns population
-// k: the value (FP64) or the pair hi + lo (FP32).
-template <typename real>
-struct NodeMoments;
-template <>
-struct NodeMoments<double> {
-    double n, dp, ux, uy, T;
-    bool ok;
-};
-template <>
-struct NodeMoments<float> {
-    float2 n, dp, T, E;  // hi + lo pairs (E = sum |p|^2 f)
-    float ux, uy;
-    bool ok;
-};
-
-template <typename real, typename Get>
-__device__ __forceinline__ NodeMoments<real> node_moments(Get get, const Geo &g, const Tab<real> &t)
-{
-    NodeMoments<real> m;
-    if constexpr (sizeof(real) == 8) {
-        // row and column sums of the 5 x 5 populations; the middle root is 0
-        // (R[2] = R2[2] = 0), so its sums drop out of j and e
-        double sx[NQ], sy[NQ];
-#pragma unroll
-        for (int k1 = 0; k1 < NQ; ++k1) {
-            double s = get(NQ * k1);
-            if (k1 == 0) sy[0] = s;
-            else sy[0] += s;
-#pragma unroll
-            for (int k2 = 1; k2 < NQ; ++k2) {
-                const double v = get(NQ * k1 + k2);
-                s += v;
-                if (k1 == 0) sy[k2] = v;
-                else sy[k2] += v;
-            }
-            sx[k1] = s;
-        }
-        double n = sx[0];
-        double jx = t.R[0] * sx[0];
-        double jy = t.R[0] * sy[0];
-        double en = t.R2[0] * (sx[0] + sy[0]);
-#pragma unroll
-        for (int k = 1; k < NQ; ++k) {
-            n += sx[k];
-            if (k == 2) continue;
-            jx = fma(t.R[k], sx[k], jx);
-            jy = fma(t.R[k], sy[k], jy);
-            en = fma(t.R2[k], sx[k] + sy[k], en);
-        }
-        const double inv_n = recip_nr(n);
-        const double ux = jx * inv_n, uy = jy * inv_n;
-        const double T = 0.5 * fma(en, inv_n, -fma(ux, ux, uy * uy));
-        // Delta p = n T - p^w, p^w = n T / (1 - b n) - a n^2 (Eq. vdw)
-        const double nT = n * T;
-        m.n = n;
-        m.dp = nT - fma(nT, recip_nr(1.0 - g.b * n), -g.a * n * n);
-        m.ux = ux;
-        m.uy = uy;
-        m.T = T;
-        m.ok = (n > 0.0) && (T > 0.0) && (g.b * n < 1.0) && isfinite(n) && isfinite(T) && isfinite(ux) && isfinite(uy);
-    } else {
-        // FP32, compensated storage: row and column sums of the 5 x 5 pairs
-        // as double-float values; n and e = sum |p|^2 f from them in
-        // double-float arithmetic.  j needs FP32 accuracy of j itself:
-        // R_4 (sx_4 - sx_0) + R_3 (sx_3 - sx_1) with the differences of the
-        // double-float sums (R_0 = -R_4, R_1 = -R_3, R_2 = 0).
-        f2 sx[NQ], sy[NQ];
-        {
-            float h[NQ], l[NQ];
-#pragma unroll
-            for (int k1 = 0; k1 < NQ; ++k1) {
-#pragma unroll
-                for (int k2 = 0; k2 < NQ; ++k2) {
-                    const float2 v = get(NQ * k1 + k2);
-                    h[k2] = v.x;
-                    l[k2] = v.y;
-                }
-                sx[k1] = pair_sum5(h, l);
-            }
-#pragma unroll
-            for (int k2 = 0; k2 < NQ; ++k2) {
-#pragma unroll
-                for (int k1 = 0; k1 < NQ; ++k1) {
-                    const float2 v = get(NQ * k1 + k2);
-                    h[k1] = v.x;
-                    l[k1] = v.y;
-                }
-                sy[k2] = pair_sum5(h, l);
-            }
-        }
-        const f2 one{1.0f, 0.0f};
-        const f2 vdw_a = f2_of(g.a), vdw_b = f2_of(g.b);
-        const f2 N = f2_add(f2_add(f2_add(sx[0], sx[4]), f2_add(sx[1], sx[3])), sx[2]);
-        const float jx = fmaf(t.R[4], pdiff(sx[4].hi, sx[4].lo, sx[0].hi, sx[0].lo),
-                              t.R[3] * pdiff(sx[3].hi, sx[3].lo, sx[1].hi, sx[1].lo));
-        const float jy = fmaf(t.R[4], pdiff(sy[4].hi, sy[4].lo, sy[0].hi, sy[0].lo),
-                              t.R[3] * pdiff(sy[3].hi, sy[3].lo, sy[1].hi, sy[1].lo));
-        const f2 S4 = f2_add(f2_add(sx[0], sx[4]), f2_add(sy[0], sy[4]));
-        const f2 S3 = f2_add(f2_add(sx[1], sx[3]), f2_add(sy[1], sy[3]));
-        const f2 R24{t.R2[4], t.R2lo[4]}, R23{t.R2[3], t.R2lo[3]};
-        const f2 Ea = f2_cmul(R24, S4.hi, S4.lo), Eb = f2_cmul(R23, S3.hi, S3.lo);
-        const f2 E = f2_add(fast_two_sum(Ea.hi, Ea.lo), fast_two_sum(Eb.hi, Eb.lo));
-        // u, T and Delta p = n T - p^w = n^2 (a - b T / (1 - b n)) (Eq. vdw):
-        // T and Delta p in double-float arithmetic, so that the stencils of n
-        // and Delta p see ~44-bit values without the FP64 pipe
-        const f2 IN = f2_div(one, N);
-        const float UX = jx * IN.hi, UY = jy * IN.hi;
-        const f2 T = f2_scale(f2_add_f(f2_mul(E, IN), -fmaf(UX, UX, UY * UY)), 0.5f);
-        const f2 BN = f2_mul(vdw_b, N);
-        const f2 Q = f2_div(f2_mul(vdw_b, T), f2_add(one, f2_neg(BN)));
-        const f2 DP = f2_mul(f2_mul(N, N), f2_add(vdw_a, f2_neg(Q)));
-        m.n = make_float2(N.hi, N.lo);
-        m.dp = make_float2(DP.hi, DP.lo);
-        m.T = make_float2(T.hi, T.lo);
-        m.E = make_float2(E.hi, E.lo);
-        m.ux = UX;
-        m.uy = UY;
-        m.ok = (N.hi > 0.0f) && (T.hi > 0.0f) && (BN.hi < 1.0f) && isfinite(N.hi) && isfinite(T.hi) && isfinite(UX) &&
-               isfinite(UY);
-    }
-    return m;
-}
-
-// Fields of the per-node pre-pass (k_fields), [ny][pitch] each: n and
-// Delta p (FP32: hi + lo pairs), u_x, u_y, T (FP32: T a pair, and e = sum
-// |p|^2 f as a pair for the equilibrium's correction).
-template <typename real>
-struct StageFields {
-    using fld = typename FieldT<real>::type;
-    fld *n, *dp, *T, *E;
-    real *ux, *uy;
-};
-
-// Pointers of the fields in a buffer of 5 planes of pitch * ny 8-byte
-// elements (fields_bytes): FP64 n, Delta p, T, u_x, u_y; FP32 n, Delta p,
-// T, e (float2 each), then u_x and u_y (float) sharing the last plane.
-template <typename real>
-__host__ __device__ inline StageFields<real> fields_of(void *base, const Geo &g)
-{
-    StageFields<real> f{};
-    char *b = static_cast<char *>(base);
-    const size_t plane = (size_t)g.plane * 8;
-    f.n = reinterpret_cast<typename FieldT<real>::type *>(b);
-    f.dp = reinterpret_cast<typename FieldT<real>::type *>(b + plane);
-    f.T = reinterpret_cast<typename FieldT<real>::type *>(b + 2 * plane);
-    if constexpr (sizeof(real) == 8) {
-        f.E = nullptr;
-        f.ux = reinterpret_cast<real *>(b + 3 * plane);
-        f.uy = reinterpret_cast<real *>(b + 4 * plane);
-    } else {
-        f.E = reinterpret_cast<typename FieldT<real>::type *>(b + 3 * plane);
-        f.ux = reinterpret_cast<real *>(b + 4 * plane);
-        f.uy = reinterpret_cast<real *>(b + 4 * plane + plane / 2);
-    }
-    return f;
-}
-
-// One thread per node: the moments of f_s, stored for the stage kernel,
-// which then reads them on its tile and halo instead of recomputing them
-// at every halo position; inadmissible moments set bit 0 of the status.
-template <typename real>
-__global__ void __launch_bounds__(256) k_fields(const real *__restrict__ fs, StageFields<real> out, int *status,
-                                                const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t)
-{
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)g.nx * g.ny) return;
-    const int j = (int)(idx / g.nx), i = (int)(idx - (long long)j * g.nx);
-    const long long o = (long long)j * g.pitch + i;
-    NodeMoments<real> m;
-    if constexpr (sizeof(real) == 8)
-        m = node_moments<real>([&](int k) { return __ldg(fs + k * g.plane + o); }, g, t);
-    else
-        m = node_moments<real>(
-            [&](int k) { return make_float2(__ldg(fs + k * g.plane + o), __ldg(fs + (NK + k) * g.plane + o)); }, g, t);
-    out.n[o] = m.n;
-    out.dp[o] = m.dp;
-    out.ux[o] = m.ux;
-    out.uy[o] = m.uy;
-    out.T[o] = m.T;
-    if constexpr (sizeof(real) == 4) out.E[o] = m.E;
-    if (!m.ok) atomicOr(status, 1);
-}
-
-// ---------------------------------------------------------------- TMA staging
-// Iterations of the bounded wait for the copy (each try_wait suspends for at
-// most a short, hardware-defined time): far above the microseconds a copy of
-// a tile's region takes, far below a hang.
-constexpr int TMA_WAIT_LIMIT = 1 << 16;
-
-__device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
-{
-    for (int i = 0; i < TMA_WAIT_LIMIT; ++i) {
-        unsigned done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
-// Phase 1 for a tile whose staged region lies inside the grid: TMA copies of the
-// boxes at (x0, y0) of the tensor maps (TmaMap) into the staging arrays (FP32:
-// pop, then the lo planes, contiguous in the box's order), completion tracked by
-// an mbarrier.  tma_issue starts the copies (all threads call it; it
-// synchronises); tma_finish waits for them with the bounded wait.  If the wait
-// runs out, bit 1 of the status word is set, the copies are waited for once more
-// (bounded) and false is returned: the caller leaves the tile untouched and the
-// CTA stops.  After completed copies the barrier is invalidated.
-__device__ __forceinline__ void tma_load(unsigned dst, const unsigned char *map, int x, int y, unsigned mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(dst),
-        "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(0), "r"(mbar)
-        : "memory");
-}
-template <int TX, int TY, int KP>
-__device__ __forceinline__ unsigned tma_bytes(const Smem32<TX, TY, KP> &sm)
-{
-    return sizeof(sm.pop) + sizeof(sm.pl);
-}
-template <int TX, int TY, int KP>
-__device__ __forceinline__ void tma_copies(Smem32<TX, TY, KP> &sm, const TmaMap *m, int x0, int y0, unsigned mbar)
-{
-    tma_load((unsigned)__cvta_generic_to_shared(&sm.pop[0][0][0]), m->bytes[0], x0 - 4, y0 - 3, mbar);
-}
-template <int TX, int TY, int KP, bool LEARNED>
-__device__ __forceinline__ unsigned tma_bytes(const Smem64<TX, TY, KP, LEARNED> &sm)
-{
-    return sizeof(sm.mid) + sizeof(sm.below) + sizeof(sm.above);
-}
-template <int TX, int TY, int KP, bool LEARNED>
-__device__ __forceinline__ void tma_copies(Smem64<TX, TY, KP, LEARNED> &sm, const TmaMap *m, int x0, int y0, unsigned mbar)
-{
-    tma_load((unsigned)__cvta_generic_to_shared(&sm.mid[0][0][0]), m->bytes[0], x0 - 4, y0, mbar);
-    tma_load((unsigned)__cvta_generic_to_shared(&sm.below[0][0][0]), m->bytes[1], x0, y0 - 3, mbar);
-    tma_load((unsigned)__cvta_generic_to_shared(&sm.above[0][0][0]), m->bytes[1], x0, y0 + TY, mbar);
-}
-template <typename Smem>
-__device__ __forceinline__ void tma_issue(Smem &sm, const TmaMap *tmap, int x0, int y0)
-{
-    const unsigned mbar = (unsigned)__cvta_generic_to_shared(&sm.mbar);
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(tma_bytes(sm)) : "memory");
-        tma_copies(sm, tmap, x0, y0, mbar);
-    }
-    __syncthreads();  // the barrier is initialised before anyone waits on it
-}
-template <typename Smem>
-__device__ __forceinline__ bool tma_finish(Smem &sm, int *status)
-{
-    const unsigned mbar = (unsigned)__cvta_generic_to_shared(&sm.mbar);
-    const bool ok = mbar_wait(mbar, 0);
-    if (__syncthreads_or(!ok)) {
-        if (threadIdx.x == 0) atomicOr(status, 2);
-        mbar_wait(mbar, 0);
-        return false;
-    }
-    // every thread has passed its wait (the barrier above)
-    if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(mbar) : "memory");
-    return true;
 }
 
 // ---------------------------------------------------------------- force and update of an FP32 tile
@@ -898,45 +582,34 @@ __device__ __forceinline__ bool advance32(Smem32<TX, TY, KP> &sm, const float *f
 
 // One stage for the tile whose lower-left node is (x0, y0); all threads of
 // the CTA call it (it synchronises).  ca, cb, cc: the stage's coefficients of
-// f^n, f_s and dt L (Eq. rk3), in the population precision; ca_lo, cb_lo:
-// their remainders (FP32: 1/3 and 2/3 as double-float constants; 0 in FP64).
-// g and t may live in parameter space (single grid) or shared memory
-// (batch); tw: the table of the wall entries (geqw, inv_den), t itself for
-// a single grid, the run's own in a batch, whose velocity tables t are common
-// to all runs and passed as a kernel parameter; mlp: the learned network's
-// parameters in shared memory (LEARNED
-// only); tmap: TMA map of fs (of this run, in a batch) for this tile shape,
-// or nullptr; fields: the moments of fs from k_fields.  Returns false when the TMA copy timed out (the CTA must stop).
-template <typename real, int TX, int TY, int KP, bool LEARNED = false>
-__device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, LEARNED>::type &sm, const real *__restrict__ fs,
-                                           const real *fn, real *out, int *__restrict__ status, const Geo &g,
-                                           const Tab<real> &t, const Tab<real> &tw, const int x0, const int y0,
-                                           const real ca,
-                                           const real cb, const real cc, const real ca_lo, const real cb_lo,
-                                           const StageK &sk, const float *mlp, const TmaMap *tmap,
-                                           const StageFields<real> &fields)
+// f^n, f_s and dt L (Eq. rk3), in FP32; ca_lo, cb_lo: their remainders (1/3 and
+// 2/3 as double-float constants).  g and t may live in parameter space (single
+// grid) or shared memory (batch); tw: the table of the wall entries (geqw,
+// inv_den), t itself for a single grid, the run's own in a batch, whose velocity
+// tables t are common to all runs and passed as a kernel parameter; mlp: the
+// learned network's parameters in shared memory (LEARNED only); tmap: TMA map of
+// fs (of this run, in a batch) for this tile shape, or nullptr; fields: the
+// moments of fs from k_fields.  Returns false when the TMA copy timed out (the
+// CTA must stop).
+template <int TX, int TY, int KP, bool LEARNED>
+__device__ __forceinline__ bool stage_tile32(Smem32<TX, TY, KP> &sm, const float *__restrict__ fs, const float *fn,
+                                             float *out, int *__restrict__ status, const Geo &g, const Tab<float> &t,
+                                             const Tab<float> &tw, int x0, int y0, float ca, float cb, float cc,
+                                             float ca_lo, float cb_lo, const float *mlp, const TmaMap *tmap,
+                                             const StageFields<float> &fields)
 {
-    using S = typename StageSmem<real, TX, TY, KP, LEARNED>::type;
+    using S = Smem32<TX, TY, KP>;
     constexpr int NT = S::NT, HX = S::HX, HY = S::HY;
-
     const int tid = threadIdx.x;
 
     // ---- 1. populations of the region (c <-> x = x0 - 4 + c, r <-> y = y0 - 3 + r)
-    //    A region inside the grid comes in one TMA copy.  Otherwise:
-    //    periodic sides wrap.  Ghost layers 0..2 of a specular side hold the
-    //    populations of the first three nodes inside with the normal
-    //    velocity component reversed (Sec. 3.4.1); diffuse-wall ghosts are
-    //    set in phase 3; anything further out is never read and holds 0.
     const bool inside = tmap != nullptr && x0 >= 4 && x0 + TX + 4 <= g.nx && y0 >= 3 && y0 + TY + 3 <= g.ny;
-    // the pre-pass fields of this thread's first moment position (phase 2's
-    // item e = tid) are fetched into registers now, so that their latency
-    // overlaps the staging of the populations
-    using fld = typename FieldT<real>::type;
-    if constexpr (sizeof(real) == 8) {
-        if (tid == 0) sm.top = 0;  // ordered before phase 2 by phase 1's barrier
-    }
+    // the pre-pass fields of this thread's first position (phase 2's item e = tid)
+    // are fetched into registers now, so that their latency overlaps the staging
+    // of the populations
+    using fld = FieldT<float>::type;
     fld pf_n{}, pf_dp{}, pf_T{}, pf_E{};
-    real pf_ux = 0, pf_uy = 0;
+    float pf_ux = 0, pf_uy = 0;
     bool pf_ok = false, pf_node = false;
     int pf_r = 0, pf_c = 0;
     if (tid < HY * (HX - 2)) {
@@ -954,106 +627,33 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
                 pf_ux = fields.ux[o];
                 pf_uy = fields.uy[o];
                 pf_T = fields.T[o];
-                if constexpr (sizeof(real) == 4) pf_E = fields.E[o];
+                pf_E = fields.E[o];
             }
         }
     }
     // A tile inside the grid touches its staged populations first in the face
     // pass (no walls, no sides), so phases 2-4 run while the copy is in flight
-    if (inside) {
-        tma_issue(sm, tmap, x0, y0);
-    } else {
-        for (int e = tid; e < HY * HX; e += NT) {
-            const int r = e / HX, c = e - r * HX;
-            if (!S::staged(r, c)) continue;
-            real *dst = sm.at(0, r, c);
-            const int dp = S::plane(r);
-            int gy = y0 - 3 + r, gx = x0 - 4 + c;
-            bool flip_x = false, flip_y = false, zero = false;
-            if (gy < 0 || gy >= g.ny) {
-                if (!g.spec_y) {
-                    gy = wrap(gy, g.ny);
-                } else if ((gy < 0 ? -1 - gy : gy - g.ny) <= 2) {
-                    gy = gy < 0 ? -1 - gy : 2 * g.ny - 1 - gy;
-                    flip_y = true;
-                } else {
-                    zero = true;
-                }
-            }
-            if (gx < 0 || gx >= g.nx) {
-                const bool lo = gx < 0;
-                if (!g.walls) {
-                    gx = wrap(gx, g.nx);
-                } else if ((lo ? g.spec_lo : g.spec_hi) && (lo ? -1 - gx : gx - g.nx) <= 2) {
-                    gx = lo ? -1 - gx : 2 * g.nx - 1 - gx;
-                    flip_x = true;
-                } else {
-                    zero = true;
-                }
-            }
-            if (zero) {
-#pragma unroll 5
-                for (int k = 0; k < NK; ++k) {
-                    dst[k * dp] = real(0);
-                    if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = 0.0f;
-                }
-                continue;
-            }
-            const real *src = fs + (long long)gy * g.pitch + gx;
-            if (!flip_x && !flip_y) {
-#pragma unroll 5
-                for (int k = 0; k < NK; ++k) {
-                    dst[k * dp] = __ldg(src + k * g.plane);
-                    if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = __ldg(src + (NK + k) * g.plane);
-                }
-            } else {
-#pragma unroll
-                for (int k1 = 0; k1 < NQ; ++k1)
-#pragma unroll
-                    for (int k2 = 0; k2 < NQ; ++k2) {
-                        const int kk = NQ * (flip_x ? NQ - 1 - k1 : k1) + (flip_y ? NQ - 1 - k2 : k2);
-                        dst[(NQ * k1 + k2) * dp] = __ldg(src + kk * g.plane);
-                        if constexpr (sizeof(real) == 4) sm.pl.lo[NQ * k1 + k2][r][c] = __ldg(src + (NK + kk) * g.plane);
-                    }
-            }
-        }
-    }
+    if (inside) tma_issue(sm, tmap, x0, y0);
+    else load_region(sm, fs, g, x0, y0);
     __syncthreads();
 
     // ---- 2. fields at every fluid position of the region that the 7 x 7
     // force stencils reach (columns 1 .. HX-2; ghost positions of walls and
-    // specular sides take the reflected fields in phase 3).  A tile at a
-    // diffuse wall also computes here, on warps of their own, the wall-face
-    // flux of every outgoing velocity in every tile row (Sec. 3.4.2: the
-    // WENO-5 face value at the wall from the three nearest fluid nodes and the
-    // two ghosts extrapolated from them) and stores those two ghosts.
+    // specular sides take the reflected fields in phase 3): n and Delta p on the
+    // region, u, T and e at the tile nodes.  A tile at a diffuse wall also
+    // computes here, on warps of their own, its wall fluxes.
     const bool x_lo = g.walls && x0 == 0;                // ghost columns at x = 0
     const bool x_hi = g.walls && (x0 + TX + 3 >= g.nx);  // ghost columns at x = nx ds
     const bool left_wall = x_lo && g.wall_lo;
     const bool right_wall = x_hi && g.wall_hi;
-    // wall-flux items start on the first warp after the moment positions
-    constexpr int e_flux = (HY * (HX - 2) + 31) / 32 * 32;
-    const int nflux = ((int)left_wall + (int)right_wall) * TY * 16;
-    // FP64: high word of this thread's largest finite n (the tile's scale)
-    int top = 0;
-    auto note_n = [&](fld n) {
-        if constexpr (sizeof(real) == 8) {
-            const int a = __double2hiint(n) & 0x7fffffff;
-            top = max(top, a < 0x7ff00000 ? a : 0);
-        }
-    };
-    // moments from the per-node pre-pass (k_fields): n and Delta p on the
-    // region, u, T (FP32: and e) at the tile nodes; item tid was fetched
-    // before phase 1
     if (pf_ok) {
-        note_n(pf_n);
         sm.n[pf_r][pf_c] = pf_n;
         sm.dp[pf_r][pf_c] = pf_dp;
         if (pf_node) {
             sm.ux[pf_r - 3][pf_c - 4] = pf_ux;
             sm.uy[pf_r - 3][pf_c - 4] = pf_uy;
             sm.T[pf_r - 3][pf_c - 4] = pf_T;
-            if constexpr (sizeof(real) == 4) sm.eng[pf_r - 3][pf_c - 4] = pf_E;
+            sm.eng[pf_r - 3][pf_c - 4] = pf_E;
         }
     }
     for (int e = tid + NT; e < HY * (HX - 2); e += NT) {
@@ -1062,85 +662,23 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
         if (g.walls && (gx < 0 || gx >= g.nx)) continue;
         if (g.spec_y && (gyr < 0 || gyr >= g.ny)) continue;
         const long long o = (long long)wrap(gyr, g.ny) * g.pitch + wrap(gx, g.nx);
-        const fld n = fields.n[o];
-        note_n(n);
-        sm.n[r][c] = n;
+        sm.n[r][c] = fields.n[o];
         sm.dp[r][c] = fields.dp[o];
         const int tr = r - 3, tc = c - 4;
         if (tr >= 0 && tr < TY && tc >= 0 && tc < TX) {
             sm.ux[tr][tc] = fields.ux[o];
             sm.uy[tr][tc] = fields.uy[o];
             sm.T[tr][tc] = fields.T[o];
-            if constexpr (sizeof(real) == 4) sm.eng[tr][tc] = fields.E[o];
+            sm.eng[tr][tc] = fields.E[o];
         }
     }
-    if constexpr (sizeof(real) == 8) {
-        top = __reduce_max_sync(0xffffffffu, top);
-        if ((tid & 31) == 0) atomicMax(&sm.top, top);
-    }
-    // wall flux item f runs on thread (e_flux + f) mod NT: on the warps after
-    // those with moment positions.  Each tile row of a wall takes a
-    // half-warp: lanes v = 0..9 compute the flux of outgoing velocity v (the
-    // half-range p_x < 0 at x = 0, p_x > 0 at x = nx ds), lanes 10..15 add 0,
-    // and a shuffle reduction over the half-warp gives the row's sum.  (e_flux
-    // and NT are multiples of 32, so f runs over whole half-warps.)
-    for (int f = (tid - e_flux % NT + NT) % NT; f < nflux; f += NT) {
-        // (wall, tile row tr, outgoing velocity v); the left wall's items first
-        const int side = (f >= TY * 16 || !left_wall) ? 1 : 0;
-        const int fr = f >= TY * 16 ? f - TY * 16 : f;
-        const int tr = fr >> 4, v = fr & 15;
-        const int k1 = side ? 3 + v / 5 : v / 5;
-        const int k = NQ * k1 + v % 5;
-        // nearest three fluid nodes, nearest first; ghost layers 0 and 1
-        // are the next two columns outwards
-        const int c0 = side ? g.nx - 1 - (x0 - 4) : 0 - (x0 - 4);
-        const int dc = side ? -1 : 1;
-        real wf = 0;
-        if (v >= 10) {
-            // idle lane of the row's half-warp
-        } else if constexpr (sizeof(real) == 8) {
-            const real a0 = *sm.at(k, tr + 3, c0), a1 = *sm.at(k, tr + 3, c0 + dc);
-            const real a2 = *sm.at(k, tr + 3, c0 + 2 * dc);
-            const real g0 = fma(real(3), a0 - a1, a2);
-            const real g1 = fma(real(6), a0, fma(real(-8), a1, real(3) * a2));
-            if (c0 - dc >= 0 && c0 - dc < HX) *sm.at(k, tr + 3, c0 - dc) = g0;
-            if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) *sm.at(k, tr + 3, c0 - 2 * dc) = g1;
-            wf = t.R[k1] * face_value<LEARNED>(mlp, a2, a1, a0, g0, g1);
-        } else {
-            // pairs: the ghosts 3a0 - 3a1 + a2 and 6a0 - 8a1 + 3a2 as a0 plus
-            // combinations of the differences D1 = a0 - a1, D2 = a1 - a2, and
-            // the stencil (a2, a1, a0, g0, g1) by its first differences
-            // (D2, D1, 2 D1 - D2, 3 D1 - 2 D2)
-            const int row = tr + 3;
-            const float h0 = sm.pop[k][row][c0], l0 = sm.pl.lo[k][row][c0];
-            const float h1 = sm.pop[k][row][c0 + dc], l1 = sm.pl.lo[k][row][c0 + dc];
-            const float h2 = sm.pop[k][row][c0 + 2 * dc], l2 = sm.pl.lo[k][row][c0 + 2 * dc];
-            const float D1 = pdiff(h0, l0, h1, l1), D2 = pdiff(h1, l1, h2, l2);
-            const float e0 = fmaf(2.0f, D1, -D2), e1 = fmaf(5.0f, D1, -3.0f * D2);
-            const f2 G0 = f2_add_f(f2{h0, l0}, e0), G1 = f2_add_f(f2{h0, l0}, e1);
-            if (c0 - dc >= 0 && c0 - dc < HX) {
-                sm.pop[k][row][c0 - dc] = G0.hi;
-                sm.pl.lo[k][row][c0 - dc] = G0.lo;
-            }
-            if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) {
-                sm.pop[k][row][c0 - 2 * dc] = G1.hi;
-                sm.pl.lo[k][row][c0 - 2 * dc] = G1.lo;
-            }
-            const float corr = face_corr<LEARNED>(mlp, D2, D1, e0, fmaf(3.0f, D1, -2.0f * D2));
-            wf = t.R[k1] * (h0 + (l0 + corr));
-        }
-        const unsigned half = (tid & 16) ? 0xffff0000u : 0x0000ffffu;
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) wf += __shfl_xor_sync(half, wf, o);
-        if (v == 0) sm.wnw[side][tr] = -wf * tw.inv_den[side];
-    }
+    // wall-flux items start on the first warp after the field positions
+    if (left_wall || right_wall)
+        wall_flux<float, LEARNED>(sm, g, t, tw, mlp, x0, (HY * (HX - 2) + 31) / 32 * 32, left_wall, right_wall);
 
     // ---- 3. sides: n and Delta p reflected evenly into the ghost layers of
     // walls and specular planes (Sec. 3.4.3; y first, then x over every row,
-    // which makes the corners a double reflection); at diffuse walls the
-    // incoming ghosts of the tile rows, f^eq_w = n_w g g (Sec. 3.4.2, Eq.
-    // diffuse_flux), with the wall density n_w of Eq. nw from the sum of the
-    // row's outgoing fluxes
+    // which makes the corners a double reflection); the incoming ghosts at walls
     if (g.spec_y && (y0 == 0 || y0 + TY + 2 >= g.ny)) {
         __syncthreads();
         for (int e = tid; e < HY * HX; e += NT) {
@@ -1155,40 +693,23 @@ __device__ __forceinline__ bool stage_tile(typename StageSmem<real, TX, TY, KP, 
     }
     if (x_lo || x_hi) {
         __syncthreads();
-        constexpr int e_in = (HY * HX + 31) / 32 * 32;  // first incoming-ghost item, on a warp boundary
-        const int nin = ((int)left_wall + (int)right_wall) * TY * 30;
-        for (int e = tid; e < e_in + nin; e += NT) {
-            if (e < HY * HX) {
-                const int r = e / HX, c = e - r * HX;
-                const int gx = x0 - 4 + c;
-                if (gx >= 0 && gx < g.nx) continue;
-                const bool right = gx >= g.nx;
-                if ((right ? gx - g.nx : -1 - gx) > 2) continue;  // beyond ghost layer 2
-                const int cm = (right ? 2 * g.nx - 1 - gx : -1 - gx) - (x0 - 4);
-                sm.n[r][c] = sm.n[r][cm];
-                sm.dp[r][c] = sm.dp[r][cm];
-            } else if (e >= e_in) {
-                // (wall, tile row tr, ghost layer m, incoming velocity v)
-                const int f = e - e_in;
-                const int side = (f >= TY * 30 || !left_wall) ? 1 : 0;
-                const int fr = f >= TY * 30 ? f - TY * 30 : f;
-                const int tr = fr / 30, m = (fr - 30 * tr) / 10, v = fr - 30 * tr - 10 * m;
-                const int c = side ? g.nx + m - (x0 - 4) : -1 - m - (x0 - 4);
-                if (c < 0 || c >= HX) continue;
-                const int k = NQ * (side ? v / 5 : 3 + v / 5) + v % 5;
-                *sm.at(k, tr + 3, c) = sm.wnw[side][tr] * tw.geqw[side][k];
-                if constexpr (sizeof(real) == 4) sm.pl.lo[k][tr + 3][c] = 0.0f;
-            }
+        for (int e = tid; e < HY * HX; e += NT) {
+            const int r = e / HX, c = e - r * HX;
+            const int gx = x0 - 4 + c;
+            if (gx >= 0 && gx < g.nx) continue;
+            const bool right = gx >= g.nx;
+            if ((right ? gx - g.nx : -1 - gx) > 2) continue;  // beyond ghost layer 2
+            const int cm = (right ? 2 * g.nx - 1 - gx : -1 - gx) - (x0 - 4);
+            sm.n[r][c] = sm.n[r][cm];
+            sm.dp[r][c] = sm.dp[r][cm];
         }
+        wall_ghosts<float>(sm, g, tw, x0, (HY * HX + 31) / 32 * 32, left_wall, right_wall);
     }
     __syncthreads();
 
     // ---- 4, 5. force, fluxes, collision and RK-3 combination
-    auto wait = [&] { return !inside || tma_finish(sm, status); };
-    if constexpr (sizeof(real) == 8)
-        return advance64<TX, TY, KP, LEARNED>(sm, fn, out, g, t, t.ff, sk, x0, y0, mlp, wait);
-    else
-        return advance32<TX, TY, KP, LEARNED>(sm, fn, out, g, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, mlp, wait);
+    return advance32<TX, TY, KP, LEARNED>(sm, fn, out, g, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, mlp,
+                                          [&] { return !inside || tma_finish(sm, status); });
 }
 
 // Shared memory of the single-grid kernel: the tile staging, then (learned
@@ -1208,11 +729,12 @@ constexpr size_t fused_smem_bytes()
     constexpr size_t mlp_floats = sizeof(real) == 4 ? MLP_SCRATCH_OFF + S::NT / 32 * MLP_WARP_SCRATCH : MLP_P + 1;
     return LEARNED ? mlp_offset<real, TX, TY, KP>() + mlp_floats * sizeof(float) : sizeof(S);
 }
-// Threads of a shape's CTA: KP lanes of the tile's nodes, rounded up to warps.
-template <int TX, int TY, int KP>
+// Threads of a shape's CTA: FP32: KP lanes of the tile's nodes, rounded up to
+// warps; FP64: Plan64.
+template <typename real, int TX, int TY, int KP>
 constexpr int stage_threads()
 {
-    return (TX * TY + 31) / 32 * 32 * KP;
+    return StageSmem<real, TX, TY, KP, false>::type::NT;
 }
 
 // CTAs per SM that the register allocation must leave room for: as many as
@@ -1227,18 +749,14 @@ constexpr int fused_min_ctas(size_t smem_bytes, int threads, int cap = 0)
     return n < 1 ? 1 : (cap > 0 && n > cap ? cap : n);
 }
 
-// FP64's lines of faces need more than the 40 registers that three CTAs of eight
-// lanes leave.
-constexpr int stage_cta_cap(bool fp64, int kp) { return fp64 && kp > 5 ? 2 : 0; }
-
 // Single grid: one CTA per tile.  Learned-weight instances leave their network the registers
 // it needs: FP32 (tensor-pipe network) at most two CTAs per SM, FP64 (per-thread
 // network) one.
 template <typename real, int TX, int TY, int KP, bool LEARNED>
-__global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
+__global__ void __launch_bounds__((stage_threads<real, TX, TY, KP>()),
                                   fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, LEARNED>(),
-                                                 stage_threads<TX, TY, KP>(),
-                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : stage_cta_cap(sizeof(real) == 8, KP)))
+                                                 stage_threads<real, TX, TY, KP>(),
+                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : 0))
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
         real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
@@ -1257,8 +775,12 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
         }
         // made visible by the first barrier inside stage_tile
     }
-    stage_tile<real, TX, TY, KP, LEARNED>(sm, fs, fn, out, status, g, t, t, blockIdx.x * TX, blockIdx.y * TY, ca, cb,
-                                          cc, ca_lo, cb_lo, sk, mlp_sm, tma.on ? &tma.map : nullptr,
+    const TmaMap *tm = tma.on ? &tma.map : nullptr;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    if constexpr (sizeof(real) == 8)
+        stage_tile64<KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, sk, mlp_sm, tm, fields);
+    else
+        stage_tile32<TX, TY, KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, mlp_sm, tm,
                                           fields);
 }
 
@@ -1269,26 +791,10 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
 // tile_start[r] is the first item of run r (prefix sum, tile_start[nruns] =
 // total).  Each run has its populations at offset `off` of the three shared
 // buffers and its own status word.
-// 16-byte aligned and sized: the kernel copies one descriptor into shared
-// memory with 16-byte loads, so consecutive array elements must stay aligned
-// and the whole struct must be covered by whole int4 words.
-template <typename real>
-struct __align__(16) BatchRun {
-    Geo g;
-    Tab<real> t;
-    long long off;   // populations: element offset in the three buffers
-    long long foff;  // stage fields: byte offset in the fields buffer
-    int ntx, pad;
-    StageK k[3];  // constants of the three RK-3 stages (FP64)
-    long long pad2;
-};
-static_assert(sizeof(BatchRun<double>) % 16 == 0, "BatchRun<double> must be a whole number of int4 words");
-static_assert(sizeof(BatchRun<float>) % 16 == 0, "BatchRun<float> must be a whole number of int4 words");
-
 template <typename real, int TX, int TY, int KP>
-__global__ void __launch_bounds__((stage_threads<TX, TY, KP>()),
+__global__ void __launch_bounds__((stage_threads<real, TX, TY, KP>()),
                                   fused_min_ctas(fused_smem_bytes<real, TX, TY, KP, false>() + sizeof(BatchRun<real>),
-                                                 stage_threads<TX, TY, KP>(), stage_cta_cap(sizeof(real) == 8, KP)))
+                                                 stage_threads<real, TX, TY, KP>()))
 k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
               const BatchRun<real> *__restrict__ runs, const int *__restrict__ tile_start, int nruns,
               const __grid_constant__ Tab<real> tv, real ca, real cb, real ccoef, real ca_lo, real cb_lo, int st,
@@ -1298,12 +804,7 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
     auto &sm = *reinterpret_cast<typename StageSmem<real, TX, TY, KP, false>::type *>(smem_raw);
     __shared__ __align__(16) BatchRun<real> run;
     const int item = blockIdx.x;
-    int lo = 0, hi = nruns - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(tile_start + mid) <= item) lo = mid;
-        else hi = mid - 1;
-    }
+    const int lo = run_of(tile_start, nruns, item);
     {
         const int4 *src = reinterpret_cast<const int4 *>(runs + lo);
         int4 *dst = reinterpret_cast<int4 *>(&run);
@@ -1321,49 +822,12 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
     if (tm && threadIdx.x == 0)
         for (int k = 0; k < 2; ++k)
             asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm->bytes[k]) : "memory");
-    stage_tile<real, TX, TY, KP>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
-                                 ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, run.k[st], nullptr, tm, fl);
-}
-
-// The moments pre-pass for a batch: one thread per node of every run (a
-// grid-stride loop over the prefix sum node_start of the runs' node counts),
-// writing each run's fields at its offset of the fields buffer.
-template <typename real>
-__global__ void __launch_bounds__(256) k_fields_batch(const real *__restrict__ fs, char *fields,
-                                                      const BatchRun<real> *__restrict__ runs,
-                                                      const long long *__restrict__ node_start, int nruns,
-                                                      long long total, int *status)
-{
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nruns - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(node_start + mid) <= idx) lo = mid;
-            else hi = mid - 1;
-        }
-        const BatchRun<real> &run = runs[lo];
-        const Geo &g = run.g;
-        const long long q = idx - __ldg(node_start + lo);
-        const int j = (int)(q / g.nx), i = (int)(q - (long long)j * g.nx);
-        const long long o = (long long)j * g.pitch + i;
-        const real *f = fs + run.off;
-        NodeMoments<real> m;
-        if constexpr (sizeof(real) == 8)
-            m = node_moments<real>([&](int k) { return __ldg(f + k * g.plane + o); }, g, run.t);
-        else
-            m = node_moments<real>(
-                [&](int k) { return make_float2(__ldg(f + k * g.plane + o), __ldg(f + (NK + k) * g.plane + o)); }, g,
-                run.t);
-        const StageFields<real> out = fields_of<real>(fields + run.foff, g);
-        out.n[o] = m.n;
-        out.dp[o] = m.dp;
-        out.ux[o] = m.ux;
-        out.uy[o] = m.uy;
-        out.T[o] = m.T;
-        if constexpr (sizeof(real) == 4) out.E[o] = m.E;
-        if (!m.ok) atomicOr(status + lo, 1);
-    }
+    if constexpr (sizeof(real) == 8)
+        stage_tile64<KP, false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
+                                run.k[st], nullptr, tm, fl);
+    else
+        stage_tile32<TX, TY, KP, false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0,
+                                        y0, ca, cb, ccoef * (real)run.g.dt, ca_lo, cb_lo, nullptr, tm, fl);
 }
 
 template <typename real, int TX, int TY, int KP, bool LEARNED = false>
@@ -1372,9 +836,11 @@ cudaError_t fused_prepare_one()
     cudaError_t e = cudaFuncSetAttribute(k_fused<real, TX, TY, KP, LEARNED>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)fused_smem_bytes<real, TX, TY, KP, LEARNED>());
-    if (e != cudaSuccess || LEARNED) return e;
-    return cudaFuncSetAttribute(k_fused_batch<real, TX, TY, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)fused_smem_bytes<real, TX, TY, KP, false>());
+    if constexpr (!LEARNED)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fused_batch<real, TX, TY, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)fused_smem_bytes<real, TX, TY, KP, false>());
+    return e;
 }
 
 template <typename real, int TX, int TY, int KP, bool LEARNED = false>
@@ -1392,9 +858,14 @@ cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *sta
     const StageFields<real> fl = fields_of<real>(fields, g);
     const long long N = (long long)g.nx * g.ny;
     k_fields<real><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
-    k_fused<real, TX, TY, KP, LEARNED><<<grid, stage_threads<TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, LEARNED>(), s>>>(
+    StageK sk{};
+    if constexpr (sizeof(real) == 8) {
+        sk = stage_constants(g, c);
+        k_force<<<dim3((g.nx + FORCE_X - 1) / FORCE_X, (g.ny + FORCE_Y - 1) / FORCE_Y), FORCE_THREADS, 0, s>>>(fl, g, sk);
+    }
+    k_fused<real, TX, TY, KP, LEARNED><<<grid, stage_threads<real, TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, LEARNED>(), s>>>(
         fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
-        (real)(c.cb - (double)(real)c.cb), sizeof(real) == 8 ? stage_constants(g, c) : StageK{}, mlp, tma, fl);
+        (real)(c.cb - (double)(real)c.cb), sk, mlp, tma, fl);
     return cudaGetLastError();
 }
 
@@ -1402,7 +873,7 @@ template <typename real, int TX, int TY, int KP>
 cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, int *status, const void *runs,
                                    const int *tile_start, int nruns, int total, const Tab<real> &t, StageCoef c,
                                    int st, void *fields, const long long *node_start, long long total_nodes,
-                                   const TmaMap *tmaps, cudaStream_t s)
+                                   const int *force_start, int force_blocks, const TmaMap *tmaps, cudaStream_t s)
 {
     if (total < 1) return cudaSuccess;
     if (total_nodes > 0) {
@@ -1414,7 +885,10 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
             fs, static_cast<char *>(fields), static_cast<const BatchRun<real> *>(runs), node_start, nruns, total_nodes,
             status);
     }
-    k_fused_batch<real, TX, TY, KP><<<total, stage_threads<TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, false>(), s>>>(
+    if constexpr (sizeof(real) == 8)
+        k_force_batch<<<force_blocks, FORCE_THREADS, 0, s>>>(
+            static_cast<char *>(fields), static_cast<const BatchRun<double> *>(runs), force_start, nruns, st);
+    k_fused_batch<real, TX, TY, KP><<<total, stage_threads<real, TX, TY, KP>(), fused_smem_bytes<real, TX, TY, KP, false>(), s>>>(
         fs, fn, out, status, static_cast<const BatchRun<real> *>(runs), tile_start, nruns, t, (real)c.ca, (real)c.cb,
         (real)c.cc, (real)(c.ca - (double)(real)c.ca), (real)(c.cb - (double)(real)c.cb), st, static_cast<char *>(fields),
         tmaps);
@@ -1428,7 +902,7 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
 #define OLB_FUSED_SHAPES_float(DO) \
     DO(float, 8, 8, 4) DO(float, 16, 8, 2) DO(float, 16, 8, 1) DO(float, 32, 8, 1) DO(float, 32, 16, 1) \
     DO(float, 8, 8, 8) DO(float, 7, 8, 8) DO(float, 8, 8, 5)
-#define OLB_FUSED_SHAPES_double(DO) DO(double, 8, 8, 4) DO(double, 8, 8, 8) DO(double, 7, 8, 8) DO(double, 8, 8, 5)
+#define OLB_FUSED_SHAPES_double(DO) DO(double, 8, 8, 8) DO(double, 8, 8, 5)
 #define OLB_FUSED_LEARNED_float(DO) DO(float, 8, 8, 4) DO(float, 16, 8, 2) DO(float, 32, 16, 1)
 #define OLB_FUSED_LEARNED_double(DO) DO(double, 8, 8, 4)
 #define OLB_FUSED_PREP_CASE(real, A, B, C) \
@@ -1444,7 +918,8 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
 #define OLB_FUSED_BATCH_CASE(real, A, B, C)                                                                  \
     if (sh.tx == A && sh.ty == B && sh.kp == C)                                                              \
         return fused_batch_launch_one<real, A, B, C>(fs, fn, out, status, runs, tile_start, nruns, total, t,     \
-                                                     c, st, fields, node_start, total_nodes, tmaps, s);
+                                                     c, st, fields, node_start, total_nodes, force_start,       \
+                                                     force_blocks, tmaps, s);
 #define OLB_DEFINE_FUSED(real)                                                                                \
     cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned)                                   \
     {                                                                                                         \
@@ -1465,7 +940,7 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
     cudaError_t launch_fused_batch(const real *fs, const real *fn, real *out, int *status, const void *runs,  \
                                    const int *tile_start, int nruns, int total, const Tab<real> &t,         \
                                    StageCoef c, int st, int tx, int ty, int kp, void *fields,                 \
-                                   const long long *node_start, long long total_nodes, const TmaMap *tmaps,   \
+                                   const long long *node_start, long long total_nodes, const int *force_start, int force_blocks, const TmaMap *tmaps,   \
                                    cudaStream_t s)                                                            \
     {                                                                                                         \
         const Shape sh = stage_shape(sizeof(real) == 8, false, tx, ty, kp);                                   \

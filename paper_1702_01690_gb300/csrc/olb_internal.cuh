@@ -126,16 +126,17 @@ __host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);
 
-// The compiled shape that advances tiles of a shape: FP64 tiles of more than 64
-// nodes are advanced as 8 x 8 tiles (their faces, factors and differences fit in
-// shared memory beside the populations; the larger shapes kept one velocity's
-// faces at a time and recomputed per-node terms 25 times).
+// The compiled shape that advances tiles of a shape: FP64 tiles are advanced as
+// 8 x 8 tiles (their faces, factors and differences fit in shared memory beside
+// the populations; larger shapes kept one velocity's faces at a time and
+// recomputed per-node terms 25 times), those with eight lanes by 320 threads of
+// one node, the others by 160 threads of two (Plan64 in olb_stage64.cuh).
 struct Shape {
     int tx, ty, kp;
 };
 inline Shape stage_shape(bool fp64, bool learned, int tx, int ty, int kp)
 {
-    if (fp64 && tx * ty > 64) return {8, 8, learned ? 4 : 5};
+    if (fp64) return {8, 8, learned ? 4 : kp == 8 ? 8 : 5};
     return {tx, ty, kp};
 }
 
@@ -159,6 +160,7 @@ StageK stage_constants(const Geo &g, StageCoef c);
                                    const Tab<real> &t, StageCoef c, int st, int tx, int ty, int kp,    \
                                    void *fields,                                                       \
                                    const long long *node_start, long long total_nodes,                 \
+                                   const int *force_start, int force_blocks,                           \
                                    const TmaMap *tmaps, cudaStream_t s);                               \
     size_t batch_run_bytes(real *);                                                                    \
     void batch_run_fill(real *, void *dst, const Geo &g, const Tab<real> &t, long long off,            \
@@ -175,9 +177,11 @@ StageK stage_constants(const Geo &g, StageCoef c);
 OLB_DECLARE_LAUNCHERS(double)
 OLB_DECLARE_LAUNCHERS(float)
 
-// Bytes of the per-node moment fields of the stage pre-pass: 5 planes of
-// pitch * ny 8-byte elements.
-inline size_t fields_bytes(const Geo &g) { return (size_t)5 * g.plane * 8; }
+// Bytes of the per-node fields of the stage (fields_of in olb_fields.cuh): 7
+// (FP64) or 5 planes of pitch * ny 8-byte elements.
+inline size_t fields_bytes(const Geo &g, bool fp64) { return (size_t)(fp64 ? 7 : 5) * g.plane * 8; }
+// Blocks of the force kernel (32 x 8 nodes each) of a grid.
+inline int force_blocks(const Geo &g) { return ((g.nx + 31) / 32) * ((g.ny + 7) / 8); }
 
 // Global sums (olb_totals): fixed grid of the first reduction pass, whose
 // per-block partial sums (4 each) the second pass adds in a fixed order.

@@ -14,27 +14,63 @@
 //
 // Measured, one step (three stages) of a 4096^2 grid: 106.6 ms with the force and
 // the node updates in FP64 (1070 FP64 instructions a node and stage beside 60
-// differences), 56.8 ms like this (228); 24-run sweep, 8 steps: 39.7 -> 24.1 ms.
+// differences), 56.8 ms like this (228), 51.8 ms with three CTAs an SM, 46.5 ms
+// with the force in a kernel of its own (k_force) and two nodes a thread.
 // Against 80-bit arithmetic the populations are closer than the FP64 form's
 // (12 steps of a 167 x 109 drop: 5.7e-16 instead of 1.2e-15 of their norm, and
 // its loss of 1e-15 of the mass is gone): Delta is summed before the one
 // rounding at the size of f.
+//
+// What bounds it now (ncu, 1024^2): no pipe; FP64 57 %, issue slots 50 %, and
+// what three CTAs of five warps leave of latency (tiles hold 70 KB, and two nodes
+// a thread take 125 registers).
 #pragma once
 
-#include "olb_ff.cuh"
-#include "olb_internal.cuh"
-#include "olb_mlp.cuh"
+#include "olb_tile.cuh"
 
 namespace olb {
 
 // ---------------------------------------------------------------- shared memory
-template <int TX, int TY, int KP, bool LEARNED>
+// A float-float of the nodes (x, y) and (x, y + 4) of the tile: threads that take
+// two nodes (vf2) read and write it whole, threads that take one a half of it.
+struct __align__(16) ffp {
+    float h[2], l[2];
+    template <typename V>
+    __device__ __forceinline__ ffv<V> get(int half) const
+    {
+        if constexpr (V::W == 1) return {{h[half]}, {l[half]}};
+        else {
+            const float4 a = *reinterpret_cast<const float4 *>(this);
+            return {vf2::pair(a.x, a.y), vf2::pair(a.z, a.w)};
+        }
+    }
+    template <typename V>
+    __device__ __forceinline__ void put(int half, ffv<V> v)
+    {
+        if constexpr (V::W == 1) {
+            h[half] = v.h[0];
+            l[half] = v.l[0];
+        } else {
+            *reinterpret_cast<float4 *>(this) = make_float4(v.h[0], v.h[1], v.l[0], v.l[1]);
+        }
+    }
+};
+
+// Tile of 8 x 8 nodes.  KP selects the threads: 5: 160, two nodes or lines a
+// thread; 8: 320, one; 4: 256, one, with learned weights (whose network needs the
+// registers).  Time of a stage, 160 and 320 threads: 64 x 4 (8 tiles) 26.7 and
+// 24.2 us, 1024 x 8 (128) 29.4 and 26.9, 192 x 128 (384) 37.8 and 38.0, 512^2
+// (4096) 233 and 247, 1024^2 868 and 931: grids of at most one tile an SM take 320.
+template <int KP>
+struct Plan64 {
+    using V = typename std::conditional<KP == 5, vf2, vf1>::type;
+    static constexpr int NT = KP == 5 ? 160 : KP == 8 ? 320 : 256;
+};
+
+template <int KP, bool LEARNED>
 struct Smem64 {
-    // LS: threads per velocity lane, the tile's nodes rounded up to whole
-    // warps; NT threads in all; HP: pitch of a staged row of populations
-    static constexpr int HX = TX + 8, HY = TY + 6, NN = TX * TY, LS = (NN + 31) / 32 * 32, NT = LS * KP;
-    static constexpr int HP = region_pitch(TX, true);
-    static_assert(NN <= 64, "FP64 tiles hold at most 64 nodes");
+    static constexpr int TX = 8, TY = 8, HX = TX + 8, HY = TY + 6, NN = TX * TY, NT = Plan64<KP>::NT;
+    static constexpr int HP = region_pitch(TX, true);  // pitch of a staged row of populations
     // populations of the tile's rows (columns x0 - 4 ...) and of the three rows
     // below and above its nodes
     alignas(128) double mid[NK][TY][HP];
@@ -42,35 +78,20 @@ struct Smem64 {
     alignas(128) double above[NK][3][TX];
     double ex[NQ][NN];  // n g_q(u_x, T) and g_q(u_y, T) of the tile nodes
     double ey[NQ][NN];
-    ff G[2][NN];        // c F
-    union {
-        // phases 2 to 4: fields of the region, and differences v(+l) - v(-l),
-        // l = 1..3, of Delta p and n, along x for every row of the region and
-        // along y for every column that a stencil of the tile reaches: a value
-        // serves the seven nodes of a stencil row
-        struct {
-            double n[HY][HX];
-            double dp[HY][HX];
-            double ux[TY][TX];
-            double uy[TY][TX];
-            double T[TY][TX];
-            ff dx[2][3][HY][TX];
-            ff dy[2][3][TY][TX + 6];
-        };
-        // phase 5: flux differences times 6 (weno5_flux6) across the nodes of
-        // each row along x and column along y, of the 20 velocities that move
-        // along the axis (slot_x, slot_y; learned weights: first the faces'
-        // non-linear parts, one more than nodes, which the flux differences then
-        // replace); then, in place of one of a velocity's flux differences (inc),
-        // the sum of its advection and y force terms
-        struct {
-            ff ax[20][TY][TX + 1];
-            ff ay[20][TX][TY + 1];
-            ff rest[NN];
-        };
-    };
+    ffp G[2][NN / 2];   // c F
+    // flux differences times 6 (weno5_flux6) across the nodes of each row along x
+    // and column along y, of the 20 velocities that move along the axis (slot_x,
+    // slot_y; learned weights: first the faces' non-linear parts, one more than
+    // nodes, which the flux differences then replace); then, in place of one of a
+    // velocity's flux differences (inc), the sum of its advection and force
+    // terms.  Entry i of a column sits in half i / 4 of element i mod 4 (face 8:
+    // in element 4); the fifth element and the one at the end keep the banks of
+    // columns apart.
+    ffp ax[20][TY / 2][TX + 1];
+    ffp ay[20][TX * (TY / 2 + 1) + 1];
+    ffp rest[NN / 2];
     double wnw[2][TY];        // wall density of each tile row (Eq. nw)
-    int top;                  // high word of the largest n of the region (the tile's scale)
+    int top;                  // high word of the largest n of the tile (its scale)
     unsigned long long mbar;  // completion barrier of the TMA copies
 
     // the staged population k at row r and column c of the region; planes lie
@@ -84,9 +105,19 @@ struct Smem64 {
         return (r >= 3 && r < TY + 3) || (c >= 4 && c < TX + 4);
     }
     __device__ __forceinline__ static constexpr int plane(int r) { return r >= 3 && r < TY + 3 ? TY * HP : 3 * TX; }
-    __device__ __forceinline__ ff &inc(int k1, int k2, int x, int y)
+    static constexpr int TMA_BYTES = NK * (TY * HP + 6 * TX) * 8;
+    __device__ __forceinline__ void tma(const TmaMap *m, int x0, int y0, unsigned mbar)
     {
-        return k1 != 2 ? ax[NQ * (k1 < 2 ? k1 : k1 - 1) + k2][y][x] : k2 != 2 ? ay[8 + (k2 < 2 ? k2 : k2 - 1)][x][y] : rest[y * TX + x];
+        tma_load((unsigned)__cvta_generic_to_shared(&mid[0][0][0]), m->bytes[0], x0 - 4, y0, mbar);
+        tma_load((unsigned)__cvta_generic_to_shared(&below[0][0][0]), m->bytes[1], x0, y0 - 3, mbar);
+        tma_load((unsigned)__cvta_generic_to_shared(&above[0][0][0]), m->bytes[1], x0, y0 + TY, mbar);
+    }
+    __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i == 8 ? 4 : i & 3)]; }
+    __device__ __forceinline__ ffp &inc(int k1, int k2, int x, int y4)
+    {
+        return k1 != 2   ? ax[NQ * (k1 < 2 ? k1 : k1 - 1) + k2][y4][x]
+               : k2 != 2 ? ay[8 + (k2 < 2 ? k2 : k2 - 1)][5 * x + y4]
+                         : rest[8 * y4 + x];
     }
 };
 
@@ -94,57 +125,26 @@ struct Smem64 {
 __device__ __forceinline__ int slot_x(int k1, int k2) { return NQ * (k1 < 2 ? k1 : k1 - 1) + k2; }
 __device__ __forceinline__ int slot_y(int k1, int k2) { return 4 * k1 + (k2 < 2 ? k2 : k2 - 1); }
 
-// ---------------------------------------------------------------- stencils
-// The weights of the 49-point stencils (Eqs. stencil_grad, stencil_glap) as
-// whole numbers: 5040 l w(l, |m|) and 2160 c(|m|, l).
-__host__ __device__ constexpr int whole(double v) { return (int)(v < 0 ? v - 0.5 : v + 0.5); }
-
-// sum over l, m of weight(l, |m|) d(l, m), d giving the difference at offsets
-// +l, -l in the row (column) m away
-template <bool LAPLACIAN, typename D>
-__device__ __forceinline__ ff stencil_sum(D d)
-{
-    ff s = {0.0f, 0.0f};
-#pragma unroll
-    for (int l = 1; l <= 3; ++l)
-#pragma unroll
-        for (int m = -3; m <= 3; ++m) {
-            const int am = m < 0 ? -m : m;
-            const float w = LAPLACIAN ? (float)whole(2160.0 * glap_c(am, l)) : (float)whole(5040.0 * l * grad_w(l, am));
-            if (w != 0.0f) {
-                const ff v = d(l, m);
-                const float z = w * v.h;
-                s.l += fmaf(w, v.l, fmaf(w, v.h, -z));
-                ff_acc(s, z);
-            }
-        }
-    return s;
-}
-
 // ---------------------------------------------------------------- momentum derivative
 // (d_p f)_k of one axis (Eq. derf) from the five populations f of a row or
 // column: the matrix is odd under p -> -p, so with a_m = f_{2+m} - f_{2-m} and
 // s_m = f_{2+m} + f_{2-m}
 //   (d_p f)_{2 +- m} = (E_m2 a_2 + E_m1 a_1) +- (O_m2 s_2 + O_m1 s_1 + O_m0 f_2).
-__device__ __forceinline__ void dp_line(const FfTab &t, const ff f[NQ], ff out[NQ])
+template <typename V>
+__device__ __forceinline__ void dp_line(const FfTab &t, const ffv<V> f[NQ], ffv<V> out[NQ])
 {
-    auto add = [](ff a, ff b) {
-        ff s = {a.h, a.l + b.l};
-        ff_acc(s, b.h);
-        return s;
+    auto add = [](ffv<V> a, ffv<V> b) {
+        ff_acc(a, b);
+        return a;
     };
-    auto neg = [](ff a) { return ff{-a.h, -a.l}; };
-    auto mul = [](ff c, ff a) {
-        const float p = c.h * a.h;
-        return ff{p, fmaf(c.l, a.h, fmaf(c.h, a.l, fmaf(c.h, a.h, -p)))};
-    };
-    const ff a2 = ff_norm(add(f[4], neg(f[0]))), s2 = add(f[4], f[0]);
-    const ff a1 = ff_norm(add(f[3], neg(f[1]))), s1 = add(f[3], f[1]);
-    out[2] = add(mul(t.E[0][1], a2), mul(t.E[0][0], a1));
+    auto neg = [](ffv<V> a) { return ffv<V>{-a.h, -a.l}; };
+    const ffv<V> a2 = add(f[4], neg(f[0])), s2 = add(f[4], f[0]);
+    const ffv<V> a1 = add(f[3], neg(f[1])), s1 = add(f[3], f[1]);
+    out[2] = add(ff_mul(t.E[0][1], a2), ff_mul(t.E[0][0], a1));
 #pragma unroll
     for (int m = 1; m <= 2; ++m) {
-        const ff e = add(mul(t.E[m][1], a2), mul(t.E[m][0], a1));
-        const ff o = add(add(mul(t.O[m - 1][2], s2), mul(t.O[m - 1][1], s1)), mul(t.O[m - 1][0], f[2]));
+        const ffv<V> e = add(ff_mul(t.E[m][1], a2), ff_mul(t.E[m][0], a1));
+        const ffv<V> o = add(add(ff_mul(t.O[m - 1][2], s2), ff_mul(t.O[m - 1][1], s1)), ff_mul(t.O[m - 1][0], f[2]));
         out[2 + m] = add(o, e);
         out[2 - m] = add(neg(o), e);
     }
@@ -174,75 +174,67 @@ __device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, dou
 }
 
 // ---------------------------------------------------------------- the stage of one tile
-// tid: the thread's index in the CTA; all threads call it.  sm holds the
-// fields of phases 1 to 3, and the populations too, unless wait() still has to
-// be called for them (it returns false when the copy timed out).
-template <int TX, int TY, int KP, bool LEARNED, typename Wait>
-__device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const double *fn, double *out, const Geo &g,
-                                          const Tab<double> &t, const FfTab &ft, const StageK &c, int x0, int y0,
-                                          const float *mlp, Wait wait)
+// One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
+// call it.  fields: the moments and c F of fs (k_fields, k_force); tw: the table
+// of the wall entries; tmap: TMA maps of fs, or nullptr; mlp: the learned
+// network's parameters in shared memory (LEARNED only).  A thread takes V::W nodes
+// (y and y + 4 of a column) or lines (rows or columns 4 apart) at a time.
+// Returns false when the TMA copy timed out (the CTA must stop).
+template <int KP, bool LEARNED>
+__device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const double *__restrict__ fs, const double *fn,
+                                             double *out, int *__restrict__ status, const Geo &g, const Tab<double> &t,
+                                             const Tab<double> &tw, int x0, int y0, const StageK &c, const float *mlp,
+                                             const TmaMap *tmap, const StageFields<double> &fields)
 {
-    using S = Smem64<TX, TY, KP, LEARNED>;
-    constexpr int NT = S::NT, NN = S::NN, HY = S::HY, HP = S::HP;
+    using S = Smem64<KP, LEARNED>;
+    using V = typename Plan64<KP>::V;
+    constexpr int W = V::W, NT = S::NT, TX = S::TX, TY = S::TY, NN = S::NN, NI = NN / W, HP = S::HP;
     const int tid = threadIdx.x;
+    const FfTab &ft = t.ff;
+
+    // ---- 1. the fields of a node and axis (threads 0 .. 2 NN - 1), then the
+    // populations: copies in flight during phase 2 for a tile inside the grid
+    const int a = tid / NN, node = tid % NN, nx = node % TX, ny = node / TX;
+    const bool has = tid < 2 * NN && x0 + nx < g.nx && y0 + ny < g.ny;
+    double fn_ = 0.0, fu = 0.0, fT = 1.0;
+    ff fG = {0.0f, 0.0f};
+    if (has) {
+        const long long o = (long long)(y0 + ny) * g.pitch + (x0 + nx);
+        fn_ = fields.n[o];
+        fu = a == 0 ? fields.ux[o] : fields.uy[o];
+        fT = fields.T[o];
+        fG = (a == 0 ? fields.G[0] : fields.G[1])[o];
+    }
+    if (tid == 0) sm.top = 0;
+    const bool inside = tmap != nullptr && x0 >= 4 && x0 + TX + 4 <= g.nx && y0 >= 3 && y0 + TY + 3 <= g.ny;
+    if (inside) tma_issue(sm, tmap, x0, y0);
+    else load_region(sm, fs, g, x0, y0);
+    __syncthreads();
+
+    // ---- 2. equilibrium factors (FP64), the tile's scale (its largest density)
+    if (tid < 2 * NN) {
+        double w[NQ];
+        eq_factors64(t, fu, fT, w);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) (a == 0 ? sm.ex : sm.ey)[q][node] = a == 0 ? fn_ * w[q] : w[q];
+        ffp &G = sm.G[a][8 * (ny & 3) + nx];
+        G.h[ny >> 2] = fG.h;
+        G.l[ny >> 2] = fG.l;
+        const int hw = __double2hiint(fn_) & 0x7fffffff, top = __reduce_max_sync(0xffffffffu, hw < 0x7ff00000 ? hw : 0);
+        if ((tid & 31) == 0) atomicMax(&sm.top, top);
+    }
+    // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
+    const bool left = x0 == 0 && g.wall_lo, right = x0 + TX + 3 >= g.nx && g.wall_hi;
+    if (left || right) {
+        wall_flux<double, LEARNED>(sm, g, t, tw, mlp, x0, 2 * NN, left, right);
+        __syncthreads();
+        wall_ghosts<double>(sm, g, tw, x0, 0, left, right);
+    }
+    if (inside && !tma_finish(sm, status)) return false;
+    __syncthreads();
     const FfScale sc = ff_scale(sm.top);
 
-    // ---- 4a. differences of the fields
-    constexpr int NX = 3 * HY * TX, NY = 3 * TY * (TX + 6);
-    for (int e = tid; e < 2 * (NX + NY); e += NT) {
-        const int field = e >= NX + NY;
-        const double(*v)[S::HX] = field ? sm.n : sm.dp;
-        int q = field ? e - (NX + NY) : e;
-        if (q < NX) {
-            const int l = q / (HY * TX) + 1, r = q % (HY * TX) / TX, x = q % TX;
-            (&sm.dx[field][0][0][0])[q] = ff_split(v[r][x + 4 + l] - v[r][x + 4 - l], sc);
-        } else {
-            q -= NX;
-            const int l = q / (TY * (TX + 6)) + 1, y = q % (TY * (TX + 6)) / (TX + 6), x = q % (TX + 6);
-            (&sm.dy[field][0][0][0])[q] = ff_split(v[y + 3 + l][x + 1] - v[y + 3 - l][x + 1], sc);
-        }
-    }
-    __syncthreads();
-
-    // ---- 4b. on the first 128 threads G = c F = (c/ds) sum_dp / n + (c sigma/ds^3)
-    // sum_n from the stencil sums of grad(Delta p) and grad(Laplacian n), a node
-    // and axis a thread (the scale that the differences carry is taken out of
-    // 1/n and sum_n); on the next 128, meanwhile, the equilibrium factors (FP64)
-    static_assert(NT >= 256, "phase 4b takes 256 threads");
-    if (tid < 2 * NN) {
-        const int a = tid / NN, node = tid - a * NN, x = node % TX, y = node / TX;
-        ff sp, sn;
-        if (a == 0) {
-            sp = stencil_sum<false>([&](int l, int m) { return sm.dx[0][l - 1][y + 3 + m][x]; });
-            sn = stencil_sum<true>([&](int l, int m) { return sm.dx[1][l - 1][y + 3 + m][x]; });
-        } else {
-            sp = stencil_sum<false>([&](int l, int m) { return sm.dy[0][l - 1][y][x + 3 + m]; });
-            sn = stencil_sum<true>([&](int l, int m) { return sm.dy[1][l - 1][y][x + 3 + m]; });
-        }
-        const ff n = ff_split(sm.n[y + 3][x + 4], sc);
-        const float r = rcp_seed(n.h);
-        const ff inv = {r, r * fmaf(-r, n.l, fmaf(-r, n.h, 1.0f))};
-        ff v = ff_mul(ff_mul(sp, inv), c.kp);
-        const ff w = ff_mul(sn, c.kn);
-        // sum_n in the populations' units is 2^k of the scaled one
-        const int k = 127 - 1023 - (sc.off >> 20);
-        const int k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
-        const float u1 = f32_make((unsigned)(k1 + 127) << 23), u2 = f32_make((unsigned)(k2 + 127) << 23);
-        v.l += w.l * u1 * u2;
-        ff_acc(v, w.h * u1 * u2);
-        sm.G[a][node] = ff_norm(v);
-    } else if (tid >= 128 && tid < 128 + 2 * NN) {
-        const int a = (tid - 128) / NN, node = tid - 128 - a * NN, x = node % TX, y = node / TX;
-        double w[NQ];
-        eq_factors64(t, a == 0 ? sm.ux[y][x] : sm.uy[y][x], sm.T[y][x], w);
-        const double n = sm.n[y + 3][x + 4];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) (a == 0 ? sm.ex : sm.ey)[q][node] = a == 0 ? n * w[q] : w[q];
-    }
-    if (!wait()) return false;
-    __syncthreads();
-
-    // ---- 5a. flux differences, a tile row or column a thread
+    // ---- 5a. flux differences, W rows or columns a thread
     if constexpr (LEARNED) {
         // the faces of the 20 velocities with xi_x != 0, then of the 20 with xi_y != 0
         constexpr int nfx = (TX + 1) * TY, nfy = TX * (TY + 1);
@@ -262,20 +254,19 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
             // z = d1 + 2 d2 - 6 (F - v2)
             const ff f1 = ff_split(d1, sc), f2 = ff_split(d2, sc);
             const float c6 = 6.0f * corr.h;
-            ff z = {2.0f * f2.h, fmaf(2.0f, f2.l, f1.l) - fmaf(6.0f, corr.l, fmaf(6.0f, corr.h, -c6))};
-            ff_acc(z, f1.h);
-            ff_acc(z, -c6);
-            if (along_x) sm.ax[q][r][cc] = z;
-            else sm.ay[q][cc][r] = z;
+            ffv<vf1> z = {{2.0f * f2.h}, {fmaf(2.0f, f2.l, f1.l) - fmaf(6.0f, corr.l, fmaf(6.0f, corr.h, -c6))}};
+            ff_acc(z, vf1{f1.h});
+            ff_acc(z, vf1{-c6});
+            if (along_x) sm.ax[q][r & 3][cc].put(r >> 2, z);
+            else sm.col(q, cc, r).put(r == 8 ? 0 : r >> 2, z);
         }
         __syncthreads();
     }
-    // (one call for rows and columns of one length: a second copy of the code
-    // would not fit the instruction cache beside the first)
-    auto line = [&](auto n, bool along_x, int q, int i) {
+    for (int e = tid; e < 40 * (TX / W); e += NT) {
+        const bool along_x = e < 20 * (TX / W);
+        const int e2 = along_x ? e : e - 20 * (TX / W), q = e2 / (TX / W), i = e2 - q * (TX / W);
         const int k = along_x ? (q < 2 * NQ ? q : q + NQ) : (q >> 2) * NQ + ((q & 3) < 2 ? (q & 3) : (q & 3) + 1);
         const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-        constexpr int N = decltype(n)::value;
         // the three nodes behind the line, its nodes, and the two ahead
         const double *p0, *p1, *p2;
         int step = up ? 1 : -1, halo = step;
@@ -291,102 +282,116 @@ __device__ __forceinline__ bool advance64(Smem64<TX, TY, KP, LEARNED> &sm, const
             p1 = &sm.mid[k][up ? 0 : TY - 1][4 + i];
             p2 = up ? &sm.above[k][0][i] : &sm.below[k][2][i];
         }
-        ff *o = along_x ? &sm.ax[q][i][0] : &sm.ay[q][i][0];
-        // (the flux difference across a node takes the place of a face that it has used)
+        auto store = [&](int j, ffv<V> v) {
+            const int at = up ? j : TX - 1 - j;
+            if (along_x) {
+                sm.ax[q][i & 3][at].put(i >> 2, v);
+            } else {
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    ffp &o = sm.col(q, i + 4 * w, at);
+                    o.h[at >> 2] = v.h[w];
+                    o.l[at >> 2] = v.l[w];
+                }
+            }
+        };
+        // (learned: the flux difference across a node takes the place of a face that it has used)
         if constexpr (LEARNED)
-            weno5_row<N>(p0, p1, p2, halo, step, o + (up ? 0 : N - 1), up ? 1 : -1, sc,
-                         [&](int j) { return o[up ? j : N - j]; });
+            weno5_line<TX, V>(p0, p1, p2, along_x ? 4 * HP : 4, halo, step, sc, store, [&](int j) {
+                const int at = up ? j : TX - j;
+                return along_x ? sm.ax[q][i & 3][at].template get<V>(i >> 2)
+                               : sm.col(q, i, at).template get<V>(at == 8 ? 0 : at >> 2);
+            });
         else
-            weno5_row<N>(p0, p1, p2, halo, step, o + (up ? 0 : N - 1), up ? 1 : -1, sc);
-    };
-    for (int e = tid; e < 20 * (TY + TX); e += NT) {
-        const bool along_x = e < 20 * TY;
-        const int e2 = along_x ? e : e - 20 * TY, w = along_x ? TY : TX, q = e2 / w, i = e2 - q * w;
-        if constexpr (TX == TY) {
-            line(std::integral_constant<int, TX>(), along_x, q, i);
-        } else {
-            if (along_x) line(std::integral_constant<int, TX>(), true, q, i);
-            else line(std::integral_constant<int, TY>(), false, q, i);
-        }
+            weno5_line<TX, V>(p0, p1, p2, along_x ? 4 * HP : 4, halo, step, sc, store);
     }
     __syncthreads();
 
-    // f^n of the velocities that this thread advances in 5c, fetched now (with
-    // five lanes it advances one column)
-    constexpr int LINES = (NQ * NN + NT - 1) / NT;
-    double f0[LINES][NQ];
+    // f^n of the velocities that this thread advances in 5c, fetched now
+    constexpr int LINES = (NQ * NI + NT - 1) / NT;
+    double f0[LINES][NQ][W];
     if (c.ca.h != 0.0f)
 #pragma unroll
         for (int w = 0; w < LINES; ++w) {
-            const int e = tid + w * NT, k2 = e / NN, node = e - k2 * NN, x = node % TX, y = node / TX;
-            if (e >= NQ * NN || x0 + x >= g.nx || y0 + y >= g.ny) continue;
+            const int e = tid + w * NT, k2 = e / NI, it = e - k2 * NI, x = it % TX, y = it / TX;
 #pragma unroll
-            for (int k1 = 0; k1 < NQ; ++k1)
-                f0[w][k1] = fn[(NQ * k1 + k2) * g.plane + (long long)(y0 + y) * g.pitch + (x0 + x)];
+            for (int i = 0; i < W; ++i) {
+                if (e >= NQ * NI || x0 + x >= g.nx || y0 + y + 4 * i >= g.ny) continue;
+#pragma unroll
+                for (int k1 = 0; k1 < NQ; ++k1)
+                    f0[w][k1][i] = fn[(NQ * k1 + k2) * g.plane + (long long)(y0 + y + 4 * i) * g.pitch + (x0 + x)];
+            }
         }
 
-    // ---- 5b. a row of velocities (k1; k2 = 0..4) of a node a thread: the y force
-    // term and both advection terms of its velocities
-    for (int e = tid; e < NQ * NN; e += NT) {
-        const int k1 = e / NN, node = e - k1 * NN, x = node % TX, y = node / TX;
-        ff f[NQ], d[NQ];
+    // ---- 5b. a row of velocities (k1; k2 = 0..4) of W nodes a thread: both
+    // advection terms, and the y force term; then a column (k2; k1 = 0..4): the x
+    // force term, collision and RK-3 combination.  (One loop for both axes: the
+    // instructions of a stage have to stay in the cache, see weno5_line.)
+#pragma unroll 1
+    for (int axis = 1; axis >= 0; --axis) {
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) f[q] = ff_split(sm.mid[NQ * k1 + q][y][x + 4], sc);
-        dp_line(ft, f, d);
-        const ff Gy = sm.G[1][node];
-        const ff K1 = c.adv[k1 < 2 ? 2 - k1 : k1 - 2];
-#pragma unroll
-        for (int k2 = 0; k2 < NQ; ++k2) {
-            ff s = ff_mul(Gy, d[k2]);
-            if (k2 != 2) {
-                const ff v = ff_mul(sm.ay[slot_y(k1, k2)][x][y], c.adv[k2 < 2 ? 2 - k2 : k2 - 2]);
-                s.l += v.l;
-                ff_acc(s, v.h);
+        for (int w = 0; w < LINES; ++w) {
+            const int e = tid + w * NT, line = e / NI, it = e - line * NI, x = it % TX, y = it / TX;
+            if (e >= NQ * NI || x0 + x >= g.nx || y0 + y >= g.ny) continue;
+            // velocity k0 + q dk is (line, q) in a row, (q, line) in a column
+            const int k0 = axis ? NQ * line : line, dk = axis ? 1 : NQ;
+            if (axis) {
+                const ff K1 = c.adv[line < 2 ? 2 - line : line - 2];
+#pragma unroll 1
+                for (int k2 = 0; k2 < NQ; ++k2) {
+                    ffv<V> s = {V::all(0.0f), V::all(0.0f)};
+                    if (line != 2) s = ff_mul(K1, sm.ax[slot_x(line, k2)][y & 3][x].template get<V>(y >> 2));
+                    if (k2 != 2)
+                        ff_acc(s, ff_mul(c.adv[k2 < 2 ? 2 - k2 : k2 - 2],
+                                         sm.ay[slot_y(line, k2)][5 * x + (y & 3)].template get<V>(y >> 2)));
+                    sm.inc(line, k2, x, y & 3).put(y >> 2, s);
+                }
             }
-            if (k1 != 2) {
-                const ff v = ff_mul(sm.ax[slot_x(k1, k2)][y][x], K1);
-                s.l += v.l;
-                ff_acc(s, v.h);
+            double fv[NQ][W];
+            ffv<V> f[NQ], d[NQ];
+            const double *p = &sm.mid[k0][y][x + 4];
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+                for (int i = 0; i < W; ++i) fv[q][i] = p[q * dk * (TY * HP) + 4 * i * HP];
+                f[q] = ff_split<V>(fv[q], sc);
             }
-            sm.inc(k1, k2, x, y) = s;
-        }
-    }
-    __syncthreads();
-
-    // ---- 5c. a column of velocities (k2; k1 = 0..4) of a node a thread: the x
-    // force term, collision and RK-3 combination
+            dp_line(ft, f, d);
+            const ffv<V> G = sm.G[axis][8 * (y & 3) + x].template get<V>(y >> 2);
 #pragma unroll
-    for (int w = 0; w < LINES; ++w) {
-        const int e = tid + w * NT, k2 = e / NN, node = e - k2 * NN, x = node % TX, y = node / TX;
-        if (e >= NQ * NN || x0 + x >= g.nx || y0 + y >= g.ny) continue;
-        double fv[NQ];
-        ff f[NQ], d[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            fv[q] = sm.mid[NQ * q + k2][y][x + 4];
-            f[q] = ff_split(fv[q], sc);
-        }
-        dp_line(ft, f, d);
-        const ff Gx = sm.G[0][node];
-        const double gy = sm.ey[k2][node];
-        const long long o = (long long)(y0 + y) * g.pitch + (x0 + x);
-#pragma unroll
-        for (int k1 = 0; k1 < NQ; ++k1) {
-            const int k = NQ * k1 + k2;
-            const long long at = k * g.plane + o;
-            // (c/tau) (f^eq - f)
-            ff s = ff_mul(ff_split(fma(sm.ex[k1][node], gy, -fv[k1]), sc), c.cit);
-            if (c.ca.h != 0.0f) {
-                const ff v = ff_mul(ff_split(f0[w][k1] - fv[k1], sc), c.ca);
-                s.l += v.l;
-                ff_acc(s, v.h);
+            for (int q = 0; q < NQ; ++q) {
+                ffp &o = sm.inc(axis ? line : q, axis ? q : line, x, y & 3);
+                ffv<V> s = ff_mul(G, d[q]);
+                ff_acc(s, o.template get<V>(y >> 2));
+                o.put(y >> 2, s);
             }
-            const ff a = sm.inc(k1, k2, x, y), b = ff_mul(Gx, d[k1]);
-            s.l -= a.l + b.l;
-            ff_acc(s, -a.h);
-            ff_acc(s, -b.h);
-            out[at] = fv[k1] + ff_widen(ff_norm(s), sc);
+            if (axis) continue;
+            double gy[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) gy[i] = sm.ey[line][it + 32 * i];
+            double *o = out + line * g.plane + (long long)(y0 + y) * g.pitch + (x0 + x);
+#pragma unroll
+            for (int k1 = 0; k1 < NQ; ++k1) {
+                double q[W];
+                // (c/tau) (f^eq - f)
+#pragma unroll
+                for (int i = 0; i < W; ++i) q[i] = fma(sm.ex[k1][it + 32 * i], gy[i], -fv[k1][i]);
+                ffv<V> s = ff_mul(c.cit, ff_split<V>(q, sc));
+                if (c.ca.h != 0.0f) {
+#pragma unroll
+                    for (int i = 0; i < W; ++i) q[i] = f0[w][k1][i] - fv[k1][i];
+                    ff_acc(s, ff_mul(c.ca, ff_split<V>(q, sc)));
+                }
+                const ffv<V> a = sm.inc(k1, line, x, y & 3).template get<V>(y >> 2);
+                s.l = s.l - a.l;
+                ff_acc(s, -a.h);
+#pragma unroll
+                for (int i = 0; i < W; ++i)
+                    if (i == 0 || y0 + y + 4 * i < g.ny)
+                        o[k1 * NQ * g.plane + 4 * i * g.pitch] = fv[k1][i] + ff_widen(ff_lane(s, i), sc);
+            }
         }
+        if (axis) __syncthreads();
     }
     return true;
 }

@@ -25,9 +25,9 @@ using namespace olb;
 namespace {
 
 constexpr long long kMaxNodes = OLB_STATIC_MAX_NODES;
-// f^(1), f^(2) as [25][ny][nx] each, then the stage fields (fields_bytes: five
+// f^(1), f^(2) as [25][ny][nx] each, then the stage fields (fields_bytes: seven
 // values a node) and 256 bytes for the status word.
-constexpr long long kScratchDoubles = (2LL * NK + 5) * kMaxNodes + 32;
+constexpr long long kScratchDoubles = (2LL * NK + 7) * kMaxNodes + 32;
 
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
@@ -112,7 +112,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
     double *f1 = scratch;
     double *f2 = scratch + (long long)NK * g.plane;
     double *fields = scratch + 2LL * NK * kMaxNodes;
-    int *status = reinterpret_cast<int *>(fields + 5 * kMaxNodes);
+    int *status = reinterpret_cast<int *>(fields + 7 * kMaxNodes);
     cudaStream_t s = (cudaStream_t)stream;
 
     // shape, as olb_create picks it for FP64: 8 x 8 nodes with 5 velocity
@@ -123,12 +123,8 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
         cudaGetLastError();
         return OLB_ERR_CUDA;
     }
-    auto most_nodes = [&](int tx_, int ty_) {
-        const long long tiles = (long long)((g.nx + tx_ - 1) / tx_) * ((g.ny + ty_ - 1) / ty_);
-        return (tiles + sms - 1) / sms * tx_ * ty_;
-    };
-    const bool narrow = most_nodes(7, 8) < most_nodes(8, 8);
-    const int tx = narrow ? 7 : 8, ty = 8, kp = narrow ? 8 : 5;
+    const long long tiles = (long long)((g.nx + 7) / 8) * ((g.ny + 7) / 8);
+    const int tx = 8, ty = 8, kp = tiles <= sms ? 8 : 5;
     cudaError_t e = prepare_fused((double *)nullptr, tx, ty, kp, false);
     // the scratch keeps the previous call's contents: the status word must start at zero
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
