@@ -55,35 +55,10 @@ __device__ __forceinline__ NodeMoments<real> node_moments(Get get, const Geo &g,
 {
     NodeMoments<real> m;
     if constexpr (sizeof(real) == 8) {
-        // row and column sums of the 5 x 5 populations; the middle root is 0
-        // (R[2] = R2[2] = 0), so its sums drop out of j and e
-        double sx[NQ], sy[NQ];
-#pragma unroll
-        for (int k1 = 0; k1 < NQ; ++k1) {
-            double s = get(NQ * k1);
-            if (k1 == 0) sy[0] = s;
-            else sy[0] += s;
-#pragma unroll
-            for (int k2 = 1; k2 < NQ; ++k2) {
-                const double v = get(NQ * k1 + k2);
-                s += v;
-                if (k1 == 0) sy[k2] = v;
-                else sy[k2] += v;
-            }
-            sx[k1] = s;
-        }
-        double n = sx[0];
-        double jx = t.R[0] * sx[0];
-        double jy = t.R[0] * sy[0];
-        double en = t.R2[0] * (sx[0] + sy[0]);
-#pragma unroll
-        for (int k = 1; k < NQ; ++k) {
-            n += sx[k];
-            if (k == 2) continue;
-            jx = fma(t.R[k], sx[k], jx);
-            jy = fma(t.R[k], sy[k], jy);
-            en = fma(t.R2[k], sx[k] + sy[k], en);
-        }
+        const NodeSums s = node_sums64(get);
+        const double n = s.n;
+        const double jx = fma(t.R[4], s.a4x, t.R[3] * s.a3x), jy = fma(t.R[4], s.a4y, t.R[3] * s.a3y);
+        const double en = fma(t.R2[4], s.s4, t.R2[3] * s.s3);
         const double inv_n = recip_nr(n);
         const double ux = jx * inv_n, uy = jy * inv_n;
         const double T = 0.5 * fma(en, inv_n, -fma(ux, ux, uy * uy));

@@ -395,36 +395,131 @@ __device__ __forceinline__ void eq_correction(const Tab<float> &t, const float E
     gamma = 0.25f * Da;
 }
 
+// ---------------------------------------------------------------- sums of a node's populations
+// Sums over the 25 populations of a node in fixed point: 64-bit integers in units
+// of 2^-57 of the binade above the largest, so that the 48 additions (and the
+// differences that the momentum needs, exactly) run on the integer pipe; an FP64
+// addition takes the time of 64 FP32 or 32 integer instructions on a GB300.  A
+// population below 2^-4 of the largest is cut at 2^-57 of it, against 2^-54 that
+// one FP64 addition rounds away.  Measured on
+// 2048^2: the FP64 moments pre-pass 0.666 -> 0.384 ms; one FP64 step of 4096^2 with
+// its initial fields and moments 46.5 -> 40.2 ms, two FP32 steps 57.1 -> 52.1 ms.
+//
+// The sums that n, j and e = sum |p|^2 f are made of: n, sums and differences of
+// the rows and columns of velocity +-R_4 and +-R_3 (the middle root is 0).
+struct NodeSums {
+    double n, a4x, a3x, a4y, a3y, s4, s3;
+};
+
+// The larger of |a| and |b| as high words.
+__device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// v in units of 2^-57 of 2^(top's exponent + 1), cut towards zero
+__device__ __forceinline__ long long to_fixed(double v, int top)
+{
+    const int hw = __double2hiint(v);
+    const unsigned long long m =
+        ((unsigned long long)(unsigned)((hw & 0x000fffff) | 0x00100000) << 32 | (unsigned)__double2loint(v)) << 4;
+    const int s = (top >> 20) - ((hw >> 20) & 0x7ff);
+    const long long q = (long long)(m >> (s < 63 ? s : 63));
+    return hw < 0 ? -q : q;
+}
+// the same for a pair of floats (FP32 storage); |lo| is at most an ulp of hi
+__device__ __forceinline__ long long to_fixed(float v, int top)
+{
+    const int b = __float_as_int(v);
+    const unsigned long long m = (unsigned long long)((b & 0x007fffff) | 0x00800000) << 33;
+    const int s = (top >> 23) - ((b >> 23) & 0xff);
+    const long long q = (long long)(m >> (s < 63 ? s : 63));
+    return b < 0 ? -q : q;
+}
+
+// get(k): population k in FP64.
+template <typename Get>
+__device__ __forceinline__ NodeSums plain_sums(Get get)
+{
+    double sx[NQ], sy[NQ];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) sx[k] = sy[k] = 0.0;
+#pragma unroll
+    for (int k1 = 0; k1 < NQ; ++k1)
+#pragma unroll
+        for (int k2 = 0; k2 < NQ; ++k2) {
+            const double v = get(NQ * k1 + k2);
+            sx[k1] += v;
+            sy[k2] += v;
+        }
+    return {sx[0] + sx[1] + sx[2] + sx[3] + sx[4], sx[4] - sx[0], sx[3] - sx[1], sy[4] - sy[0], sy[3] - sy[1],
+            (sx[4] + sx[0]) + (sy[4] + sy[0]), (sx[3] + sx[1]) + (sy[3] + sy[1])};
+}
+
+// fixed(k): population k as a 64-bit integer in units of 2^-57 of 2^e.
+template <typename Fixed>
+__device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, double unit)
+{
+    long long sx[NQ], sy[NQ];
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) sx[k] = sy[k] = 0;
+#pragma unroll
+    for (int k1 = 0; k1 < NQ; ++k1)
+#pragma unroll
+        for (int k2 = 0; k2 < NQ; ++k2) {
+            const long long v = fixed(NQ * k1 + k2);
+            sx[k1] += v;
+            sy[k2] += v;
+        }
+    auto val = [&](long long v) { return (double)v * unit; };
+    return {val(sx[0] + sx[1] + sx[2] + sx[3] + sx[4]), val(sx[4] - sx[0]), val(sx[3] - sx[1]), val(sy[4] - sy[0]),
+            val(sy[3] - sy[1]), val(sx[4] + sx[0] + sy[4] + sy[0]), val(sx[3] + sx[1] + sy[3] + sy[1])};
+}
+
+// The sums of a node's populations, get(k) giving population k (FP64) or its hi
+// and lo parts (FP32).  Infinities, NaN and populations near the ends of the range
+// are summed in FP64.
+template <typename Get>
+__device__ __forceinline__ NodeSums node_sums64(Get get)
+{
+    int top = 0;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) top = max(top, abs_hi(get(k)));
+    if (top >= (2046 << 20) || top < (128 << 20)) return plain_sums(get);
+    // 2^(e - 56), e the exponent of the largest
+    return fixed_sums([&](int k) { return to_fixed(get(k), top); }, __hiloint2double((top & 0x7ff00000) - (56 << 20), 0));
+}
+template <typename Get>
+__device__ __forceinline__ NodeSums node_sums32(Get get)
+{
+    int top = 0;
+#pragma unroll
+    for (int k = 0; k < NK; ++k) top = max(top, __float_as_int(get(k).x) & 0x7fffffff);
+    if (top >= (254 << 23) || top < (64 << 23))
+        return plain_sums([&](int k) {
+            const float2 v = get(k);
+            return (double)v.x + (double)v.y;
+        });
+    return fixed_sums(
+        [&](int k) {
+            const float2 v = get(k);
+            return to_fixed(v.x, top) + to_fixed(v.y, top);
+        },
+        __hiloint2double(((top >> 23) - 127 + 1023 - 56) << 20, 0));
+}
+
 // Moments of the 25 populations at one node in FP64: n, jx, jy, e (FP32
-// storage: hi + lo of each population, summed in FP64; output kernels only).
+// storage: hi + lo of each population; output kernels only).
 template <typename real>
 __device__ __forceinline__ void node_sums(const real *__restrict__ f, long long plane, long long o,
                                           const Tab<double> &t, double &n, double &jx, double &jy, double &e)
 {
-    double sx[NQ], sy[NQ];
-#pragma unroll
-    for (int k = 0; k < NQ; ++k) sy[k] = 0.0;
-#pragma unroll
-    for (int k1 = 0; k1 < NQ; ++k1) {
-        double r = 0.0;
-#pragma unroll
-        for (int k2 = 0; k2 < NQ; ++k2) {
-            const long long q = (NQ * k1 + k2) * plane + o;
-            double v = (double)__ldg(f + q);
-            if constexpr (sizeof(real) == 4) v += (double)__ldg(f + NK * plane + q);
-            r += v;
-            sy[k2] += v;
-        }
-        sx[k1] = r;
-    }
-    n = jx = jy = e = 0.0;
-#pragma unroll
-    for (int k = 0; k < NQ; ++k) {
-        n += sx[k];
-        jx = fma(t.R[k], sx[k], jx);
-        jy = fma(t.R[k], sy[k], jy);
-        e = fma(t.R2[k], sx[k] + sy[k], e);
-    }
+    NodeSums s;
+    if constexpr (sizeof(real) == 8)
+        s = node_sums64([&](int k) { return __ldg(f + k * plane + o); });
+    else
+        s = node_sums32([&](int k) { return make_float2(__ldg(f + k * plane + o), __ldg(f + (NK + k) * plane + o)); });
+    n = s.n;
+    jx = fma(t.R[4], s.a4x, t.R[3] * s.a3x);
+    jy = fma(t.R[4], s.a4y, t.R[3] * s.a3y);
+    e = fma(t.R2[4], s.s4, t.R2[3] * s.s3);
 }
 
 // Store the FP64 value v of population plane offset q: FP64 as is, FP32 as
@@ -432,9 +527,25 @@ __device__ __forceinline__ void node_sums(const real *__restrict__ f, long long 
 __device__ __forceinline__ void store_pop(double *f, long long, long long q, double v) { f[q] = v; }
 __device__ __forceinline__ void store_pop(float *f, long long plane, long long q, double v)
 {
-    const float hi = __double2float_rn(v);
+    const int hw = __double2hiint(v), e = (hw >> 20) & 0x7ff;
+    const unsigned lw = (unsigned)__double2loint(v);
+    float hi, lo;
+    if (e > 1023 - 60 && e < 1023 + 120) {
+        // v rounded to 24 bits (to even) and the rest, a 29-bit integer with a
+        // sign, rounded: on the integer pipe (the conversions between FP64 and
+        // FP32 run at the FP64 rate)
+        const unsigned up = 0x0fffffffu + ((lw >> 29) & 1u), lr = lw + up;
+        const unsigned sign = (unsigned)hw & 0x80000000u;
+        const unsigned b = ((unsigned)(hw & 0x7fffffff) - (896u << 20) + (lr < lw ? 1u : 0u)) << 3 | lr >> 29;
+        hi = __uint_as_float(b | sign);
+        const int r = (int)(lw & 0x1fffffffu) - (((lr >> 29) & 7u) != (lw >> 29) ? 0x20000000 : 0);
+        lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 896 - 52) << 23 | sign);
+    } else {
+        hi = __double2float_rn(v);
+        lo = __double2float_rn(v - (double)hi);
+    }
     f[q] = hi;
-    f[NK * plane + q] = __double2float_rn(v - (double)hi);
+    f[NK * plane + q] = lo;
 }
 __device__ __forceinline__ double load_pop(const double *f, long long, long long q) { return f[q]; }
 __device__ __forceinline__ double load_pop(const float *f, long long plane, long long q)
@@ -473,11 +584,11 @@ __global__ void k_moments_out(const real *__restrict__ f, double *__restrict__ o
     const long long o = (long long)j * g.pitch + i;
     double n, jx, jy, e;
     node_sums<real>(f, g.plane, o, t, n, jx, jy, e);
-    const double ux = jx / n, uy = jy / n;
+    const double inv = 1.0 / n, ux = jx * inv, uy = jy * inv;
     if (on) on[idx] = n;
     if (oux) oux[idx] = ux;
     if (ouy) ouy[idx] = uy;
-    if (oT) oT[idx] = 0.5 * (e / n - fma(ux, ux, uy * uy));
+    if (oT) oT[idx] = 0.5 * fma(e, inv, -fma(ux, ux, uy * uy));
 }
 
 template <typename real>
