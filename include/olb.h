@@ -220,9 +220,9 @@ int olb_profile(olb_ctx *ctx, int nsteps, double *ms, int *launches);
  * (32,16,1), (8,8,8), (7,8,8), (8,8,5); olb_create picks one from the
  * grid size ((8,8,5), FP64: or (8,8,8) on grids of at most one tile an SM;
  * (8,8,4) with learned weights).  With
- * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  FP64 tiles are
- * advanced as 8 x 8 tiles whatever the shape, by 320 threads each with kp = 8
- * and by 160 otherwise (learned weights: 256).  olb_set_tile returns
+ * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  Whatever the
+ * shape, tiles are advanced as 8 x 8 nodes, in FP64 by 320 threads with kp = 8 and
+ * by 160 otherwise.  olb_set_tile returns
  * OLB_ERR_ARG for any other shape; results do not depend on the shape.
  * Not part of the paper (a tuning knob). */
 int olb_set_tile(olb_ctx *ctx, int tx, int ty, int kp);

@@ -44,7 +44,7 @@ bool olb::tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int
 {
     static_assert(sizeof(TmaMap) == 2 * sizeof(CUtensorMap), "TmaMap must hold two CUtensorMaps");
     const size_t elt = fp64 ? 8 : 4;
-    const unsigned hx = (unsigned)region_pitch(tx, fp64), hy = (unsigned)ty + 6;
+    const unsigned hx = (unsigned)region_pitch(tx, fp64);
     // the boxes' rows must be whole 16-byte units, and their x starts x0 - 4
     // and x0 (x0 a multiple of tx) must sit on a 16-byte boundary for every tile
     if ((hx * elt) % 16 != 0 || ((size_t)tx * elt) % 16 != 0 || (4 * elt) % 16 != 0) return false;
@@ -54,9 +54,9 @@ bool olb::tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int
     const cuuint32_t planes = fp64 ? (cuuint32_t)pop_planes<double>() : (cuuint32_t)pop_planes<float>();
     const cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, planes};
     const cuuint64_t strides[2] = {(cuuint64_t)g.pitch * elt, (cuuint64_t)g.plane * elt};
-    const cuuint32_t box[2][3] = {{hx, fp64 ? (cuuint32_t)ty : hy, planes}, {(cuuint32_t)tx, 3, planes}};
+    const cuuint32_t box[2][3] = {{hx, (cuuint32_t)ty, planes}, {(cuuint32_t)tx, 3, planes}};
     const cuuint32_t estr[3] = {1, 1, 1};
-    for (int k = 0; k < (fp64 ? 2 : 1); ++k) {
+    for (int k = 0; k < 2; ++k) {
         CUtensorMap m;
         const CUresult r = fn(&m, fp64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
                               const_cast<void *>(base), dims, strides, box[k], estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

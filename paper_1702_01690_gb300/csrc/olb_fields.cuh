@@ -2,6 +2,8 @@
 // moments (one thread per node), and in FP64 the force.
 #pragma once
 
+#include <type_traits>
+
 #include "olb_kernels.cuh"
 
 namespace olb {
@@ -141,12 +143,13 @@ struct StageFields {
     using fld = typename FieldT<real>::type;
     fld *n, *dp, *T, *E;
     real *ux, *uy;
-    ff *G[2];  // FP64: c F along x and y (k_force)
+    typename std::conditional<sizeof(real) == 8, ff, float>::type *G[2];  // c F along x and y (k_force)
 };
 
 // Pointers of the fields in a buffer of planes of pitch * ny 8-byte elements
 // (fields_bytes): FP64 n, Delta p, T, u_x, u_y, c F_x, c F_y; FP32 n, Delta p,
-// T, e (float2 each), then u_x and u_y (float) sharing the last plane.
+// T, e (float2 each), then u_x and u_y (float) sharing a plane, and c F_x and c
+// F_y.
 template <typename real>
 __host__ __device__ inline StageFields<real> fields_of(void *base, const Geo &g)
 {
@@ -166,6 +169,8 @@ __host__ __device__ inline StageFields<real> fields_of(void *base, const Geo &g)
         f.E = reinterpret_cast<typename FieldT<real>::type *>(b + 3 * plane);
         f.ux = reinterpret_cast<real *>(b + 4 * plane);
         f.uy = reinterpret_cast<real *>(b + 4 * plane + plane / 2);
+        f.G[0] = reinterpret_cast<real *>(b + 5 * plane);
+        f.G[1] = reinterpret_cast<real *>(b + 5 * plane + plane / 2);
     }
     return f;
 }
@@ -262,7 +267,7 @@ __global__ void __launch_bounds__(256) k_fields_batch(const real *__restrict__ f
     }
 }
 
-// ---------------------------------------------------------------- force (FP64)
+// ---------------------------------------------------------------- force
 // c F = (c/ds) sum_dp / n + (c sigma/ds^3) sum_n at every node from the 49-point
 // stencils of Delta p and n (Eqs. F_def, stencil_grad, stencil_glap), in a launch
 // of its own between the moments and the stage: inside the stage kernel it took
@@ -271,7 +276,7 @@ __global__ void __launch_bounds__(256) k_fields_batch(const real *__restrict__ f
 // clock64), and three tiles are all that an SM holds.  Here blocks are small, 32
 // x 8 nodes share a halo, and two nodes a thread keep the FP32 pipe busy.
 //
-// Differences v(+l) - v(-l), l = 1..3, along x for every row of the block's region
+// FP64: differences v(+l) - v(-l), l = 1..3, along x for every row of the block's region
 // and along y for every column are taken once in FP64 (a value serves the seven
 // nodes of a stencil row) and summed in float-float arithmetic.
 
@@ -413,22 +418,108 @@ __device__ __forceinline__ void force_block(ForceSmem &sm, const StageFields<dou
     }
 }
 
-static __global__ void __launch_bounds__(FORCE_THREADS) k_force(StageFields<double> f, const __grid_constant__ Geo g,
-                                                                const __grid_constant__ StageK c)
+// FP32: n and Delta p as pairs hi + lo.  grad(Delta p) in FP32 from differences of
+// pairs; the capillary stencil cancels its O(ds) terms down to O(ds^3) (a factor
+// ~1/(ds k)^2 on fine grids), so its weighted differences are summed in
+// double-float arithmetic with double-float weights (exact products of the hi
+// parts, TwoSum accumulation): the sum keeps FP32 accuracy of itself, not of its
+// terms.
+struct ForceSmem32 {
+    static constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
+    float2 dp[HY][HX], n[HY][HX];
+};
+// sums along x (y) at the node whose field is *v, fields sl apart along the
+// direction of the derivative and sm across it
+__device__ __forceinline__ float grad_sum32(const float2 *v, int sl, int sm)
 {
-    __shared__ ForceSmem sm;
-    force_block(sm, f, g, c, blockIdx.x * FORCE_X, blockIdx.y * FORCE_Y);
+    float acc = 0.0f;
+#pragma unroll
+    for (int l = 1; l <= 3; ++l)
+#pragma unroll
+        for (int m = -3; m <= 3; ++m) {
+            const int am = m < 0 ? -m : m;
+            if (grad_w(l, am) != 0.0)
+                acc = fmaf((float)(l * grad_w(l, am)), field_diff(v[m * sm + l * sl], v[m * sm - l * sl]), acc);
+        }
+    return acc;
+}
+__device__ __forceinline__ float glap_sum32(const float2 *v, int sl, int sm)
+{
+    f2 sum{0.0f, 0.0f};
+#pragma unroll
+    for (int l = 1; l <= 3; ++l)
+#pragma unroll
+        for (int m = -3; m <= 3; ++m) {
+            const int am = m < 0 ? -m : m;
+            if (glap_c(am, l) != 0.0) {
+                const float wh = (float)glap_c(am, l);
+                const float wl = (float)(glap_c(am, l) - (double)(float)glap_c(am, l));
+                const float2 a = v[m * sm + l * sl], b = v[m * sm - l * sl];
+                const f2 dh = two_sum(a.x, -b.x);
+                const float dl = dh.lo + (a.y - b.y);
+                const float p = wh * dh.hi;
+                const float e = fmaf(wh, dh.hi, -p);
+                const float tl = fmaf(wh, dl, fmaf(wl, dh.hi, e));
+                const f2 t2 = two_sum(sum.hi, p);
+                sum = f2{t2.hi, t2.lo + (sum.lo + tl)};
+            }
+        }
+    return sum.hi + sum.lo;
+}
+// cc: the stage's coefficient of dt L
+__device__ __forceinline__ void force_block32(ForceSmem32 &sm, const StageFields<float> &f, const Geo &g, float cc, int x0,
+                                              int y0)
+{
+    constexpr int HX = ForceSmem32::HX, HY = ForceSmem32::HY;
+    for (int e = threadIdx.x; e < HY * HX; e += 2 * FORCE_THREADS) {
+        const int r = e / HX, x = e - r * HX;
+        const long long o = (long long)field_index(y0 - 3 + r, g.ny, g.spec_y) * g.pitch + field_index(x0 - 3 + x, g.nx, g.walls);
+        sm.dp[r][x] = f.dp[o];
+        sm.n[r][x] = f.n[o];
+    }
+    __syncthreads();
+    const int x = threadIdx.x % FORCE_X, y = threadIdx.x / FORCE_X;
+    if (x0 + x >= g.nx || y0 + y >= g.ny) return;
+    const float2 *dp = &sm.dp[y + 3][x + 3], *n = &sm.n[y + 3][x + 3];
+    const float dn = (float)g.inv_ds / field_val(*n), sg3 = (float)g.sigma * (float)g.inv_ds3;
+    const long long o = (long long)(y0 + y) * g.pitch + (x0 + x);
+    f.G[0][o] = cc * fmaf(grad_sum32(dp, 1, HX), dn, sg3 * glap_sum32(n, 1, HX));
+    f.G[1][o] = cc * fmaf(grad_sum32(dp, HX, 1), dn, sg3 * glap_sum32(n, HX, 1));
+}
+
+template <typename real>
+struct ForceOf {
+    using Smem = ForceSmem;
+    static constexpr int NT = FORCE_THREADS;
+};
+template <>
+struct ForceOf<float> {
+    using Smem = ForceSmem32;
+    static constexpr int NT = 2 * FORCE_THREADS;
+};
+template <typename real>
+__global__ void __launch_bounds__(ForceOf<real>::NT) k_force(StageFields<real> f, const __grid_constant__ Geo g,
+                                                             const __grid_constant__ StageK c, real cc)
+{
+    __shared__ typename ForceOf<real>::Smem sm;
+    if constexpr (sizeof(real) == 8) force_block(sm, f, g, c, blockIdx.x * FORCE_X, blockIdx.y * FORCE_Y);
+    else force_block32(sm, f, g, cc, blockIdx.x * FORCE_X, blockIdx.y * FORCE_Y);
 }
 
 // the blocks of every run, in the order of force_start (prefix sum of their numbers)
-static __global__ void __launch_bounds__(FORCE_THREADS) k_force_batch(char *fields, const BatchRun<double> *__restrict__ runs,
-                                                                      const int *__restrict__ force_start, int nruns, int st)
+template <typename real>
+__global__ void __launch_bounds__(ForceOf<real>::NT) k_force_batch(char *fields, const BatchRun<real> *__restrict__ runs,
+                                                                   const int *__restrict__ force_start, int nruns, int st,
+                                                                   real ccoef)
 {
-    __shared__ ForceSmem sm;
+    __shared__ typename ForceOf<real>::Smem sm;
     const int lo = run_of(force_start, nruns, (int)blockIdx.x);
-    const BatchRun<double> &run = runs[lo];
+    const BatchRun<real> &run = runs[lo];
     const int b = blockIdx.x - __ldg(force_start + lo), nbx = (run.g.nx + FORCE_X - 1) / FORCE_X;
-    force_block(sm, fields_of<double>(fields + run.foff, run.g), run.g, run.k[st], b % nbx * FORCE_X, b / nbx * FORCE_Y);
+    const StageFields<real> f = fields_of<real>(fields + run.foff, run.g);
+    const int x0 = b % nbx * FORCE_X, y0 = b / nbx * FORCE_Y;
+    if constexpr (sizeof(real) == 8) force_block(sm, f, run.g, run.k[st], x0, y0);
+    else force_block32(sm, f, run.g, ccoef * (real)run.g.dt, x0, y0);
 }
 
 }  // namespace olb

@@ -102,12 +102,11 @@ void set_sides(Geo *g, const ::olb_params *p);
 int cuda_status(cudaError_t e);
 
 // TMA tensor maps (CUtensorMap, 128 bytes, 64-byte aligned) over one population
-// buffer as a 3-D tensor [planes][ny][nx] with row stride pitch.  FP32: one box
-// (pitch of a staged row) x (TY + 6) x planes, the staged region of a tile.
-// FP64: the rows of the tile, (pitch of a staged row) x TY x planes, and the
-// three rows above or below its nodes, TX x 3 x planes: the corners of the
-// region, which no face reads, are left out (39 KB instead of 51 KB for an
-// 8 x 8 tile, and three CTAs on an SM instead of two).
+// buffer as a 3-D tensor [planes][ny][nx] with row stride pitch: a box of the rows
+// of a tile, (pitch of a staged row) x TY x planes, and one of the three rows
+// above or below its nodes, TX x 3 x planes.  The corners of the region, which no
+// face reads, are left out (39 KB instead of 51 KB for an FP64 tile, and three
+// CTAs on an SM instead of two).
 struct alignas(64) TmaMap {
     unsigned char bytes[2][128];
 };
@@ -117,27 +116,30 @@ struct alignas(64) TmaArg {
     TmaMap map;
     int on;
 };
-// Pitch (elements) of a staged row of a tile's region, TX + 8 nodes wide: FP64
-// rows of even tiles get two more, so that the strips of the eight rows of a
-// tile start 4 banks apart (rows of TX + 8 doubles are whole multiples of the 32
-// banks or halves of it, and the strips of a warp would queue for two banks).
-__host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 8 + (fp64 && tx % 2 == 0 ? 2 : 0); }
+// Pitch (elements) of a staged row of a tile's region, TX + 8 nodes wide, with two
+// (FP64) or four (FP32) more: the lines of the eight rows of a tile then start in
+// different banks (rows of TX + 8 are whole multiples of the 32 banks or halves of
+// it, and the lines of a warp would queue for one or two).
+__host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 8 + (fp64 ? 2 : 4); }
 // Encode the maps of buffer `base` for tile shape tx x ty (olb_api.cu); false
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);
 
-// The compiled shape that advances tiles of a shape: FP64 tiles are advanced as
-// 8 x 8 tiles (their faces, factors and differences fit in shared memory beside
-// the populations; larger shapes kept one velocity's faces at a time and
-// recomputed per-node terms 25 times), those with eight lanes by 320 threads of
-// one node, the others by 160 threads of two (Plan64 in olb_stage64.cuh).
+// The compiled shape that advances tiles of a shape: all tiles are advanced as 8 x 8
+// tiles (their flux differences and factors fit in shared memory beside the
+// populations; larger shapes kept one velocity's faces at a time and recomputed
+// per-node terms 25 times: FP32 4096^2 14 ms a stage with 32 x 16 against 8).
+// FP64 shapes with eight lanes take 320 threads of one node, the others 160 of
+// two (Plan64 in olb_stage64.cuh).
 struct Shape {
     int tx, ty, kp;
 };
-inline Shape stage_shape(bool fp64, bool learned, int tx, int ty, int kp)
+inline Shape stage_shape(bool fp64, bool learned, int, int, int kp) { return {8, 8, learned ? 4 : fp64 && kp == 8 ? 8 : 5}; }
+
+// Shapes that olb_set_tile accepts with learned weights.
+inline bool learned_shape(int tx, int ty, int kp)
 {
-    if (fp64) return {8, 8, learned ? 4 : kp == 8 ? 8 : 5};
-    return {tx, ty, kp};
+    return (tx == 8 && ty == 8 && kp == 4) || (tx == 16 && ty == 8 && kp == 2) || (tx == 32 && ty == 16 && kp == 1);
 }
 
 // RK-3 stage coefficients: out = ca f^n + cb f_s + cc L[f_s] (Eq. rk3).
@@ -178,8 +180,8 @@ OLB_DECLARE_LAUNCHERS(double)
 OLB_DECLARE_LAUNCHERS(float)
 
 // Bytes of the per-node fields of the stage (fields_of in olb_fields.cuh): 7
-// (FP64) or 5 planes of pitch * ny 8-byte elements.
-inline size_t fields_bytes(const Geo &g, bool fp64) { return (size_t)(fp64 ? 7 : 5) * g.plane * 8; }
+// (FP64) or 6 planes of pitch * ny 8-byte elements.
+inline size_t fields_bytes(const Geo &g, bool fp64) { return (size_t)(fp64 ? 7 : 6) * g.plane * 8; }
 // Blocks of the force kernel (32 x 8 nodes each) of a grid.
 inline int force_blocks(const Geo &g) { return ((g.nx + 31) / 32) * ((g.ny + 7) / 8); }
 
@@ -187,8 +189,8 @@ inline int force_blocks(const Geo &g) { return ((g.nx + 31) / 32) * ((g.ny + 7) 
 // per-block partial sums (4 each) the second pass adds in a fixed order.
 constexpr int TOTALS_BLOCKS = 1024, TOTALS_THREADS = 256;
 
-// Stage-kernel shapes compiled for both precisions: TX x TY nodes per CTA
-// and KP velocities advanced at once.
+// Shapes that olb_set_tile accepts: TX x TY nodes and KP velocities at once
+// (stage_shape: what advances them).
 constexpr int NUM_TILES = 8;
 constexpr int TILE_X[NUM_TILES] = {8, 16, 16, 32, 32, 8, 7, 8};
 constexpr int TILE_Y[NUM_TILES] = {8, 8, 8, 8, 16, 8, 8, 8};

@@ -68,14 +68,8 @@ struct Plan64 {
 };
 
 template <int KP, bool LEARNED>
-struct Smem64 {
-    static constexpr int TX = 8, TY = 8, HX = TX + 8, HY = TY + 6, NN = TX * TY, NT = Plan64<KP>::NT;
-    static constexpr int HP = region_pitch(TX, true);  // pitch of a staged row of populations
-    // populations of the tile's rows (columns x0 - 4 ...) and of the three rows
-    // below and above its nodes
-    alignas(128) double mid[NK][TY][HP];
-    alignas(128) double below[NK][3][TX];
-    alignas(128) double above[NK][3][TX];
+struct Smem64 : Staged<double> {
+    static constexpr int NT = Plan64<KP>::NT;
     double ex[NQ][NN];  // n g_q(u_x, T) and g_q(u_y, T) of the tile nodes
     double ey[NQ][NN];
     ffp G[2][NN / 2];   // c F
@@ -90,28 +84,8 @@ struct Smem64 {
     ffp ax[20][TY / 2][TX + 1];
     ffp ay[20][TX * (TY / 2 + 1) + 1];
     ffp rest[NN / 2];
-    double wnw[2][TY];        // wall density of each tile row (Eq. nw)
-    int top;                  // high word of the largest n of the tile (its scale)
-    unsigned long long mbar;  // completion barrier of the TMA copies
+    int top;            // high word of the largest n of the tile (its scale)
 
-    // the staged population k at row r and column c of the region; planes lie
-    // plane(r) apart; the corners of the region are not staged
-    __device__ __forceinline__ double *at(int k, int r, int c)
-    {
-        return r < 3 ? &below[k][r][c - 4] : r < TY + 3 ? &mid[k][r - 3][c] : &above[k][r - TY - 3][c - 4];
-    }
-    __device__ __forceinline__ static constexpr bool staged(int r, int c)
-    {
-        return (r >= 3 && r < TY + 3) || (c >= 4 && c < TX + 4);
-    }
-    __device__ __forceinline__ static constexpr int plane(int r) { return r >= 3 && r < TY + 3 ? TY * HP : 3 * TX; }
-    static constexpr int TMA_BYTES = NK * (TY * HP + 6 * TX) * 8;
-    __device__ __forceinline__ void tma(const TmaMap *m, int x0, int y0, unsigned mbar)
-    {
-        tma_load((unsigned)__cvta_generic_to_shared(&mid[0][0][0]), m->bytes[0], x0 - 4, y0, mbar);
-        tma_load((unsigned)__cvta_generic_to_shared(&below[0][0][0]), m->bytes[1], x0, y0 - 3, mbar);
-        tma_load((unsigned)__cvta_generic_to_shared(&above[0][0][0]), m->bytes[1], x0, y0 + TY, mbar);
-    }
     __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i == 8 ? 4 : i & 3)]; }
     __device__ __forceinline__ ffp &inc(int k1, int k2, int x, int y4)
     {
@@ -241,7 +215,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
         for (int e = tid; e < 20 * (nfx + nfy); e += NT) {
             const bool along_x = e < 20 * nfx;
             const int e2 = along_x ? e : e - 20 * nfx, nf = along_x ? nfx : nfy, q = e2 / nf, f = e2 - q * nf;
-            const int k = along_x ? (q < 2 * NQ ? q : q + NQ) : (q >> 2) * NQ + ((q & 3) < 2 ? (q & 3) : (q & 3) + 1);
+            const int k = line_velocity(along_x, q);
             const int r = along_x ? f / (TX + 1) : f / TX, cc = along_x ? f - r * (TX + 1) : f - r * TX;
             if (along_x ? (y0 + r >= g.ny || x0 + cc > g.nx) : (x0 + cc >= g.nx || y0 + r > g.ny)) continue;
             const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
@@ -265,23 +239,8 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
     for (int e = tid; e < 40 * (TX / W); e += NT) {
         const bool along_x = e < 20 * (TX / W);
         const int e2 = along_x ? e : e - 20 * (TX / W), q = e2 / (TX / W), i = e2 - q * (TX / W);
-        const int k = along_x ? (q < 2 * NQ ? q : q + NQ) : (q >> 2) * NQ + ((q & 3) < 2 ? (q & 3) : (q & 3) + 1);
-        const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-        // the three nodes behind the line, its nodes, and the two ahead
-        const double *p0, *p1, *p2;
-        int step = up ? 1 : -1, halo = step;
-        if (along_x) {
-            const double *row = &sm.mid[k][i][0];
-            p0 = row + (up ? 1 : TX + 6);
-            p1 = row + (up ? 4 : TX + 3);
-            p2 = row + (up ? TX + 4 : 3);
-        } else {
-            halo = step * TX;
-            step *= HP;
-            p0 = up ? &sm.below[k][0][i] : &sm.above[k][2][i];
-            p1 = &sm.mid[k][up ? 0 : TY - 1][4 + i];
-            p2 = up ? &sm.above[k][0][i] : &sm.below[k][2][i];
-        }
+        const Line<double> ln = line_of<double>(sm, along_x, q, i);
+        const bool up = ln.up;
         auto store = [&](int j, ffv<V> v) {
             const int at = up ? j : TX - 1 - j;
             if (along_x) {
@@ -297,13 +256,13 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
         };
         // (learned: the flux difference across a node takes the place of a face that it has used)
         if constexpr (LEARNED)
-            weno5_line<TX, V>(p0, p1, p2, along_x ? 4 * HP : 4, halo, step, sc, store, [&](int j) {
+            weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store, [&](int j) {
                 const int at = up ? j : TX - j;
                 return along_x ? sm.ax[q][i & 3][at].template get<V>(i >> 2)
                                : sm.col(q, i, at).template get<V>(at == 8 ? 0 : at >> 2);
             });
         else
-            weno5_line<TX, V>(p0, p1, p2, along_x ? 4 * HP : 4, halo, step, sc, store);
+            weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
     }
     __syncthreads();
 

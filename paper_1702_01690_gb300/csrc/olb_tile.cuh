@@ -55,8 +55,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned mbar, unsigned parity)
 }
 
 // Phase 1 for a tile whose staged region lies inside the grid: TMA copies of the
-// boxes at (x0, y0) of the tensor maps (TmaMap) into the staging arrays (FP32:
-// pop, then the lo planes, contiguous in the box's order), completion tracked by
+// boxes of the tensor maps (TmaMap) into the staging arrays, completion tracked by
 // an mbarrier.  tma_issue starts the copies (all threads call it; it
 // synchronises); tma_finish waits for them with the bounded wait.  If the wait
 // runs out, bit 1 of the status word is set, the copies are waited for once more
@@ -96,6 +95,76 @@ __device__ __forceinline__ bool tma_finish(Smem &sm, int *status)
     // every thread has passed its wait (the barrier above)
     if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(mbar) : "memory");
     return true;
+}
+
+// Staged populations of an 8 x 8 tile: P planes (FP64 25; FP32 25 hi, then 25 lo)
+// of the tile's rows (columns x0 - 4 ...) and of the three rows below and above
+// its nodes.
+template <typename real>
+struct Staged {
+    static constexpr int TX = 8, TY = 8, HX = TX + 8, HY = TY + 6, NN = TX * TY, P = pop_planes<real>();
+    static constexpr int HP = region_pitch(TX, sizeof(real) == 8);  // pitch of a staged row
+    alignas(128) real mid[P][TY][HP];
+    alignas(128) real below[P][3][TX];
+    alignas(128) real above[P][3][TX];
+    real wnw[2][TY];          // wall density of each tile row (Eq. nw)
+    unsigned long long mbar;  // completion barrier of the TMA copies
+
+    // plane k at row r and column c of the region (r: y = y0 - 3 + r, c: x = x0 - 4 +
+    // c); planes lie plane(r) apart; the corners of the region are not staged
+    __device__ __forceinline__ real *at(int k, int r, int c)
+    {
+        return r < 3 ? &below[k][r][c - 4] : r < TY + 3 ? &mid[k][r - 3][c] : &above[k][r - TY - 3][c - 4];
+    }
+    __device__ __forceinline__ static constexpr bool staged(int r, int c)
+    {
+        return (r >= 3 && r < TY + 3) || (c >= 4 && c < TX + 4);
+    }
+    __device__ __forceinline__ static constexpr int plane(int r) { return r >= 3 && r < TY + 3 ? TY * HP : 3 * TX; }
+    static constexpr int TMA_BYTES = P * (TY * HP + 6 * TX) * (int)sizeof(real);
+    __device__ __forceinline__ void tma(const TmaMap *m, int x0, int y0, unsigned bar)
+    {
+        tma_load((unsigned)__cvta_generic_to_shared(&mid[0][0][0]), m->bytes[0], x0 - 4, y0, bar);
+        tma_load((unsigned)__cvta_generic_to_shared(&below[0][0][0]), m->bytes[1], x0, y0 - 3, bar);
+        tma_load((unsigned)__cvta_generic_to_shared(&above[0][0][0]), m->bytes[1], x0, y0 + TY, bar);
+    }
+};
+
+// A line of an 8 x 8 tile in the upwind direction of a velocity: row i (20
+// velocities with xi_x != 0) or column i (20 with xi_y != 0), q counting the
+// velocities.  p0[0], p0[halo], p0[2 halo] are the three nodes behind it, p1[j
+// step] its nodes, p2[0] and p2[halo] the two ahead.
+template <typename real>
+struct Line {
+    const real *p0, *p1, *p2;
+    int halo, step;
+    bool up;
+};
+__device__ __forceinline__ int line_velocity(bool along_x, int q)
+{
+    return along_x ? (q < 2 * NQ ? q : q + NQ) : (q >> 2) * NQ + ((q & 3) < 2 ? (q & 3) : (q & 3) + 1);
+}
+template <typename real>
+__device__ __forceinline__ Line<real> line_of(const Staged<real> &sm, bool along_x, int q, int i)
+{
+    constexpr int TX = Staged<real>::TX, TY = Staged<real>::TY, HP = Staged<real>::HP;
+    const int k = line_velocity(along_x, q);
+    Line<real> l;
+    l.up = along_x ? k / NQ > 2 : k % NQ > 2;
+    l.step = l.halo = l.up ? 1 : -1;
+    if (along_x) {
+        const real *row = &sm.mid[k][i][0];
+        l.p0 = row + (l.up ? 1 : TX + 6);
+        l.p1 = row + (l.up ? 4 : TX + 3);
+        l.p2 = row + (l.up ? TX + 4 : 3);
+    } else {
+        l.halo *= TX;
+        l.step *= HP;
+        l.p0 = l.up ? &sm.below[k][0][i] : &sm.above[k][2][i];
+        l.p1 = &sm.mid[k][l.up ? 0 : TY - 1][4 + i];
+        l.p2 = l.up ? &sm.above[k][0][i] : &sm.below[k][2][i];
+    }
+    return l;
 }
 
 // ---------------------------------------------------------------- element by element
@@ -141,7 +210,7 @@ __device__ __forceinline__ void load_region(S &sm, const real *__restrict__ fs, 
 #pragma unroll 5
             for (int k = 0; k < NK; ++k) {
                 dst[k * dp] = real(0);
-                if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = 0.0f;
+                if constexpr (sizeof(real) == 4) dst[(NK + k) * dp] = 0.0f;
             }
             continue;
         }
@@ -150,7 +219,7 @@ __device__ __forceinline__ void load_region(S &sm, const real *__restrict__ fs, 
 #pragma unroll 5
             for (int k = 0; k < NK; ++k) {
                 dst[k * dp] = __ldg(src + k * g.plane);
-                if constexpr (sizeof(real) == 4) sm.pl.lo[k][r][c] = __ldg(src + (NK + k) * g.plane);
+                if constexpr (sizeof(real) == 4) dst[(NK + k) * dp] = __ldg(src + (NK + k) * g.plane);
             }
         } else {
 #pragma unroll
@@ -159,7 +228,7 @@ __device__ __forceinline__ void load_region(S &sm, const real *__restrict__ fs, 
                 for (int k2 = 0; k2 < NQ; ++k2) {
                     const int kk = NQ * (flip_x ? NQ - 1 - k1 : k1) + (flip_y ? NQ - 1 - k2 : k2);
                     dst[(NQ * k1 + k2) * dp] = __ldg(src + kk * g.plane);
-                    if constexpr (sizeof(real) == 4) sm.pl.lo[NQ * k1 + k2][r][c] = __ldg(src + (NK + kk) * g.plane);
+                    if constexpr (sizeof(real) == 4) dst[(NK + NQ * k1 + k2) * dp] = __ldg(src + (NK + kk) * g.plane);
                 }
         }
     }
@@ -209,19 +278,19 @@ __device__ __forceinline__ void wall_flux(S &sm, const Geo &g, const Tab<real> &
             // the stencil (a2, a1, a0, g0, g1) by its first differences
             // (D2, D1, 2 D1 - D2, 3 D1 - 2 D2)
             const int row = tr + 3;
-            const float h0 = sm.pop[k][row][c0], l0 = sm.pl.lo[k][row][c0];
-            const float h1 = sm.pop[k][row][c0 + dc], l1 = sm.pl.lo[k][row][c0 + dc];
-            const float h2 = sm.pop[k][row][c0 + 2 * dc], l2 = sm.pl.lo[k][row][c0 + 2 * dc];
+            const float h0 = *sm.at(k, row, c0), l0 = *sm.at(NK + k, row, c0);
+            const float h1 = *sm.at(k, row, c0 + dc), l1 = *sm.at(NK + k, row, c0 + dc);
+            const float h2 = *sm.at(k, row, c0 + 2 * dc), l2 = *sm.at(NK + k, row, c0 + 2 * dc);
             const float D1 = pdiff(h0, l0, h1, l1), D2 = pdiff(h1, l1, h2, l2);
             const float e0 = fmaf(2.0f, D1, -D2), e1 = fmaf(5.0f, D1, -3.0f * D2);
             const f2 G0 = f2_add_f(f2{h0, l0}, e0), G1 = f2_add_f(f2{h0, l0}, e1);
             if (c0 - dc >= 0 && c0 - dc < HX) {
-                sm.pop[k][row][c0 - dc] = G0.hi;
-                sm.pl.lo[k][row][c0 - dc] = G0.lo;
+                *sm.at(k, row, c0 - dc) = G0.hi;
+                *sm.at(NK + k, row, c0 - dc) = G0.lo;
             }
             if (c0 - 2 * dc >= 0 && c0 - 2 * dc < HX) {
-                sm.pop[k][row][c0 - 2 * dc] = G1.hi;
-                sm.pl.lo[k][row][c0 - 2 * dc] = G1.lo;
+                *sm.at(k, row, c0 - 2 * dc) = G1.hi;
+                *sm.at(NK + k, row, c0 - 2 * dc) = G1.lo;
             }
             const float corr = face_corr<LEARNED>(mlp, D2, D1, e0, fmaf(3.0f, D1, -2.0f * D2));
             wf = t.R[k1] * (h0 + (l0 + corr));
@@ -250,7 +319,7 @@ __device__ __forceinline__ void wall_ghosts(S &sm, const Geo &g, const Tab<real>
         if (c < 0 || c >= HX) continue;
         const int k = NQ * (side ? v / 5 : 3 + v / 5) + v % 5;
         *sm.at(k, tr + 3, c) = sm.wnw[side][tr] * tw.geqw[side][k];
-        if constexpr (sizeof(real) == 4) sm.pl.lo[k][tr + 3][c] = 0.0f;
+        if constexpr (sizeof(real) == 4) *sm.at(NK + k, tr + 3, c) = 0.0f;
     }
 }
 

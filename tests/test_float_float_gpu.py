@@ -88,3 +88,15 @@ def test_infinities_and_nan_reach_their_neighbours(olb, bad):
     assert not np.isfinite(g[:, 12, 12]).any()
     assert not np.isfinite(g[24, 12, 10:15]).any() and not np.isfinite(g[24, 10:15, 12]).any()
     assert np.isfinite(g[:, 0, 0]).all()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_learned_weights_take_their_three_shapes_only(olb, precision):
+    ctx = olb.create(_params(24, 24), precision=precision, weno_mode=olb.WENO_LEARNED)
+    for shape in ((8, 8, 4), (16, 8, 2), (32, 16, 1)):
+        ctx.set_tile(*shape)
+        assert ctx.get_tile() == shape
+    for shape in ((8, 8, 5), (8, 8, 8), (7, 8, 8), (16, 8, 1), (32, 8, 1), (16, 16, 1)):
+        with pytest.raises(olb.OlbError):
+            ctx.set_tile(*shape)
+        assert ctx.get_tile() == (32, 16, 1)
