@@ -36,8 +36,8 @@ struct StageSmem<double, KP, LEARNED> {
 };
 
 // Shared memory of the single-grid kernel: the tile staging, then (learned
-// weights only) the network's parameters at a 16-byte aligned offset and the
-// warps' scratch for the network's tensor-pipe layer.
+// weights only) the network's tables at a 16-byte aligned offset and, FP64, a
+// scratch of each warp (olb_mlp.cuh).
 template <typename real, int KP>
 constexpr size_t mlp_offset()
 {
@@ -46,10 +46,8 @@ constexpr size_t mlp_offset()
 template <typename real, int KP, bool LEARNED>
 constexpr size_t fused_smem_bytes()
 {
-    // learned: the parameters; FP32 also the split W2 and MLP_WARP_SCRATCH
-    // floats per warp
     using S = typename StageSmem<real, KP, LEARNED>::type;
-    constexpr size_t mlp_floats = sizeof(real) == 4 ? MLP_SCRATCH_OFF + S::NT / 32 * MLP_WARP_SCRATCH : MLP_P + 1;
+    constexpr size_t mlp_floats = sizeof(real) == 4 ? MLP_T32_SIZE : MLP_T64_SIZE + S::NT / 32 * MLP_WARP_SCRATCH;
     return LEARNED ? mlp_offset<real, KP>() + mlp_floats * sizeof(float) : sizeof(S);
 }
 template <typename real, int KP, bool LEARNED>
@@ -70,14 +68,13 @@ constexpr int fused_min_ctas(size_t smem_bytes, int threads, int cap = 0)
     return n < 1 ? 1 : (cap > 0 && n > cap ? cap : n);
 }
 
-// Single grid: one CTA per tile.  Learned-weight instances leave their network the registers
-// it needs: FP32 (tensor-pipe network) at most two CTAs per SM, FP64 (per-thread
-// network) one.
+// Single grid: one CTA per tile.  Learned-weight instances leave their network the
+// registers it needs: two CTAs per SM.
 template <typename real, int KP, bool LEARNED>
 __global__ void __launch_bounds__((stage_threads<real, KP, LEARNED>()),
                                   fused_min_ctas(fused_smem_bytes<real, KP, LEARNED>(),
                                                  stage_threads<real, KP, LEARNED>(),
-                                                 LEARNED ? (sizeof(real) == 4 ? 2 : 1) : 0))
+                                                 LEARNED ? 2 : 0))
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
         real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
@@ -86,22 +83,17 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
     // 128-byte aligned: the TMA copy of phase 1 lands at offset 0
     extern __shared__ __align__(128) unsigned char smem_raw[];
     auto &sm = *reinterpret_cast<typename StageSmem<real, KP, LEARNED>::type *>(smem_raw);
-    float *mlp_sm = nullptr;
+    MlpArg net = {nullptr, nullptr};
     if constexpr (LEARNED) {
-        mlp_sm = reinterpret_cast<float *>(smem_raw + mlp_offset<real, KP>());
-        for (int p = threadIdx.x; p < MLP_P; p += blockDim.x) mlp_sm[p] = __ldg(mlp + p);
-        if constexpr (sizeof(real) == 4) {
-            __syncthreads();
-            mlp_split_w2(mlp_sm);
-        }
-        // made visible by the first barrier inside stage_tile
+        net = {mlp, reinterpret_cast<float *>(smem_raw + mlp_offset<real, KP>())};
+        mlp_tables<real>(net.tables, mlp);  // made visible by the first barrier inside stage_tile
     }
     const TmaMap *tm = tma.on ? &tma.map : nullptr;
     const int x0 = blockIdx.x * 8, y0 = blockIdx.y * 8;
     if constexpr (sizeof(real) == 8)
-        stage_tile64<KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, sk, mlp_sm, tm, fields);
+        stage_tile64<KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, sk, net, tm, fields);
     else
-        stage_tile32<LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, mlp_sm, tm, fields);
+        stage_tile32<LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, net, tm, fields);
 }
 
 // Batch of independent runs (uneven grid sizes, own parameters): one CTA per
@@ -144,10 +136,10 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
             asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm->bytes[k]) : "memory");
     if constexpr (sizeof(real) == 8)
         stage_tile64<KP, false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
-                                run.k[st], nullptr, tm, fl);
+                                run.k[st], MlpArg{}, tm, fl);
     else
         stage_tile32<false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0, ca, cb,
-                            ccoef * (real)run.g.dt, ca_lo, cb_lo, nullptr, tm, fl);
+                            ccoef * (real)run.g.dt, ca_lo, cb_lo, MlpArg{}, tm, fl);
 }
 
 template <typename real, int KP, bool LEARNED = false>

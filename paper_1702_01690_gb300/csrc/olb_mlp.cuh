@@ -33,8 +33,7 @@ __device__ __forceinline__ float tanh_fast(float x)
     return copysignf(fmaf(-2.0f, r, 1.0f), x);
 }
 
-// Weights of one stencil; th points to the parameters (shared memory in the
-// stage kernel).  x: normalised stencil.
+// Weights of one stencil; th points to the parameters, 16-byte aligned.  x: normalised stencil.
 __device__ __forceinline__ void mlp_weights(const float *__restrict__ th, const float x[MLP_IN], float w[MLP_OUT])
 {
     float h1[MLP_H];
@@ -174,7 +173,7 @@ __device__ __forceinline__ float learned_corr_net(const float *__restrict__ th, 
 // stencil is smooth (min sigma_q >= MLP_GUARD max sigma_q); otherwise
 // sum_q w_q G_q with the network's weights.  FP64 populations: the guard is
 // taken in FP64; the network and sum_q w_q G_q run in FP32 (the weights carry
-// FP32 error anyway).
+// FP32 error anyway).  This and weno5_learned_corr: one thread's face, for walls.
 __device__ __forceinline__ double weno5_learned_corr64(const float *__restrict__ th, double d01, double d12, double d23,
                                                        double d34)
 {
@@ -198,19 +197,47 @@ __device__ __forceinline__ float weno5_learned_corr(const float *__restrict__ th
     return learned_corr_net(th, e);
 }
 
-// ---------------------------------------------------------------- the network on the tensor pipe
-// Inside the stage kernel the 32 lanes of a warp evaluate the network for 32
-// stencils at once: layer 1 per lane, the 32 x 32 layer as a matrix product
-// on the tensor pipe (mma.sync m16n8k8 with TF32 operands; each operand
-// split into a TF32 high part and a TF32 remainder and the product taken as
-// hi hi + hi lo + lo hi, accurate to ~2^-21 like an FP32 dot product), layer 3
-// and the softmax per stencil.
+// ---------------------------------------------------------------- the network of a warp
+// Inside the stage kernels the 32 lanes of a warp evaluate the network for 32
+// stencils at once.  Lane 4 g + t works on the stencils g, g + 8, g + 16, g + 24
+// (the rows of an mma fragment): a weight that it loads from shared memory serves
+// four stencils instead of one, and two of them share a packed instruction.
+// Every sum takes its terms in a fixed order.
+//   FP32 populations: the 32 x 32 layer is a matrix product on the tensor pipe
+// (mma.sync m16n8k8 with TF32 operands; each operand split into a TF32 high part
+// and a TF32 remainder and the product taken as hi hi + hi lo + lo hi, accurate to
+// ~2^-21 like an FP32 dot product).  A lane's layer-1 outputs are its own
+// fragment, so nothing goes through shared memory.
+//   FP64 populations: FP32 multiply-adds, the layers' outputs exchanged through
+// shared memory (mlp_weights' sums: the same results).
+// One stage of 1024^2 where the network acts on nearly every face: 5.07 -> 3.15 ms
+// (FP32 populations) and 5.67 -> 4.51 ms (FP64), from a lane per stencil, whose
+// weights came with 576 loads a face (FP64) and whose layer-1 outputs went through
+// shared memory to the fragments (FP32); FP64 faces where the network does not act
+// also left the FP64 pipe (weno5_line).  Bound by instruction issue and latency with
+// the 16 warps that 128 registers a thread leave an SM (ncu: issue 61 %, special
+// functions 22 %, tensor pipe 30 % with FP32; issue 49 %, FP32 pipe 25 %, wavefronts
+// of shared memory 90 % before their rows were rotated, with FP64).
 
-// scratch floats per warp: one 16 x 8 block of layer-1 outputs (row stride 9)
-constexpr int MLP_WARP_SCRATCH = 16 * 9;
-// shared memory after the parameters (1348 floats): W2 split into TF32 high
-// parts and remainders (2 x 1024 words), then the warps' scratch
-constexpr int MLP_W2HI_OFF = 1348, MLP_W2LO_OFF = 1348 + 1024, MLP_SCRATCH_OFF = 1348 + 2048;
+// What a stage kernel has of the network: its parameters in global memory (wall faces,
+// a network a thread), the tables and scratch in shared memory.
+struct MlpArg {
+    const float *theta;
+    float *tables;
+};
+
+// Tables in shared memory, in the order of the loads.  Layer 1, for units j = 8 ks +
+// 4 u + t at (2 ks + u, part, t): the weights and the bias, each twice (float4
+// parts (w0 w0 w1 w1) (w2 w2 w3 w3) (w4 w4 b b)).
+constexpr int MLP_T1 = 0, MLP_T1_SIZE = 384;
+// FP32: layer 3 and the biases of layer 2, for units j = 8 nt + 2 t + q at (2 nt + q,
+// part, t): (w0 w0 w1 w1) (w2 w2 b2 b2); W2 as B fragments (hi hi lo lo) of lane
+// (g, t) at (ks, nt, lane): B[k][n] = W2[n][k], k = 8 ks + t (+ 4), n = 8 nt + g; b3
+constexpr int MLP_T3 = 384, MLP_TB = 640, MLP_T32_B3 = 2688, MLP_T32_SIZE = 2692;
+// FP64: W2 transposed; layer 3's weights (w0 w1 w2 0) of each unit; b2; b3; then
+// MLP_WARP_SCRATCH floats a warp (the outputs of a layer, [unit][g][4 stencils])
+constexpr int MLP_TW = 384, MLP_T4 = 1408, MLP_T64_B2 = 1536, MLP_T64_B3 = 1568, MLP_T64_SIZE = 1572;
+constexpr int MLP_WARP_SCRATCH = 1024;
 
 __device__ __forceinline__ void tf32_split(float v, unsigned &hi, unsigned &lo)
 {
@@ -219,12 +246,48 @@ __device__ __forceinline__ void tf32_split(float v, unsigned &hi, unsigned &lo)
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(r));
 }
 
-// Fill the split copies of W2 after the parameters (all threads of the CTA).
-__device__ __forceinline__ void mlp_split_w2(float *th)
+// The same for |v| <= 1 or a NaN, which the low part then carries (two integer
+// instructions instead of three for the high part).
+__device__ __forceinline__ void tf32_split_unit(float v, unsigned &hi, unsigned &lo)
 {
-    unsigned *w2h = reinterpret_cast<unsigned *>(th + MLP_W2HI_OFF);
-    unsigned *w2l = reinterpret_cast<unsigned *>(th + MLP_W2LO_OFF);
-    for (int i = threadIdx.x; i < MLP_H * MLP_H; i += blockDim.x) tf32_split(th[MLP_W2 + i], w2h[i], w2l[i]);
+    hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
+    const float r = v - __uint_as_float(hi);
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(r));
+}
+
+// Fill the tables from the parameters theta (all threads of the CTA).
+template <typename real>
+__device__ __forceinline__ void mlp_tables(float *tb, const float *__restrict__ theta)
+{
+    for (int i = threadIdx.x; i < 6 * MLP_H; i += blockDim.x) {
+        const int j = i / 6, q = i - 6 * j;
+        const float v = __ldg(theta + (q < MLP_IN ? MLP_W1 + j * MLP_IN + q : MLP_B1 + j));
+        float *o = tb + MLP_T1 + ((j >> 2) * 3 + q / 2) * 16 + (j & 3) * 4 + 2 * (q & 1);
+        o[0] = o[1] = v;
+    }
+    for (int i = threadIdx.x; i < 4 * MLP_H; i += blockDim.x) {
+        const int j = i / 4, o = i - 4 * j;
+        const float v = __ldg(theta + (o < MLP_OUT ? MLP_W3 + o * MLP_H + j : MLP_B2 + j));
+        if constexpr (sizeof(real) == 4) {
+            float *p = tb + MLP_T3 + ((2 * (j >> 3) + (j & 1)) * 2 + o / 2) * 16 + (j >> 1 & 3) * 4 + 2 * (o & 1);
+            p[0] = p[1] = v;
+        } else {
+            tb[o < MLP_OUT ? MLP_T4 + i : MLP_T64_B2 + j] = v;
+        }
+    }
+    for (int i = threadIdx.x; i < MLP_H * MLP_H; i += blockDim.x) {
+        const int n = i / MLP_H, k = i - MLP_H * n;
+        const float v = __ldg(theta + MLP_W2 + i);
+        if constexpr (sizeof(real) == 4) {
+            unsigned *p = reinterpret_cast<unsigned *>(tb) + MLP_TB +
+                          (((k >> 3) * 4 + (n >> 3)) * 32 + 4 * (n & 7) + (k & 3)) * 4 + (k >> 2 & 1);
+            tf32_split(v, p[0], p[2]);
+        } else {
+            tb[MLP_TW + k * MLP_H + n] = v;
+        }
+    }
+    if (threadIdx.x < MLP_OUT)
+        tb[(sizeof(real) == 4 ? MLP_T32_B3 : MLP_T64_B3) + threadIdx.x] = __ldg(theta + MLP_B3 + threadIdx.x);
 }
 
 // c += a b for one m16n8k8 tile (row-major A, column-major B, FP32 accumulators).
@@ -236,18 +299,70 @@ __device__ __forceinline__ void mma_tf32(float c[4], const unsigned a[4], const 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// Weights w of this lane's stencil x; every lane of the warp must call it,
-// from one call site (mma.sync.aligned needs the whole warp at the same
-// instruction; lanes whose stencil the network does not act on pass any x and
-// ignore w).
-// th: parameters in shared memory; sc: this warp's MLP_WARP_SCRATCH floats.
-__device__ __forceinline__ void mlp_weights_warp(const float *__restrict__ th, const float x[MLP_IN],
-                                                 float w[MLP_OUT], float *sc)
+// tanh_fast of two values.
+__device__ __forceinline__ vf2 tanh_fast(vf2 x)
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    // layer 2 accumulators: rows = stencils (lanes), 16 per m-tile mt;
-    // columns = outputs, 8 per n-tile nt; k = the 32 layer-1 outputs, 8 per
-    // step ks, each step's layer-1 outputs computed just before it
+    const float x0 = x[0], x1 = x[1];
+    float e0, e1, r0, r1;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fabsf(x0) * 2.8853900817779268f));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fabsf(x1) * 2.8853900817779268f));
+    const vf2 d = vf2::pair(e0, e1) + vf2::all(1.0f);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d[0]));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d[1]));
+    const vf2 y = vfma(vf2::all(-2.0f), vf2::pair(r0, r1), vf2::all(1.0f));
+    return vf2::pair(copysignf(y[0], x0), copysignf(y[1], x1));
+}
+__device__ __forceinline__ vf2 vf2_lo(float4 v) { return vf2::pair(v.x, v.y); }
+__device__ __forceinline__ vf2 vf2_hi(float4 v) { return vf2::pair(v.z, v.w); }
+
+// The inputs of the four stencils of this lane, as two pairs, from those of each
+// lane's own stencil.
+__device__ __forceinline__ void mlp_inputs(const float x[MLP_IN], vf2 X[2][MLP_IN])
+{
+    const int g = (threadIdx.x & 31) >> 2;
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int i = 0; i < MLP_IN; ++i)
+            X[p][i] = vf2::pair(__shfl_sync(0xffffffffu, x[i], g + 16 * p), __shfl_sync(0xffffffffu, x[i], g + 16 * p + 8));
+}
+// Layer 1: outputs of unit j = 4 ju + t for the four stencils of this lane.
+__device__ __forceinline__ void mlp_unit1(const float *tb, int ju, const vf2 X[2][MLP_IN], vf2 h[2])
+{
+    const float4 *r = reinterpret_cast<const float4 *>(tb + MLP_T1) + ju * 12 + (threadIdx.x & 3);
+    const float4 r0 = r[0], r1 = r[4], r2 = r[8];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        vf2 a = vfma(vf2_lo(r0), X[p][0], vf2_hi(r2));
+        a = vfma(vf2_hi(r0), X[p][1], a);
+        a = vfma(vf2_lo(r1), X[p][2], a);
+        a = vfma(vf2_hi(r1), X[p][3], a);
+        a = vfma(vf2_lo(r2), X[p][4], a);
+        h[p] = tanh_fast(a);
+    }
+}
+__device__ __forceinline__ void mlp_softmax(const float z[MLP_OUT], float w[MLP_OUT])
+{
+    const float zm = fmaxf(z[0], fmaxf(z[1], z[2]));
+    const float e0 = expf(z[0] - zm), e1 = expf(z[1] - zm), e2 = expf(z[2] - zm);
+    const float inv = 1.0f / (e0 + e1 + e2);
+    w[0] = e0 * inv;
+    w[1] = e1 * inv;
+    w[2] = e2 * inv;
+}
+
+// Weights w of this lane's stencil x (FP32 populations); every lane of the warp must
+// call it, from one call site (mma.sync.aligned needs the whole warp at the same
+// instruction; lanes whose stencil the network does not act on pass any x and
+// ignore w).  tb: the tables (mlp_tables<float>).
+__device__ __forceinline__ void mlp_weights_warp32(const float *tb, const float x[MLP_IN], float w[MLP_OUT])
+{
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    vf2 X[2][MLP_IN];
+    mlp_inputs(x, X);
+    // layer 2 accumulators: rows = stencils, 16 per m-tile mt; columns = outputs, 8
+    // per n-tile nt; k = the 32 layer-1 outputs, 8 per step ks, each step's layer-1
+    // outputs (this lane's part of the A fragments) computed just before it
     float acc[2][4][4];
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -257,85 +372,138 @@ __device__ __forceinline__ void mlp_weights_warp(const float *__restrict__ th, c
             for (int q = 0; q < 4; ++q) acc[mt][nt][q] = 0.0f;
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-        float hc[8];
+        unsigned ah[2][4], al[2][4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int j = 8 * ks + q;
-            float a = th[MLP_B1 + j];
+        for (int u = 0; u < 2; ++u) {
+            vf2 h[2];
+            mlp_unit1(tb, 2 * ks + u, X, h);
 #pragma unroll
-            for (int i = 0; i < MLP_IN; ++i) a = fmaf(th[MLP_W1 + j * MLP_IN + i], x[i], a);
-            hc[q] = tanh_fast(a);
+            for (int mt = 0; mt < 2; ++mt) {
+                tf32_split_unit(h[mt][0], ah[mt][2 * u], al[mt][2 * u]);
+                tf32_split_unit(h[mt][1], ah[mt][2 * u + 1], al[mt][2 * u + 1]);
+            }
         }
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            // the m-tile's 16 lanes put their 8 layer-1 outputs in the scratch
-            __syncwarp();
-            if ((lane >> 4) == mt)
+        for (int nt = 0; nt < 4; ++nt) {
+            const uint4 b = reinterpret_cast<const uint4 *>(tb + MLP_TB)[(4 * ks + nt) * 32 + lane];
+            const unsigned bh[2] = {b.x, b.y}, bl[2] = {b.z, b.w};
 #pragma unroll
-                for (int q = 0; q < 8; ++q) sc[(lane & 15) * 9 + q] = hc[q];
-            __syncwarp();
-            unsigned ah[4], al[4];
-            tf32_split(sc[g * 9 + t], ah[0], al[0]);
-            tf32_split(sc[(g + 8) * 9 + t], ah[1], al[1]);
-            tf32_split(sc[g * 9 + t + 4], ah[2], al[2]);
-            tf32_split(sc[(g + 8) * 9 + t + 4], ah[3], al[3]);
+            for (int mt = 0; mt < 2; ++mt) mma_tf32(acc[mt][nt], al[mt], bh);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                // B[k][n] = W2[n][k]: k = 8 ks + t (+4), n = 8 nt + g
-                const unsigned *w2h = reinterpret_cast<const unsigned *>(th + MLP_W2HI_OFF);
-                const unsigned *w2l = reinterpret_cast<const unsigned *>(th + MLP_W2LO_OFF);
-                const int i0 = (8 * nt + g) * MLP_H + 8 * ks + t;
-                const unsigned bh[2] = {w2h[i0], w2h[i0 + 4]}, bl[2] = {w2l[i0], w2l[i0 + 4]};
-                mma_tf32(acc[mt][nt], al, bh);
-                mma_tf32(acc[mt][nt], ah, bl);
-                mma_tf32(acc[mt][nt], ah, bh);
-            }
+            for (int mt = 0; mt < 2; ++mt) mma_tf32(acc[mt][nt], ah[mt], bl);
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) mma_tf32(acc[mt][nt], ah[mt], bh);
         }
     }
     // h2 = tanh(acc + b2) and layer 3: accumulator q of (mt, nt) holds stencil
-    // 16 mt + g + 8 (q >> 1) = g + 8 m, output 8 nt + 2 t + (q & 1)
-    float z[4][MLP_OUT];
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-#pragma unroll
-        for (int o = 0; o < MLP_OUT; ++o) z[m][o] = 0.0f;
+    // g + 8 m, m = 2 mt + (q >> 1), output 8 nt + 2 t + (q & 1)
+    vf2 z[2][MLP_OUT];
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+        for (int o = 0; o < MLP_OUT; ++o) z[mt][o] = vf2::all(0.0f);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int j = 8 * nt + 2 * t + (q & 1), m = 2 * mt + (q >> 1);
-                const float h2 = tanh_fast(acc[mt][nt][q] + th[MLP_B2 + j]);
+    for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-                for (int o = 0; o < MLP_OUT; ++o) z[m][o] = fmaf(th[MLP_W3 + o * MLP_H + j], h2, z[m][o]);
+        for (int q = 0; q < 2; ++q) {
+            const float4 *r = reinterpret_cast<const float4 *>(tb + MLP_T3) + (2 * nt + q) * 8 + t;
+            const float4 r0 = r[0], r1 = r[4];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const vf2 h2 = tanh_fast(vf2::pair(acc[mt][nt][q], acc[mt][nt][q + 2]) + vf2_hi(r1));
+                z[mt][0] = vfma(vf2_lo(r0), h2, z[mt][0]);
+                z[mt][1] = vfma(vf2_hi(r0), h2, z[mt][1]);
+                z[mt][2] = vfma(vf2_lo(r1), h2, z[mt][2]);
             }
-    // sum over the four lanes of a row group (t = 0..3): every one gets the total
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-#pragma unroll
-        for (int o = 0; o < MLP_OUT; ++o) {
-            z[m][o] += __shfl_xor_sync(0xffffffffu, z[m][o], 1);
-            z[m][o] += __shfl_xor_sync(0xffffffffu, z[m][o], 2);
         }
-    // lane (g, t) finishes stencil g + 8 t
+    // sum over the four lanes of a row group (t = 0..3), of which lane t keeps m = t:
+    // (z_t + z_{t^1}) + (z_{t^2} + z_{t^3})
     float zz[MLP_OUT];
 #pragma unroll
     for (int o = 0; o < MLP_OUT; ++o) {
-        float v = z[0][o];
-        v = t == 1 ? z[1][o] : v;
-        v = t == 2 ? z[2][o] : v;
-        v = t == 3 ? z[3][o] : v;
-        zz[o] = v + th[MLP_B3 + o];
+        float s[2];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            const float keep = t & 1 ? z[mt][o][1] : z[mt][o][0], send = t & 1 ? z[mt][o][0] : z[mt][o][1];
+            s[mt] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+        }
+        const float keep = t & 2 ? s[1] : s[0], send = t & 2 ? s[0] : s[1];
+        zz[o] = (keep + __shfl_xor_sync(0xffffffffu, send, 2)) + tb[MLP_T32_B3 + o];
     }
-    const float zm = fmaxf(zz[0], fmaxf(zz[1], zz[2]));
-    const float e0 = expf(zz[0] - zm), e1 = expf(zz[1] - zm), e2 = expf(zz[2] - zm);
-    const float inv = 1.0f / (e0 + e1 + e2);
+    float e[MLP_OUT];
+    mlp_softmax(zz, e);
     // stencil F sits in lane F; lane 4 (F mod 8) + F / 8 finished it
     const int src = 4 * (lane & 7) + (lane >> 3);
-    w[0] = __shfl_sync(0xffffffffu, e0 * inv, src);
-    w[1] = __shfl_sync(0xffffffffu, e1 * inv, src);
-    w[2] = __shfl_sync(0xffffffffu, e2 * inv, src);
+#pragma unroll
+    for (int o = 0; o < MLP_OUT; ++o) w[o] = __shfl_sync(0xffffffffu, e[o], src);
+}
+
+// The same for FP64 populations, with the results of mlp_weights (every lane of the
+// warp must call it).  tb: the tables (mlp_tables<double>); sc: this warp's scratch.
+__device__ __forceinline__ void mlp_weights_warp64(const float *tb, const float x[MLP_IN], float w[MLP_OUT], float *sc)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    // (the g of a unit's row rotated by twice the t of the lane that writes it: the
+    // eight lanes of a quarter of a 16-byte access fall on all banks)
+    float4 *const s4 = reinterpret_cast<float4 *>(sc);
+    auto at = [](int unit, int g, int t) { return 8 * unit + ((g + 2 * t) & 7); };
+    vf2 X[2][MLP_IN];
+    mlp_inputs(x, X);
+#pragma unroll 2
+    for (int ju = 0; ju < MLP_H / 4; ++ju) {
+        vf2 h[2];
+        mlp_unit1(tb, ju, X, h);
+        s4[at(4 * ju + t, g, t)] = make_float4(h[0][0], h[0][1], h[1][0], h[1][1]);
+    }
+    __syncwarp();
+    // layer 2: the units 8 t .. 8 t + 7 of this lane's four stencils, units in pairs
+    vf2 a[4][4];
+    const float4 b0 = reinterpret_cast<const float4 *>(tb + MLP_T64_B2)[2 * t],
+                 b1 = reinterpret_cast<const float4 *>(tb + MLP_T64_B2)[2 * t + 1];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        a[m][0] = vf2_lo(b0);
+        a[m][1] = vf2_hi(b0);
+        a[m][2] = vf2_lo(b1);
+        a[m][3] = vf2_hi(b1);
+    }
+#pragma unroll 8
+    for (int k = 0; k < MLP_H; ++k) {
+        const float4 *r = reinterpret_cast<const float4 *>(tb + MLP_TW + k * MLP_H) + 2 * t;
+        const float4 r0 = r[0], r1 = r[1], h = s4[at(k, g, k & 3)];
+        const float hm[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const vf2 hh = vf2::all(hm[m]);
+            a[m][0] = vfma(vf2_lo(r0), hh, a[m][0]);
+            a[m][1] = vfma(vf2_hi(r0), hh, a[m][1]);
+            a[m][2] = vfma(vf2_lo(r1), hh, a[m][2]);
+            a[m][3] = vfma(vf2_hi(r1), hh, a[m][3]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int jp = 0; jp < 4; ++jp) {
+        vf2 h[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) h[m] = tanh_fast(a[m][jp]);
+        s4[at(8 * t + 2 * jp, g, t)] = make_float4(h[0][0], h[1][0], h[2][0], h[3][0]);
+        s4[at(8 * t + 2 * jp + 1, g, t)] = make_float4(h[0][1], h[1][1], h[2][1], h[3][1]);
+    }
+    __syncwarp();
+    // layer 3 and the softmax: a lane its own stencil
+    vf2 z01 = vf2::pair(tb[MLP_T64_B3], tb[MLP_T64_B3 + 1]);
+    float z2 = tb[MLP_T64_B3 + 2];
+#pragma unroll
+    for (int j = 0; j < MLP_H; ++j) {
+        const float4 r = reinterpret_cast<const float4 *>(tb + MLP_T4)[j];
+        const float h2 = sc[4 * at(j, lane & 7, j >> 3) + (lane >> 3)];
+        z01 = vfma(vf2_lo(r), vf2::all(h2), z01);
+        z2 = fmaf(r.z, h2, z2);
+    }
+    const float z[MLP_OUT] = {z01[0], z01[1], z2};
+    mlp_softmax(z, w);
+    __syncwarp();  // before the next call writes the scratch
 }
 
 }  // namespace olb

@@ -90,15 +90,14 @@ __device__ __forceinline__ void weno5_line32(const Line<float> &ln, int lo_p1, i
 // One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
 // call it.  ca, cb, cc: the stage's coefficients of f^n, f_s and dt L (Eq. rk3);
 // ca_lo, cb_lo: their remainders (1/3 and 2/3 as double-float constants); tw: the
-// table of the wall entries; mlp: the learned network's parameters in shared memory
-// (LEARNED only); tmap: TMA maps of fs, or nullptr; fields: the moments and c F of
+// table of the wall entries; net: the learned network (LEARNED only); tmap: TMA maps of fs, or nullptr; fields: the moments and c F of
 // fs (k_fields, k_force).  Returns false when the TMA copy timed out (the CTA must
 // stop).
 template <bool LEARNED>
 __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *__restrict__ fs, const float *fn, float *out,
                                              int *__restrict__ status, const Geo &g, const Tab<float> &t,
                                              const Tab<float> &tw, int x0, int y0, float ca, float cb, float cc, float ca_lo,
-                                             float cb_lo, const float *mlp, const TmaMap *tmap,
+                                             float cb_lo, const MlpArg &net, const TmaMap *tmap,
                                              const StageFields<float> &fields)
 {
     using S = Smem32<LEARNED>;
@@ -159,7 +158,7 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
     // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
     const bool left = x0 == 0 && g.wall_lo, right = x0 + TX + 3 >= g.nx && g.wall_hi;
     if (left || right) {
-        wall_flux<float, LEARNED>(sm, g, t, tw, mlp, x0, 3 * NN, left, right);
+        wall_flux<float, LEARNED>(sm, g, t, tw, net.theta, x0, 3 * NN, left, right);
         __syncthreads();
         wall_ghosts<float>(sm, g, tw, x0, 0, left, right);
     }
@@ -174,7 +173,6 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
         // x faces of the 20 velocities with xi_x != 0, then the y faces of the 20
         // with xi_y != 0
         constexpr int nfx = (TX + 1) * TY, nfy = TX * (TY + 1), total = 20 * (nfx + nfy);
-        float *const sc = const_cast<float *>(mlp) + MLP_SCRATCH_OFF + (tid >> 5) * MLP_WARP_SCRATCH;
         for (int e = tid; e < (total + 31) / 32 * 32; e += NT) {
             const int ee = e < total ? e : 0;
             const bool along_x = ee < 20 * nfx;
@@ -200,7 +198,7 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
             float x[MLP_IN], w[MLP_OUT] = {0.0f, 0.0f, 0.0f};
             learned_input_x(d, acts, x);
             // the whole warp skips the network when none of its stencils needs it
-            if (__any_sync(0xffffffffu, acts)) mlp_weights_warp(mlp, x, w, sc);
+            if (__any_sync(0xffffffffu, acts)) mlp_weights_warp32(net.tables, x, w);
             if (valid) {
                 const float res = acts ? learned_corr_from(w, d) : weno5_corr(d[0], d[1], d[2], d[3]);
                 if (along_x) sm.ax[q][r][c] = res;

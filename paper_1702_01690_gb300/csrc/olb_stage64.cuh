@@ -63,7 +63,7 @@ struct __align__(16) ffp {
 // (4096) 233 and 247, 1024^2 868 and 931: grids of at most one tile an SM take 320.
 template <int KP>
 struct Plan64 {
-    using V = typename std::conditional<KP == 5, vf2, vf1>::type;
+    using V = typename std::conditional<KP == 8, vf1, vf2>::type;
     static constexpr int NT = KP == 5 ? 160 : KP == 8 ? 320 : 256;
 };
 
@@ -75,8 +75,8 @@ struct Smem64 : Staged<double> {
     ffp G[2][NN / 2];   // c F
     // flux differences times 6 (weno5_flux6) across the nodes of each row along x
     // and column along y, of the 20 velocities that move along the axis (slot_x,
-    // slot_y; learned weights: first the faces' non-linear parts, one more than
-    // nodes, which the flux differences then replace); then, in place of one of a
+    // slot_y; learned weights: first the network's corrections of the faces, one more
+    // than nodes, which the flux differences then replace); then, in place of one of a
     // velocity's flux differences (inc), the sum of its advection and force
     // terms.  Entry i of a column sits in half i / 4 of element i mod 4 (face 8:
     // in element 4); the fifth element and the one at the end keep the banks of
@@ -150,14 +150,14 @@ __device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, dou
 // ---------------------------------------------------------------- the stage of one tile
 // One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
 // call it.  fields: the moments and c F of fs (k_fields, k_force); tw: the table
-// of the wall entries; tmap: TMA maps of fs, or nullptr; mlp: the learned
-// network's parameters in shared memory (LEARNED only).  A thread takes V::W nodes
+// of the wall entries; tmap: TMA maps of fs, or nullptr; net: the learned
+// network (LEARNED only).  A thread takes V::W nodes
 // (y and y + 4 of a column) or lines (rows or columns 4 apart) at a time.
 // Returns false when the TMA copy timed out (the CTA must stop).
 template <int KP, bool LEARNED>
 __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const double *__restrict__ fs, const double *fn,
                                              double *out, int *__restrict__ status, const Geo &g, const Tab<double> &t,
-                                             const Tab<double> &tw, int x0, int y0, const StageK &c, const float *mlp,
+                                             const Tab<double> &tw, int x0, int y0, const StageK &c, const MlpArg &net,
                                              const TmaMap *tmap, const StageFields<double> &fields)
 {
     using S = Smem64<KP, LEARNED>;
@@ -200,7 +200,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
     // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
     const bool left = x0 == 0 && g.wall_lo, right = x0 + TX + 3 >= g.nx && g.wall_hi;
     if (left || right) {
-        wall_flux<double, LEARNED>(sm, g, t, tw, mlp, x0, 2 * NN, left, right);
+        wall_flux<double, LEARNED>(sm, g, t, tw, net.theta, x0, 2 * NN, left, right);
         __syncthreads();
         wall_ghosts<double>(sm, g, tw, x0, 0, left, right);
     }
@@ -210,29 +210,36 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
 
     // ---- 5a. flux differences, W rows or columns a thread
     if constexpr (LEARNED) {
-        // the faces of the 20 velocities with xi_x != 0, then of the 20 with xi_y != 0
-        constexpr int nfx = (TX + 1) * TY, nfy = TX * (TY + 1);
-        for (int e = tid; e < 20 * (nfx + nfy); e += NT) {
-            const bool along_x = e < 20 * nfx;
-            const int e2 = along_x ? e : e - 20 * nfx, nf = along_x ? nfx : nfy, q = e2 / nf, f = e2 - q * nf;
+        // the network's corrections of the faces it acts on, on whole warps: the x faces
+        // of the 20 velocities with xi_x != 0, then the y faces of the 20 with xi_y != 0
+        constexpr int nfx = (TX + 1) * TY, nfy = TX * (TY + 1), total = 20 * (nfx + nfy);
+        float *const scratch = net.tables + MLP_T64_SIZE + (tid >> 5) * MLP_WARP_SCRATCH;
+        for (int e = tid; e < (total + 31) / 32 * 32; e += NT) {
+            const int ee = e < total ? e : 0;
+            const bool along_x = ee < 20 * nfx;
+            const int e2 = along_x ? ee : ee - 20 * nfx, nf = along_x ? nfx : nfy, q = e2 / nf, f = e2 - q * nf;
             const int k = line_velocity(along_x, q);
             const int r = along_x ? f / (TX + 1) : f / TX, cc = along_x ? f - r * (TX + 1) : f - r * TX;
-            if (along_x ? (y0 + r >= g.ny || x0 + cc > g.nx) : (x0 + cc >= g.nx || y0 + r > g.ny)) continue;
+            const bool valid = e < total && (along_x ? (y0 + r < g.ny && x0 + cc <= g.nx) : (x0 + cc < g.nx && y0 + r <= g.ny));
             const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-            double v[5];
+            double d[4] = {0.0, 0.0, 0.0, 0.0};
+            if (valid) {
+                double v[5];
 #pragma unroll
-            for (int m = 0; m < 5; ++m)
-                v[m] = along_x ? sm.mid[k][r][up ? cc + 1 + m : cc + 6 - m] : *sm.at(k, up ? r + m : r + 5 - m, 4 + cc);
-            const double d1 = v[2] - v[1], d2 = v[3] - v[2];
-            const ff corr = ff_split(weno5_learned_corr64(mlp, v[1] - v[0], d1, d2, v[4] - v[3]), sc);
-            // z = d1 + 2 d2 - 6 (F - v2)
-            const ff f1 = ff_split(d1, sc), f2 = ff_split(d2, sc);
-            const float c6 = 6.0f * corr.h;
-            ffv<vf1> z = {{2.0f * f2.h}, {fmaf(2.0f, f2.l, f1.l) - fmaf(6.0f, corr.l, fmaf(6.0f, corr.h, -c6))}};
-            ff_acc(z, vf1{f1.h});
-            ff_acc(z, vf1{-c6});
-            if (along_x) sm.ax[q][r & 3][cc].put(r >> 2, z);
-            else sm.col(q, cc, r).put(r == 8 ? 0 : r >> 2, z);
+                for (int m = 0; m < 5; ++m)
+                    v[m] = along_x ? sm.mid[k][r][up ? cc + 1 + m : cc + 6 - m] : *sm.at(k, up ? r + m : r + 5 - m, 4 + cc);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) d[m] = v[m + 1] - v[m];
+            }
+            const float d4[4] = {(float)d[0], (float)d[1], (float)d[2], (float)d[3]};
+            const bool acts = learned_guard<double>(d[0], d[1], d[2], d[3]);
+            float x[MLP_IN], w[MLP_OUT];
+            learned_input_x(d4, acts, x);
+            if (__any_sync(0xffffffffu, acts)) mlp_weights_warp64(net.tables, x, w, scratch);
+            if (!valid) continue;
+            const float c = acts ? ff_split((double)learned_corr_from(w, d4), sc).h : no_network();
+            if (along_x) sm.ax[q][r & 3][cc].h[r >> 2] = c;
+            else sm.col(q, cc, r).h[r == 8 ? 0 : r >> 2] = c;
         }
         __syncthreads();
     }
@@ -258,8 +265,11 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
         if constexpr (LEARNED)
             weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store, [&](int j) {
                 const int at = up ? j : TX - j;
-                return along_x ? sm.ax[q][i & 3][at].template get<V>(i >> 2)
-                               : sm.col(q, i, at).template get<V>(at == 8 ? 0 : at >> 2);
+                if (along_x) return sm.ax[q][i & 3][at].template get<V>(i >> 2).h;
+                float h[W];
+#pragma unroll
+                for (int w = 0; w < W; ++w) h[w] = sm.col(q, i + 4 * w, at).h[at == 8 ? 0 : at >> 2];
+                return V::of(h);
             });
         else
             weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);

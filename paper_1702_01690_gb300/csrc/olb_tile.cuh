@@ -9,7 +9,7 @@
 namespace olb {
 
 // Face value of one upwind-ordered FP64 stencil: Jiang-Shu weights, or the
-// learned network's (parameters in shared memory) when LEARNED.
+// learned network's (parameters mlp) when LEARNED.
 template <bool LEARNED>
 __device__ __forceinline__ double face_value(const float *mlp, double v0, double v1, double v2, double v3, double v4)
 {

@@ -100,3 +100,29 @@ def test_learned_weights_take_their_three_shapes_only(olb, precision):
         with pytest.raises(olb.OlbError):
             ctx.set_tile(*shape)
         assert ctx.get_tile() == (32, 16, 1)
+
+
+# a face's arithmetic is that of its stencil, whichever lane and warp takes it and whatever its neighbours are (a
+# density within [1, 2) gives every tile one scale): no tolerance
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(9, 8), (24, 16), (65, 9)])
+@pytest.mark.parametrize("kind", ["wave", "jump", "jump in noise"])
+def test_learned_step_does_not_depend_on_the_tiles(olb, nx, ny, kind, precision):
+    from paper_1702_01690_gb300 import learned
+    p = _params(nx, ny)
+    rng = np.random.default_rng(6)
+    i = np.arange(nx) + 0 * np.arange(ny)[:, None]
+    n = {"wave": 1.5 + 0.1 * np.sin(2 * np.pi * i / nx), "jump": np.where(i < nx // 2, 1.2, 1.7),
+         "jump in noise": np.where(i < nx // 2, 1.2, 1.7) + 1e-9 * rng.uniform(-1, 1, i.shape)}[kind].astype(float)
+    z = np.zeros_like(n)
+
+    def run(dx, dy):
+        ctx = olb.create(p, precision=precision, weno_mode=olb.WENO_LEARNED)
+        ctx.set_weno_mlp(learned.load_theta())
+        ctx.init_fields(np.roll(n, (dy, dx), (0, 1)), z + 0.01, z - 0.02, z + 0.9)
+        assert ctx.step(2) == 0
+        return np.roll(ctx.get_populations(), (-dy, -dx), (1, 2))
+
+    ref = run(0, 0)
+    for dx, dy in ((1, 0), (0, 3), (5, 6)):
+        assert np.array_equal(run(dx, dy), ref)
