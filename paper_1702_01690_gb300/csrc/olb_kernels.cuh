@@ -187,6 +187,28 @@ __device__ __forceinline__ void eq_factors(const Tab<real> &t, real u, real T, r
         g[k] = fma(t.wHe[k][4], c4, fma(t.wHe[k][3], c3, fma(t.wHe[k][2], c2, fma(t.wHe[k][1], c1, t.wHe[k][0]))));
 }
 
+// The same in FP64 by the parity of the Hermite orders: 26 instead of 34
+// FP64 operations.
+__device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, double T, double g[NQ])
+{
+    const double th = T - 1.0, u2 = u * u;
+    const double c2 = 0.5 * (u2 + th);
+    const double c3 = u * fma(u2, 1.0 / 6.0, 0.5 * th);
+    const double c4 = fma(u2, fma(u2, 1.0 / 24.0, 0.25 * th), 0.125 * th * th);
+#pragma unroll
+    for (int m = 0; m <= 2; ++m) {
+        const int k = 2 + m;
+        const double even = fma(t.wHe[k][4], c4, fma(t.wHe[k][2], c2, t.wHe[k][0]));
+        if (m == 0) {
+            g[2] = even;
+        } else {
+            const double odd = fma(t.wHe[k][3], c3, t.wHe[k][1] * u);
+            g[2 + m] = even + odd;
+            g[2 - m] = even - odd;
+        }
+    }
+}
+
 // The same factors split by Hermite order parity: ge_k from the even orders
 // l = 0, 2, 4 and go_k from the odd ones l = 1, 3 (g_k = ge_k + go_k).  The
 // tables give w_k He_l(p_k) exactly even or odd under p_k -> -p_k
@@ -525,6 +547,14 @@ __device__ __forceinline__ void node_sums(const real *__restrict__ f, long long 
 // Store the FP64 value v of population plane offset q: FP64 as is, FP32 as
 // the pair hi + lo.
 __device__ __forceinline__ void store_pop(double *f, long long, long long q, double v) { f[q] = v; }
+// (not inlined: the compiler would otherwise convert every value and select, 75
+// operations of a node on the FP64 pipe; initialisation of 4096^2 nodes 5.8 ms)
+static __device__ __noinline__ void store_pop_converted(float *f, long long plane, long long q, double v)
+{
+    const float hi = __double2float_rn(v);
+    f[q] = hi;
+    f[NK * plane + q] = __double2float_rn(v - (double)hi);
+}
 __device__ __forceinline__ void store_pop(float *f, long long plane, long long q, double v)
 {
     const int hw = __double2hiint(v), e = (hw >> 20) & 0x7ff;
@@ -541,8 +571,8 @@ __device__ __forceinline__ void store_pop(float *f, long long plane, long long q
         const int r = (int)(lw & 0x1fffffffu) - (((lr >> 29) & 7u) != (lw >> 29) ? 0x20000000 : 0);
         lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 896 - 52) << 23 | sign);
     } else {
-        hi = __double2float_rn(v);
-        lo = __double2float_rn(v - (double)hi);
+        store_pop_converted(f, plane, q, v);
+        return;
     }
     f[q] = hi;
     f[NK * plane + q] = lo;
@@ -554,7 +584,8 @@ __device__ __forceinline__ double load_pop(const float *f, long long plane, long
 }
 
 // ---------------------------------------------------------------- init / output
-// f = f^eq(n, u, T) (Eq. feq), evaluated in FP64 for both storages.
+// f = f^eq(n, u, T) (Eq. feq), evaluated in FP64 for both storages.  Bound by its 82
+// (FP64 populations) or 98 FP64 operations a node.
 template <typename real>
 __global__ void k_init(real *__restrict__ f, const double *__restrict__ n, const double *__restrict__ ux,
                        const double *__restrict__ uy, const double *__restrict__ T, Geo g, Tab<double> t)
@@ -564,8 +595,13 @@ __global__ void k_init(real *__restrict__ f, const double *__restrict__ n, const
     const int j = (int)(idx / g.nx), i = (int)(idx - (long long)j * g.nx);
     const long long o = (long long)j * g.pitch + i;
     double gx[NQ], gy[NQ];
-    eq_factors<double>(t, ux[idx], T[idx], gx);
-    eq_factors<double>(t, uy[idx], T[idx], gy);
+    if constexpr (sizeof(real) == 8) {
+        eq_factors64(t, ux[idx], T[idx], gx);
+        eq_factors64(t, uy[idx], T[idx], gy);
+    } else {
+        eq_factors<double>(t, ux[idx], T[idx], gx);
+        eq_factors<double>(t, uy[idx], T[idx], gy);
+    }
     const double nn = n[idx];
 #pragma unroll
     for (int k1 = 0; k1 < NQ; ++k1)

@@ -124,29 +124,6 @@ __device__ __forceinline__ void dp_line(const FfTab &t, const ffv<V> f[NQ], ffv<
     }
 }
 
-// ---------------------------------------------------------------- equilibrium
-// g_q(u, T) (eq_factors) by the parity of the Hermite orders: 26 instead of 34
-// FP64 operations.
-__device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, double T, double g[NQ])
-{
-    const double th = T - 1.0, u2 = u * u;
-    const double c2 = 0.5 * (u2 + th);
-    const double c3 = u * fma(u2, 1.0 / 6.0, 0.5 * th);
-    const double c4 = fma(u2, fma(u2, 1.0 / 24.0, 0.25 * th), 0.125 * th * th);
-#pragma unroll
-    for (int m = 0; m <= 2; ++m) {
-        const int k = 2 + m;
-        const double even = fma(t.wHe[k][4], c4, fma(t.wHe[k][2], c2, t.wHe[k][0]));
-        if (m == 0) {
-            g[2] = even;
-        } else {
-            const double odd = fma(t.wHe[k][3], c3, t.wHe[k][1] * u);
-            g[2 + m] = even + odd;
-            g[2 - m] = even - odd;
-        }
-    }
-}
-
 // ---------------------------------------------------------------- the stage of one tile
 // One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
 // call it.  fields: the moments and c F of fs (k_fields, k_force); tw: the table
