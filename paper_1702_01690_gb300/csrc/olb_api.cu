@@ -280,7 +280,7 @@ static cudaError_t enqueue_stage(olb_ctx *c, int st, cudaStream_t s)
     real *dst[3] = {f1, f2, f0};
     const StageCoef coef = stage_coef(c->p.dt, st);
     const int src_buf[3] = {0, 1, 2};
-    return launch_fused(src[st], f0, dst[st], c->status, c->geo, ctx_tab<real>(c), coef, c->tx, c->ty, c->kp,
+    return launch_fused(src[st], f0, dst[st], c->status, c->geo, ctx_tab<real>(c), coef,
                         c->p.weno_mode == OLB_WENO_LEARNED ? c->mlp : nullptr,
                         c->tma_ok ? &c->tma[src_buf[st]] : nullptr, c->fields, s);
 }
@@ -388,28 +388,25 @@ static cudaError_t prepare_tile(olb_ctx *c)
     // TMA maps of the three buffers for this shape (tiles whose region lies
     // inside the grid then load it with one copy); without them every tile
     // takes the per-element loads
-    const Shape s = stage_shape(is_fp64(c), learned, c->tx, c->ty, c->kp);
     c->tma_ok = true;
     for (int k = 0; k < 3 && c->tma_ok; ++k)
-        c->tma_ok = tma_encode(&c->tma[k], c->f[k], is_fp64(c), c->geo, s.tx, s.ty);
+        c->tma_ok = tma_encode(&c->tma[k], c->f[k], is_fp64(c), c->geo, STAGE_TX, STAGE_TY);
     return cudaSuccess;
 }
 
-// Default shape, the fastest measured on a GB300 for each precision: 8 x 8
-// nodes with 5 velocity lanes (FP32: the faces of all 25 velocities fit in shared
-// memory, so a stage has one face pass and one barrier; FP64: 160 threads, two
-// nodes each), FP64 grids of at most one tile an SM 8 lanes (320 threads, Plan64
-// in olb_stage64.cuh).  Learned weights: 4 lanes.  olb_set_tile overrides.
-static void default_tile(olb_ctx *c)
+int olb::stage_kind(bool learned, int tiles)
 {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
-    const bool learned = c->p.weno_mode == OLB_WENO_LEARNED;
-    const bool fp64 = is_fp64(c);
-    const long long tiles = (long long)((c->geo.nx + 7) / 8) * ((c->geo.ny + 7) / 8);
-    int k = learned ? 0 : 7;
-    if (fp64 && !learned && tiles <= sms) k = 5;
+    return learned ? (tiles <= sms ? 6 : 4) : tiles <= sms ? 8 : 5;
+}
+
+// Default shape: 8 x 8 nodes with 4 velocity lanes (FP64, learned weights) or 5.
+// olb_set_tile overrides.
+static void default_tile(olb_ctx *c)
+{
+    const int k = is_fp64(c) || c->p.weno_mode == OLB_WENO_LEARNED ? 0 : 7;
     c->tx = TILE_X[k];
     c->ty = TILE_Y[k];
     c->kp = TILE_K[k];

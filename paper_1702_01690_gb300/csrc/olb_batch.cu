@@ -90,11 +90,10 @@ static cudaError_t batch_upload(olb_batch *b)
     const size_t rb = b_fp64(b) ? batch_run_bytes((double *)nullptr) : batch_run_bytes((float *)nullptr);
     std::vector<char> host(rb * b->count);
     std::vector<int> start(b->count + 1);
-    const Shape sh = stage_shape(b_fp64(b), false, b->tx, b->ty, b->kp);
     int acc = 0;
     for (int r = 0; r < b->count; ++r) {
         const Geo &g = b->geo[r];
-        const int ntx = (g.nx + sh.tx - 1) / sh.tx, nty = (g.ny + sh.ty - 1) / sh.ty;
+        const int ntx = stage_tiles(g.nx, 1), nty = stage_tiles(1, g.ny);
         start[r] = acc;
         acc += ntx * nty;
         if (b_fp64(b))
@@ -111,7 +110,7 @@ static cudaError_t batch_upload(olb_batch *b)
     for (int k = 0; k < 3 && b->tma_ok; ++k)
         for (int r = 0; r < b->count && b->tma_ok; ++r)
             b->tma_ok = tma_encode(&maps[(size_t)k * b->count + r], (const char *)b->f[k] + b->off[r] * b->elt,
-                                   b_fp64(b), b->geo[r], sh.tx, sh.ty);
+                                   b_fp64(b), b->geo[r], STAGE_TX, STAGE_TY);
     cudaError_t e = cudaMemcpyAsync(b->runs, host.data(), host.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->tile_start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream);
@@ -143,7 +142,7 @@ static cudaError_t batch_stage(olb_batch *b, int st, cudaStream_t s)
     // src[st] is buffer st: its maps are row st of tmaps
     const TmaMap *maps = b->tma_ok ? b->tmaps + (size_t)st * b->count : nullptr;
     return launch_fused_batch(src[st], f0, dst[st], b->status, b->runs, b->tile_start, b->count, b->total_tiles,
-                              batch_tab(b, (real *)nullptr), coef[st], st, b->tx, b->ty, b->kp, b->fields, b->node_start,
+                              batch_tab(b, (real *)nullptr), coef[st], st, b->fields, b->node_start,
                               b->total_nodes, b->force_start, b->total_force, maps, s);
 }
 
@@ -525,8 +524,7 @@ extern "C" int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, in
             b->tx = TILE_X[q];
             b->ty = TILE_Y[q];
             b->kp = TILE_K[q];
-            const Shape sh = stage_shape(b_fp64(b), false, b->tx, b->ty, b->kp);
-            if (sh.tx != b->tx || sh.ty != b->ty || sh.kp != b->kp) continue;  // advanced as another shape of the list
+            if (b->tx != STAGE_TX || b->ty != STAGE_TY || b->kp != 5) continue;  // all are advanced alike
             if (batch_prepare(b) != cudaSuccess) {
                 cudaGetLastError();
                 continue;  // shape does not fit this precision

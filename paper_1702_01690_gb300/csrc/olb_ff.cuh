@@ -420,17 +420,12 @@ __host__ __device__ __forceinline__ double weno5_face(double v2, double d0, doub
 // nodes behind a line, p1[i step] its nodes, p2[0] and p2[halo] the two ahead.
 // store(i, v) takes the flux difference across node i (weno5_flux6).
 // Differences, their squares and products and the third differences are formed
-// once for the line.  Z: gives the correction F - v2 of face j (scaled floats) to be
-// used instead of the Jiang-Shu weights, no_network() where they are to be used.
-// The loop over the faces is unrolled by three: unrolled whole, a line is some 2000
-// instructions and the warps waited for the instruction cache.
-__host__ __device__ __forceinline__ float no_network() { return f32_make(0x7fffdeadu); }  // (a NaN that no operation gives)
-struct NoFaces {};
-template <int N, typename V, typename Store, typename Z = NoFaces>
+// once for the line.  The loop over the faces is unrolled by three: unrolled whole, a
+// line is some 2000 instructions and the warps waited for the instruction cache.
+template <int N, typename V, typename Store>
 __device__ __forceinline__ void weno5_line(const double *p0, const double *p1, const double *p2, int lane, int halo,
-                                           int step, FfScale s, Store store, Z given = {})
+                                           int step, FfScale s, Store store)
 {
-    constexpr bool JS = std::is_same<Z, NoFaces>::value;
     double v[V::W];
 #pragma unroll
     for (int i = 0; i < V::W; ++i) v[i] = p0[i * lane];
@@ -459,29 +454,7 @@ __device__ __forceinline__ void weno5_line(const double *p0, const double *p1, c
         const ffv<V> f3 = next(p);
         p += step;
         const ffv<V> q3 = ff_sqr(f3), x2 = ff_mul(f2, f3), t1 = ff_diff2(f1, f2, f3);
-        ffv<V> z1;
-        if constexpr (JS) {
-            z1 = weno5_ff(q0, q1, q2, q3, x0, x1, x2, t0, t1);
-        } else {
-            // z = d1 + 2 d2 - 6 (F - v2)
-            const V c = given(j), c6 = 6.0f * c;
-            z1 = {2.0f * f2.h, vfma(2.0f, f2.l, f1.l) - vfma(6.0f, c, -c6)};
-            ff_acc(z1, f1.h);
-            ff_acc(z1, -c6);
-            bool none[V::W], any = false;
-#pragma unroll
-            for (int i = 0; i < V::W; ++i) any |= none[i] = f32_bits(c[i]) == f32_bits(no_network());
-            if (any) {
-                const ffv<V> js = weno5_ff(q0, q1, q2, q3, x0, x1, x2, t0, t1);
-                float h[V::W], l[V::W];
-#pragma unroll
-                for (int i = 0; i < V::W; ++i) {
-                    h[i] = none[i] ? js.h[i] : z1.h[i];
-                    l[i] = none[i] ? js.l[i] : z1.l[i];
-                }
-                z1 = {V::of(h), V::of(l)};
-            }
-        }
+        const ffv<V> z1 = weno5_ff(q0, q1, q2, q3, x0, x1, x2, t0, t1);
         q0 = q1; q1 = q2; q2 = q3;
         x0 = x1; x1 = x2;
         t0 = t1;

@@ -37,7 +37,8 @@ __device__ __forceinline__ float field_val(float2 a) { return a.x + a.y; }
 // n, u, T and Delta p of one node from its 25 populations (Sec. 2.2; T from
 // the trace of Eq. sigmaq_def; Delta p = n T - p^w, Eq. vdw), and whether they
 // are admissible (finite, n > 0, T > 0, b n < 1).  get(k) returns population
-// k: the value (FP64) or the pair hi + lo (FP32).
+// k: the value (FP64) or the pair hi + lo (FP32).  SEQ: FP64 sums in FP64, one term
+// after the other (olb_stage64l.cuh).
 template <typename real>
 struct NodeMoments;
 template <>
@@ -52,15 +53,49 @@ struct NodeMoments<float> {
     bool ok;
 };
 
-template <typename real, typename Get>
+template <typename real, bool SEQ = false, typename Get>
 __device__ __forceinline__ NodeMoments<real> node_moments(Get get, const Geo &g, const Tab<real> &t)
 {
     NodeMoments<real> m;
     if constexpr (sizeof(real) == 8) {
-        const NodeSums s = node_sums64(get);
-        const double n = s.n;
-        const double jx = fma(t.R[4], s.a4x, t.R[3] * s.a3x), jy = fma(t.R[4], s.a4y, t.R[3] * s.a3y);
-        const double en = fma(t.R2[4], s.s4, t.R2[3] * s.s3);
+        double n, jx, jy, en;
+        if constexpr (SEQ) {
+            // row and column sums of the 5 x 5 populations; the middle root is 0
+            // (R[2] = R2[2] = 0), so its sums drop out of j and e
+            double sx[NQ], sy[NQ];
+#pragma unroll
+            for (int k1 = 0; k1 < NQ; ++k1) {
+                double s = get(NQ * k1);
+                if (k1 == 0) sy[0] = s;
+                else sy[0] += s;
+#pragma unroll
+                for (int k2 = 1; k2 < NQ; ++k2) {
+                    const double v = get(NQ * k1 + k2);
+                    s += v;
+                    if (k1 == 0) sy[k2] = v;
+                    else sy[k2] += v;
+                }
+                sx[k1] = s;
+            }
+            n = sx[0];
+            jx = t.R[0] * sx[0];
+            jy = t.R[0] * sy[0];
+            en = t.R2[0] * (sx[0] + sy[0]);
+#pragma unroll
+            for (int k = 1; k < NQ; ++k) {
+                n += sx[k];
+                if (k == 2) continue;
+                jx = fma(t.R[k], sx[k], jx);
+                jy = fma(t.R[k], sy[k], jy);
+                en = fma(t.R2[k], sx[k] + sy[k], en);
+            }
+        } else {
+            const NodeSums s = node_sums64(get);
+            n = s.n;
+            jx = fma(t.R[4], s.a4x, t.R[3] * s.a3x);
+            jy = fma(t.R[4], s.a4y, t.R[3] * s.a3y);
+            en = fma(t.R2[4], s.s4, t.R2[3] * s.s3);
+        }
         const double inv_n = recip_nr(n);
         const double ux = jx * inv_n, uy = jy * inv_n;
         const double T = 0.5 * fma(en, inv_n, -fma(ux, ux, uy * uy));
@@ -178,7 +213,7 @@ __host__ __device__ inline StageFields<real> fields_of(void *base, const Geo &g)
 // One thread per node: the moments of f_s, stored for the stage kernel,
 // which then reads them on its tile and halo instead of recomputing them
 // at every halo position; inadmissible moments set bit 0 of the status.
-template <typename real>
+template <typename real, bool SEQ = false>
 __global__ void __launch_bounds__(256) k_fields(const real *__restrict__ fs, StageFields<real> out, int *status,
                                                 const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t)
 {
@@ -188,7 +223,7 @@ __global__ void __launch_bounds__(256) k_fields(const real *__restrict__ fs, Sta
     const long long o = (long long)j * g.pitch + i;
     NodeMoments<real> m;
     if constexpr (sizeof(real) == 8)
-        m = node_moments<real>([&](int k) { return __ldg(fs + k * g.plane + o); }, g, t);
+        m = node_moments<real, SEQ>([&](int k) { return __ldg(fs + k * g.plane + o); }, g, t);
     else
         m = node_moments<real>(
             [&](int k) { return make_float2(__ldg(fs + k * g.plane + o), __ldg(fs + (NK + k) * g.plane + o)); }, g, t);
@@ -338,18 +373,72 @@ __device__ __forceinline__ int field_index(int i, int n, bool mirror)
 }
 
 constexpr int FORCE_X = 32, FORCE_Y = 8, FORCE_THREADS = FORCE_X * FORCE_Y / 2;
+template <int FX, int FY>
 struct ForceSmem {
-    static constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
+    static constexpr int HX = FX + 6, HY = FY + 6;
     double v[2][HY][HX];  // Delta p, n
-    float dx[2][2][3][HY][FORCE_X];
-    float dy[2][2][3][FORCE_Y][HX];
+    float dx[2][2][3][HY][FX];
+    float dy[2][2][3][FY][HX];
     int top;
 };
 
-__device__ __forceinline__ void force_block(ForceSmem &sm, const StageFields<double> &f, const Geo &g, const StageK &c,
-                                            int x0, int y0)
+// differences of the block's fields v, by all NT threads
+template <int NT, int FX, int FY>
+__device__ __forceinline__ void force_differences(ForceSmem<FX, FY> &sm, FfScale sc)
 {
-    constexpr int HX = ForceSmem::HX, HY = ForceSmem::HY;
+    constexpr int HX = FX + 6, HY = FY + 6;
+    // a row of the region, or a row of the block, at a time per warp lane
+    for (int e = threadIdx.x; e < 2 * HY * FX; e += NT) {
+        const int x = e % FX, r = e / FX % HY, k = e / (FX * HY);
+        const double *v = &sm.v[k][r][x + 3];
+#pragma unroll
+        for (int l = 1; l <= 3; ++l) {
+            const ff d = ff_split(v[l] - v[-l], sc);
+            sm.dx[k][0][l - 1][r][x] = d.h;
+            sm.dx[k][1][l - 1][r][x] = d.l;
+        }
+    }
+    for (int e = threadIdx.x; e < 2 * FY * HX; e += NT) {
+        const int x = e % HX, y = e / HX % FY, k = e / (HX * FY);
+        const double *v = &sm.v[k][y + 3][x];
+#pragma unroll
+        for (int l = 1; l <= 3; ++l) {
+            const ff d = ff_split(v[l * HX] - v[-l * HX], sc);
+            sm.dy[k][0][l - 1][y][x] = d.h;
+            sm.dy[k][1][l - 1][y][x] = d.l;
+        }
+    }
+}
+// c F along axis a at node (x, y) of the block and, two lanes, (x, y + 4)
+template <typename V, int FX, int FY>
+__device__ __forceinline__ ffv<V> force_at(const ForceSmem<FX, FY> &sm, FfScale sc, const StageK &c, int a, int x, int y)
+{
+    constexpr int HX = FX + 6, HY = FY + 6;
+    double nd[V::W];
+#pragma unroll
+    for (int i = 0; i < V::W; ++i) nd[i] = sm.v[1][y + 3 + 4 * i][x + 3];
+    const ffv<V> n = ff_split<V>(nd, sc);
+    const V r = rcp_seed(n.h);
+    const ffv<V> inv = {r, r * vfma(-r, n.l, vfma(-r, n.h, V::all(1.0f)))};
+    // sum_n in the populations' units is 2^k of the scaled one
+    const int k = 127 - 1023 - (sc.off >> 20), k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
+    const float u1 = f32_make((unsigned)(k1 + 127) << 23), u2 = f32_make((unsigned)(k2 + 127) << 23);
+    const float *d = a == 0 ? &sm.dx[0][0][0][y + 3][x] : &sm.dy[0][0][0][y][x + 3];
+    constexpr int NX = 3 * HY * FX, NY = 3 * FY * HX;
+    const int part = a == 0 ? NX : NY, lane = 4 * (a == 0 ? FX : HX), sr = a == 0 ? FX : 1;
+    const ffv<V> sp = stencil_sum<false, V>(d, d + part, lane, part / 3, sr);
+    const ffv<V> sn = stencil_sum<true, V>(d + 2 * part, d + 3 * part, lane, part / 3, sr);
+    ffv<V> v = ff_mul(c.kp, ff_mul(sp, inv));
+    const ffv<V> w = ff_mul(c.kn, sn);
+    v.l = v.l + u2 * (u1 * w.l);
+    ff_acc(v, u2 * (u1 * w.h));
+    return ff_norm(v);
+}
+
+__device__ __forceinline__ void force_block(ForceSmem<FORCE_X, FORCE_Y> &sm, const StageFields<double> &f, const Geo &g,
+                                            const StageK &c, int x0, int y0)
+{
+    constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
     const int tid = threadIdx.x;
     if (tid == 0) sm.top = 0;
     __syncthreads();
@@ -367,50 +456,12 @@ __device__ __forceinline__ void force_block(ForceSmem &sm, const StageFields<dou
     if ((tid & 31) == 0) atomicMax(&sm.top, top);
     __syncthreads();
     const FfScale sc = ff_scale(sm.top);
-    // differences: a row of the region, or a row of the block, at a time per warp lane
-    for (int e = tid; e < 2 * HY * FORCE_X; e += FORCE_THREADS) {
-        const int x = e % FORCE_X, r = e / FORCE_X % HY, k = e / (FORCE_X * HY);
-        const double *v = &sm.v[k][r][x + 3];
-#pragma unroll
-        for (int l = 1; l <= 3; ++l) {
-            const ff d = ff_split(v[l] - v[-l], sc);
-            sm.dx[k][0][l - 1][r][x] = d.h;
-            sm.dx[k][1][l - 1][r][x] = d.l;
-        }
-    }
-    for (int e = tid; e < 2 * FORCE_Y * HX; e += FORCE_THREADS) {
-        const int x = e % HX, y = e / HX % FORCE_Y, k = e / (HX * FORCE_Y);
-        const double *v = &sm.v[k][y + 3][x];
-#pragma unroll
-        for (int l = 1; l <= 3; ++l) {
-            const ff d = ff_split(v[l * HX] - v[-l * HX], sc);
-            sm.dy[k][0][l - 1][y][x] = d.h;
-            sm.dy[k][1][l - 1][y][x] = d.l;
-        }
-    }
+    force_differences<FORCE_THREADS>(sm, sc);
     __syncthreads();
-    // nodes (x, y) and (x, y + 4)
-    using V = vf2;
     const int x = tid % FORCE_X, y = tid / FORCE_X;
-    const double nd[2] = {sm.v[1][y + 3][x + 3], sm.v[1][y + 7][x + 3]};
-    const ffv<V> n = ff_split<V>(nd, sc);
-    const V r = rcp_seed(n.h);
-    const ffv<V> inv = {r, r * vfma(-r, n.l, vfma(-r, n.h, V::all(1.0f)))};
-    // sum_n in the populations' units is 2^k of the scaled one
-    const int k = 127 - 1023 - (sc.off >> 20), k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
-    const float u1 = f32_make((unsigned)(k1 + 127) << 23), u2 = f32_make((unsigned)(k2 + 127) << 23);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        const float *d = a == 0 ? &sm.dx[0][0][0][y + 3][x] : &sm.dy[0][0][0][y][x + 3];
-        constexpr int NX = 3 * HY * FORCE_X, NY = 3 * FORCE_Y * HX;
-        const int part = a == 0 ? NX : NY, lane = 4 * (a == 0 ? FORCE_X : HX), sr = a == 0 ? FORCE_X : 1;
-        const ffv<V> sp = stencil_sum<false, V>(d, d + part, lane, part / 3, sr);
-        const ffv<V> sn = stencil_sum<true, V>(d + 2 * part, d + 3 * part, lane, part / 3, sr);
-        ffv<V> v = ff_mul(c.kp, ff_mul(sp, inv));
-        const ffv<V> w = ff_mul(c.kn, sn);
-        v.l = v.l + u2 * (u1 * w.l);
-        ff_acc(v, u2 * (u1 * w.h));
-        v = ff_norm(v);
+        const ffv<vf2> v = force_at<vf2>(sm, sc, c, a, x, y);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
             if (x0 + x < g.nx && y0 + y + 4 * i < g.ny)
@@ -424,8 +475,9 @@ __device__ __forceinline__ void force_block(ForceSmem &sm, const StageFields<dou
 // double-float arithmetic with double-float weights (exact products of the hi
 // parts, TwoSum accumulation): the sum keeps FP32 accuracy of itself, not of its
 // terms.
+template <int FX, int FY>
 struct ForceSmem32 {
-    static constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
+    static constexpr int HX = FX + 6, HY = FY + 6;
     float2 dp[HY][HX], n[HY][HX];
 };
 // sums along x (y) at the node whose field is *v, fields sl apart along the
@@ -466,11 +518,20 @@ __device__ __forceinline__ float glap_sum32(const float2 *v, int sl, int sm)
         }
     return sum.hi + sum.lo;
 }
-// cc: the stage's coefficient of dt L
-__device__ __forceinline__ void force_block32(ForceSmem32 &sm, const StageFields<float> &f, const Geo &g, float cc, int x0,
-                                              int y0)
+// c F along axis a at node (x, y) of the block; cc: the stage's coefficient of dt L
+template <int FX, int FY>
+__device__ __forceinline__ float force_at32(const ForceSmem32<FX, FY> &sm, const Geo &g, float cc, int a, int x, int y)
 {
-    constexpr int HX = ForceSmem32::HX, HY = ForceSmem32::HY;
+    constexpr int HX = FX + 6;
+    const float2 *dp = &sm.dp[y + 3][x + 3], *n = &sm.n[y + 3][x + 3];
+    const float dn = (float)g.inv_ds / field_val(*n), sg3 = (float)g.sigma * (float)g.inv_ds3;
+    const int sl = a == 0 ? 1 : HX, sm_ = a == 0 ? HX : 1;
+    return cc * fmaf(grad_sum32(dp, sl, sm_), dn, sg3 * glap_sum32(n, sl, sm_));
+}
+__device__ __forceinline__ void force_block32(ForceSmem32<FORCE_X, FORCE_Y> &sm, const StageFields<float> &f, const Geo &g,
+                                              float cc, int x0, int y0)
+{
+    constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
     for (int e = threadIdx.x; e < HY * HX; e += 2 * FORCE_THREADS) {
         const int r = e / HX, x = e - r * HX;
         const long long o = (long long)field_index(y0 - 3 + r, g.ny, g.spec_y) * g.pitch + field_index(x0 - 3 + x, g.nx, g.walls);
@@ -480,21 +541,19 @@ __device__ __forceinline__ void force_block32(ForceSmem32 &sm, const StageFields
     __syncthreads();
     const int x = threadIdx.x % FORCE_X, y = threadIdx.x / FORCE_X;
     if (x0 + x >= g.nx || y0 + y >= g.ny) return;
-    const float2 *dp = &sm.dp[y + 3][x + 3], *n = &sm.n[y + 3][x + 3];
-    const float dn = (float)g.inv_ds / field_val(*n), sg3 = (float)g.sigma * (float)g.inv_ds3;
     const long long o = (long long)(y0 + y) * g.pitch + (x0 + x);
-    f.G[0][o] = cc * fmaf(grad_sum32(dp, 1, HX), dn, sg3 * glap_sum32(n, 1, HX));
-    f.G[1][o] = cc * fmaf(grad_sum32(dp, HX, 1), dn, sg3 * glap_sum32(n, HX, 1));
+#pragma unroll
+    for (int a = 0; a < 2; ++a) f.G[a][o] = force_at32(sm, g, cc, a, x, y);
 }
 
 template <typename real>
 struct ForceOf {
-    using Smem = ForceSmem;
+    using Smem = ForceSmem<FORCE_X, FORCE_Y>;
     static constexpr int NT = FORCE_THREADS;
 };
 template <>
 struct ForceOf<float> {
-    using Smem = ForceSmem32;
+    using Smem = ForceSmem32<FORCE_X, FORCE_Y>;
     static constexpr int NT = 2 * FORCE_THREADS;
 };
 template <typename real>
@@ -520,6 +579,62 @@ __global__ void __launch_bounds__(ForceOf<real>::NT) k_force_batch(char *fields,
     const int x0 = b % nbx * FORCE_X, y0 = b / nbx * FORCE_Y;
     if constexpr (sizeof(real) == 8) force_block(sm, f, run.g, run.k[st], x0, y0);
     else force_block32(sm, f, run.g, ccoef * (real)run.g.dt, x0, y0);
+}
+
+// ---------------------------------------------------------------- fields of one tile
+// Moments and stencils' input of an 8 x 8 tile whose CTA takes them itself (stage
+// kernels with KP 8): n and Delta p of the 14 x 14 nodes that the stencils of its
+// nodes read, the other moments of its nodes.
+template <typename real>
+struct TileFields;
+template <>
+struct TileFields<double> {
+    ForceSmem<8, 8> force;
+    double T[64], ux[64], uy[64];
+};
+template <>
+struct TileFields<float> {
+    ForceSmem32<8, 8> force;
+    float2 T[64], E[64];
+    float ux[64], uy[64];
+};
+constexpr int OWN_THREADS = 7 * 32;  // 14 x 14 nodes, one a thread
+// Threads 0 .. OWN_THREADS - 1, whole warps: the moments of a node (those of k_fields,
+// from the nodes that k_force's blocks take), the status of the tile's own nodes.
+template <typename real>
+__device__ __forceinline__ void tile_moments(TileFields<real> &own, int *top, const real *__restrict__ fs, int *status,
+                                             const Geo &g, const Tab<real> &t, int x0, int y0)
+{
+    const int tid = threadIdx.x, r = tid / 14, x = tid - 14 * r;
+    int a = 0;
+    if (r < 14) {
+        const real *f = fs + (long long)field_index(y0 - 3 + r, g.ny, g.spec_y) * g.pitch + field_index(x0 - 3 + x, g.nx, g.walls);
+        NodeMoments<real> m;
+        const bool mine = r >= 3 && r < 11 && x >= 3 && x < 11;
+        const int node = 8 * (r - 3) + x - 3;
+        if constexpr (sizeof(real) == 8) {
+            m = node_moments<real>([&](int k) { return __ldg(f + k * g.plane); }, g, t);
+            own.force.v[0][r][x] = m.dp;
+            own.force.v[1][r][x] = m.n;
+            a = __double2hiint(m.n) & 0x7fffffff;
+        } else {
+            m = node_moments<real>([&](int k) { return make_float2(__ldg(f + k * g.plane), __ldg(f + (NK + k) * g.plane)); },
+                                   g, t);
+            own.force.dp[r][x] = m.dp;
+            own.force.n[r][x] = m.n;
+            if (mine) own.E[node] = m.E;
+        }
+        if (mine) {
+            own.ux[node] = m.ux;
+            own.uy[node] = m.uy;
+            own.T[node] = m.T;
+            if (!m.ok && x0 + x - 3 < g.nx && y0 + r - 3 < g.ny) atomicOr(status, 1);
+        }
+    }
+    if constexpr (sizeof(real) == 8) {
+        a = __reduce_max_sync(0xffffffffu, a < 0x7ff00000 ? a : 0);
+        if ((tid & 31) == 0) atomicMax(top, a);
+    }
 }
 
 }  // namespace olb

@@ -22,17 +22,22 @@
 #include "olb_fields.cuh"
 #include "olb_stage32.cuh"
 #include "olb_stage64.cuh"
+#include "olb_stage64l.cuh"
 #include "olb_tile.cuh"
 
 namespace olb {
 
 template <typename real, int KP, bool LEARNED>
 struct StageSmem {
-    using type = Smem32<LEARNED>;
+    using type = Smem32<KP, LEARNED>;
 };
-template <int KP, bool LEARNED>
-struct StageSmem<double, KP, LEARNED> {
-    using type = Smem64<KP, LEARNED>;
+template <int KP>
+struct StageSmem<double, KP, false> {
+    using type = Smem64<KP>;
+};
+template <int KP>
+struct StageSmem<double, KP, true> {
+    using type = Smem64L<KP>;
 };
 
 // Shared memory of the single-grid kernel: the tile staging, then (learned
@@ -43,12 +48,20 @@ constexpr size_t mlp_offset()
 {
     return (sizeof(typename StageSmem<real, KP, true>::type) + 15) / 16 * 16;
 }
+// KP 8: the CTA's own fields.
+template <typename real>
+constexpr size_t own_offset()
+{
+    return (sizeof(typename StageSmem<real, 8, false>::type) + 15) / 16 * 16;
+}
 template <typename real, int KP, bool LEARNED>
 constexpr size_t fused_smem_bytes()
 {
     using S = typename StageSmem<real, KP, LEARNED>::type;
     constexpr size_t mlp_floats = sizeof(real) == 4 ? MLP_T32_SIZE : MLP_T64_SIZE + S::NT / 32 * MLP_WARP_SCRATCH;
-    return LEARNED ? mlp_offset<real, KP>() + mlp_floats * sizeof(float) : sizeof(S);
+    return LEARNED   ? mlp_offset<real, KP>() + mlp_floats * sizeof(float)
+           : KP == 8 ? own_offset<real>() + sizeof(TileFields<real>)
+                     : sizeof(S);
 }
 template <typename real, int KP, bool LEARNED>
 constexpr int stage_threads()
@@ -69,12 +82,12 @@ constexpr int fused_min_ctas(size_t smem_bytes, int threads, int cap = 0)
 }
 
 // Single grid: one CTA per tile.  Learned-weight instances leave their network the
-// registers it needs: two CTAs per SM.
+// registers it needs: 512 threads per SM.
 template <typename real, int KP, bool LEARNED>
 __global__ void __launch_bounds__((stage_threads<real, KP, LEARNED>()),
                                   fused_min_ctas(fused_smem_bytes<real, KP, LEARNED>(),
                                                  stage_threads<real, KP, LEARNED>(),
-                                                 LEARNED ? 2 : 0))
+                                                 KP == 4 ? 2 : KP == 5 ? 0 : 1))
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
         real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
@@ -88,12 +101,15 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
         net = {mlp, reinterpret_cast<float *>(smem_raw + mlp_offset<real, KP>())};
         mlp_tables<real>(net.tables, mlp);  // made visible by the first barrier inside stage_tile
     }
+    TileFields<real> *own = KP == 8 ? reinterpret_cast<TileFields<real> *>(smem_raw + own_offset<real>()) : nullptr;
     const TmaMap *tm = tma.on ? &tma.map : nullptr;
     const int x0 = blockIdx.x * 8, y0 = blockIdx.y * 8;
-    if constexpr (sizeof(real) == 8)
-        stage_tile64<KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, sk, net, tm, fields);
+    if constexpr (sizeof(real) == 8 && LEARNED)
+        stage_tile64l<KP>(sm, fs, fn, out, status, g, t, x0, y0, ca, cb, cc, net, tm, fields);
+    else if constexpr (sizeof(real) == 8)
+        stage_tile64<KP>(sm, fs, fn, out, status, g, t, t, x0, y0, sk, tm, fields, own);
     else
-        stage_tile32<LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, net, tm, fields);
+        stage_tile32<KP, LEARNED>(sm, fs, fn, out, status, g, t, t, x0, y0, ca, cb, cc, ca_lo, cb_lo, net, tm, fields, own);
 }
 
 // Batch of independent runs (uneven grid sizes, own parameters): one CTA per
@@ -106,7 +122,7 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
 template <typename real, int KP>
 __global__ void __launch_bounds__((stage_threads<real, KP, false>()),
                                   fused_min_ctas(fused_smem_bytes<real, KP, false>() + sizeof(BatchRun<real>),
-                                                 stage_threads<real, KP, false>()))
+                                                 stage_threads<real, KP, false>(), KP == 8 ? 1 : 0))
 k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
               const BatchRun<real> *__restrict__ runs, const int *__restrict__ tile_start, int nruns,
               const __grid_constant__ Tab<real> tv, real ca, real cb, real ccoef, real ca_lo, real cb_lo, int st,
@@ -134,12 +150,13 @@ k_fused_batch(const real *__restrict__ fs, const real *fn, real *out, int *__res
     if (tm && threadIdx.x == 0)
         for (int k = 0; k < 2; ++k)
             asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(tm->bytes[k]) : "memory");
+    TileFields<real> *own = KP == 8 ? reinterpret_cast<TileFields<real> *>(smem_raw + own_offset<real>()) : nullptr;
     if constexpr (sizeof(real) == 8)
-        stage_tile64<KP, false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
-                                run.k[st], MlpArg{}, tm, fl);
+        stage_tile64<KP>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0,
+                                run.k[st], tm, fl, own);
     else
-        stage_tile32<false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0, ca, cb,
-                            ccoef * (real)run.g.dt, ca_lo, cb_lo, MlpArg{}, tm, fl);
+        stage_tile32<KP, false>(sm, fs + run.off, fn + run.off, out + run.off, status + lo, run.g, tv, run.t, x0, y0, ca, cb,
+                            ccoef * (real)run.g.dt, ca_lo, cb_lo, MlpArg{}, tm, fl, own);
 }
 
 template <typename real, int KP, bool LEARNED = false>
@@ -166,13 +183,17 @@ cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *sta
         tma.map = *tmap;
         tma.on = 1;
     }
-    // the moments of fs first (one thread per node), then the stage
+    // the moments of fs first (one thread per node) and the force, then the stage
     const StageFields<real> fl = fields_of<real>(fields, g);
-    const long long N = (long long)g.nx * g.ny;
-    k_fields<real><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
     const StageK sk = sizeof(real) == 8 ? stage_constants(g, c) : StageK{};
-    k_force<real><<<dim3((g.nx + FORCE_X - 1) / FORCE_X, (g.ny + FORCE_Y - 1) / FORCE_Y), ForceOf<real>::NT, 0, s>>>(
-        fl, g, sk, (real)c.cc);
+    if (KP != 8) {
+        const long long N = (long long)g.nx * g.ny;
+        constexpr bool SEQ = LEARNED && sizeof(real) == 8;
+        k_fields<real, SEQ><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
+        const dim3 blocks((g.nx + FORCE_X - 1) / FORCE_X, (g.ny + FORCE_Y - 1) / FORCE_Y);
+        if constexpr (SEQ) k_force_learned<real><<<blocks, 2 * FORCE_THREADS, 0, s>>>(fl, g, c.cc);
+        else k_force<real><<<blocks, ForceOf<real>::NT, 0, s>>>(fl, g, sk, (real)c.cc);
+    }
     k_fused<real, KP, LEARNED><<<grid, stage_threads<real, KP, LEARNED>(), fused_smem_bytes<real, KP, LEARNED>(), s>>>(
         fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
         (real)(c.cb - (double)(real)c.cb), sk, mlp, tma, fl);
@@ -186,7 +207,7 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
                                    const int *force_start, int force_blocks, const TmaMap *tmaps, cudaStream_t s)
 {
     if (total < 1) return cudaSuccess;
-    if (total_nodes > 0) {
+    if (KP != 8 && total_nodes > 0) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -195,8 +216,9 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
             fs, static_cast<char *>(fields), static_cast<const BatchRun<real> *>(runs), node_start, nruns, total_nodes,
             status);
     }
-    k_force_batch<real><<<force_blocks, ForceOf<real>::NT, 0, s>>>(
-        static_cast<char *>(fields), static_cast<const BatchRun<real> *>(runs), force_start, nruns, st, (real)c.cc);
+    if (KP != 8)
+        k_force_batch<real><<<force_blocks, ForceOf<real>::NT, 0, s>>>(
+            static_cast<char *>(fields), static_cast<const BatchRun<real> *>(runs), force_start, nruns, st, (real)c.cc);
     k_fused_batch<real, KP><<<total, stage_threads<real, KP, false>(), fused_smem_bytes<real, KP, false>(), s>>>(
         fs, fn, out, status, static_cast<const BatchRun<real> *>(runs), tile_start, nruns, t, (real)c.ca, (real)c.cb,
         (real)c.cc, (real)(c.ca - (double)(real)c.ca), (real)(c.cb - (double)(real)c.cb), st, static_cast<char *>(fields),
@@ -204,44 +226,33 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
     return cudaGetLastError();
 }
 
-// Compiled instances (stage_shape): KP 8 and 5 in FP64, 5 in FP32, 4 with learned
-// weights.
-#define OLB_FUSED_CASES_double(DO) DO(double, 8, false) DO(double, 5, false)
-#define OLB_FUSED_CASES_float(DO) DO(float, 5, false)
-#define OLB_FUSED_PREP_CASE(real, C, L) \
-    if (learned == L && sh.kp == C) return fused_prepare_one<real, C, L>();
-#define OLB_FUSED_LAUNCH_CASE(real, C, L)    \
-    if ((mlp != nullptr) == L && sh.kp == C) \
-        return fused_launch_one<real, C, L>(fs, fn, out, status, g, t, c, mlp, tma, fields, s);
-#define OLB_FUSED_BATCH_CASE(real, C, L)                                                                     \
-    if (sh.kp == C)                                                                                          \
-        return fused_batch_launch_one<real, C>(fs, fn, out, status, runs, tile_start, nruns, total, t, c, st,    \
-                                               fields, node_start, total_nodes, force_start, force_blocks, tmaps, s);
+// Compiled instances (stage_kind): KP 8 and 5, 6 and 4 with learned weights.
 #define OLB_DEFINE_FUSED(real)                                                                                \
     cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned)                                   \
     {                                                                                                         \
         if (learned && !learned_shape(tx, ty, kp)) return cudaErrorInvalidValue;                              \
-        const Shape sh = stage_shape(sizeof(real) == 8, learned, tx, ty, kp);                                 \
-        OLB_FUSED_CASES_##real(OLB_FUSED_PREP_CASE) OLB_FUSED_PREP_CASE(real, 4, true)                        \
-        return cudaErrorInvalidValue;                                                                         \
+        const cudaError_t e = learned ? fused_prepare_one<real, 6, true>() : fused_prepare_one<real, 8>();    \
+        return e != cudaSuccess ? e : learned ? fused_prepare_one<real, 4, true>() : fused_prepare_one<real, 5>(); \
     }                                                                                                         \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,            \
-                             const Tab<real> &t, StageCoef c, int tx, int ty, int kp, const float *mlp,       \
-                             const TmaMap *tma, void *fields, cudaStream_t s)                                 \
+                             const Tab<real> &t, StageCoef c, const float *mlp, const TmaMap *tma,            \
+                             void *fields, cudaStream_t s)                                                    \
     {                                                                                                         \
-        const Shape sh = stage_shape(sizeof(real) == 8, mlp != nullptr, tx, ty, kp);                          \
-        OLB_FUSED_CASES_##real(OLB_FUSED_LAUNCH_CASE) OLB_FUSED_LAUNCH_CASE(real, 4, true)                    \
-        return cudaErrorInvalidValue;                                                                         \
+        const int kind = stage_kind(mlp != nullptr, stage_tiles(g.nx, g.ny));                                 \
+        if (kind == 4) return fused_launch_one<real, 4, true>(fs, fn, out, status, g, t, c, mlp, tma, fields, s); \
+        if (kind == 6) return fused_launch_one<real, 6, true>(fs, fn, out, status, g, t, c, mlp, tma, fields, s); \
+        return kind == 8 ? fused_launch_one<real, 8>(fs, fn, out, status, g, t, c, nullptr, tma, fields, s)   \
+                         : fused_launch_one<real, 5>(fs, fn, out, status, g, t, c, nullptr, tma, fields, s);  \
     }                                                                                                         \
     cudaError_t launch_fused_batch(const real *fs, const real *fn, real *out, int *status, const void *runs,  \
-                                   const int *tile_start, int nruns, int total, const Tab<real> &t,         \
-                                   StageCoef c, int st, int tx, int ty, int kp, void *fields,                 \
-                                   const long long *node_start, long long total_nodes, const int *force_start, int force_blocks, const TmaMap *tmaps,   \
-                                   cudaStream_t s)                                                            \
+                                   const int *tile_start, int nruns, int total, const Tab<real> &t,           \
+                                   StageCoef c, int st, void *fields, const long long *node_start,            \
+                                   long long total_nodes, const int *force_start, int force_blocks,           \
+                                   const TmaMap *tmaps, cudaStream_t s)                                       \
     {                                                                                                         \
-        const Shape sh = stage_shape(sizeof(real) == 8, false, tx, ty, kp);                                   \
-        OLB_FUSED_CASES_##real(OLB_FUSED_BATCH_CASE)                                                          \
-        return cudaErrorInvalidValue;                                                                         \
+        const auto go = stage_kind(false, total) == 8 ? fused_batch_launch_one<real, 8> : fused_batch_launch_one<real, 5>; \
+        return go(fs, fn, out, status, runs, tile_start, nruns, total, t, c, st, fields, node_start, total_nodes, \
+                  force_start, force_blocks, tmaps, s);                                                       \
     }                                                                                                         \
     size_t batch_run_bytes(real *) { return sizeof(BatchRun<real>); }                                         \
     void batch_run_fill(real *, void *dst, const Geo &g, const Tab<real> &t, long long off, long long foff,   \

@@ -125,16 +125,20 @@ __host__ __device__ constexpr int region_pitch(int tx, bool fp64) { return tx + 
 // if the shape's rows are not a multiple of 16 bytes or the driver refuses.
 bool tma_encode(TmaMap *out, const void *base, bool fp64, const Geo &g, int tx, int ty);
 
-// The compiled shape that advances tiles of a shape: all tiles are advanced as 8 x 8
-// tiles (their flux differences and factors fit in shared memory beside the
-// populations; larger shapes kept one velocity's faces at a time and recomputed
-// per-node terms 25 times: FP32 4096^2 14 ms a stage with 32 x 16 against 8).
-// FP64 shapes with eight lanes take 320 threads of one node, the others 160 of
-// two (Plan64 in olb_stage64.cuh).
-struct Shape {
-    int tx, ty, kp;
-};
-inline Shape stage_shape(bool fp64, bool learned, int, int, int kp) { return {8, 8, learned ? 4 : fp64 && kp == 8 ? 8 : 5}; }
+// All grids are advanced as tiles of 8 x 8 nodes, whatever shape was set (their flux
+// differences and factors fit in shared memory beside the populations; larger shapes
+// kept one velocity's faces at a time and recomputed per-node terms 25 times: FP32
+// 4096^2 14 ms a stage with 32 x 16 against 8).
+constexpr int STAGE_TX = 8, STAGE_TY = 8;
+inline int stage_tiles(int nx, int ny) { return ((nx + STAGE_TX - 1) / STAGE_TX) * ((ny + STAGE_TY - 1) / STAGE_TY); }
+// The compiled stage that advances so many tiles.  At most one tile an SM, 8: one launch of 512 threads a tile that take the moments and the
+// force of the tile too (of its 14 x 14 nodes, three times the work of k_fields);
+// else 5: three launches.  A stage, three launches and one, FP64: 8 tiles 26.4 and
+// 14.7 us, 128 tiles 27.4 and 15.7, 256 tiles 32.6 and 30.4, 384 tiles 35.1 and 45.0,
+// 4096 tiles 214 and 408; FP32: 13.1 and 7.2, 14.3 and 8.0, 15.7 and 15.0, 17.8 and
+// 21.8, 96 and 188.  Learned weights: at most one tile an SM, 6 (512 threads a tile), else
+// 4 (256, two tiles an SM): 39 tiles 70 and 60 us (FP64), 51 and 38 us (FP32).
+int stage_kind(bool learned, int tiles);
 
 // Shapes that olb_set_tile accepts with learned weights.
 inline bool learned_shape(int tx, int ty, int kp)
@@ -155,12 +159,11 @@ StageK stage_constants(const Geo &g, StageCoef c);
 #define OLB_DECLARE_LAUNCHERS(real)                                                                    \
     cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned);                           \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,     \
-                             const Tab<real> &t, StageCoef c, int tx, int ty, int kp,                  \
-                             const float *mlp, const TmaMap *tma, void *fields, cudaStream_t s);       \
+                             const Tab<real> &t, StageCoef c, const float *mlp,                        \
+                             const TmaMap *tma, void *fields, cudaStream_t s);                         \
     cudaError_t launch_fused_batch(const real *fs, const real *fn, real *out, int *status,             \
                                    const void *runs, const int *tile_start, int nruns, int total,      \
-                                   const Tab<real> &t, StageCoef c, int st, int tx, int ty, int kp,    \
-                                   void *fields,                                                       \
+                                   const Tab<real> &t, StageCoef c, int st, void *fields,              \
                                    const long long *node_start, long long total_nodes,                 \
                                    const int *force_start, int force_blocks,                           \
                                    const TmaMap *tmaps, cudaStream_t s);                               \
@@ -190,7 +193,7 @@ inline int force_blocks(const Geo &g) { return ((g.nx + 31) / 32) * ((g.ny + 7) 
 constexpr int TOTALS_BLOCKS = 1024, TOTALS_THREADS = 256;
 
 // Shapes that olb_set_tile accepts: TX x TY nodes and KP velocities at once
-// (stage_shape: what advances them).
+// (all are advanced as tiles of STAGE_TX x STAGE_TY).
 constexpr int NUM_TILES = 8;
 constexpr int TILE_X[NUM_TILES] = {8, 16, 16, 32, 32, 8, 7, 8};
 constexpr int TILE_Y[NUM_TILES] = {8, 8, 8, 8, 16, 8, 8, 8};

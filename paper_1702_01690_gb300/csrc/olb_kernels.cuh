@@ -68,12 +68,8 @@ __device__ __forceinline__ double recip_nr1(double d)
     return fma(r, fma(-d, r, 1.0), r);
 }
 
-// Jiang-Shu correction of an interface in FP64, for the stencils that the learned
-// weights leave to Jiang-Shu in FP64 contexts: a warp takes this beside the
-// network, which fills the FP32 pipe, so it stays on the FP64 pipe (as weno5_ff
-// it measured 50.6 ms against 43.8 ms for two steps of 1024^2, when the node
-// updates were in FP64).  Same forms as
-// weno5_ff (olb_ff.cuh).
+// Jiang-Shu value of an interface in FP64, for the stencils that the learned
+// weights leave to Jiang-Shu in FP64 contexts (olb_stage64l.cuh).
 //
 // Weights: wbar_q is proportional to delta_q / sigma_q^2.  Multiplying every
 // term by 10 (sigma_1 sigma_2 sigma_3)^2 gives weights proportional to
@@ -84,7 +80,7 @@ __device__ __forceinline__ double recip_nr1(double d)
 // the vanishing set).  If the products underflow without an exact zero the
 // min-scaled form delta_q (s/sigma_q)^2 is used instead.
 __device__ __forceinline__ double weno5_core(double d01, double d12, double d23, double d34, double q23, double h12,
-                                             double h23)
+                                             double h23, double v2)
 {
     const double s1 = fma(d01, fma(-2.75, d12, d01), h12);
     const double s2 = fma(d12, fma(-1.25, d23, d12), q23);
@@ -114,7 +110,7 @@ __device__ __forceinline__ double weno5_core(double d01, double d12, double d23,
         }
         den = A1 + A2 + A3;
     }
-    return fma(A1, G1, fma(A2, G2, A3 * G3)) * recip_nr1(6.0 * den);
+    return fma(fma(A1, G1, fma(A2, G2, A3 * G3)), recip_nr1(6.0 * den), v2);
 }
 // FP32 populations: the correction c of an interface value (the value minus
 // its upwind node v2, sum_q wbar_q (Fhat^q - v2)) from the first differences
@@ -185,28 +181,6 @@ __device__ __forceinline__ void eq_factors(const Tab<real> &t, real u, real T, r
 #pragma unroll
     for (int k = 0; k < NQ; ++k)
         g[k] = fma(t.wHe[k][4], c4, fma(t.wHe[k][3], c3, fma(t.wHe[k][2], c2, fma(t.wHe[k][1], c1, t.wHe[k][0]))));
-}
-
-// The same in FP64 by the parity of the Hermite orders: 26 instead of 34
-// FP64 operations.
-__device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, double T, double g[NQ])
-{
-    const double th = T - 1.0, u2 = u * u;
-    const double c2 = 0.5 * (u2 + th);
-    const double c3 = u * fma(u2, 1.0 / 6.0, 0.5 * th);
-    const double c4 = fma(u2, fma(u2, 1.0 / 24.0, 0.25 * th), 0.125 * th * th);
-#pragma unroll
-    for (int m = 0; m <= 2; ++m) {
-        const int k = 2 + m;
-        const double even = fma(t.wHe[k][4], c4, fma(t.wHe[k][2], c2, t.wHe[k][0]));
-        if (m == 0) {
-            g[2] = even;
-        } else {
-            const double odd = fma(t.wHe[k][3], c3, t.wHe[k][1] * u);
-            g[2 + m] = even + odd;
-            g[2 - m] = even - odd;
-        }
-    }
 }
 
 // The same factors split by Hermite order parity: ge_k from the even orders
@@ -584,8 +558,8 @@ __device__ __forceinline__ double load_pop(const float *f, long long plane, long
 }
 
 // ---------------------------------------------------------------- init / output
-// f = f^eq(n, u, T) (Eq. feq), evaluated in FP64 for both storages.  Bound by its 82
-// (FP64 populations) or 98 FP64 operations a node.
+// f = f^eq(n, u, T) (Eq. feq), evaluated in FP64 for both storages.  Bound by its 98 FP64
+// operations a node.
 template <typename real>
 __global__ void k_init(real *__restrict__ f, const double *__restrict__ n, const double *__restrict__ ux,
                        const double *__restrict__ uy, const double *__restrict__ T, Geo g, Tab<double> t)
@@ -595,13 +569,8 @@ __global__ void k_init(real *__restrict__ f, const double *__restrict__ n, const
     const int j = (int)(idx / g.nx), i = (int)(idx - (long long)j * g.nx);
     const long long o = (long long)j * g.pitch + i;
     double gx[NQ], gy[NQ];
-    if constexpr (sizeof(real) == 8) {
-        eq_factors64(t, ux[idx], T[idx], gx);
-        eq_factors64(t, uy[idx], T[idx], gy);
-    } else {
-        eq_factors<double>(t, ux[idx], T[idx], gx);
-        eq_factors<double>(t, uy[idx], T[idx], gy);
-    }
+    eq_factors<double>(t, ux[idx], T[idx], gx);
+    eq_factors<double>(t, uy[idx], T[idx], gy);
     const double nn = n[idx];
 #pragma unroll
     for (int k1 = 0; k1 < NQ; ++k1)

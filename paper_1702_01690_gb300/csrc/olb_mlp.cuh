@@ -79,54 +79,54 @@ __device__ __forceinline__ void mlp_weights(const float *__restrict__ th, const 
 // compared on the integer pipe (they are >= 0, and their bit patterns order
 // like their values; x == 0 of either sign is a zero pattern without the sign
 // bit).
-template <typename real>
-__device__ __forceinline__ bool learned_guard(real d01, real d12, real d23, real d34)
+__device__ __forceinline__ bool learned_guard(float d01, float d12, float d23, float d34)
 {
-    if constexpr (sizeof(real) == 8) {
-        // a_q = b_q = 0 exactly when both differences of sub-stencil q are 0
-        // (a difference of two numbers is 0 only when they are equal, and an
-        // FMA is exact before its one rounding)
-        auto z = [](double v) { return (__double_as_longlong(v) << 1) == 0; };
-        if ((z(d01) && z(d12)) || (z(d12) && z(d23)) || (z(d23) && z(d34))) return false;
-        // FP32 pre-check: each sigma_q is a positive-definite quadratic form in
-        // two differences (condition number ~18), so from the differences
-        // rounded to FP32 it carries a relative error below ~3e-6; outside a
-        // band of 1e-4 around the threshold the FP32 comparison is the FP64
-        // one.  Inside the band, or with squares near FP32's range limits,
-        // the FP64 test below decides.
-        const float e01 = (float)d01, e12 = (float)d12, e23 = (float)d23, e34 = (float)d34;
-        const float fa1 = e12 - e01, fb1 = fmaf(3.0f, e12, -e01);
-        const float fa2 = e23 - e12, fb2 = e12 + e23;
-        const float fa3 = e34 - e23, fb3 = fmaf(-3.0f, e23, e34);
-        const float f1 = fmaf(13.0f * fa1, fa1, 3.0f * fb1 * fb1);
-        const float f2v = fmaf(13.0f * fa2, fa2, 3.0f * fb2 * fb2);
-        const float f3 = fmaf(13.0f * fa3, fa3, 3.0f * fb3 * fb3);
-        const float fmn = fminf(f1, fminf(f2v, f3)), fmx = fmaxf(f1, fmaxf(f2v, f3));
-        if (fmx > 1e-30f && fmx < 1e30f) {
-            if (fmn < (float)(MLP_GUARD * (1.0 - 1e-4)) * fmx) return true;
-            if (fmn > (float)(MLP_GUARD * (1.0 + 1e-4)) * fmx) return false;
-        }
+    const float a1 = d12 - d01, b1 = fmaf(3.0f, d12, -d01);
+    const float a2 = d23 - d12, b2 = d12 + d23;
+    const float a3 = d34 - d23, b3 = fmaf(-3.0f, d23, d34);
+    const float s1 = fmaf(13.0f * a1, a1, 3.0f * b1 * b1);
+    const float s2 = fmaf(13.0f * a2, a2, 3.0f * b2 * b2);
+    const float s3 = fmaf(13.0f * a3, a3, 3.0f * b3 * b3);
+    const float smin = fminf(s1, fminf(s2, s3)), smax = fmaxf(s1, fmaxf(s2, s3));
+    const bool zero = (a1 == 0.0f && b1 == 0.0f) || (a2 == 0.0f && b2 == 0.0f) || (a3 == 0.0f && b3 == 0.0f);
+    return !zero && smin < (float)MLP_GUARD * smax;
+}
+// d: the differences d01 .. d34; e: the same rounded to FP32
+__device__ __forceinline__ bool learned_guard(const double d[4], const float e[4])
+{
+    // a_q = b_q = 0 exactly when both differences of sub-stencil q are 0
+    // (a difference of two numbers is 0 only when they are equal, and an
+    // FMA is exact before its one rounding)
+    auto z = [](double v) { return (__double_as_longlong(v) << 1) == 0; };
+    if ((z(d[0]) && z(d[1])) || (z(d[1]) && z(d[2])) || (z(d[2]) && z(d[3]))) return false;
+    // FP32 pre-check: each sigma_q is a positive-definite quadratic form in
+    // two differences (condition number ~18), so from the differences
+    // rounded to FP32 it carries a relative error below ~3e-6; outside a
+    // band of 1e-4 around the threshold the FP32 comparison is the FP64
+    // one.  Inside the band, or with squares near FP32's range limits,
+    // the FP64 test below decides.
+    const float fa1 = e[1] - e[0], fb1 = fmaf(3.0f, e[1], -e[0]);
+    const float fa2 = e[2] - e[1], fb2 = e[1] + e[2];
+    const float fa3 = e[3] - e[2], fb3 = fmaf(-3.0f, e[2], e[3]);
+    const float f1 = fmaf(13.0f * fa1, fa1, 3.0f * fb1 * fb1);
+    const float f2v = fmaf(13.0f * fa2, fa2, 3.0f * fb2 * fb2);
+    const float f3 = fmaf(13.0f * fa3, fa3, 3.0f * fb3 * fb3);
+    const float fmn = fminf(f1, fminf(f2v, f3)), fmx = fmaxf(f1, fmaxf(f2v, f3));
+    if (fmx > 1e-30f && fmx < 1e30f) {
+        if (fmn < (float)(MLP_GUARD * (1.0 - 1e-4)) * fmx) return true;
+        if (fmn > (float)(MLP_GUARD * (1.0 + 1e-4)) * fmx) return false;
     }
-    const real a1 = d12 - d01, b1 = fma(real(3), d12, -d01);
-    const real a2 = d23 - d12, b2 = d12 + d23;
-    const real a3 = d34 - d23, b3 = fma(real(-3), d23, d34);
-    const real s1 = fma(real(13) * a1, a1, real(3) * b1 * b1);
-    const real s2 = fma(real(13) * a2, a2, real(3) * b2 * b2);
-    const real s3 = fma(real(13) * a3, a3, real(3) * b3 * b3);
-    real smin, smax;
-    bool zero;
-    if constexpr (sizeof(real) == 8) {
-        const long long i1 = __double_as_longlong(s1), i2 = __double_as_longlong(s2), i3 = __double_as_longlong(s3);
-        smin = i1 < i2 ? (i1 < i3 ? s1 : s3) : (i2 < i3 ? s2 : s3);
-        smax = i1 > i2 ? (i1 > i3 ? s1 : s3) : (i2 > i3 ? s2 : s3);
-        auto z = [](real v) { return (__double_as_longlong(v) << 1) == 0; };
-        zero = (z(a1) && z(b1)) || (z(a2) && z(b2)) || (z(a3) && z(b3));
-    } else {
-        smin = fminf(s1, fminf(s2, s3));
-        smax = fmaxf(s1, fmaxf(s2, s3));
-        zero = (a1 == 0.0f && b1 == 0.0f) || (a2 == 0.0f && b2 == 0.0f) || (a3 == 0.0f && b3 == 0.0f);
-    }
-    return !zero && smin < real(MLP_GUARD) * smax;
+    const double a1 = d[1] - d[0], b1 = fma(3.0, d[1], -d[0]);
+    const double a2 = d[2] - d[1], b2 = d[1] + d[2];
+    const double a3 = d[3] - d[2], b3 = fma(-3.0, d[2], d[3]);
+    const double s1 = fma(13.0 * a1, a1, 3.0 * b1 * b1);
+    const double s2 = fma(13.0 * a2, a2, 3.0 * b2 * b2);
+    const double s3 = fma(13.0 * a3, a3, 3.0 * b3 * b3);
+    const long long i1 = __double_as_longlong(s1), i2 = __double_as_longlong(s2), i3 = __double_as_longlong(s3);
+    const double smin = i1 < i2 ? (i1 < i3 ? s1 : s3) : (i2 < i3 ? s2 : s3);
+    const double smax = i1 > i2 ? (i1 > i3 ? s1 : s3) : (i2 > i3 ? s2 : s3);
+    const bool zero = (z(a1) && z(b1)) || (z(a2) && z(b2)) || (z(a3) && z(b3));
+    return !zero && smin < MLP_GUARD * smax;
 }
 
 // The network's input from the stencil's first differences in FP32: the
@@ -166,24 +166,25 @@ __device__ __forceinline__ float learned_corr_net(const float *__restrict__ th, 
     return learned_corr_from(w, e);
 }
 
-// Learned WENO-5 correction (interface value minus its upwind node, without p/m)
-// from the first differences of the upwind-ordered stencil: where any
+// Learned WENO-5 face value of one upwind-ordered stencil: where any
 // smoothness indicator vanishes the Jiang-Shu weights with Table tab:weno apply
 // (constant ghost layers keep their exact flux), and so do they where the
 // stencil is smooth (min sigma_q >= MLP_GUARD max sigma_q); otherwise
 // sum_q w_q G_q with the network's weights.  FP64 populations: the guard is
 // taken in FP64; the network and sum_q w_q G_q run in FP32 (the weights carry
 // FP32 error anyway).  This and weno5_learned_corr: one thread's face, for walls.
-__device__ __forceinline__ double weno5_learned_corr64(const float *__restrict__ th, double d01, double d12, double d23,
-                                                       double d34)
+__device__ __forceinline__ double weno5_js(const double d[4], double v2)
 {
-    if (!learned_guard<double>(d01, d12, d23, d34)) {
-        // Jiang-Shu on the same differences
-        const double q12 = d12 * d12, q23 = d23 * d23;
-        return weno5_core(d01, d12, d23, d34, q23, 2.5 * q12, 2.5 * q23);
-    }
-    const float e[4] = {(float)d01, (float)d12, (float)d23, (float)d34};
-    return (double)learned_corr_net(th, e);
+    const double q12 = d[1] * d[1], q23 = d[2] * d[2];
+    return weno5_core(d[0], d[1], d[2], d[3], q23, 2.5 * q12, 2.5 * q23, v2);
+}
+__device__ __forceinline__ double weno5_learned(const float *__restrict__ th, double v0, double v1, double v2, double v3,
+                                                double v4)
+{
+    const double d[4] = {v1 - v0, v2 - v1, v3 - v2, v4 - v3};
+    const float e[4] = {(float)d[0], (float)d[1], (float)d[2], (float)d[3]};
+    if (!learned_guard(d, e)) return weno5_js(d, v2);
+    return v2 + (double)learned_corr_net(th, e);
 }
 
 // The same for the compensated FP32 storage: the correction sum_q w_q G_q (the
@@ -192,7 +193,7 @@ __device__ __forceinline__ double weno5_learned_corr64(const float *__restrict__
 __device__ __forceinline__ float weno5_learned_corr(const float *__restrict__ th, float d01, float d12, float d23,
                                                    float d34)
 {
-    if (!learned_guard<float>(d01, d12, d23, d34)) return weno5_corr(d01, d12, d23, d34);
+    if (!learned_guard(d01, d12, d23, d34)) return weno5_corr(d01, d12, d23, d34);
     const float e[4] = {d01, d12, d23, d34};
     return learned_corr_net(th, e);
 }
@@ -210,14 +211,13 @@ __device__ __forceinline__ float weno5_learned_corr(const float *__restrict__ th
 // fragment, so nothing goes through shared memory.
 //   FP64 populations: FP32 multiply-adds, the layers' outputs exchanged through
 // shared memory (mlp_weights' sums: the same results).
-// One stage of 1024^2 where the network acts on nearly every face: 5.07 -> 3.15 ms
-// (FP32 populations) and 5.67 -> 4.51 ms (FP64), from a lane per stencil, whose
-// weights came with 576 loads a face (FP64) and whose layer-1 outputs went through
-// shared memory to the fragments (FP32); FP64 faces where the network does not act
-// also left the FP64 pipe (weno5_line).  Bound by instruction issue and latency with
-// the 16 warps that 128 registers a thread leave an SM (ncu: issue 61 %, special
-// functions 22 %, tensor pipe 30 % with FP32; issue 49 %, FP32 pipe 25 %, wavefronts
-// of shared memory 90 % before their rows were rotated, with FP64).
+// One stage of 1024^2 where the network acts on nearly every face: 5.0 -> 3.1 ms (FP32
+// populations) and 7.2 -> 4.95 ms (FP64), from a lane per stencil, whose weights came
+// with 576 loads a face (FP64) and whose layer-1 outputs went through shared memory to
+// the fragments (FP32).  Bound by instruction issue and latency with the 16 warps that
+// 128 registers a thread leave an SM (ncu: FP32 issue 61 %, special functions 22 %,
+// tensor pipe 30 %; FP64, before the rows of its scratch were rotated, wavefronts of
+// shared memory 90 %).
 
 // What a stage kernel has of the network: its parameters in global memory (wall faces,
 // a network a thread), the tables and scratch in shared memory.

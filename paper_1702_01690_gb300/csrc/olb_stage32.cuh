@@ -23,11 +23,13 @@
 
 namespace olb {
 
-// 320 threads: a line of the tile (Line), then a node and velocity column, each;
-// with learned weights 256 (whose network needs the registers).
-template <bool LEARNED>
+// KP (stage_kind) 5: 320 threads, a line of the tile (Line), then a node and velocity
+// column, each; 8: 512, which take the tile's moments and force too (OWN); 4: 256,
+// with learned weights (whose network needs the registers), 6: 512 with them.
+template <int KP, bool LEARNED>
 struct Smem32 : Staged<float> {
-    static constexpr int NT = LEARNED ? 256 : 320;
+    static constexpr bool OWN = KP == 8;
+    static constexpr int NT = OWN || KP == 6 ? 512 : LEARNED ? 256 : 320;
     // per tile node: the even and odd equilibrium parts n ge_q(u_x, T), n go_q(u_x,
     // T), ge_q(u_y, T), go_q(u_y, T), the correction alpha, beta, gamma
     // (eq_correction), and c F
@@ -93,14 +95,15 @@ __device__ __forceinline__ void weno5_line32(const Line<float> &ln, int lo_p1, i
 // table of the wall entries; net: the learned network (LEARNED only); tmap: TMA maps of fs, or nullptr; fields: the moments and c F of
 // fs (k_fields, k_force).  Returns false when the TMA copy timed out (the CTA must
 // stop).
-template <bool LEARNED>
-__device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *__restrict__ fs, const float *fn, float *out,
+template <int KP, bool LEARNED>
+__device__ __forceinline__ bool stage_tile32(Smem32<KP, LEARNED> &sm, const float *__restrict__ fs, const float *fn, float *out,
                                              int *__restrict__ status, const Geo &g, const Tab<float> &t,
                                              const Tab<float> &tw, int x0, int y0, float ca, float cb, float cc, float ca_lo,
                                              float cb_lo, const MlpArg &net, const TmaMap *tmap,
-                                             const StageFields<float> &fields)
+                                             const StageFields<float> &fields, TileFields<float> *own = nullptr)
 {
-    using S = Smem32<LEARNED>;
+    using S = Smem32<KP, LEARNED>;
+    constexpr bool OWN = S::OWN;
     constexpr int NT = S::NT, TX = S::TX, TY = S::TY, NN = S::NN, HP = S::HP;
     const int tid = threadIdx.x;
 
@@ -111,7 +114,7 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
     const bool has = part < 3 && x0 + tx < g.nx && y0 + ty < g.ny;
     float2 fN = {1.0f, 0.0f}, fT = {1.0f, 0.0f}, fE = {0.0f, 0.0f};
     float ux = 0.0f, uy = 0.0f, G = 0.0f;
-    if (has) {
+    if (!OWN && has) {
         const long long o = (long long)(y0 + ty) * g.pitch + (x0 + tx);
         fN = fields.n[o];
         fT = fields.T[o];
@@ -122,8 +125,21 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
     }
     const bool inside = tmap != nullptr && x0 >= 4 && x0 + TX + 4 <= g.nx && y0 >= 3 && y0 + TY + 3 <= g.ny;
     if (inside) tma_issue(sm, tmap, x0, y0);
-    else load_region(sm, fs, g, x0, y0);
-    __syncthreads();
+    if constexpr (OWN) {
+        if (tid < OWN_THREADS) tile_moments(*own, nullptr, fs, status, g, t, x0, y0);
+        else if (!inside) load_region(sm, fs, g, x0, y0, OWN_THREADS);
+        __syncthreads();
+        if (has) {
+            fN = own->force.n[ty + 3][tx + 3];
+            fT = own->T[node];
+            ux = own->ux[node];
+            uy = own->uy[node];
+            if (part == 2) fE = own->E[node];
+        }
+    } else {
+        if (!inside) load_region(sm, fs, g, x0, y0);
+        __syncthreads();
+    }
 
     // ---- 2. equilibrium factors and the correction of their rounding
     if (part < 3) {
@@ -153,12 +169,14 @@ __device__ __forceinline__ bool stage_tile32(Smem32<LEARNED> &sm, const float *_
         } else {
             eq_correction(t, a, c, fN, fE, ux, uy, sm.corr[0][node], sm.corr[1][node], sm.corr[2][node]);
         }
-        if (part < 2) sm.G[part][node] = G;
+        if (!OWN && part < 2) sm.G[part][node] = G;
+    } else if (OWN && part < 5) {
+        sm.G[part - 3][node] = force_at32(own->force, g, cc, part - 3, tx, ty);
     }
     // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
     const bool left = x0 == 0 && g.wall_lo, right = x0 + TX + 3 >= g.nx && g.wall_hi;
     if (left || right) {
-        wall_flux<float, LEARNED>(sm, g, t, tw, net.theta, x0, 3 * NN, left, right);
+        wall_flux<float, LEARNED>(sm, g, t, tw, net.theta, x0, OWN ? 5 * NN : 3 * NN, left, right);
         __syncthreads();
         wall_ghosts<float>(sm, g, tw, x0, 0, left, right);
     }

@@ -56,18 +56,16 @@ struct __align__(16) ffp {
     }
 };
 
-// Tile of 8 x 8 nodes.  KP selects the threads: 5: 160, two nodes or lines a
-// thread; 8: 320, one; 4: 256, one, with learned weights (whose network needs the
-// registers).  Time of a stage, 160 and 320 threads: 64 x 4 (8 tiles) 26.7 and
-// 24.2 us, 1024 x 8 (128) 29.4 and 26.9, 192 x 128 (384) 37.8 and 38.0, 512^2
-// (4096) 233 and 247, 1024^2 868 and 931: grids of at most one tile an SM take 320.
+// Tile of 8 x 8 nodes.  KP selects the threads (stage_kind): 5: 160, two nodes or
+// lines a thread; 8: 512, one, which take the tile's moments and force too (OWN).
 template <int KP>
 struct Plan64 {
     using V = typename std::conditional<KP == 8, vf1, vf2>::type;
-    static constexpr int NT = KP == 5 ? 160 : KP == 8 ? 320 : 256;
+    static constexpr int NT = KP == 5 ? 160 : 512;
+    static constexpr bool OWN = KP == 8;
 };
 
-template <int KP, bool LEARNED>
+template <int KP>
 struct Smem64 : Staged<double> {
     static constexpr int NT = Plan64<KP>::NT;
     double ex[NQ][NN];  // n g_q(u_x, T) and g_q(u_y, T) of the tile nodes
@@ -75,18 +73,16 @@ struct Smem64 : Staged<double> {
     ffp G[2][NN / 2];   // c F
     // flux differences times 6 (weno5_flux6) across the nodes of each row along x
     // and column along y, of the 20 velocities that move along the axis (slot_x,
-    // slot_y; learned weights: first the network's corrections of the faces, one more
-    // than nodes, which the flux differences then replace); then, in place of one of a
-    // velocity's flux differences (inc), the sum of its advection and force
-    // terms.  Entry i of a column sits in half i / 4 of element i mod 4 (face 8:
-    // in element 4); the fifth element and the one at the end keep the banks of
-    // columns apart.
+    // slot_y); then, in place of one of a velocity's flux differences (inc), the sum of
+    // its advection and force terms.  Entry i of a column sits in half i / 4 of element i
+    // mod 4; the ninth element of a row, the fifth of a column and the one at the end
+    // keep the banks of rows and columns apart.
     ffp ax[20][TY / 2][TX + 1];
     ffp ay[20][TX * (TY / 2 + 1) + 1];
     ffp rest[NN / 2];
     int top;            // high word of the largest n of the tile (its scale)
 
-    __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i == 8 ? 4 : i & 3)]; }
+    __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i & 3)]; }
     __device__ __forceinline__ ffp &inc(int k1, int k2, int x, int y4)
     {
         return k1 != 2   ? ax[NQ * (k1 < 2 ? k1 : k1 - 1) + k2][y4][x]
@@ -124,20 +120,44 @@ __device__ __forceinline__ void dp_line(const FfTab &t, const ffv<V> f[NQ], ffv<
     }
 }
 
+// ---------------------------------------------------------------- equilibrium
+// g_q(u, T) (eq_factors) by the parity of the Hermite orders: 26 instead of 34
+// FP64 operations.
+__device__ __forceinline__ void eq_factors64(const Tab<double> &t, double u, double T, double g[NQ])
+{
+    const double th = T - 1.0, u2 = u * u;
+    const double c2 = 0.5 * (u2 + th);
+    const double c3 = u * fma(u2, 1.0 / 6.0, 0.5 * th);
+    const double c4 = fma(u2, fma(u2, 1.0 / 24.0, 0.25 * th), 0.125 * th * th);
+#pragma unroll
+    for (int m = 0; m <= 2; ++m) {
+        const int k = 2 + m;
+        const double even = fma(t.wHe[k][4], c4, fma(t.wHe[k][2], c2, t.wHe[k][0]));
+        if (m == 0) {
+            g[2] = even;
+        } else {
+            const double odd = fma(t.wHe[k][3], c3, t.wHe[k][1] * u);
+            g[2 + m] = even + odd;
+            g[2 - m] = even - odd;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- the stage of one tile
 // One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
 // call it.  fields: the moments and c F of fs (k_fields, k_force); tw: the table
-// of the wall entries; tmap: TMA maps of fs, or nullptr; net: the learned
-// network (LEARNED only).  A thread takes V::W nodes
+// of the wall entries; tmap: TMA maps of fs, or nullptr; own: KP 8's room for its own
+// fields.  A thread takes V::W nodes
 // (y and y + 4 of a column) or lines (rows or columns 4 apart) at a time.
 // Returns false when the TMA copy timed out (the CTA must stop).
-template <int KP, bool LEARNED>
-__device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const double *__restrict__ fs, const double *fn,
+template <int KP>
+__device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__restrict__ fs, const double *fn,
                                              double *out, int *__restrict__ status, const Geo &g, const Tab<double> &t,
-                                             const Tab<double> &tw, int x0, int y0, const StageK &c, const MlpArg &net,
-                                             const TmaMap *tmap, const StageFields<double> &fields)
+                                             const Tab<double> &tw, int x0, int y0, const StageK &c, const TmaMap *tmap,
+                                              const StageFields<double> &fields,
+                                             TileFields<double> *own = nullptr)
 {
-    using S = Smem64<KP, LEARNED>;
+    using S = Smem64<KP>;
     using V = typename Plan64<KP>::V;
     constexpr int W = V::W, NT = S::NT, TX = S::TX, TY = S::TY, NN = S::NN, NI = NN / W, HP = S::HP;
     const int tid = threadIdx.x;
@@ -145,11 +165,12 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
 
     // ---- 1. the fields of a node and axis (threads 0 .. 2 NN - 1), then the
     // populations: copies in flight during phase 2 for a tile inside the grid
+    constexpr bool OWN = Plan64<KP>::OWN;
     const int a = tid / NN, node = tid % NN, nx = node % TX, ny = node / TX;
     const bool has = tid < 2 * NN && x0 + nx < g.nx && y0 + ny < g.ny;
     double fn_ = 0.0, fu = 0.0, fT = 1.0;
     ff fG = {0.0f, 0.0f};
-    if (has) {
+    if (!OWN && has) {
         const long long o = (long long)(y0 + ny) * g.pitch + (x0 + nx);
         fn_ = fields.n[o];
         fu = a == 0 ? fields.ux[o] : fields.uy[o];
@@ -159,7 +180,20 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
     if (tid == 0) sm.top = 0;
     const bool inside = tmap != nullptr && x0 >= 4 && x0 + TX + 4 <= g.nx && y0 >= 3 && y0 + TY + 3 <= g.ny;
     if (inside) tma_issue(sm, tmap, x0, y0);
-    else load_region(sm, fs, g, x0, y0);
+    if constexpr (OWN) {
+        __syncthreads();
+        if (tid < OWN_THREADS) tile_moments(*own, &sm.top, fs, status, g, t, x0, y0);
+        else if (!inside) load_region(sm, fs, g, x0, y0, OWN_THREADS);
+        __syncthreads();
+        force_differences<NT>(own->force, ff_scale(sm.top));
+        if (has) {
+            fn_ = own->force.v[1][ny + 3][nx + 3];
+            fu = a == 0 ? own->ux[node] : own->uy[node];
+            fT = own->T[node];
+        }
+    } else if (!inside) {
+        load_region(sm, fs, g, x0, y0);
+    }
     __syncthreads();
 
     // ---- 2. equilibrium factors (FP64), the tile's scale (its largest density)
@@ -168,16 +202,21 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
         eq_factors64(t, fu, fT, w);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) (a == 0 ? sm.ex : sm.ey)[q][node] = a == 0 ? fn_ * w[q] : w[q];
-        ffp &G = sm.G[a][8 * (ny & 3) + nx];
-        G.h[ny >> 2] = fG.h;
-        G.l[ny >> 2] = fG.l;
-        const int hw = __double2hiint(fn_) & 0x7fffffff, top = __reduce_max_sync(0xffffffffu, hw < 0x7ff00000 ? hw : 0);
-        if ((tid & 31) == 0) atomicMax(&sm.top, top);
+        if constexpr (!OWN) {
+            ffp &G = sm.G[a][8 * (ny & 3) + nx];
+            G.h[ny >> 2] = fG.h;
+            G.l[ny >> 2] = fG.l;
+            const int hw = __double2hiint(fn_) & 0x7fffffff, top = __reduce_max_sync(0xffffffffu, hw < 0x7ff00000 ? hw : 0);
+            if ((tid & 31) == 0) atomicMax(&sm.top, top);
+        }
+    } else if (OWN && tid < 4 * NN) {
+        const ffv<vf1> v = force_at<vf1>(own->force, ff_scale(sm.top), c, a - 2, nx, ny);
+        sm.G[a - 2][8 * (ny & 3) + nx].put(ny >> 2, v);
     }
     // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
     const bool left = x0 == 0 && g.wall_lo, right = x0 + TX + 3 >= g.nx && g.wall_hi;
     if (left || right) {
-        wall_flux<double, LEARNED>(sm, g, t, tw, net.theta, x0, 2 * NN, left, right);
+        wall_flux<double, false>(sm, g, t, tw, nullptr, x0, OWN ? 4 * NN : 2 * NN, left, right);
         __syncthreads();
         wall_ghosts<double>(sm, g, tw, x0, 0, left, right);
     }
@@ -186,40 +225,6 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
     const FfScale sc = ff_scale(sm.top);
 
     // ---- 5a. flux differences, W rows or columns a thread
-    if constexpr (LEARNED) {
-        // the network's corrections of the faces it acts on, on whole warps: the x faces
-        // of the 20 velocities with xi_x != 0, then the y faces of the 20 with xi_y != 0
-        constexpr int nfx = (TX + 1) * TY, nfy = TX * (TY + 1), total = 20 * (nfx + nfy);
-        float *const scratch = net.tables + MLP_T64_SIZE + (tid >> 5) * MLP_WARP_SCRATCH;
-        for (int e = tid; e < (total + 31) / 32 * 32; e += NT) {
-            const int ee = e < total ? e : 0;
-            const bool along_x = ee < 20 * nfx;
-            const int e2 = along_x ? ee : ee - 20 * nfx, nf = along_x ? nfx : nfy, q = e2 / nf, f = e2 - q * nf;
-            const int k = line_velocity(along_x, q);
-            const int r = along_x ? f / (TX + 1) : f / TX, cc = along_x ? f - r * (TX + 1) : f - r * TX;
-            const bool valid = e < total && (along_x ? (y0 + r < g.ny && x0 + cc <= g.nx) : (x0 + cc < g.nx && y0 + r <= g.ny));
-            const bool up = along_x ? k / NQ > 2 : k % NQ > 2;
-            double d[4] = {0.0, 0.0, 0.0, 0.0};
-            if (valid) {
-                double v[5];
-#pragma unroll
-                for (int m = 0; m < 5; ++m)
-                    v[m] = along_x ? sm.mid[k][r][up ? cc + 1 + m : cc + 6 - m] : *sm.at(k, up ? r + m : r + 5 - m, 4 + cc);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) d[m] = v[m + 1] - v[m];
-            }
-            const float d4[4] = {(float)d[0], (float)d[1], (float)d[2], (float)d[3]};
-            const bool acts = learned_guard<double>(d[0], d[1], d[2], d[3]);
-            float x[MLP_IN], w[MLP_OUT];
-            learned_input_x(d4, acts, x);
-            if (__any_sync(0xffffffffu, acts)) mlp_weights_warp64(net.tables, x, w, scratch);
-            if (!valid) continue;
-            const float c = acts ? ff_split((double)learned_corr_from(w, d4), sc).h : no_network();
-            if (along_x) sm.ax[q][r & 3][cc].h[r >> 2] = c;
-            else sm.col(q, cc, r).h[r == 8 ? 0 : r >> 2] = c;
-        }
-        __syncthreads();
-    }
     for (int e = tid; e < 40 * (TX / W); e += NT) {
         const bool along_x = e < 20 * (TX / W);
         const int e2 = along_x ? e : e - 20 * (TX / W), q = e2 / (TX / W), i = e2 - q * (TX / W);
@@ -238,18 +243,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP, LEARNED> &sm, const doub
                 }
             }
         };
-        // (learned: the flux difference across a node takes the place of a face that it has used)
-        if constexpr (LEARNED)
-            weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store, [&](int j) {
-                const int at = up ? j : TX - j;
-                if (along_x) return sm.ax[q][i & 3][at].template get<V>(i >> 2).h;
-                float h[W];
-#pragma unroll
-                for (int w = 0; w < W; ++w) h[w] = sm.col(q, i + 4 * w, at).h[at == 8 ? 0 : at >> 2];
-                return V::of(h);
-            });
-        else
-            weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
+        weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
     }
     __syncthreads();
 

@@ -115,17 +115,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
     int *status = reinterpret_cast<int *>(fields + 7 * kMaxNodes);
     cudaStream_t s = (cudaStream_t)stream;
 
-    // shape, as olb_create picks it for FP64: 8 x 8 nodes with 5 velocity
-    // lanes, or 7 x 8 nodes with 8 lanes when that lowers the most nodes one
-    // SM advances (grids here have at most 256 tiles, a wave or two)
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1) {
-        cudaGetLastError();
-        return OLB_ERR_CUDA;
-    }
-    const long long tiles = (long long)((g.nx + 7) / 8) * ((g.ny + 7) / 8);
-    const int tx = 8, ty = 8, kp = tiles <= sms ? 8 : 5;
-    cudaError_t e = prepare_fused((double *)nullptr, tx, ty, kp, false);
+    cudaError_t e = prepare_fused((double *)nullptr, STAGE_TX, STAGE_TY, 5, false);
     // the scratch keeps the previous call's contents: the status word must start at zero
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
     const double dt = p->dt;
@@ -134,7 +124,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
     double *dst[3] = {f1, f2, f};
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k)
         for (int st = 0; st < 3 && e == cudaSuccess; ++st)
-            e = launch_fused(src[st], f, dst[st], status, g, tab, coef[st], tx, ty, kp, nullptr, nullptr, fields, s);
+            e = launch_fused(src[st], f, dst[st], status, g, tab, coef[st], nullptr, nullptr, fields, s);
     int hstatus = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, status, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

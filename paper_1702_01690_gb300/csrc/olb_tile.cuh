@@ -14,7 +14,7 @@ template <bool LEARNED>
 __device__ __forceinline__ double face_value(const float *mlp, double v0, double v1, double v2, double v3, double v4)
 {
     if constexpr (LEARNED)
-        return v2 + weno5_learned_corr64(mlp, v1 - v0, v2 - v1, v3 - v2, v4 - v3);
+        return weno5_learned(mlp, v0, v1, v2, v3, v4);
     else
     {
         auto high = [](double v) { return __double2hiint(v) & 0x7fffffff; };
@@ -172,13 +172,12 @@ __device__ __forceinline__ Line<real> line_of(const Staged<real> &sm, bool along
 // c): periodic sides wrap.  Ghost layers 0..2 of a specular side hold the
 // populations of the first three nodes inside with the normal velocity component
 // reversed (Sec. 3.4.1); diffuse-wall ghosts are set later; anything further out
-// is never read and holds 0.
+// is never read and holds 0.  By the threads from `first` on.
 template <typename real, typename S>
-__device__ __forceinline__ void load_region(S &sm, const real *__restrict__ fs, const Geo &g, int x0, int y0)
+__device__ __forceinline__ void load_region(S &sm, const real *__restrict__ fs, const Geo &g, int x0, int y0, int first = 0)
 {
     constexpr int HX = S::HX, HY = S::HY, NT = S::NT;
-    const int tid = threadIdx.x;
-    for (int e = tid; e < HY * HX; e += NT) {
+    for (int e = (int)threadIdx.x - first; e < HY * HX; e += NT - first) {
         const int r = e / HX, c = e - r * HX;
         if (!S::staged(r, c)) continue;
         real *dst = sm.at(0, r, c);
