@@ -1,5 +1,6 @@
 // olb_fields.cuh -- what a stage needs at a node besides its populations: the
-// moments (one thread per node), and in FP64 the force.
+// moments (k_fields, one thread per node) and the force (k_force); for grids of at
+// most one tile an SM both are taken by the stage's own CTAs (TileFields).
 #pragma once
 
 #include <type_traits>
@@ -8,7 +9,7 @@
 
 namespace olb {
 
-// n and Delta p of the region, kept for the 49-point stencils.  The stencils
+// n and Delta p as the 49-point stencils read them.  The stencils
 // cancel to O(ds^k) of their terms on fine grids, so the FP32 kernel keeps
 // each value as an unevaluated sum hi + lo of two floats (hi = the value
 // rounded to FP32, lo = the FP64 remainder rounded to FP32): differences of
@@ -22,15 +23,7 @@ struct FieldT<float> {
     using type = float2;
 };
 
-__device__ __forceinline__ double make_field(double v, double) { return v; }
-__device__ __forceinline__ float2 make_field(double v, float)
-{
-    const float hi = __double2float_rn(v);
-    return make_float2(hi, __double2float_rn(v - (double)hi));
-}
-__device__ __forceinline__ double field_diff(double a, double b) { return a - b; }
 __device__ __forceinline__ float field_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
-__device__ __forceinline__ double field_val(double a) { return a; }
 __device__ __forceinline__ float field_val(float2 a) { return a.x + a.y; }
 
 // ---------------------------------------------------------------- moments of a node

@@ -74,8 +74,7 @@ __device__ __forceinline__ double recip_nr1(double d)
 // Weights: wbar_q is proportional to delta_q / sigma_q^2.  Multiplying every
 // term by 10 (sigma_1 sigma_2 sigma_3)^2 gives weights proportional to
 // A_q = 10 delta_q (prod_{r != q} sigma_r)^2, which needs one reciprocal
-// (recip_nr1),
-// equals the table row for a single vanishing indicator, and is 0/0 only when
+// (recip_nr1), equals the table row for a single vanishing indicator, and is 0/0 only when
 // two or three vanish; those cases take Table tab:weno (the ideal weights of
 // the vanishing set).  If the products underflow without an exact zero the
 // min-scaled form delta_q (s/sigma_q)^2 is used instead.
@@ -112,6 +111,7 @@ __device__ __forceinline__ double weno5_core(double d01, double d12, double d23,
     }
     return fma(fma(A1, G1, fma(A2, G2, A3 * G3)), recip_nr1(6.0 * den), v2);
 }
+
 // FP32 populations: the correction c of an interface value (the value minus
 // its upwind node v2, sum_q wbar_q (Fhat^q - v2)) from the first differences
 // d01 = v1 - v0, ..., d34 = v4 - v3 of the stencil v0..v4 = f_{i-2} .. f_{i+2} in
@@ -129,8 +129,8 @@ __device__ __forceinline__ double weno5_core(double d01, double d12, double d23,
 // Table tab:weno).  The products of four squared indicators underflow in
 // single precision, so the weights are the min-scaled 10 delta_q (s/sigma_q)^2,
 // with Table tab:weno (the ideal weights of the vanishing set) when an
-// indicator vanishes.  q23 = d23^2, h12 = 2.5 d12^2, h23 = 2.5 d23^2: strips of
-// consecutive faces carry those values from face to face.
+// indicator vanishes.  q23 = d23^2, h12 = 2.5 d12^2, h23 = 2.5 d23^2: lines of
+// faces carry those values from face to face.
 __device__ __forceinline__ float weno5_core(float d01, float d12, float d23, float d34, float q23, float h12, float h23)
 {
     const float s1 = fmaf(d01, fmaf(-2.75f, d12, d01), h12);
@@ -153,18 +153,12 @@ __device__ __forceinline__ float weno5_core(float d01, float d12, float d23, flo
     }
     return fmaf(fmaf(w1, G1, fmaf(w2, G2, w3 * G3)), __fdividef(1.0f, 6.0f * (w1 + w2 + w3)), 0.0f);
 }
+
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ int wrap(int i, int n)
 {
     int r = i % n;
     return r < 0 ? r + n : r;
-}
-
-// Even extension of a field about both wall faces (Sec. 3.4.3): period 2 nx.
-__device__ __forceinline__ int reflect(int i, int n)
-{
-    int r = wrap(i, 2 * n);
-    return r >= n ? 2 * n - 1 - r : r;
 }
 
 // Equilibrium factors g_k(u, T), k = 0..4 (Eq. g_alpha with m = 1):
@@ -308,29 +302,6 @@ __device__ __forceinline__ float weno5_corr(float d01, float d12, float d23, flo
 {
     const float q12 = d12 * d12, q23 = d23 * d23;
     return weno5_core(d01, d12, d23, d34, q23, 2.5f * q12, 2.5f * q23);
-}
-
-// S consecutive faces along a row or column, in the upwind direction: the
-// stencil of face j is (ph, pl)[(j + m) step], m = 0..4, the corrections go to
-// out[j ostep].  Neighbouring faces share three first differences of the pairs
-// and one scaled square, which are carried instead of recomputed.
-template <int S>
-__device__ __forceinline__ void weno5_strip_c(const float *ph, const float *pl, int step, float *out, int ostep)
-{
-    float d01 = pdiff(ph[step], pl[step], ph[0], pl[0]);
-    float d12 = pdiff(ph[2 * step], pl[2 * step], ph[step], pl[step]);
-    float d23 = pdiff(ph[3 * step], pl[3 * step], ph[2 * step], pl[2 * step]);
-    float h12 = 2.5f * (d12 * d12);
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-        const float d34 = pdiff(ph[(j + 4) * step], pl[(j + 4) * step], ph[(j + 3) * step], pl[(j + 3) * step]);
-        const float q23 = d23 * d23, h23 = 2.5f * q23;
-        out[j * ostep] = weno5_core(d01, d12, d23, d34, q23, h12, h23);
-        d01 = d12;
-        d12 = d23;
-        d23 = d34;
-        h12 = h23;
-    }
 }
 
 // FP32: the symmetric part s_kappa = Ex[k1] gy[k2] of the equilibrium, as

@@ -129,6 +129,20 @@ __device__ __forceinline__ bool learned_guard(const double d[4], const float e[4
     return !zero && smin < MLP_GUARD * smax;
 }
 
+// An FP64 value rounded to FP32 (to even) on the integer pipe, by conversion (on the
+// FP64 pipe) where it is neither zero nor a normal FP32 number.
+static __device__ __noinline__ float f32_converted(double v) { return (float)v; }
+__device__ __forceinline__ float f32_rounded(double v)
+{
+    const int hw = __double2hiint(v), e = (hw >> 20) & 0x7ff;
+    const unsigned lw = (unsigned)__double2loint(v), sign = (unsigned)hw & 0x80000000u;
+    if (e > 1023 - 126 && e < 1023 + 127) {
+        const unsigned lr = lw + 0x0fffffffu + ((lw >> 29) & 1u);
+        return __uint_as_float((((unsigned)(hw & 0x7fffffff) - (896u << 20) + (lr < lw ? 1u : 0u)) << 3 | lr >> 29) | sign);
+    }
+    return ((unsigned)hw << 1 | lw) == 0 ? __uint_as_float(sign) : f32_converted(v);
+}
+
 // The network's input from the stencil's first differences in FP32: the
 // normalised stencil x = (v - mean) / (max - min), taken relative to v0
 // (shift invariant); all zero where the network does not act.
@@ -211,8 +225,8 @@ __device__ __forceinline__ float weno5_learned_corr(const float *__restrict__ th
 // fragment, so nothing goes through shared memory.
 //   FP64 populations: FP32 multiply-adds, the layers' outputs exchanged through
 // shared memory (mlp_weights' sums: the same results).
-// One stage of 1024^2 where the network acts on nearly every face: 5.0 -> 3.1 ms (FP32
-// populations) and 7.2 -> 4.95 ms (FP64), from a lane per stencil, whose weights came
+// One stage of 1024^2 where the network acts on nearly every face: 4.9 -> 3.1 ms (FP32
+// populations) and 6.84 -> 4.9 ms (FP64), from a lane per stencil, whose weights came
 // with 576 loads a face (FP64) and whose layer-1 outputs went through shared memory to
 // the fragments (FP32).  Bound by instruction issue and latency with the 16 warps that
 // 128 registers a thread leave an SM (ncu: FP32 issue 61 %, special functions 22 %,

@@ -9,10 +9,13 @@
 // olb_stage64.cuh (with which two runs of 100 steps of 308 x 4 nodes differed by 1.5e-8
 // of u, one of 44 x 188 by 4.5e-8).
 //
-// One stage of 1024^2 (with moments and force): 7.2 -> 4.95 ms.  The network takes most
-// of it (olb_mlp.cuh); the FP64 operations, some 1200 a node, run beside it on the two
-// tiles that an SM holds.  Faces that the network leaves to Jiang-Shu, a few in every
-// warp, gathered for whole warps: 5.14 -> 4.95 ms.
+// One stage of 1024^2 (with moments and force), the network acting on nearly every
+// face: 6.84 -> 4.9 ms; on few (a drop): 6.55 -> 5.6 ms.  The network takes most of the
+// first (olb_mlp.cuh), with the FP64 operations beside it on the two tiles that an SM
+// holds; the second is bound by the FP64 pipe, some 2500 operations a node.  Faces that
+// the network leaves to Jiang-Shu among others are gathered for whole warps (5.14 ->
+// 4.95 ms, noise); differences are rounded to FP32 on the integer pipe (drop 6.17 ->
+// 5.95 ms); a warp of Jiang-Shu faces only takes them at once (5.95 -> 5.6 ms).
 #pragma once
 
 #include "olb_tile.cuh"
@@ -155,21 +158,23 @@ __device__ __forceinline__ bool stage_tile64l(Smem64L<KP> &sm, const double *__r
     if (inside && !tma_finish(sm, status)) return false;
     __syncthreads();
 
-    // ---- 4. faces: those that the network acts on, whole warps; the others are
-    // collected and taken by whole warps then (a warp's FP64 instruction costs the same
-    // for one lane as for all)
+    // ---- 4. faces: those that the network acts on, whole warps; the others, unless they
+    // fill a warp, are collected and taken by whole warps then (a warp's FP64 instruction
+    // costs the same for one lane as for all)
     float *const scratch = net.tables + MLP_T64_SIZE + (tid >> 5) * MLP_WARP_SCRATCH;
     for (int e = tid; e < (S::FACES + 31) / 32 * 32; e += NT) {
         LearnedFace f{};
         const bool valid = e < S::FACES && learned_face(sm, g, x0, y0, e, f);
-        const float d[4] = {(float)f.d[0], (float)f.d[1], (float)f.d[2], (float)f.d[3]};
+        const float d[4] = {f32_rounded(f.d[0]), f32_rounded(f.d[1]), f32_rounded(f.d[2]), f32_rounded(f.d[3])};
         const bool acts = valid && learned_guard(f.d, d);
         float x[MLP_IN], w[MLP_OUT];
         learned_input_x(d, acts, x);
         if (__any_sync(0xffffffffu, acts)) mlp_weights_warp64(net.tables, x, w, scratch);
         if (acts) *f.at = f.v2 + (double)learned_corr_from(w, d);
         const unsigned rest = __ballot_sync(0xffffffffu, valid && !acts);
-        if (rest) {
+        if (rest == 0xffffffffu) {
+            *f.at = weno5_js(f.d, f.v2);
+        } else if (rest) {
             int first = 0;
             if ((tid & 31) == 0) first = atomicAdd(&sm.njs, __popc(rest));
             first = __shfl_sync(0xffffffffu, first, 0);
