@@ -535,22 +535,25 @@ __device__ __forceinline__ void force_block32(ForceSmem32<FORCE_X, FORCE_Y> &sm,
     const int x = threadIdx.x % FORCE_X, y = threadIdx.x / FORCE_X;
     if (x0 + x >= g.nx || y0 + y >= g.ny) return;
     const long long o = (long long)(y0 + y) * g.pitch + (x0 + x);
-#pragma unroll
-    for (int a = 0; a < 2; ++a) f.G[a][o] = force_at32(sm, g, cc, a, x, y);
+    f.G[0][o] = force_at32(sm, g, cc, 0, x, y);
+    // (one axis after the other, 64 registers: the compiler had mixed them in 114, k_force
+    // of 2048^2 0.18 ms)
+    asm volatile("" ::: "memory");
+    f.G[1][o] = force_at32(sm, g, cc, 1, x, y);
 }
 
 template <typename real>
 struct ForceOf {
     using Smem = ForceSmem<FORCE_X, FORCE_Y>;
-    static constexpr int NT = FORCE_THREADS;
+    static constexpr int NT = FORCE_THREADS, CTAS = 5;
 };
 template <>
 struct ForceOf<float> {
     using Smem = ForceSmem32<FORCE_X, FORCE_Y>;
-    static constexpr int NT = 2 * FORCE_THREADS;
+    static constexpr int NT = 2 * FORCE_THREADS, CTAS = 4;
 };
 template <typename real>
-__global__ void __launch_bounds__(ForceOf<real>::NT) k_force(StageFields<real> f, const __grid_constant__ Geo g,
+__global__ void __launch_bounds__(ForceOf<real>::NT, ForceOf<real>::CTAS) k_force(StageFields<real> f, const __grid_constant__ Geo g,
                                                              const __grid_constant__ StageK c, real cc)
 {
     __shared__ typename ForceOf<real>::Smem sm;
@@ -560,7 +563,7 @@ __global__ void __launch_bounds__(ForceOf<real>::NT) k_force(StageFields<real> f
 
 // the blocks of every run, in the order of force_start (prefix sum of their numbers)
 template <typename real>
-__global__ void __launch_bounds__(ForceOf<real>::NT) k_force_batch(char *fields, const BatchRun<real> *__restrict__ runs,
+__global__ void __launch_bounds__(ForceOf<real>::NT, ForceOf<real>::CTAS) k_force_batch(char *fields, const BatchRun<real> *__restrict__ runs,
                                                                    const int *__restrict__ force_start, int nruns, int st,
                                                                    real ccoef)
 {

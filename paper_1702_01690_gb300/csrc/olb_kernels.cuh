@@ -420,9 +420,21 @@ __device__ __forceinline__ NodeSums plain_sums(Get get)
             (sx[4] + sx[0]) + (sy[4] + sy[0]), (sx[3] + sx[1]) + (sy[3] + sy[1])};
 }
 
-// fixed(k): population k as a 64-bit integer in units of 2^-57 of 2^e.
+// v times 2^(unit - 1023) in FP64, rounded to even as a conversion rounds, on the
+// integer pipe (a conversion and a multiplication take twice 64 of its issue slots).
+__device__ __forceinline__ double fixed_value(long long v, int unit)
+{
+    const unsigned long long m = v < 0 ? -v : v;
+    const int z = __clzll(m);
+    const unsigned long long q = m << (z & 63), h = q >> 11;
+    const unsigned up = (((unsigned)q & 0x7ffu) + 0x3ffu + ((unsigned)h & 1u)) >> 11;
+    const unsigned long long b = ((unsigned long long)(unsigned)(unit + 62 - z) << 52) + h + up;
+    return m == 0 ? 0.0 : __longlong_as_double(v < 0 ? b | 0x8000000000000000ull : b);
+}
+
+// fixed(k): population k as a 64-bit integer in units of 2^(unit - 1023).
 template <typename Fixed>
-__device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, double unit)
+__device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, int unit)
 {
     long long sx[NQ], sy[NQ];
 #pragma unroll
@@ -435,7 +447,7 @@ __device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, double unit)
             sx[k1] += v;
             sy[k2] += v;
         }
-    auto val = [&](long long v) { return (double)v * unit; };
+    auto val = [&](long long v) { return fixed_value(v, unit); };
     return {val(sx[0] + sx[1] + sx[2] + sx[3] + sx[4]), val(sx[4] - sx[0]), val(sx[3] - sx[1]), val(sy[4] - sy[0]),
             val(sy[3] - sy[1]), val(sx[4] + sx[0] + sy[4] + sy[0]), val(sx[3] + sx[1] + sy[3] + sy[1])};
 }
@@ -451,7 +463,7 @@ __device__ __forceinline__ NodeSums node_sums64(Get get)
     for (int k = 0; k < NK; ++k) top = max(top, abs_hi(get(k)));
     if (top >= (2046 << 20) || top < (128 << 20)) return plain_sums(get);
     // 2^(e - 56), e the exponent of the largest
-    return fixed_sums([&](int k) { return to_fixed(get(k), top); }, __hiloint2double((top & 0x7ff00000) - (56 << 20), 0));
+    return fixed_sums([&](int k) { return to_fixed(get(k), top); }, (top >> 20) - 56);
 }
 template <typename Get>
 __device__ __forceinline__ NodeSums node_sums32(Get get)
@@ -469,7 +481,7 @@ __device__ __forceinline__ NodeSums node_sums32(Get get)
             const float2 v = get(k);
             return to_fixed(v.x, top) + to_fixed(v.y, top);
         },
-        __hiloint2double(((top >> 23) - 127 + 1023 - 56) << 20, 0));
+        (top >> 23) - 127 + 1023 - 56);
 }
 
 // Moments of the 25 populations at one node in FP64: n, jx, jy, e (FP32
