@@ -12,8 +12,8 @@ GPU, each with its own stage time and roofline fraction:
   batch_fp64/32 64 independent runs of uneven size (32^2 .. 1024^2, 13.5 M
                 nodes) in one launch per stage, autotuned shape
 A "step" is one full RK-3 step of the whole grid: three stages, each the
-per-node moments pre-pass and the fused stage kernel (force, WENO-5 fluxes,
-collision and RK combination), six launches in all.
+moments kernel, the force kernel and the stage kernel (WENO-5 fluxes, collision
+and RK combination), nine launches in all.
 
 Timing: W untimed warm-up steps, then K steps each bracketed by CUDA events
 on the context's stream, with a 256 MiB buffer written between steps (the
@@ -67,15 +67,15 @@ MLP_FLOPS = 2 * (5 * 32 + 32 * 32 + 32 * 3)
 # (50), stages 2 and 3 read f^n and f_s and write (75 each): 200 per step,
 # 8 bytes each in both paths (FP32 stores hi + lo pairs).
 VALUES_PER_NODE_STEP = 200
-# DRAM bytes (read + write) per stage launch from one ncu capture of exactly
+# DRAM bytes (read + write) per launch of the stage kernel from one ncu capture of
 # this kernel build, on the Laplace 2048^2 grid (4.19 M nodes; the 4096^2
 # grid is too large to capture), scaled by 4 to the 16.8 M nodes of the
 # 4096^2 grid (traffic grows with the node count).  Any other kernel or
 # workload reports null.
 DRAM_TRAFFIC_PER_LAUNCH = {
-    # 2048^2, stages 1, 2, 3: 1.820, 2.669, 2.658 GB (FP64) and 1.818, 2.668, 2.655 GB (FP32); mean x 4
-    ("phase", None, "k_fused<double,8,8,4>"): 4 * (1.820 + 2.669 + 2.658) / 3 * 1e9,
-    ("phase", None, "k_fused<float,8,8,5>"): 4 * (1.818 + 2.668 + 2.655) / 3 * 1e9,
+    # 2048^2, stages 1, 2, 3: 1.850, 2.700, 2.689 GB (FP64) and 1.817, 2.667, 2.655 GB (FP32); mean x 4
+    ("phase", None, "k_fused<double>"): 4 * (1.850 + 2.700 + 2.689) / 3 * 1e9,
+    ("phase", None, "k_fused<float>"): 4 * (1.817 + 2.667 + 2.655) / 3 * 1e9,
 }
 
 
@@ -338,9 +338,9 @@ def time_steps(ctx, steps, warmup, flush, stream):
 
 def timed_leg(olb, p, dev_fields, prec, steps, warmup, flush, stream, world, peak, weno=0, theta=None,
               clocks=None, mlp_acts=None):
-    """One timed leg: value, ms per step, stage time and roofline of the stage
-    kernel.  The step is exactly three launches of the stage kernel, so the
-    average launch takes a third of the timed step."""
+    """One timed leg: value, ms per step, stage time and roofline of a stage.  The
+    step is exactly three stages, so the average stage (its moments, force and
+    stage kernels) takes a third of the timed step."""
     import torch
     N = p.nx * p.ny
     ctx = olb.create(p, prec, stream, weno_mode=weno)
@@ -362,9 +362,8 @@ def timed_leg(olb, p, dev_fields, prec, steps, warmup, flush, stream, world, pea
     if mlp_acts is not None:
         flops += mlp_acts * MLP_FLOPS
     ach = flops / (stage_ms * 1e-3) / 1e12
-    tile = ctx.get_tile()
     kind = "double" if prec == olb.FP64 else "float"
-    kname = f"k_fused<{kind},{tile[0]},{tile[1]},{tile[2]}{',learned' if weno else ''}>"
+    kname = f"k_fused<{kind}{',learned' if weno else ''}>"
     prof = ctx.profile(3)
     leg = {"value": job_value(world, N, steps, total), "ms_per_step": ms_step,
            "roofline": {"kernel": kname, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
@@ -399,6 +398,8 @@ def run_ours(args, rank, world):
     roof["traffic"] = DRAM_TRAFFIC_PER_LAUNCH.get((args.workload, args.size, kname))
     roof["peak_source"] = (f"FP64 units x max SM clock: 2 DFMA/SM/clk x {sms} SMs x {mhz:.0f} MHz x 2 flop "
                            f"(no FP64 entry in MEASURED_PEAKS.json)")
+    roof["note"] = ("flops of the equations, counted once; the kernel takes most of them in float-float arithmetic on the "
+                    "FP32 pipe (several FP32 operations each), so the FP64 peak does not bound it")
     # mass and energy from the GPU's FP64 reduction after the timed steps
     # (the context is then at step warmup + steps + 3 profiled steps)
     tot_after = ctx.totals()
@@ -475,7 +476,7 @@ def run_ours(args, rank, world):
             "totals_fp64_gpu": {"mass_initial": tot0[0], "energy_initial": tot0[3],
                                 "mass_after_timed_steps": tot_after[0], "energy_after_timed_steps": tot_after[3],
                                 "mass_rel_change": float((tot_after[0] - tot0[0]) / tot0[0])},
-            "gpu_launches": 6 * args.steps, "clocks": clk.summary()}
+            "gpu_launches": 9 * args.steps, "clocks": clk.summary()}
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         line.update(oracle_leg(args, p, fields, dev_fields, theta, stream))
     if rank == 0:

@@ -127,8 +127,8 @@ int olb_set_allocator(olb_alloc_fn alloc, olb_free_fn release, void *user);
 
 /* Validate *p and create a context on the current CUDA device, using
  * `stream` (a cudaStream_t, or NULL for the legacy default stream) for all
- * its work.  Device memory (3 population buffers of 25 nx ny values and the
- * stage fields) is allocated here and nothing is launched.  Rejects
+ * its work.  Device memory (3 population buffers of 25 nx ny values, rows
+ * padded to 32 nodes, and the stage fields, 56 or 48 bytes a node) is allocated here and nothing is launched.  Rejects
  * nx, ny < 1, nx < 3 with walls, ds, dt, tau <= 0, sigma < 0, b < 0,
  * Tw <= 0 with walls, unknown enums (OLB_ERR_ARG) and
  * p_max dt / ds >= 1 or dt > 2.5 tau (OLB_ERR_CFL; CFL rule of Sec. 4.1,
@@ -208,30 +208,27 @@ int olb_set_populations(olb_ctx *ctx, const double *f);
 
 /* Per-kernel timing (not part of the paper; the tracing hook of the
  * library).  Runs nsteps >= 1 RK-3 steps on the context's stream as
- * individual launches of the stage kernel, each bracketed by CUDA events,
+ * individual launches of the three stages, each bracketed by CUDA events,
  * synchronises, and writes the mean device time in milliseconds of one
- * launch to ms[0] and the number of launches to launches[0] (either may be
+ * stage to ms[0] and the number of stages to launches[0] (either may be
  * NULL).  The populations advance exactly as with olb_step. */
 int olb_profile(olb_ctx *ctx, int nsteps, double *ms, int *launches);
 
 /* Shape of the stage kernel: tx x ty nodes per CTA, kp velocities advanced
- * at once (kp lanes of tx*ty threads, each rounded up to whole warps).
- * Compiled shapes (tx, ty, kp): (8,8,4), (16,8,2), (16,8,1), (32,8,1),
- * (32,16,1), (8,8,8), (7,8,8), (8,8,5); olb_create picks one from the
- * grid size ((8,8,5), FP64: or (8,8,8) on grids of at most one tile an SM;
- * (8,8,4) with learned weights).  With
- * OLB_WENO_LEARNED only (8,8,4), (16,8,2), (32,16,1).  Whatever the
- * shape, tiles are advanced as 8 x 8 nodes, in FP64 by 320 threads with kp = 8 and
- * by 160 otherwise.  olb_set_tile returns
- * OLB_ERR_ARG for any other shape; results do not depend on the shape.
- * Not part of the paper (a tuning knob). */
+ * at once.  Accepted shapes (tx, ty, kp): (8,8,4), (16,8,2), (16,8,1),
+ * (32,8,1), (32,16,1), (8,8,8), (7,8,8), (8,8,5); with OLB_WENO_LEARNED
+ * only (8,8,4), (16,8,2), (32,16,1).  olb_create sets (8,8,4) (FP64,
+ * learned weights) or (8,8,5).  Whatever the shape, grids are advanced as
+ * tiles of 8 x 8 nodes by the kernel that suits their number, and results
+ * do not depend on it.  olb_set_tile returns OLB_ERR_ARG for any other
+ * shape.  Not part of the paper. */
 int olb_set_tile(olb_ctx *ctx, int tx, int ty, int kp);
 int olb_get_tile(olb_ctx *ctx, int *tx, int *ty, int *kp);
 
 /* ------------------------------------------------------------------------
  * Batches: many independent runs (uneven grid sizes, each with its own
- * olb_params) advanced together, one launch per RK-3 stage with one CTA per
- * (run, tile) work item, replayed from CUDA graphs.  Not
+ * olb_params) advanced together, each kernel of an RK-3 stage in one launch,
+ * the stage kernel with one CTA per (run, tile) work item, replayed from CUDA graphs.  Not
  * part of the paper: it serves parameter sweeps (ds, T_w, drop radius) whose
  * single grids are too small to fill the GPU.  All runs must share the
  * precision.  Conventions as for single contexts; `run` indexes the array
@@ -267,8 +264,8 @@ int olb_batch_get_populations(olb_batch *b, int run, double *f);
 int olb_batch_set_tile(olb_batch *b, int tx, int ty, int kp);
 int olb_batch_get_tile(olb_batch *b, int *tx, int *ty, int *kp);
 
-/* Autotuner: times nsteps steps with every compiled shape (on a copy of the
- * state, which is restored), keeps the fastest and reports it; the choice is
+/* Autotuner: times nsteps steps with the compiled shape (on a copy of the
+ * state, which is restored), keeps it and reports it; the choice is
  * cached per process for the batch's precision, device and grid list. */
 int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, int *kp);
 

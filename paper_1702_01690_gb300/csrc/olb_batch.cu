@@ -1,14 +1,14 @@
-// olb_batch.cu -- many independent runs (uneven grids, own parameters) in one
-// launch per RK-3 stage (one CTA per tile of every run), replayed from CUDA
-// graphs, with an autotuner that times the compiled stage shapes.
+// olb_batch.cu -- many independent runs (uneven grids, own parameters), each kernel
+// of an RK-3 stage in one launch for all (the stage kernel with one CTA per tile of
+// every run), replayed from CUDA graphs.
 //
 // Device layout: the populations of all runs share three buffers (f^n, f^(1),
 // f^(2)); run r occupies 25 x ny_r x pitch_r values at offset off_r of each.
 // A descriptor per run (geometry, velocity and wall tables, offset, tiles per
 // row) and the prefix sum of tiles per run drive the stage kernel
 // (k_fused_batch in olb_fused.cuh); each run has its own status word.  Where
-// the tile shape suits TMA, each run also has a tensor map per buffer
-// ([3][count], in device memory): tiles inside a run are staged by one copy.
+// the tile shape suits TMA, each run also has its tensor maps per
+// buffer ([3][count], in device memory), with which tiles inside a run are staged.
 #include <cmath>
 #include <algorithm>
 #include <cstring>

@@ -2,11 +2,12 @@
 // model for a grid (k_fused) or a batch of grids (k_fused_batch), and their
 // launches.
 //
-// A stage is three launches.  k_fields computes the moments n, u, T, Delta p of f_s
+// A stage is three launches (one on small grids, see stage_kind).  k_fields computes the moments n, u, T, Delta p of f_s
 // once per node (Sec. 2.2, Eq. vdw), k_force the force F = grad(Delta p)/n + sigma
 // grad(Laplacian n) from the 49-point stencils (Eqs. F_def, stencil_grad,
 // stencil_glap; Sec. 3.4.3 at walls and mirror planes), both in olb_fields.cuh.
-// Then one CTA per tile of 8 x 8 nodes (olb_stage64.cuh, olb_stage32.cuh):
+// Then one CTA per tile of 8 x 8 nodes (olb_stage64.cuh, olb_stage32.cuh, FP64 with
+// learned weights olb_stage64l.cuh):
 //   1. stages the populations of the tile and three nodes around it in shared
 //      memory (olb_tile.cuh; TMA for tiles inside the grid);
 //   2. forms the equilibrium factors of its nodes (Eqs. feq, g_alpha);

@@ -369,8 +369,9 @@ __device__ __forceinline__ void eq_correction(const Tab<float> &t, const float E
 // addition takes the time of 64 FP32 or 32 integer instructions on a GB300.  A
 // population below 2^-4 of the largest is cut at 2^-57 of it, against 2^-54 that
 // one FP64 addition rounds away.  Measured on
-// 2048^2: the FP64 moments pre-pass 0.666 -> 0.384 ms; one FP64 step of 4096^2 with
-// its initial fields and moments 46.5 -> 40.2 ms, two FP32 steps 57.1 -> 52.1 ms.
+// 2048^2: the FP64 moments kernel 0.666 -> 0.384 ms, 0.276 with the sums converted to
+// FP64 on the integer pipe too (fixed_value); one FP64 step of 4096^2
+// with its initial fields and moments 46.5 -> 40.2 -> 38.7 ms.
 //
 // The sums that n, j and e = sum |p|^2 f are made of: n, sums and differences of
 // the rows and columns of velocity +-R_4 and +-R_3 (the middle root is 0).

@@ -16,7 +16,7 @@
 // instead of faces: 17 shared-memory loads a node and velocity less), the force
 // moved to its own kernel (with its 14 x 14 fields a tile), and rows of the staged
 // tile got a pitch of 20 floats (57 % of the shared-memory wavefronts were bank
-// conflicts); moments and force take 0.22 and 0.14 ms beside it.
+// conflicts); moments and force take 0.22 and 0.13 ms beside it.
 #pragma once
 
 #include "olb_tile.cuh"
@@ -92,8 +92,8 @@ __device__ __forceinline__ void weno5_line32(const Line<float> &ln, int lo_p1, i
 // One stage for the tile whose lower-left node is (x0, y0); all threads of the CTA
 // call it.  ca, cb, cc: the stage's coefficients of f^n, f_s and dt L (Eq. rk3);
 // ca_lo, cb_lo: their remainders (1/3 and 2/3 as double-float constants); tw: the
-// table of the wall entries; net: the learned network (LEARNED only); tmap: TMA maps of fs, or nullptr; fields: the moments and c F of
-// fs (k_fields, k_force).  Returns false when the TMA copy timed out (the CTA must
+// table of the wall entries; net: the learned network (LEARNED only); tmap: TMA maps of fs, or nullptr; fields: the moments
+// and c F of fs (k_fields, k_force); own: KP 8's room for its own fields.  Returns false when the TMA copy timed out (the CTA must
 // stop).
 template <int KP, bool LEARNED>
 __device__ __forceinline__ bool stage_tile32(Smem32<KP, LEARNED> &sm, const float *__restrict__ fs, const float *fn, float *out,

@@ -15,7 +15,8 @@
 // Measured, one step (three stages) of a 4096^2 grid: 106.6 ms with the force and
 // the node updates in FP64 (1070 FP64 instructions a node and stage beside 60
 // differences), 56.8 ms like this (228), 51.8 ms with three CTAs an SM, 46.5 ms
-// with the force in a kernel of its own (k_force) and two nodes a thread.
+// with the force in a kernel of its own (k_force) and two nodes a thread, 38.7 ms
+// with the moments' sums in fixed point (olb_kernels.cuh).
 // Against 80-bit arithmetic the populations are closer than the FP64 form's
 // (12 steps of a 167 x 109 drop: 5.7e-16 instead of 1.2e-15 of their norm, and
 // its loss of 1e-15 of the mass is gone): Delta is summed before the one
