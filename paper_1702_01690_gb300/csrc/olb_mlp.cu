@@ -316,8 +316,9 @@ extern "C" int olb_mlp_train(float *theta, const float *x, const float *g, const
     const int ctas = grad_ctas(std::min(batch, n));
     // the CTAs' gradients, then m, v and the per-epoch loss
     const size_t grads = (size_t)ctas * GRAD_STRIDE, state = 2 * MLP_P + epochs + 8;
+    // (from the stream's memory pool: cudaMalloc and cudaFree took 0.15 ms of a call)
     float *work = nullptr;
-    cudaError_t e = cudaMalloc((void **)&work, (grads + state) * sizeof(float));
+    cudaError_t e = cudaMallocAsync((void **)&work, (grads + state) * sizeof(float), s);
     if (e != cudaSuccess) return cuda_status(e);
     float *m = work + grads, *v = m + MLP_P, *lhist = v + MLP_P;
     e = cudaMemsetAsync(m, 0, state * sizeof(float), s);
@@ -339,7 +340,7 @@ extern "C" int olb_mlp_train(float *theta, const float *x, const float *g, const
     std::vector<float> h(epochs, 0.f);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), lhist, epochs * sizeof(float), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(work);
+    cudaFreeAsync(work, s);
     if (e != cudaSuccess) return cuda_status(e);
     if (loss_history)
         for (int ep = 0; ep < epochs; ++ep) loss_history[ep] = h[ep] / (float)nb;
