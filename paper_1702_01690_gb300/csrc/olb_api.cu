@@ -382,8 +382,9 @@ int olb::validate_params(const olb_params *p)
 static cudaError_t prepare_tile(olb_ctx *c)
 {
     const bool learned = c->p.weno_mode == OLB_WENO_LEARNED;
-    cudaError_t e = is_fp64(c) ? prepare_fused((double *)nullptr, c->tx, c->ty, c->kp, learned)
-                               : prepare_fused((float *)nullptr, c->tx, c->ty, c->kp, learned);
+    const int tiles = stage_tiles(c->geo.nx, c->geo.ny);
+    cudaError_t e = is_fp64(c) ? prepare_fused((double *)nullptr, c->tx, c->ty, c->kp, learned, tiles)
+                               : prepare_fused((float *)nullptr, c->tx, c->ty, c->kp, learned, tiles);
     if (e != cudaSuccess) return e;
     // TMA maps of the three buffers for this shape (tiles whose region lies
     // inside the grid then load it with one copy); without them every tile

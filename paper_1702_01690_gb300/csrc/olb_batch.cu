@@ -122,8 +122,10 @@ static cudaError_t batch_upload(olb_batch *b)
 
 static cudaError_t batch_prepare(olb_batch *b)
 {
-    return b_fp64(b) ? prepare_fused((double *)nullptr, b->tx, b->ty, b->kp, false)
-                     : prepare_fused((float *)nullptr, b->tx, b->ty, b->kp, false);
+    int tiles = 0;
+    for (const Geo &g : b->geo) tiles += stage_tiles(g.nx, g.ny);
+    return b_fp64(b) ? prepare_fused((double *)nullptr, b->tx, b->ty, b->kp, false, tiles)
+                     : prepare_fused((float *)nullptr, b->tx, b->ty, b->kp, false, tiles);
 }
 
 // The velocity tables (identical in every run's Tab; only the wall entries

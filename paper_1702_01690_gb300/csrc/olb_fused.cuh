@@ -229,11 +229,14 @@ cudaError_t fused_batch_launch_one(const real *fs, const real *fn, real *out, in
 
 // Compiled instances (stage_kind): KP 8 and 5, 6 and 4 with learned weights.
 #define OLB_DEFINE_FUSED(real)                                                                                \
-    cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned)                                   \
+    cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned, int tiles)                        \
     {                                                                                                         \
         if (learned && !learned_shape(tx, ty, kp)) return cudaErrorInvalidValue;                              \
-        const cudaError_t e = learned ? fused_prepare_one<real, 6, true>() : fused_prepare_one<real, 8>();    \
-        return e != cudaSuccess ? e : learned ? fused_prepare_one<real, 4, true>() : fused_prepare_one<real, 5>(); \
+        const int kind = stage_kind(learned, tiles);                                                          \
+        return kind == 4   ? fused_prepare_one<real, 4, true>()                                               \
+               : kind == 6 ? fused_prepare_one<real, 6, true>()                                               \
+               : kind == 8 ? fused_prepare_one<real, 8>()                                                     \
+                           : fused_prepare_one<real, 5>();                                                    \
     }                                                                                                         \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,            \
                              const Tab<real> &t, StageCoef c, const float *mlp, const TmaMap *tma,            \

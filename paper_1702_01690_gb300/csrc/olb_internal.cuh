@@ -157,7 +157,7 @@ StageK stage_constants(const Geo &g, StageCoef c);
 // runs the per-node moments pre-pass into fields (a buffer of fields_bytes(g)),
 // then the stage kernel, which reads them.
 #define OLB_DECLARE_LAUNCHERS(real)                                                                    \
-    cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned);                           \
+    cudaError_t prepare_fused(real *, int tx, int ty, int kp, bool learned, int tiles);                \
     cudaError_t launch_fused(const real *fs, const real *fn, real *out, int *status, const Geo &g,     \
                              const Tab<real> &t, StageCoef c, const float *mlp,                        \
                              const TmaMap *tma, void *fields, cudaStream_t s);                         \

@@ -115,7 +115,7 @@ extern "C" int olb_step_static(const olb_params *p, void *stream, double *f, int
     int *status = reinterpret_cast<int *>(fields + 7 * kMaxNodes);
     cudaStream_t s = (cudaStream_t)stream;
 
-    cudaError_t e = prepare_fused((double *)nullptr, STAGE_TX, STAGE_TY, 5, false);
+    cudaError_t e = prepare_fused((double *)nullptr, STAGE_TX, STAGE_TY, 5, false, stage_tiles(g.nx, g.ny));
     // the scratch keeps the previous call's contents: the status word must start at zero
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
     const double dt = p->dt;
