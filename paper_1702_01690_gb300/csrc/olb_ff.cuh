@@ -134,15 +134,17 @@ __host__ __device__ __forceinline__ ff ff_split(double d, FfScale s)
     return {f32_make(h), f32_of((int)(lw << 3)) * f32_make(unit | sign)};
 }
 // A scaled float as FP64, scale undone (FP64's smallest normal number where it
-// would be less); l: a low part, whose high part carries an infinity or NaN.
-__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s, bool l)
+// would be less, no number where v is none).
+__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s)
 {
     const unsigned b = f32_bits(v);
     const int a = (int)(b & 0x7fffffffu), least = (max(s.off, 0) + (1 << 20)) << 3;
     const int m = max(a, least), hw = (m >> 3) - s.off;
-    return f64_make(!l && a >= 0x7f800000 ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
+    return f64_make(a >= 0x7f800000 ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
 }
-__host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s) { return ff_widen(v.h, s, false) + ff_widen(v.l, s, true); }
+// (either part can leave FP32's range alone: where an indicator overflows, its
+// weight's high part is zero and only the low part is no number)
+__host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s) { return ff_widen(v.h, s) + ff_widen(v.l, s); }
 
 // ---------------------------------------------------------------- one or two floats
 // The arithmetic below is written for a vector V of one float or of two (the
