@@ -10,9 +10,12 @@
 //
 // Accuracy, relative to the largest difference of the stencil, against 113-bit
 // arithmetic on 2e5 stencils each of noise, sines of 16 to 3000 nodes a wave and
-// tanh profiles: rms 2^-46.3 to 2^-49.9, at most 2^-42.0.  The FP64 form it took
-// the place of normalised its weights with a reciprocal good to 2^-39.9 (rms
-// 2^-41 to 2^-42.6), so faces are more accurate than they were.
+// tanh profiles: rms 2^-46.3 to 2^-49.9, the largest 2^-42.0 (of 4e5 of noise 2^-41.6).
+// The FP64 form it took the place of normalised its weights with a reciprocal good to
+// 2^-39.9 (rms 2^-41 to 2^-42.6), so faces are more accurate than they were.  But its
+// errors were those of the face's own candidates; here a face behind a jump of one
+// node, whose weights leave the jump out, still carries 2^-47 of it: two nodes beyond a
+// jump of more than 2^46 times their density the first stage of a step is rounding.
 //
 // Measured on a 4096^2 grid (one step, three stages): 236.1 ms with 30 FP64
 // operations a face, 106.6 ms with 1.3 differences and 3 more a face (the force
@@ -93,7 +96,9 @@ __host__ __device__ __forceinline__ float rcp_seed(float v)
 // Values are scaled by a power of two that puts the largest density of a tile
 // at 2^45: a tile's differences, from 2^-66 of it (an ulp of a population 2^-13
 // of it) to 2^18 times it, then have squares and weights inside FP32's range
-// whatever the populations' units.
+// whatever the populations' units.  Where they lie beyond (dilute nodes beside dense
+// ones of the next tile) the low parts are not finite, and the stage takes the tile's
+// lines again with the scale of its largest population (stage_tile64).
 constexpr int FF_EXP = 127 + 45;  // FP32 exponent field of the largest density
 struct FfScale {
     int off;     // added to an FP64 high word: exponent field e - emax + FF_EXP
@@ -134,17 +139,21 @@ __host__ __device__ __forceinline__ ff ff_split(double d, FfScale s)
     return {f32_make(h), f32_of((int)(lw << 3)) * f32_make(unit | sign)};
 }
 // A scaled float as FP64, scale undone (FP64's smallest normal number where it
-// would be less, no number where v is none).
-__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s)
+// would be less); l: a low part, whose high part is no number where it is none.
+__host__ __device__ __forceinline__ double ff_widen(float v, FfScale s, bool l)
 {
     const unsigned b = f32_bits(v);
     const int a = (int)(b & 0x7fffffffu), least = (max(s.off, 0) + (1 << 20)) << 3;
     const int m = max(a, least), hw = (m >> 3) - s.off;
-    return f64_make(a >= 0x7f800000 ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
+    return f64_make(!l && a >= 0x7f800000 ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
 }
 // (either part can leave FP32's range alone: where an indicator overflows, its
-// weight's high part is zero and only the low part is no number)
-__host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s) { return ff_widen(v.h, s) + ff_widen(v.l, s); }
+// weight's high part is zero and only the low part is no number, which the high
+// part takes on here)
+__host__ __device__ __forceinline__ double ff_widen(ff v, FfScale s)
+{
+    return ff_widen(fmaf(0.0f, v.l, v.h), s, false) + ff_widen(v.l, s, true);
+}
 
 // ---------------------------------------------------------------- one or two floats
 // The arithmetic below is written for a vector V of one float or of two (the

@@ -81,9 +81,20 @@ struct Smem64 : Staged<double> {
     ffp ax[20][TY / 2][TX + 1];
     ffp ay[20][TX * (TY / 2 + 1) + 1];
     ffp rest[NN / 2];
-    int top;            // high word of the largest n of the tile (its scale)
+    int top;            // high word of the largest n of the tile (its scale), or of the largest population
 
     __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i & 3)]; }
+    // top is at least the largest finite staged population, wall ghosts included (all threads)
+    __device__ __noinline__ void raise_top(int tid)
+    {
+        int a = 0;
+        for (int e = tid; e < P * HY * (TX + 6); e += NT) {
+            const int k = e / (HY * (TX + 6)), r = e / (TX + 6) % HY, c = 1 + e % (TX + 6);
+            const int v = staged(r, c) ? __double2hiint(*at(k, r, c)) & 0x7fffffff : 0;
+            a = max(a, v < 0x7ff00000 ? v : 0);
+        }
+        atomicMax(&top, a);
+    }
     __device__ __forceinline__ ffp &inc(int k1, int k2, int x, int y4)
     {
         return k1 != 2   ? ax[NQ * (k1 < 2 ? k1 : k1 - 1) + k2][y4][x]
@@ -223,30 +234,42 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
     }
     if (inside && !tma_finish(sm, status)) return false;
     __syncthreads();
-    const FfScale sc = ff_scale(sm.top);
+    FfScale sc = ff_scale(sm.top);
 
-    // ---- 5a. flux differences, W rows or columns a thread
-    for (int e = tid; e < 40 * (TX / W); e += NT) {
-        const bool along_x = e < 20 * (TX / W);
-        const int e2 = along_x ? e : e - 20 * (TX / W), q = e2 / (TX / W), i = e2 - q * (TX / W);
-        const Line<double> ln = line_of<double>(sm, along_x, q, i);
-        const bool up = ln.up;
-        auto store = [&](int j, ffv<V> v) {
-            const int at = up ? j : TX - 1 - j;
-            if (along_x) {
-                sm.ax[q][i & 3][at].put(i >> 2, v);
-            } else {
+    // ---- 5a. flux differences, W rows or columns a thread; once more with the scale of
+    // the largest population if some were beyond FP32's range (in-range tiles pay one
+    // packed FMA a flux difference for it)
+    for (bool again = false;; again = true) {
+        V sum = V::all(0.0f);  // of 0 times the low parts: not 0 if one is not finite
+        for (int e = tid; e < 40 * (TX / W); e += NT) {
+            const bool along_x = e < 20 * (TX / W);
+            const int e2 = along_x ? e : e - 20 * (TX / W), q = e2 / (TX / W), i = e2 - q * (TX / W);
+            const Line<double> ln = line_of<double>(sm, along_x, q, i);
+            const bool up = ln.up;
+            auto store = [&](int j, ffv<V> v) {
+                const int at = up ? j : TX - 1 - j;
+                sum = vfma(0.0f, v.l, sum);
+                if (along_x) {
+                    sm.ax[q][i & 3][at].put(i >> 2, v);
+                } else {
 #pragma unroll
-                for (int w = 0; w < W; ++w) {
-                    ffp &o = sm.col(q, i + 4 * w, at);
-                    o.h[at >> 2] = v.h[w];
-                    o.l[at >> 2] = v.l[w];
+                    for (int w = 0; w < W; ++w) {
+                        ffp &o = sm.col(q, i + 4 * w, at);
+                        o.h[at >> 2] = v.h[w];
+                        o.l[at >> 2] = v.l[w];
+                    }
                 }
-            }
-        };
-        weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
+            };
+            weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
+        }
+        if (!__syncthreads_or(!(sum[0] == 0.0f && sum[W - 1] == 0.0f)) || again) break;
+        const int top = sm.top;
+        __syncthreads();
+        sm.raise_top(tid);
+        __syncthreads();
+        if (sm.top == top) break;  // (infinities or NaN among the populations)
+        sc = ff_scale(sm.top);
     }
-    __syncthreads();
 
     // f^n of the velocities that this thread advances in 5c, fetched now
     constexpr int LINES = (NQ * NI + NT - 1) / NT;
