@@ -135,7 +135,7 @@ StageK stage_constants(const Geo &g, StageCoef c)
     k.cit = ff_of(c.cc * g.inv_tau);
     k.ca = ff_of(c.ca);
     k.kp = ff_of(c.cc * g.inv_ds / 5040.0);
-    k.kn = ff_of(c.cc * g.sigma * g.inv_ds3 / 2160.0);
+    k.kn = ff_of(std::frexp(c.cc * g.sigma * g.inv_ds3 / 2160.0, &k.kn_exp));
     for (int m = 0; m < 3; ++m) k.adv[m] = ff_of(c.cc * g.inv_ds * h.R[2 + m] / 6.0);
     return k;
 }

@@ -413,8 +413,8 @@ __device__ __forceinline__ ffv<V> force_at(const ForceSmem<FX, FY> &sm, FfScale 
     const ffv<V> n = ff_split<V>(nd, sc);
     const V r = rcp_seed(n.h);
     const ffv<V> inv = {r, r * vfma(-r, n.l, vfma(-r, n.h, V::all(1.0f)))};
-    // sum_n in the populations' units is 2^k of the scaled one
-    const int k = 127 - 1023 - (sc.off >> 20), k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
+    // kn sum_n is 2^k of the product of its scaled parts
+    const int k = c.kn_exp + 127 - 1023 - (sc.off >> 20), k1 = max(-126, min(127, k)), k2 = max(-126, min(127, k - k1));
     const float u1 = f32_make((unsigned)(k1 + 127) << 23), u2 = f32_make((unsigned)(k2 + 127) << 23);
     const float *d = a == 0 ? &sm.dx[0][0][0][y + 3][x] : &sm.dy[0][0][0][y][x + 3];
     constexpr int NX = 3 * HY * FX, NY = 3 * FY * HX;

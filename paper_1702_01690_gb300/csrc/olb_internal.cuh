@@ -58,7 +58,8 @@ struct FfTab {
 struct StageK {
     ff cit;     // c / tau, c the coefficient of dt L
     ff ca;      // the coefficient of f^n (cb = 1 - ca)
-    ff kp, kn;  // c / (5040 ds), c sigma / (2160 ds^3)
+    ff kp, kn;  // c / (5040 ds), c sigma / (2160 ds^3) / 2^kn_exp (one over a density: beyond FP32's
+    int kn_exp; // range in many units, so its binary exponent is kept beside it)
     ff adv[3];  // c |xi| / (6 ds), |xi| the roots 2, 3, 4
 };
 template <typename real>

@@ -93,3 +93,21 @@ def test_populations_far_above_their_density(olb, nx, ny):
     o.set_populations(f)
     o.step(1)
     assert np.max(np.abs(_stepped(olb, p, f, 1) - o.get_populations())) <= 3 * 40 * EPS * np.max(np.abs(f))
+
+
+def _noisy(p, seed=3):
+    rng = np.random.default_rng(seed)
+    n, u, v, T = rng.uniform(-1, 1, (4, p.ny, p.nx))
+    return 1.0 + 0.3 * n, 0.1 * u, 0.1 * v, 1.0 + 0.1 * T
+
+
+@pytest.mark.parametrize("shift", [-101, -64, 64, 101, 125])
+@pytest.mark.parametrize("nx,ny", [SMALL, LARGE])
+def test_units_of_density(olb, nx, ny, shift):
+    """The step with n, 1/a, 1/b and 1/sigma in another unit, a power of two: the same bits, capillary term included."""
+    p = _ideal(nx, ny, a=9.0 / 8.0, b=1.0 / 3.0, sigma=1e-4)
+    q = _ideal(nx, ny, a=np.ldexp(9.0 / 8.0, -shift), b=np.ldexp(1.0 / 3.0, -shift), sigma=np.ldexp(1e-4, -shift))
+    f = _populations(olb, p, _noisy(p))
+    one, other = _stepped(olb, p, f, 2), _stepped(olb, q, np.ldexp(f, shift), 2)
+    assert np.isfinite(one).all()
+    assert np.array_equal(np.ldexp(other, -shift), one)
