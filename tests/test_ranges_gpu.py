@@ -111,3 +111,13 @@ def test_units_of_density(olb, nx, ny, shift):
     one, other = _stepped(olb, p, f, 2), _stepped(olb, q, np.ldexp(f, shift), 2)
     assert np.isfinite(one).all()
     assert np.array_equal(np.ldexp(other, -shift), one)
+
+
+@pytest.mark.parametrize("shift", [900, 950, 1000, 1020])
+@pytest.mark.parametrize("nx,ny", [SMALL, LARGE])
+def test_largest_densities(olb, nx, ny, shift):
+    """An ideal gas up to the end of FP64's range: the same bits."""
+    p = _ideal(nx, ny)
+    f = _populations(olb, p, _noisy(p))
+    one, other = _stepped(olb, p, f, 1), _stepped(olb, p, np.ldexp(f, shift), 1)
+    assert np.array_equal(np.ldexp(other, -shift), one)
