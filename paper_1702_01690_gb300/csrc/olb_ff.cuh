@@ -102,7 +102,7 @@ __host__ __device__ __forceinline__ float rcp_seed(float v)
 constexpr int FF_EXP = 127 + 45;  // FP32 exponent field of the largest density
 struct FfScale {
     int off;     // added to an FP64 high word: exponent field e - emax + FF_EXP
-    int inf;     // bits of the first scaled float that is beyond FP64 or no number
+    float inf;   // the first scaled value that is beyond FP64 or FP32
     int lo, hi;  // high words of the smallest value that is kept (2^-60 scaled: smaller ones
                  // and zero become it, far below every rounding) and of the first beyond FP32
 };
@@ -112,7 +112,7 @@ __host__ __device__ __forceinline__ FfScale ff_scale(int top)
     const int off = (FF_EXP << 20) - (top & 0x7ff00000);
     // (densities above 2^941 leave no room beyond FP32: an infinity is then taken as 2^1024)
     const int least = (255 << 20) - 0x7ff00000;
-    return {off, (0x7ff00000 + min(off, least)) << 3, max((67 << 20) - off, 1 << 20), (255 << 20) - max(off, least)};
+    return {off, f32_make((unsigned)(0x7ff00000 + min(off, least)) << 3), max((67 << 20) - off, 1 << 20), (255 << 20) - max(off, least)};
 }
 // An int as a float (rounded).
 __host__ __device__ __forceinline__ float f32_of(int v)
@@ -149,7 +149,7 @@ __host__ __device__ __forceinline__ double ff_widen(float v, FfScale s, bool l)
     const unsigned b = f32_bits(v);
     const int a = (int)(b & 0x7fffffffu), least = (max(s.off, 0) + (1 << 20)) << 3;
     const int m = max(a, least), hw = (m >> 3) - s.off;
-    return f64_make(!l && a >= s.inf ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
+    return f64_make(!l && !(fabsf(v) < s.inf) ? 0x7ff80000 : (int)((unsigned)hw | (b & 0x80000000u)), m << 29);
 }
 // (either part can leave FP32's range alone: where an indicator overflows, its
 // weight's high part is zero and only the low part is no number, which the high

@@ -430,7 +430,8 @@ __device__ __forceinline__ double fixed_value(long long v, int unit)
     const unsigned long long q = m << (z & 63), h = q >> 11;
     const unsigned up = (((unsigned)q & 0x7ffu) + 0x3ffu + ((unsigned)h & 1u)) >> 11;
     const unsigned long long b = ((unsigned long long)(unsigned)(unit + 62 - z) << 52) + h + up;
-    return m == 0 ? 0.0 : __longlong_as_double(v < 0 ? b | 0x8000000000000000ull : b);
+    const unsigned hw = min((unsigned)(b >> 32), 0x7ff00000u);  // (not finite where it is beyond FP64)
+    return m == 0 ? 0.0 : __hiloint2double((int)(v < 0 ? hw | 0x80000000u : hw), (int)(unsigned)b);
 }
 
 // fixed(k): population k as a 64-bit integer in units of 2^(unit - 1023).
@@ -453,26 +454,16 @@ __device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, int unit)
             val(sy[3] - sy[1]), val(sx[4] + sx[0] + sy[4] + sy[0]), val(sx[3] + sx[1] + sy[3] + sy[1])};
 }
 
-// Near the ends of the range: infinities, NaN and the smallest in FP64; the largest,
-// whose sums may be beyond FP64, in a smaller unit.
-template <typename Get>
-__device__ __noinline__ NodeSums far_sums(Get get, int top)
-{
-    if (top >= (2047 << 20) || top < (128 << 20)) return plain_sums(get);
-    NodeSums s = fixed_sums([&](int k) { return to_fixed(get(k), top); }, (top >> 20) - 56 - 16);
-    for (double *v : {&s.n, &s.a4x, &s.a3x, &s.a4y, &s.a3y, &s.s4, &s.s3}) *v *= 65536.0;
-    return s;
-}
-
 // The sums of a node's populations, get(k) giving population k (FP64) or its hi
-// and lo parts (FP32).
+// and lo parts (FP32).  Infinities, NaN and populations near the lower end of the range
+// are summed in FP64.
 template <typename Get>
 __device__ __forceinline__ NodeSums node_sums64(Get get)
 {
     int top = 0;
 #pragma unroll
     for (int k = 0; k < NK; ++k) top = max(top, abs_hi(get(k)));
-    if (top >= (2040 << 20) || top < (128 << 20)) return far_sums(get, top);
+    if (top >= (2047 << 20) || top < (128 << 20)) return plain_sums(get);
     // 2^(e - 56), e the exponent of the largest
     return fixed_sums([&](int k) { return to_fixed(get(k), top); }, (top >> 20) - 56);
 }

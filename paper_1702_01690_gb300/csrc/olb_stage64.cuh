@@ -271,6 +271,9 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
         sc = ff_scale(sm.top);
     }
 
+    // (once more, not kept: 5a's registers)
+    sc = ff_scale(*(volatile int *)&sm.top);
+
     // f^n of the velocities that this thread advances in 5c, fetched now
     constexpr int LINES = (NQ * NI + NT - 1) / NT;
     double f0[LINES][NQ][W];
