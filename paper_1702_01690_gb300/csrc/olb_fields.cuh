@@ -554,11 +554,13 @@ struct ForceOf<float> {
 };
 template <typename real>
 __global__ void __launch_bounds__(ForceOf<real>::NT, ForceOf<real>::CTAS) k_force(StageFields<real> f, const __grid_constant__ Geo g,
-                                                             const __grid_constant__ StageK c, real cc)
+                                                             const __grid_constant__ StageK c, real cc,
+                                                             int row0)
 {
     __shared__ typename ForceOf<real>::Smem sm;
-    if constexpr (sizeof(real) == 8) force_block(sm, f, g, c, blockIdx.x * FORCE_X, blockIdx.y * FORCE_Y);
-    else force_block32(sm, f, g, cc, blockIdx.x * FORCE_X, blockIdx.y * FORCE_Y);
+    const int x0 = blockIdx.x * FORCE_X, y0 = (row0 + blockIdx.y) * FORCE_Y;
+    if constexpr (sizeof(real) == 8) force_block(sm, f, g, c, x0, y0);
+    else force_block32(sm, f, g, cc, x0, y0);
 }
 
 // the blocks of every run, in the order of force_start (prefix sum of their numbers)

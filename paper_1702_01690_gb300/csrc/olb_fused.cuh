@@ -92,7 +92,7 @@ __global__ void __launch_bounds__((stage_threads<real, KP, LEARNED>()),
 k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict__ status,
         const __grid_constant__ Geo g, const __grid_constant__ Tab<real> t, real ca, real cb, real cc, real ca_lo,
         real cb_lo, const __grid_constant__ StageK sk, const float *__restrict__ mlp, const __grid_constant__ TmaArg tma,
-        const __grid_constant__ StageFields<real> fields)
+        const __grid_constant__ StageFields<real> fields, int row0)
 {
     // 128-byte aligned: the TMA copy of phase 1 lands at offset 0
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -104,7 +104,9 @@ k_fused(const real *__restrict__ fs, const real *fn, real *out, int *__restrict_
     }
     TileFields<real> *own = KP == 8 ? reinterpret_cast<TileFields<real> *>(smem_raw + own_offset<real>()) : nullptr;
     const TmaMap *tm = tma.on ? &tma.map : nullptr;
-    const int x0 = blockIdx.x * 8, y0 = blockIdx.y * 8;
+    const int x0 = blockIdx.x * 8;
+    // (masked: not negative as the compiler sees it; 0.8 % of a stage of 2048^2 otherwise)
+    const int y0 = (int)(((unsigned)row0 & 0x0fffffffu) + blockIdx.y) * 8;
     if constexpr (sizeof(real) == 8 && LEARNED)
         stage_tile64l<KP>(sm, fs, fn, out, status, g, t, x0, y0, ca, cb, cc, net, tm, fields);
     else if constexpr (sizeof(real) == 8)
@@ -173,12 +175,19 @@ cudaError_t fused_prepare_one()
     return e;
 }
 
+// A launch has at most 65535 blocks along y: launch(first row of blocks, rows) for each
+// so many.
+template <typename Launch>
+void for_rows(int rows, Launch launch)
+{
+    for (int row0 = 0; row0 < rows; row0 += 65535) launch(row0, rows - row0 < 65535 ? rows - row0 : 65535);
+}
+
 template <typename real, int KP, bool LEARNED = false>
 cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *status, const Geo &g,
                              const Tab<real> &t, StageCoef c, const float *mlp, const TmaMap *tmap, void *fields,
                              cudaStream_t s)
 {
-    dim3 grid((g.nx + 7) / 8, (g.ny + 7) / 8);
     TmaArg tma{};
     if (tmap) {
         tma.map = *tmap;
@@ -191,13 +200,18 @@ cudaError_t fused_launch_one(const real *fs, const real *fn, real *out, int *sta
         const long long N = (long long)g.nx * g.ny;
         constexpr bool SEQ = LEARNED && sizeof(real) == 8;
         k_fields<real, SEQ><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(fs, fl, status, g, t);
-        const dim3 blocks((g.nx + FORCE_X - 1) / FORCE_X, (g.ny + FORCE_Y - 1) / FORCE_Y);
-        if constexpr (SEQ) k_force_learned<real><<<blocks, 2 * FORCE_THREADS, 0, s>>>(fl, g, c.cc);
-        else k_force<real><<<blocks, ForceOf<real>::NT, 0, s>>>(fl, g, sk, (real)c.cc);
+        for_rows((g.ny + FORCE_Y - 1) / FORCE_Y, [&](int row0, int rows) {
+            const dim3 blocks((g.nx + FORCE_X - 1) / FORCE_X, rows);
+            if constexpr (SEQ) k_force_learned<real><<<blocks, 2 * FORCE_THREADS, 0, s>>>(fl, g, c.cc, row0);
+            else k_force<real><<<blocks, ForceOf<real>::NT, 0, s>>>(fl, g, sk, (real)c.cc, row0);
+        });
     }
-    k_fused<real, KP, LEARNED><<<grid, stage_threads<real, KP, LEARNED>(), fused_smem_bytes<real, KP, LEARNED>(), s>>>(
-        fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
-        (real)(c.cb - (double)(real)c.cb), sk, mlp, tma, fl);
+    for_rows((g.ny + 7) / 8, [&](int row0, int rows) {
+        k_fused<real, KP, LEARNED><<<dim3((g.nx + 7) / 8, rows), stage_threads<real, KP, LEARNED>(),
+                                     fused_smem_bytes<real, KP, LEARNED>(), s>>>(
+            fs, fn, out, status, g, t, (real)c.ca, (real)c.cb, (real)c.cc, (real)(c.ca - (double)(real)c.ca),
+            (real)(c.cb - (double)(real)c.cb), sk, mlp, tma, fl, row0);
+    });
     return cudaGetLastError();
 }
 

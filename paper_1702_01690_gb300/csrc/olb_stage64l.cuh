@@ -49,11 +49,11 @@ __device__ __forceinline__ double glap_sum64(const double *v, int sl, int sm)
 }
 template <typename real>
 __global__ void __launch_bounds__(2 * FORCE_THREADS) k_force_learned(StageFields<real> f, const __grid_constant__ Geo g,
-                                                                     real cc)
+                                                                     real cc, int row0)
 {
     constexpr int HX = FORCE_X + 6, HY = FORCE_Y + 6;
     __shared__ double dp[HY][HX], n[HY][HX];
-    const int x0 = blockIdx.x * FORCE_X, y0 = blockIdx.y * FORCE_Y;
+    const int x0 = blockIdx.x * FORCE_X, y0 = (row0 + blockIdx.y) * FORCE_Y;
     for (int e = threadIdx.x; e < HY * HX; e += 2 * FORCE_THREADS) {
         const int r = e / HX, x = e - r * HX;
         const long long o = (long long)field_index(y0 - 3 + r, g.ny, g.spec_y) * g.pitch + field_index(x0 - 3 + x, g.nx, g.walls);

@@ -121,3 +121,26 @@ def test_largest_densities(olb, nx, ny, shift):
     f = _populations(olb, p, _noisy(p))
     one, other = _stepped(olb, p, f, 1), _stepped(olb, p, np.ldexp(f, shift), 1)
     assert np.array_equal(np.ldexp(other, -shift), one)
+
+
+@pytest.mark.parametrize("precision,learned", [(0, False), (1, False), (0, True), (1, True)])
+def test_grids_of_more_rows_than_a_launch_has(olb, precision, learned):
+    """65537 tiles along y; the shape (32, 16, 1) has always taken them.  Uniform along y: the moments of eight rows."""
+    from paper_1702_01690_gb300 import learned as weights
+    out = []
+    for ny in (8, 8 * 65535 + 11):
+        ds = 1.0 / 64
+        p = inputs.RunParams(nx=5, ny=ny, ds=ds, dt=inputs.stable_dt(ds), tau=5e-3, Tw=(0.9, 0.9))
+        row = 1.5 + 0.1 * np.sin(2 * np.pi * np.arange(5) / 5)
+        n = np.ascontiguousarray(np.broadcast_to(row, (ny, 5)))
+        ctx = olb.create(p, precision, weno_mode=olb.WENO_LEARNED if learned else olb.WENO_JS)
+        ctx.set_tile(32, 16, 1)
+        if learned:
+            ctx.set_weno_mlp(weights.load_theta())
+        ctx.init_fields(n, 0 * n + 0.05, 0 * n - 0.02, 0 * n + 0.9)
+        assert ctx.step(1) == 0
+        out.append(ctx.moments())
+        ctx.close()
+    for small, tall in zip(*out):
+        assert np.max(np.abs(tall - small[:1])) <= 1e-6 * np.max(np.abs(small))
+        assert precision or learned or np.array_equal(tall, np.broadcast_to(small[:1], tall.shape))
