@@ -367,8 +367,9 @@ __device__ __forceinline__ void eq_correction(const Tab<float> &t, const float E
 // of 2^-57 of the binade above the largest, so that the 48 additions (and the
 // differences that the momentum needs, exactly) run on the integer pipe; an FP64
 // addition takes the time of 64 FP32 or 32 integer instructions on a GB300.  A
-// population below 2^-4 of the largest is cut at 2^-57 of it, against 2^-54 that
-// one FP64 addition rounds away.  Measured on
+// population below 2^-4 of the largest is rounded to 2^-57 of it, against 2^-54 that
+// one FP64 addition rounds away (to nearest: cut towards zero, the sums of a fluid near
+// equilibrium were 2^-55 of n short on average).  Measured on
 // 2048^2: the FP64 moments kernel 0.666 -> 0.384 ms, 0.276 with the sums converted to
 // FP64 on the integer pipe too (fixed_value); one FP64 step of 4096^2
 // with its initial fields and moments 46.5 -> 40.2 -> 38.7 ms.
@@ -382,23 +383,29 @@ struct NodeSums {
 // The larger of |a| and |b| as high words.
 __device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
 
-// v in units of 2^-57 of 2^(top's exponent + 1), cut towards zero
+// m, less than 2^63, in units of 64 times 2^s, rounded to nearest (ties to even; what lies
+// below 2^-6 of a unit is cut)
+__device__ __forceinline__ long long fixed_rounded(unsigned long long m, int s)
+{
+    const unsigned long long t = m >> (s < 63 ? s : 63);
+    return (long long)((t + (31 + ((unsigned)t >> 6 & 1u))) >> 6);
+}
+
+// v in units of 2^-57 of 2^(top's exponent + 1)
 __device__ __forceinline__ long long to_fixed(double v, int top)
 {
     const int hw = __double2hiint(v);
     const unsigned long long m =
-        ((unsigned long long)(unsigned)((hw & 0x000fffff) | 0x00100000) << 32 | (unsigned)__double2loint(v)) << 4;
-    const int s = (top >> 20) - ((hw >> 20) & 0x7ff);
-    const long long q = (long long)(m >> (s < 63 ? s : 63));
+        ((unsigned long long)(unsigned)((hw & 0x000fffff) | 0x00100000) << 32 | (unsigned)__double2loint(v)) << 10;
+    const long long q = fixed_rounded(m, (top >> 20) - ((hw >> 20) & 0x7ff));
     return hw < 0 ? -q : q;
 }
 // the same for a pair of floats (FP32 storage); |lo| is at most an ulp of hi
 __device__ __forceinline__ long long to_fixed(float v, int top)
 {
     const int b = __float_as_int(v);
-    const unsigned long long m = (unsigned long long)((b & 0x007fffff) | 0x00800000) << 33;
-    const int s = (top >> 23) - ((b >> 23) & 0xff);
-    const long long q = (long long)(m >> (s < 63 ? s : 63));
+    const unsigned long long m = (unsigned long long)((b & 0x007fffff) | 0x00800000) << 39;
+    const long long q = fixed_rounded(m, (top >> 23) - ((b >> 23) & 0xff));
     return b < 0 ? -q : q;
 }
 
