@@ -264,9 +264,10 @@ int olb_batch_get_populations(olb_batch *b, int run, double *f);
 int olb_batch_set_tile(olb_batch *b, int tx, int ty, int kp);
 int olb_batch_get_tile(olb_batch *b, int *tx, int *ty, int *kp);
 
-/* Autotuner: times nsteps steps with the compiled shape (on a copy of the
- * state, which is restored), keeps it and reports it; the choice is
- * cached per process for the batch's precision, device and grid list. */
+/* Autotuner: sets the shape (8,8,5), by whose kernels every batch is advanced
+ * whatever its shape, and reports it (any pointer may be NULL).  The
+ * populations stay as they are; nsteps >= 1 is not used.  All runs must be
+ * initialised. */
 int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, int *kp);
 
 /* Mean device time (ms) of one stage launch over nsteps individually

@@ -12,10 +12,7 @@
 #include <cmath>
 #include <algorithm>
 #include <cstring>
-#include <map>
-#include <mutex>
 #include <new>
-#include <string>
 #include <vector>
 
 #include "../../include/olb.h"
@@ -25,10 +22,6 @@ using namespace olb;
 
 namespace {
 constexpr int BATCH_GRAPH_STEPS = 16;
-
-// Process-wide autotune results: batch signature -> shape index.
-std::mutex g_tune_lock;
-std::map<std::string, int> g_tune_cache;
 }  // namespace
 
 struct olb_batch {
@@ -51,7 +44,7 @@ struct olb_batch {
     void *fields = nullptr;              // stage fields of every run (moments pre-pass)
     std::vector<long long> foff;         // byte offset of each run's fields
     long long *node_start = nullptr;     // [count + 1] prefix sum of the runs' node counts
-    int *force_start = nullptr;          // [count + 1] prefix sum of the runs' force blocks (FP64)
+    int *force_start = nullptr;          // [count + 1] prefix sum of the runs' force blocks
     int total_force = 0;
     long long total_nodes = 0;
     long long max_nodes = 0;
@@ -496,62 +489,13 @@ extern "C" int olb_batch_profile(olb_batch *b, int nsteps, double *ms)
     return batch_time(b, nsteps, ms);
 }
 
+// Nothing is left to choose: every shape is advanced by the same kernels.
 extern "C" int olb_batch_autotune(olb_batch *b, int nsteps, int *tx, int *ty, int *kp)
 {
     if (!b || nsteps < 1) return OLB_ERR_ARG;
     for (int r = 0; r < b->count; ++r)
         if (!b->init[r]) return OLB_ERR_STATE;
-    BDevice dg(b->device);
-    std::string sig = std::to_string(b->precision) + ":" + std::to_string(b->device);
-    for (int r = 0; r < b->count; ++r)
-        sig += ";" + std::to_string(b->geo[r].nx) + "x" + std::to_string(b->geo[r].ny) + (b->geo[r].walls ? "w" : "p") +
-               std::to_string(b->geo[r].wall_lo * 8 + b->geo[r].wall_hi * 4 + b->geo[r].spec_lo * 2 + b->geo[r].spec_hi) +
-               (b->geo[r].spec_y ? "s" : "");
-    int best = -1;
-    {
-        std::lock_guard<std::mutex> guard(g_tune_lock);
-        auto it = g_tune_cache.find(sig);
-        if (it != g_tune_cache.end()) best = it->second;
-    }
-    if (best < 0) {
-        // time every shape on a copy of the state, then put the state back
-        const size_t bytes = (size_t)b->total_elems * b->elt;
-        void *backup = nullptr;
-        cudaError_t e = cudaMallocAsync(&backup, bytes, b->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(backup, b->f[0], bytes, cudaMemcpyDeviceToDevice, b->stream);
-        if (e != cudaSuccess) return cuda_status(e);
-        double best_ms = 1e300;
-        const int otx = b->tx, oty = b->ty, okp = b->kp;
-        for (int q = 0; q < NUM_TILES; ++q) {
-            b->tx = TILE_X[q];
-            b->ty = TILE_Y[q];
-            b->kp = TILE_K[q];
-            if (b->tx != STAGE_TX || b->ty != STAGE_TY || b->kp != 5) continue;  // all are advanced alike
-            if (batch_prepare(b) != cudaSuccess) {
-                cudaGetLastError();
-                continue;  // shape does not fit this precision
-            }
-            double ms = 0.0;
-            int rc = batch_upload(b) == cudaSuccess ? OLB_OK : OLB_ERR_CUDA;
-            if (rc == OLB_OK) rc = batch_time(b, 1, &ms);  // warm-up
-            if (rc == OLB_OK) rc = batch_time(b, nsteps, &ms);
-            cudaMemcpyAsync(b->f[0], backup, bytes, cudaMemcpyDeviceToDevice, b->stream);
-            if (rc == OLB_OK && ms < best_ms) {
-                best_ms = ms;
-                best = q;
-            }
-        }
-        cudaMemsetAsync(b->status, 0, (size_t)b->count * sizeof(int), b->stream);
-        cudaFreeAsync(backup, b->stream);
-        cudaStreamSynchronize(b->stream);
-        b->tx = otx;
-        b->ty = oty;
-        b->kp = okp;
-        if (best < 0) return OLB_ERR_CUDA;
-        std::lock_guard<std::mutex> guard(g_tune_lock);
-        g_tune_cache[sig] = best;
-    }
-    const int rc = olb_batch_set_tile(b, TILE_X[best], TILE_Y[best], TILE_K[best]);
+    const int rc = olb_batch_set_tile(b, STAGE_TX, STAGE_TY, 5);
     if (rc != OLB_OK) return rc;
     if (tx) *tx = b->tx;
     if (ty) *ty = b->ty;
