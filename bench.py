@@ -10,10 +10,11 @@ GPU, each with its own stage time and roofline fraction:
   learned_fp64  learned WENO weights (network in FP32, populations FP64)
   learned_fp32  learned WENO weights with the FP32 path
   batch_fp64/32 64 independent runs of uneven size (32^2 .. 1024^2, 13.5 M
-                nodes) in one launch per stage, autotuned shape
+                nodes), each kernel of a stage in one launch for all
 A "step" is one full RK-3 step of the whole grid: three stages, each the
 moments kernel, the force kernel and the stage kernel (WENO-5 fluxes, collision
-and RK combination), nine launches in all.
+and RK combination), nine launches in all; grids of at most one tile of 8 x 8
+nodes an SM take one launch a stage, three in all.
 
 Timing: W untimed warm-up steps, then K steps each bracketed by CUDA events
 on the context's stream, with a 256 MiB buffer written between steps (the
@@ -67,15 +68,15 @@ MLP_FLOPS = 2 * (5 * 32 + 32 * 32 + 32 * 3)
 # (50), stages 2 and 3 read f^n and f_s and write (75 each): 200 per step,
 # 8 bytes each in both paths (FP32 stores hi + lo pairs).
 VALUES_PER_NODE_STEP = 200
-# DRAM bytes (read + write) per launch of the stage kernel from one ncu capture of
-# this kernel build, on the Laplace 2048^2 grid (4.19 M nodes; the 4096^2
-# grid is too large to capture), scaled by 4 to the 16.8 M nodes of the
-# 4096^2 grid (traffic grows with the node count).  Any other kernel or
-# workload reports null.
-DRAM_TRAFFIC_PER_LAUNCH = {
-    # 2048^2, stages 1, 2, 3: 1.850, 2.700, 2.689 GB (FP64) and 1.817, 2.667, 2.655 GB (FP32); mean x 4
-    ("phase", None, "k_fused<double>"): 4 * (1.850 + 2.700 + 2.689) / 3 * 1e9,
-    ("phase", None, "k_fused<float>"): 4 * (1.817 + 2.667 + 2.655) / 3 * 1e9,
+# DRAM bytes (read + write) of the three kernels of a stage from one ncu capture on
+# the Laplace 2048^2 grid (4.19 M nodes; the 4096^2 grid is too large to capture),
+# scaled by 4 to the 16.8 M nodes of the 4096^2 grid (traffic grows with the node
+# count).  Any other workload reports null.
+DRAM_TRAFFIC_PER_STAGE = {
+    # 2048^2: moments and force kernels 0.989 + 0.096 GB (FP64) and 0.993 + 0.078 GB (FP32); stage kernel of stages
+    # 1, 2, 3 1.850, 2.700, 2.689 GB (FP64) and 1.817, 2.667, 2.655 GB (FP32), the mean
+    ("phase", None, "double"): 4 * (0.989 + 0.096 + (1.850 + 2.700 + 2.689) / 3) * 1e9,
+    ("phase", None, "float"): 4 * (0.993 + 0.078 + (1.817 + 2.667 + 2.655) / 3) * 1e9,
 }
 
 
@@ -95,6 +96,25 @@ def alu_peaks(device_index: int = 0):
     sms = torch.cuda.get_device_properties(device_index).multi_processor_count
     mhz = float(load_peaks().get("sm_max_mhz", 2070.0))
     return (sms * 2 * 2 * mhz * 1e6 / 1e12, sms * 128 * 2 * mhz * 1e6 / 1e12, sms, mhz)
+
+
+def stage_roofline(what, nodes, stage_ms, flops, alu_peak):
+    """Of an average stage: its algorithmic bytes against the measured copy rate, and beside them its algorithmic flops
+    (counted once; in FP64 most are taken in float-float arithmetic, several FP32 operations each) against the peak of
+    the FP64 or FP32 units.  No unit is full: the kernels are bound by instruction issue and latency."""
+    measured = load_peaks().get("hbm_gbs")
+    peak = float(measured or 6800.0)
+    nbytes = VALUES_PER_NODE_STEP * 8 * nodes / 3
+    gbs, tflops = nbytes / (stage_ms * 1e-3) / 1e9, flops / (stage_ms * 1e-3) / 1e12
+    return {"kernel": what, "bound": "instruction issue and latency", "achieved": gbs, "peak": peak, "unit": "GB/s",
+            "frac": gbs / peak, "peak_source": "measured copy rate" if measured else "copy rate measured once before",
+            "algorithmic_bytes_per_stage": nbytes, "stage_ms": stage_ms,
+            "alu": {"achieved": tflops, "unit_peak": alu_peak, "unit": "TFLOP/s", "algorithmic_flops_per_stage": flops}}
+
+
+def launches_per_step(p, sms):
+    """Launches of a step: three kernels a stage, one on grids of at most one tile of 8 x 8 nodes an SM."""
+    return 3 if -(-p.nx // 8) * -(-p.ny // 8) <= sms else 9
 
 
 def workload(name, size=None):
@@ -361,14 +381,11 @@ def timed_leg(olb, p, dev_fields, prec, steps, warmup, flush, stream, world, pea
     flops = STAGE_FLOPS_PER_NODE * N
     if mlp_acts is not None:
         flops += mlp_acts * MLP_FLOPS
-    ach = flops / (stage_ms * 1e-3) / 1e12
     kind = "double" if prec == olb.FP64 else "float"
-    kname = f"k_fused<{kind}{',learned' if weno else ''}>"
-    prof = ctx.profile(3)
-    leg = {"value": job_value(world, N, steps, total), "ms_per_step": ms_step,
-           "roofline": {"kernel": kname, "bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                        "frac": ach / peak, "algorithmic_flops_per_launch": flops, "stage_ms": stage_ms,
-                        "stage_ms_single_launches": prof["stage_ms"]}}
+    roof = stage_roofline(f"stage<{kind}{',learned' if weno else ''}>: k_fields + k_force + k_fused", N, stage_ms, flops,
+                          peak)
+    roof["stage_ms_single_launches"] = ctx.profile(3)["stage_ms"]
+    leg = {"value": job_value(world, N, steps, total), "ms_per_step": ms_step, "roofline": roof}
     return leg, ctx
 
 
@@ -394,12 +411,8 @@ def run_ours(args, rank, world):
     legs_run += 1
     value, ms_step = fp64["value"], fp64["ms_per_step"]
     roof = dict(fp64["roofline"])
-    kname = roof["kernel"]
-    roof["traffic"] = DRAM_TRAFFIC_PER_LAUNCH.get((args.workload, args.size, kname))
-    roof["peak_source"] = (f"FP64 units x max SM clock: 2 DFMA/SM/clk x {sms} SMs x {mhz:.0f} MHz x 2 flop "
-                           f"(no FP64 entry in MEASURED_PEAKS.json)")
-    roof["note"] = ("flops of the equations, counted once; the kernel takes most of them in float-float arithmetic on the "
-                    "FP32 pipe (several FP32 operations each), so the FP64 peak does not bound it")
+    roof["traffic"] = DRAM_TRAFFIC_PER_STAGE.get((args.workload, args.size, "double"))
+    roof["alu"]["peak_source"] = f"FP64 units x max SM clock: 2 DFMA/SM/clk x {sms} SMs x {mhz:.0f} MHz x 2 flop"
     # mass and energy from the GPU's FP64 reduction after the timed steps
     # (the context is then at step warmup + steps + 3 profiled steps)
     tot_after = ctx.totals()
@@ -412,8 +425,8 @@ def run_ours(args, rank, world):
     # ---- FP32 compensated
     fp32, c32 = timed_leg(olb, p, dev_fields, olb.FP32_KAHAN, args.steps, args.warmup, flush, stream, world, peak32)
     fp32["speedup_vs_fp64"] = fp32["value"] / value
-    fp32["roofline"]["peak_source"] = f"FP32 lanes x max SM clock: 128/SM x {sms} SMs x {mhz:.0f} MHz x 2 flop"
-    fp32["roofline"]["traffic"] = DRAM_TRAFFIC_PER_LAUNCH.get((args.workload, args.size, fp32["roofline"]["kernel"]))
+    fp32["roofline"]["alu"]["peak_source"] = f"FP32 lanes x max SM clock: 128/SM x {sms} SMs x {mhz:.0f} MHz x 2 flop"
+    fp32["roofline"]["traffic"] = DRAM_TRAFFIC_PER_STAGE.get((args.workload, args.size, "float"))
     c32.close()
     del c32
     torch.cuda.empty_cache()
@@ -476,7 +489,7 @@ def run_ours(args, rank, world):
             "totals_fp64_gpu": {"mass_initial": tot0[0], "energy_initial": tot0[3],
                                 "mass_after_timed_steps": tot_after[0], "energy_after_timed_steps": tot_after[3],
                                 "mass_rel_change": float((tot_after[0] - tot0[0]) / tot0[0])},
-            "gpu_launches": 9 * args.steps, "clocks": clk.summary()}
+            "gpu_launches": launches_per_step(p, sms) * args.steps, "clocks": clk.summary()}
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         line.update(oracle_leg(args, p, fields, dev_fields, theta, stream))
     if rank == 0:
@@ -543,9 +556,8 @@ def oracle_leg(args, p, fields, dev_fields, theta, stream):
 def run_batch_legs(args, world, stream, peak64, peak32):
     """64 independent runs of uneven sizes (32^2 .. 1024^2 shear and
     longitudinal waves, Laplace drops, planar wall runs; 13.5 M nodes) in one
-    launch per stage (one CTA per tile of every run), replayed from CUDA
-    graphs, shape autotuned.  The working set (3 x 25 x 13.5 M values) is far
-    larger than L2."""
+    launch per kernel of a stage, replayed from CUDA graphs.  The working set
+    (3 x 25 x 13.5 M values) is far larger than L2."""
     import torch
     from paper_1702_01690_gb300 import inputs, olb
     runs = inputs.batch_sweep()
@@ -555,7 +567,6 @@ def run_batch_legs(args, world, stream, peak64, peak32):
         b = olb.Batch([p for p, _ in runs], prec, stream)
         for r, (p, fl) in enumerate(runs):
             b.init_fields(r, *fl)
-        shape = b.autotune(2)
         b.step(args.warmup)
         torch.cuda.synchronize()
         rank_barrier()
@@ -570,11 +581,9 @@ def run_batch_legs(args, world, stream, peak64, peak32):
         if rc != 0:
             raise RuntimeError(f"batch diverged ({name})")
         stage_ms = ms / args.steps / 3.0
-        ach = STAGE_FLOPS_PER_NODE * nodes / (stage_ms * 1e-3) / 1e12
         out[name] = {"value": job_value(world, nodes, args.steps, ms), "ms_per_step": ms / args.steps,
-                     "runs": len(runs), "nodes": nodes, "shape": list(shape),
-                     "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                                  "frac": ach / peak, "stage_ms": stage_ms}}
+                     "runs": len(runs), "nodes": nodes,
+                     "roofline": stage_roofline("stage of a batch", nodes, stage_ms, STAGE_FLOPS_PER_NODE * nodes, peak)}
         b.close()
         del b
         torch.cuda.empty_cache()
