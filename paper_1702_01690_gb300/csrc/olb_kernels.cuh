@@ -366,13 +366,14 @@ __device__ __forceinline__ void eq_correction(const Tab<float> &t, const float E
 // Sums over the 25 populations of a node in fixed point: 64-bit integers in units
 // of 2^-57 of the binade above the largest, so that the 48 additions (and the
 // differences that the momentum needs, exactly) run on the integer pipe; an FP64
-// addition takes the time of 64 FP32 or 32 integer instructions on a GB300.  A
-// population below 2^-4 of the largest is rounded to 2^-57 of it, against 2^-54 that
-// one FP64 addition rounds away (to nearest: cut towards zero, the sums of a fluid near
-// equilibrium were 2^-55 of n short on average).  Measured on
-// 2048^2: the FP64 moments kernel 0.666 -> 0.384 ms, 0.276 with the sums converted to
-// FP64 on the integer pipe too (fixed_value); one FP64 step of 4096^2
-// with its initial fields and moments 46.5 -> 40.2 -> 38.7 ms.
+// addition takes the time of 64 FP32 or 32 integer instructions on a GB300.  The sums
+// of a row or column have three more bits, to which populations below 2^-7 of the
+// largest are cut, and are then rounded, against 2^-54 that one FP64 addition rounds
+// away.  (Populations cut to whole units left the sums of a fluid near equilibrium 2^-55
+// of n short on average; rounded one by one they cost a stage of one launch 0.2 us.)
+// Measured on 2048^2: the FP64 moments kernel 0.666 -> 0.384 ms, 0.28 with the sums
+// converted to FP64 on the integer pipe too (fixed_value); one FP64 step of 4096^2 with
+// its initial fields and moments 46.5 -> 40.2 -> 38.7 ms.
 //
 // The sums that n, j and e = sum |p|^2 f are made of: n, sums and differences of
 // the rows and columns of velocity +-R_4 and +-R_3 (the middle root is 0).
@@ -383,29 +384,23 @@ struct NodeSums {
 // The larger of |a| and |b| as high words.
 __device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
 
-// m, less than 2^63, in units of 64 times 2^s, rounded to nearest (ties to even; what lies
-// below 2^-6 of a unit is cut)
-__device__ __forceinline__ long long fixed_rounded(unsigned long long m, int s)
-{
-    const unsigned long long t = m >> (s < 63 ? s : 63);
-    return (long long)((t + (31 + ((unsigned)t >> 6 & 1u))) >> 6);
-}
-
-// v in units of 2^-57 of 2^(top's exponent + 1)
+// v in units of 2^-60 of 2^(top's exponent + 1), cut towards zero
 __device__ __forceinline__ long long to_fixed(double v, int top)
 {
     const int hw = __double2hiint(v);
     const unsigned long long m =
-        ((unsigned long long)(unsigned)((hw & 0x000fffff) | 0x00100000) << 32 | (unsigned)__double2loint(v)) << 10;
-    const long long q = fixed_rounded(m, (top >> 20) - ((hw >> 20) & 0x7ff));
+        ((unsigned long long)(unsigned)((hw & 0x000fffff) | 0x00100000) << 32 | (unsigned)__double2loint(v)) << 7;
+    const int s = (top >> 20) - ((hw >> 20) & 0x7ff);
+    const long long q = (long long)(m >> (s < 63 ? s : 63));
     return hw < 0 ? -q : q;
 }
 // the same for a pair of floats (FP32 storage); |lo| is at most an ulp of hi
 __device__ __forceinline__ long long to_fixed(float v, int top)
 {
     const int b = __float_as_int(v);
-    const unsigned long long m = (unsigned long long)((b & 0x007fffff) | 0x00800000) << 39;
-    const long long q = fixed_rounded(m, (top >> 23) - ((b >> 23) & 0xff));
+    const unsigned long long m = (unsigned long long)((b & 0x007fffff) | 0x00800000) << 36;
+    const int s = (top >> 23) - ((b >> 23) & 0xff);
+    const long long q = (long long)(m >> (s < 63 ? s : 63));
     return b < 0 ? -q : q;
 }
 
@@ -441,7 +436,8 @@ __device__ __forceinline__ double fixed_value(long long v, int unit)
     return m == 0 ? 0.0 : __hiloint2double((int)(v < 0 ? hw | 0x80000000u : hw), (int)(unsigned)b);
 }
 
-// fixed(k): population k as a 64-bit integer in units of 2^(unit - 1023).
+// fixed(k): population k as a 64-bit integer in units of 2^-3 of 2^(unit - 1023), of which
+// the sums of five have room; they are rounded to whole units.
 template <typename Fixed>
 __device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, int unit)
 {
@@ -456,6 +452,11 @@ __device__ __forceinline__ NodeSums fixed_sums(Fixed fixed, int unit)
             sx[k1] += v;
             sy[k2] += v;
         }
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) {
+        sx[k] = (sx[k] + 4) >> 3;
+        sy[k] = (sy[k] + 4) >> 3;
+    }
     auto val = [&](long long v) { return fixed_value(v, unit); };
     return {val(sx[0] + sx[1] + sx[2] + sx[3] + sx[4]), val(sx[4] - sx[0]), val(sx[3] - sx[1]), val(sy[4] - sy[0]),
             val(sy[3] - sy[1]), val(sx[4] + sx[0] + sy[4] + sy[0]), val(sx[3] + sx[1] + sy[3] + sy[1])};
