@@ -37,6 +37,7 @@ struct NodeMoments;
 template <>
 struct NodeMoments<double> {
     double n, dp, ux, uy, T;
+    int top;  // high word of the largest |population|, 0 if it is not finite (without SEQ)
     bool ok;
 };
 template <>
@@ -84,6 +85,7 @@ __device__ __forceinline__ NodeMoments<real> node_moments(Get get, const Geo &g,
             }
         } else {
             const NodeSums s = node_sums64(get);
+            m.top = finite_hi(s.top);
             n = s.n;
             jx = fma(t.R[4], s.a4x, t.R[3] * s.a3x);
             jy = fma(t.R[4], s.a4y, t.R[3] * s.a3y);
@@ -442,8 +444,7 @@ __device__ __forceinline__ void force_block(ForceSmem<FORCE_X, FORCE_Y> &sm, con
         const double n = f.n[o];
         sm.v[0][r][x] = f.dp[o];
         sm.v[1][r][x] = n;
-        const int a = __double2hiint(n) & 0x7fffffff;
-        top = max(top, a < 0x7ff00000 ? a : 0);
+        top = max(top, finite_hi(abs_hi(n)));
     }
     top = __reduce_max_sync(0xffffffffu, top);
     if ((tid & 31) == 0) atomicMax(&sm.top, top);
@@ -598,13 +599,14 @@ struct TileFields<float> {
 };
 constexpr int OWN_THREADS = 7 * 32;  // 14 x 14 nodes, one a thread
 // Threads 0 .. OWN_THREADS - 1, whole warps: the moments of a node (those of k_fields,
-// from the nodes that k_force's blocks take), the status of the tile's own nodes.
+// from the nodes that k_force's blocks take), the status of the tile's own nodes; FP64
+// the largest population (*top) and density (own.force.top) of the 14 x 14 nodes.
 template <typename real>
 __device__ __forceinline__ void tile_moments(TileFields<real> &own, int *top, const real *__restrict__ fs, int *status,
                                              const Geo &g, const Tab<real> &t, int x0, int y0)
 {
     const int tid = threadIdx.x, r = tid / 14, x = tid - 14 * r;
-    int a = 0;
+    int a = 0, an = 0;
     if (r < 14) {
         const real *f = fs + (long long)field_index(y0 - 3 + r, g.ny, g.spec_y) * g.pitch + field_index(x0 - 3 + x, g.nx, g.walls);
         NodeMoments<real> m;
@@ -614,7 +616,8 @@ __device__ __forceinline__ void tile_moments(TileFields<real> &own, int *top, co
             m = node_moments<real>([&](int k) { return __ldg(f + k * g.plane); }, g, t);
             own.force.v[0][r][x] = m.dp;
             own.force.v[1][r][x] = m.n;
-            a = __double2hiint(m.n) & 0x7fffffff;
+            a = m.top;
+            an = finite_hi(abs_hi(m.n));
         } else {
             m = node_moments<real>([&](int k) { return make_float2(__ldg(f + k * g.plane), __ldg(f + (NK + k) * g.plane)); },
                                    g, t);
@@ -630,8 +633,12 @@ __device__ __forceinline__ void tile_moments(TileFields<real> &own, int *top, co
         }
     }
     if constexpr (sizeof(real) == 8) {
-        a = __reduce_max_sync(0xffffffffu, a < 0x7ff00000 ? a : 0);
-        if ((tid & 31) == 0) atomicMax(top, a);
+        a = __reduce_max_sync(0xffffffffu, a);
+        an = __reduce_max_sync(0xffffffffu, an);
+        if ((tid & 31) == 0) {
+            atomicMax(top, a);
+            atomicMax(&own.force.top, an);
+        }
     }
 }
 

@@ -379,10 +379,12 @@ __device__ __forceinline__ void eq_correction(const Tab<float> &t, const float E
 // the rows and columns of velocity +-R_4 and +-R_3 (the middle root is 0).
 struct NodeSums {
     double n, a4x, a3x, a4y, a3y, s4, s3;
+    int top;  // high word of the largest |population| (node_sums64)
 };
 
-// The larger of |a| and |b| as high words.
+// |v| as its high word; 0 for infinities and NaN.
 __device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ int finite_hi(int a) { return a < 0x7ff00000 ? a : 0; }
 
 // v in units of 2^-60 of 2^(top's exponent + 1), cut towards zero
 __device__ __forceinline__ long long to_fixed(double v, int top)
@@ -471,9 +473,12 @@ __device__ __forceinline__ NodeSums node_sums64(Get get)
     int top = 0;
 #pragma unroll
     for (int k = 0; k < NK; ++k) top = max(top, abs_hi(get(k)));
-    if (top >= (2047 << 20) || top < (128 << 20)) return plain_sums(get);
-    // 2^(e - 56), e the exponent of the largest
-    return fixed_sums([&](int k) { return to_fixed(get(k), top); }, (top >> 20) - 56);
+    // (units of 2^(e - 56), e the exponent of the largest)
+    NodeSums s = top >= (2047 << 20) || top < (128 << 20)
+                     ? plain_sums(get)
+                     : fixed_sums([&](int k) { return to_fixed(get(k), top); }, (top >> 20) - 56);
+    s.top = top;
+    return s;
 }
 template <typename Get>
 __device__ __forceinline__ NodeSums node_sums32(Get get)

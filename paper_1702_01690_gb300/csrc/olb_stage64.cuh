@@ -81,7 +81,7 @@ struct Smem64 : Staged<double> {
     ffp ax[20][TY / 2][TX + 1];
     ffp ay[20][TX * (TY / 2 + 1) + 1];
     ffp rest[NN / 2];
-    int top;            // high word of the largest n of the tile (its scale), or of the largest population
+    int top;            // high word of the largest n of the tile (its scale) or of the largest population
 
     __device__ __forceinline__ ffp &col(int q, int x, int i) { return ay[q][5 * x + (i & 3)]; }
     // top is at least the largest finite staged population, wall ghosts included (all threads)
@@ -189,7 +189,10 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
         fT = fields.T[o];
         fG = (a == 0 ? fields.G[0] : fields.G[1])[o];
     }
-    if (tid == 0) sm.top = 0;
+    if (tid == 0) {
+        sm.top = 0;
+        if (OWN) own->force.top = 0;
+    }
     const bool inside = tmap != nullptr && x0 >= 4 && x0 + TX + 4 <= g.nx && y0 >= 3 && y0 + TY + 3 <= g.ny;
     if (inside) tma_issue(sm, tmap, x0, y0);
     if constexpr (OWN) {
@@ -197,7 +200,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
         if (tid < OWN_THREADS) tile_moments(*own, &sm.top, fs, status, g, t, x0, y0);
         else if (!inside) load_region(sm, fs, g, x0, y0, OWN_THREADS);
         __syncthreads();
-        force_differences<NT>(own->force, ff_scale(sm.top));
+        force_differences<NT>(own->force, ff_scale(own->force.top));
         if (has) {
             fn_ = own->force.v[1][ny + 3][nx + 3];
             fu = a == 0 ? own->ux[node] : own->uy[node];
@@ -208,7 +211,8 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
     }
     __syncthreads();
 
-    // ---- 2. equilibrium factors (FP64), the tile's scale (its largest density)
+    // ---- 2. equilibrium factors (FP64), the tile's scale (its largest density; OWN: the
+    // largest population that the lines read, which costs nothing there)
     if (tid < 2 * NN) {
         double w[NQ];
         eq_factors64(t, fu, fT, w);
@@ -222,7 +226,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
             if ((tid & 31) == 0) atomicMax(&sm.top, top);
         }
     } else if (OWN && tid < 4 * NN) {
-        const ffv<vf1> v = force_at<vf1>(own->force, ff_scale(sm.top), c, a - 2, nx, ny);
+        const ffv<vf1> v = force_at<vf1>(own->force, ff_scale(own->force.top), c, a - 2, nx, ny);
         sm.G[a - 2][8 * (ny & 3) + nx].put(ny >> 2, v);
     }
     // ---- 3. diffuse walls: fluxes and ghosts of the tile rows
@@ -230,15 +234,15 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
     if (left || right) {
         wall_flux<double, false>(sm, g, t, tw, nullptr, x0, OWN ? 4 * NN : 2 * NN, left, right);
         __syncthreads();
-        wall_ghosts<double>(sm, g, tw, x0, 0, left, right);
+        wall_ghosts<double>(sm, g, tw, x0, 0, left, right, OWN ? &sm.top : nullptr);
     }
     if (inside && !tma_finish(sm, status)) return false;
     __syncthreads();
     FfScale sc = ff_scale(sm.top);
 
-    // ---- 5a. flux differences, W rows or columns a thread; once more with the scale of
-    // the largest population if some were beyond FP32's range (in-range tiles pay one
-    // packed FMA a flux difference for it)
+    // ---- 5a. flux differences, W rows or columns a thread; unless OWN, once more with the
+    // scale of the largest population if some were beyond FP32's range (other tiles pay
+    // one packed FMA a flux difference for it)
     for (bool again = false;; again = true) {
         V sum = V::all(0.0f);  // of 0 times the low parts: not 0 if one is not finite
         for (int e = tid; e < 40 * (TX / W); e += NT) {
@@ -248,7 +252,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
             const bool up = ln.up;
             auto store = [&](int j, ffv<V> v) {
                 const int at = up ? j : TX - 1 - j;
-                sum = vfma(0.0f, v.l, sum);
+                if constexpr (!OWN) sum = vfma(0.0f, v.l, sum);
                 if (along_x) {
                     sm.ax[q][i & 3][at].put(i >> 2, v);
                 } else {
@@ -262,6 +266,10 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
             };
             weno5_line<TX, V>(ln.p0, ln.p1, ln.p2, along_x ? 4 * HP : 4, ln.halo, ln.step, sc, store);
         }
+        if constexpr (OWN) {
+            __syncthreads();
+            break;
+        }
         if (!__syncthreads_or(!(sum[0] == 0.0f && sum[W - 1] == 0.0f)) || again) break;
         const int top = sm.top;
         __syncthreads();
@@ -272,7 +280,7 @@ __device__ __forceinline__ bool stage_tile64(Smem64<KP> &sm, const double *__res
     }
 
     // (once more, not kept: 5a's registers)
-    sc = ff_scale(*(volatile int *)&sm.top);
+    if (!OWN) sc = ff_scale(*(volatile int *)&sm.top);
 
     // f^n of the velocities that this thread advances in 5c, fetched now
     constexpr int LINES = (NQ * NI + NT - 1) / NT;

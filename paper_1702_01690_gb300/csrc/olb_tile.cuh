@@ -302,10 +302,11 @@ __device__ __forceinline__ void wall_flux(S &sm, const Geo &g, const Tab<real> &
 }
 
 // The incoming ghosts of the tile rows at a wall, f^eq_w = n_w g g (Eq.
-// diffuse_flux); items start on thread `first`.
+// diffuse_flux); items start on thread `first`.  top: the high word of the largest staged
+// value, kept up to date, or nullptr.
 template <typename real, typename S>
 __device__ __forceinline__ void wall_ghosts(S &sm, const Geo &g, const Tab<real> &tw, int x0, int first, bool left_wall,
-                                            bool right_wall)
+                                            bool right_wall, int *top = nullptr)
 {
     constexpr int HX = S::HX, TY = S::TY, NT = S::NT;
     const int nin = ((int)left_wall + (int)right_wall) * TY * 30;
@@ -317,7 +318,10 @@ __device__ __forceinline__ void wall_ghosts(S &sm, const Geo &g, const Tab<real>
         const int c = side ? g.nx + m - (x0 - 4) : -1 - m - (x0 - 4);
         if (c < 0 || c >= HX) continue;
         const int k = NQ * (side ? v / 5 : 3 + v / 5) + v % 5;
-        *sm.at(k, tr + 3, c) = sm.wnw[side][tr] * tw.geqw[side][k];
+        const real ghost = sm.wnw[side][tr] * tw.geqw[side][k];
+        *sm.at(k, tr + 3, c) = ghost;
+        if constexpr (sizeof(real) == 8)
+            if (top) atomicMax(top, finite_hi(abs_hi(ghost)));
         if constexpr (sizeof(real) == 4) *sm.at(NK + k, tr + 3, c) = 0.0f;
     }
 }
