@@ -255,7 +255,7 @@ static void ctx_free_all(olb_ctx *c)
 
 static bool is_fp64(const olb_ctx *c) { return c->p.precision == OLB_FP64; }
 
-// One RK-3 step (Eq. rk3) as 3 launches of the fused stage kernel:
+// One RK-3 step (Eq. rk3) as 3 stages (launch_fused):
 //   f1 = f + dt L[f];  f2 = 3/4 f + 1/4 f1 + 1/4 dt L[f1];
 //   f  = 1/3 f + 2/3 f2 + 2/3 dt L[f2]  (written in place: f is read only at
 //   the node being written).

@@ -98,7 +98,8 @@ __host__ __device__ __forceinline__ float rcp_seed(float v)
 // of it) to 2^18 times it, then have squares and weights inside FP32's range
 // whatever the populations' units.  Where they lie beyond (dilute nodes beside dense
 // ones of the next tile) the low parts are not finite, and the stage takes the tile's
-// lines again with the scale of its largest population (stage_tile64).
+// lines again with the scale of its largest population (stage_tile64; grids of one
+// launch a stage have that from the start).
 constexpr int FF_EXP = 127 + 45;  // FP32 exponent field of the largest density
 struct FfScale {
     int off;     // added to an FP64 high word: exponent field e - emax + FF_EXP

@@ -11,8 +11,10 @@
 //                an RK increment far below FP32 resolution of f survives
 //   status       int                     bit 0: invalid moment seen; bit 1: a
 //                                        bounded wait for a TMA copy ran out
-// The stage kernel keeps moments, force and wall densities of its tile in
-// shared memory; no other global scratch is needed.
+//   fields       moments and force of the nodes (StageFields in olb_fields.cuh, 56 or
+//                48 bytes a node), for grids of more tiles than SMs
+// The stage kernel keeps what else it needs of its tile (equilibrium factors, wall
+// densities, flux differences) in shared memory.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -134,11 +136,13 @@ constexpr int STAGE_TX = 8, STAGE_TY = 8;
 inline int stage_tiles(int nx, int ny) { return ((nx + STAGE_TX - 1) / STAGE_TX) * ((ny + STAGE_TY - 1) / STAGE_TY); }
 // The compiled stage that advances so many tiles.  At most one tile an SM, 8: one launch of 512 threads a tile that take the moments and the
 // force of the tile too (of its 14 x 14 nodes, three times the work of k_fields);
-// else 5: three launches.  A stage, three launches and one, FP64: 8 tiles 26.4 and
-// 14.7 us, 128 tiles 27.4 and 15.7, 256 tiles 32.6 and 30.4, 384 tiles 35.1 and 45.0,
-// 4096 tiles 214 and 408; FP32: 13.1 and 7.2, 14.3 and 8.0, 15.7 and 15.0, 17.8 and
-// 21.8, 96 and 188.  Learned weights: at most one tile an SM, 6 (512 threads a tile), else
-// 4 (256, two tiles an SM): 39 tiles 70 and 60 us (FP64), 51 and 38 us (FP32).
+// else 5: three launches.  A stage, three launches and one, FP64: 8 tiles 27.3 and
+// 15.2 us, 128 tiles 27.1 and 15.6, 256 tiles 32.6 and 30.3, 384 tiles 35.5 and 44.9,
+// 4096 tiles 210 and 407; FP32: 13.9 and 7.4, 13.7 and 8.0, 15.8 and 15.1, 18.0 and
+// 21.7, 93 and 188 (the lines cross between two and two and a half tiles an SM; the rule
+// stops at one, up to which one launch is always the faster by far).  Learned weights: at
+// most one tile an SM, 6 (512 threads a tile), else 4 (256, two tiles an SM): 39 tiles
+// 70.8 (4) and 59.6 us (6) in FP64, 42.5 and 37.7 in FP32; 200 tiles 113 and 122, 68 and 72.
 int stage_kind(bool learned, int tiles);
 
 // Shapes that olb_set_tile accepts with learned weights.

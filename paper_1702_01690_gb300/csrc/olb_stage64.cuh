@@ -10,21 +10,27 @@
 // populations along a row, of n and Delta p across a stencil, f^n - f_s,
 // f^eq - f_s) and the sum f_s + Delta; what is done with them runs on the FP32
 // pipe in float-float arithmetic (olb_ff.cuh), whose 2^-46 of Delta is below
-// FP64's rounding of f wherever Delta < f / 128.
+// FP64's rounding of f wherever Delta < f / 128.  Where Delta is larger its errors show;
+// against 80-bit arithmetic, in units of 2.2e-16 of the largest population (FP64 form ->
+// this one): one step of 30 % noise on 32^2 nodes 6.8 -> 2.3, of jumps 0.05 | 1.6 between
+// nodes on 32^2 2.9 -> 3.3 (4 steps 16 -> 5), of a drop's interface of three nodes 7.7
+// -> 16 (8 steps 91 -> 41).  Only where a step's capillary increment is of the size of f,
+// jumps between the nodes of a fine grid (512 x 24), is it the less accurate: 6 -> 105.
 //
 // Measured, one step (three stages) of a 4096^2 grid: 106.6 ms with the force and
 // the node updates in FP64 (1070 FP64 instructions a node and stage beside 60
 // differences), 56.8 ms like this (228), 51.8 ms with three CTAs an SM, 46.5 ms
 // with the force in a kernel of its own (k_force) and two nodes a thread, 38.7 ms
-// with the moments' sums in fixed point (olb_kernels.cuh).
+// with the moments' sums in fixed point (olb_kernels.cuh), 39.1 ms with initial fields
+// and moments output as they are now and tiles checked for values beyond their scale.
 // Against 80-bit arithmetic the populations are closer than the FP64 form's
 // (12 steps of a 167 x 109 drop: 5.7e-16 instead of 1.2e-15 of their norm, and
 // its loss of 1e-15 of the mass is gone): Delta is summed before the one
 // rounding at the size of f.
 //
-// What bounds it now (ncu, 1024^2): no pipe; FP64 57 %, issue slots 50 %, and
-// what three CTAs of five warps leave of latency (tiles hold 70 KB, and two nodes
-// a thread take 125 registers).
+// What bounds it now (ncu, 2048^2): no pipe; FP64 57-59 %, issue slots 55 %, and
+// what three CTAs of five warps leave of latency (three tiles hold 210 of the 228 KB of
+// shared memory, and two nodes a thread take 126 registers: 60 of 64 K).
 #pragma once
 
 #include "olb_tile.cuh"

@@ -117,3 +117,30 @@ def test_what_the_scale_cannot_hold_is_not_finite(lib, low):
                                                 - _face_minus_upwind(v[:, :5])[0][0]))):
             got = _call(fn, w, np.array([low]))[0]
             assert not np.isfinite(got) or abs(got - ref) <= 1e-9, (at, got, ref)
+
+
+def test_parity_form_of_the_momentum_derivative_is_the_matrix():
+    """dp_line (csrc/olb_stage64.cuh) takes (d_p f)_{2 +- m} = (E_m2 a_2 + E_m1 a_1) +- (O_m2 s_2 + O_m1 s_1 + O_m0 f_2)
+    with a_q = f_{2+q} - f_{2-q}, s_q = f_{2+q} + f_{2-q} and E, O from D as fill_tab forms them: D f of Eq. derf,
+    exactly, since D is odd under p -> -p."""
+    sp = pytest.importorskip("sympy")
+    x = sp.Symbol("x")
+    He = [sp.Integer(1), x, x ** 2 - 1, x ** 3 - 3 * x, x ** 4 - 6 * x ** 2 + 3]
+    R = [-sp.sqrt(5 + sp.sqrt(10)), -sp.sqrt(5 - sp.sqrt(10)), sp.Integer(0)]
+    R += [-R[1], -R[0]]
+    W = [(7 - 2 * sp.sqrt(10)) / 60, (7 + 2 * sp.sqrt(10)) / 60, sp.Rational(8, 15)]
+    W += [W[1], W[0]]
+    D = [[-W[k] * sum(He[q + 1].subs(x, R[k]) * He[q].subs(x, R[j]) / sp.factorial(q) for q in range(4))
+          for j in range(5)] for k in range(5)]
+    f = sp.symbols("f0:5")
+    a, s = [None] + [f[2 + q] - f[2 - q] for q in (1, 2)], [f[2]] + [f[2 + q] + f[2 - q] for q in (1, 2)]
+    for m in range(3):
+        d = D[2 + m]
+        E = [None] + [(d[2 + q] - d[2 - q]) / 2 for q in (1, 2)]
+        Od = [d[2]] + [(d[2 + q] + d[2 - q]) / 2 for q in (1, 2)]
+        even, odd = E[2] * a[2] + E[1] * a[1], Od[2] * s[2] + Od[1] * s[1] + Od[0] * s[0]
+        for sign in (1, -1):
+            row = sum(D[2 + sign * m][j] * f[j] for j in range(5))
+            form = even + (sign * odd if m else 0)  # (the middle row has no part O)
+            for j in range(5):
+                assert abs(sp.N(sp.diff(row - form, f[j]), 50)) < sp.Float("1e-45")
